@@ -8,6 +8,7 @@
 #include <mutex>
 
 #include "egs_internal.cuh"
+#include "tc64.cuh"
 
 namespace egs {
 
@@ -83,7 +84,7 @@ static egs_status check_theta(const double *theta)
 }
 
 
-static Layout make_layout(const TileGeom &g)
+static Layout make_layout(const TileGeom &g, bool tc)
 {
     Layout L;
     size_t off = 0;
@@ -103,6 +104,8 @@ static Layout make_layout(const TileGeom &g)
     off += align256(EGS_MT_DOUBLES * sizeof(double));
     L.pctr = off;
     off += align256((size_t)g.T * potrf_diag_scratch_words(g.b) * sizeof(unsigned));
+    L.tc = off;
+    if (tc) off += tc64_scratch_bytes(g.b, g.T);
     L.total = off;
     return L;
 }
@@ -190,7 +193,8 @@ egs_status eval_setup(int64_t n, const double *theta, egs_precision p, const egs
     es->p = p;
     es->g = TileGeom{n, tile, (int)((n + tile - 1) / tile)};
     es->mixed = mixed_p(p) && es->g.T > es->band;
-    es->L = make_layout(es->g);
+    es->tc = !es->mixed && tc64_applies(n, tile, es->g.T);
+    es->L = make_layout(es->g, es->tc);
     es->ML = make_mixed_layout(es->g, es->band, p);
     es->need = es->mixed ? es->ML.total : es->L.total;
     es->locs_off = es->mixed ? es->ML.locs : es->L.locs;
@@ -202,6 +206,15 @@ egs_status eval_setup(int64_t n, const double *theta, egs_precision p, const egs
     es->P.metric = dist;
     es->P.radius = EGS_EARTH_RADIUS_KM;
     return EGS_OK;
+}
+
+bool eval_shrink(EvalSetup *es)
+{
+    if (es->mixed || !es->tc) return false;
+    es->tc = false;
+    es->L = make_layout(es->g, false);
+    es->need = es->L.total;
+    return true;
 }
 
 DevStatus *eval_status(const EvalSetup &es, char *ws) { return (DevStatus *)(ws + (es.mixed ? es.ML.status : es.L.status)); }
@@ -272,7 +285,7 @@ cudaError_t eval_enqueue(const EvalSetup &es, const double *dlocs, const double 
     cudaError_t e = launch_matern_tiles_f64(dlocs, dlocs + n, g, es.P, tiles, s, kt, (double *)(ws + es.L.mtab));
     if (e == cudaSuccess) {
         if (ev) cudaEventRecord(ev[1], s);
-        e = launch_potrf_tiles_f64(tiles, g, st, s, kt, (unsigned *)(ws + es.L.pctr));
+        e = launch_potrf_tiles_f64(tiles, g, st, s, kt, (unsigned *)(ws + es.L.pctr), es.tc ? ws + es.L.tc : nullptr);
     }
     if (e == cudaSuccess) {
         if (ev) cudaEventRecord(ev[2], s);
@@ -371,7 +384,7 @@ size_t egs_loglik_workspace_bytes(int64_t n, int32_t tile, egs_precision p, int3
     if (band <= 0) band = 2;
     if (n < 1 || !tile_ok(tile)) return 0;
     TileGeom g{n, tile, (int)((n + tile - 1) / tile)};
-    if (p == EGS_FP64 || (mixed_p(p) && g.T <= band)) return make_layout(g).total;
+    if (p == EGS_FP64 || (mixed_p(p) && g.T <= band)) return make_layout(g, tc64_applies(n, tile, g.T)).total;
     if (mixed_p(p) && tile % 256 == 0) return make_mixed_layout(g, band, p).total;
     return 0;
 }
@@ -425,11 +438,20 @@ egs_status egs_potrf_tiles(void *tiles, int64_t n, int32_t tile, int64_t *fail_i
     DevStatus *st = nullptr;
     const size_t sbytes = align256(sizeof(DevStatus));
     const Allocator A = current_allocator();
-    const size_t wbytes = sbytes + (size_t)g.T * potrf_diag_scratch_words(g.b) * sizeof(unsigned);
+    const size_t cbytes = align256(sbytes + (size_t)g.T * potrf_diag_scratch_words(g.b) * sizeof(unsigned));
+    bool tc = tc64_applies(n, tile, g.T);
+    size_t wbytes = cbytes + (tc ? tc64_scratch_bytes(g.b, g.T) : 0);
     cudaError_t e = dev_alloc(A, (void **)&st, wbytes, s);
+    if (e == cudaErrorMemoryAllocation && tc) {  // no room for the slices: the DFMA update
+        cudaGetLastError();
+        tc = false;
+        wbytes = cbytes;
+        e = dev_alloc(A, (void **)&st, wbytes, s);
+    }
     if (e != cudaSuccess) return cuda_error(e, "egs_potrf_tiles workspace");
     status_init(st, s);
-    e = launch_potrf_tiles_f64((double *)tiles, g, st, s, nullptr, (unsigned *)((char *)st + sbytes));
+    e = launch_potrf_tiles_f64((double *)tiles, g, st, s, nullptr, (unsigned *)((char *)st + sbytes),
+                               tc ? (char *)st + cbytes : nullptr);
     DevStatus h;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s);
     dev_free(A, st, wbytes, s);
@@ -497,11 +519,16 @@ egs_status egs_loglik_ex(const double *locs, const double *z, const double theta
     cudaError_t e = cudaSuccess;
     const Allocator A = current_allocator();
     if (opts && opts->workspace) {
+        if (opts->workspace_bytes < es.need) eval_shrink(&es);
         if (opts->workspace_bytes < es.need)
             return set_error(EGS_ERR_ARG, "workspace of %zu bytes < %zu needed", opts->workspace_bytes, es.need);
         ws = (char *)opts->workspace;
     } else {
         e = dev_alloc(A, (void **)&ws, es.need, s);
+        if (e == cudaErrorMemoryAllocation && eval_shrink(&es)) {
+            cudaGetLastError();
+            e = dev_alloc(A, (void **)&ws, es.need, s);
+        }
         if (e != cudaSuccess) return cuda_error(e, "egs_loglik workspace");
         own = true;
     }
@@ -575,6 +602,10 @@ egs_status egs_simulate(const double *locs, const double *e, const double theta[
     char *ws = nullptr;
     const Allocator A = current_allocator();
     cudaError_t err = dev_alloc(A, (void **)&ws, es.need, s);
+    if (err == cudaErrorMemoryAllocation && eval_shrink(&es)) {
+        cudaGetLastError();
+        err = dev_alloc(A, (void **)&ws, es.need, s);
+    }
     if (err != cudaSuccess) return cuda_error(err, "egs_simulate workspace");
     double *tiles = (double *)(ws + es.L.tiles);
     double *epad = (double *)(ws + es.L.zpad);
@@ -595,7 +626,9 @@ egs_status egs_simulate(const double *locs, const double *e, const double theta[
         status_init(st, s);
         err = launch_matern_tiles_f64(dlocs, dlocs + n, g, es.P, tiles, s, nullptr, (double *)(ws + es.L.mtab));
     }
-    if (err == cudaSuccess) err = launch_potrf_tiles_f64(tiles, g, st, s, nullptr, (unsigned *)(ws + es.L.pctr));
+    if (err == cudaSuccess)
+        err = launch_potrf_tiles_f64(tiles, g, st, s, nullptr, (unsigned *)(ws + es.L.pctr),
+                                     es.tc ? ws + es.L.tc : nullptr);
     if (err == cudaSuccess) err = launch_pad_vector(de, n, epad, (int64_t)g.T * g.b, s);
     if (err == cudaSuccess) err = launch_trmv_lower(tiles, g, epad, zfull, st, s);
     if (err == cudaSuccess) err = cudaMemcpyAsync(z, zfull, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, s);

@@ -17,6 +17,7 @@
 // Every output element is updated by exactly one thread in a fixed order, so
 // results are bitwise reproducible.
 #include "blocks.cuh"
+#include "tc64.cuh"
 
 namespace egs {
 
@@ -245,12 +246,20 @@ cudaError_t launch_update_f64(const Tiles &tl, int k, int64_t ntri, DevStatus *s
 }
 
 cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *st, cudaStream_t s, KernelTimer *kt,
-                                   unsigned *ctr)
+                                   unsigned *ctr, void *tc_scratch)
 {
     const int T = g.T;
     const Tiles tl{tiles, nullptr, g.b, T, T};
     cudaError_t e0 = cudaMemsetAsync(ctr, 0, (size_t)T * potrf_diag_scratch_words(g.b) * sizeof(unsigned), s);
     if (e0 != cudaSuccess) return e0;
+    F64Scratch sc{};
+    F64Maps maps;
+    if (tc_scratch) {
+        sc = tc64_scratch(tc_scratch, g.b, T);
+        e0 = make_f64_maps(sc.panel, g.b, T, &maps);
+        if (e0 == cudaSuccess) e0 = cudaMemsetAsync(sc.counters, 0, (size_t)T * sizeof(unsigned long long), s);
+        if (e0 != cudaSuccess) return e0;
+    }
     for (int k = 0; k < T; ++k) {
         if (kt) kt->step = k;
         cudaError_t e = launch_potrf_diag(tl, k, st, s, kt, ctr + (size_t)k * potrf_diag_scratch_words(g.b));
@@ -258,7 +267,13 @@ cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *
         if (k + 1 < T) {
             e = launch_trsm_f64(tl, k, T - k - 1, st, s, kt);
             if (e != cudaSuccess) return e;
-            e = launch_update_f64(tl, k, (int64_t)(T - k - 1) * (T - k) / 2, st, s, kt);
+            if (tc_scratch) {
+                e = launch_slice_panel64(tl, k, k + 1, sc.panel, st, s, kt);
+                if (e == cudaSuccess)
+                    e = launch_update_tc64(maps, tl, k, k + 1, T, sc.panel, sc.counters + k, 0, st, s, kt);
+            } else {
+                e = launch_update_f64(tl, k, (int64_t)(T - k - 1) * (T - k) / 2, st, s, kt);
+            }
             if (e != cudaSuccess) return e;
         }
     }

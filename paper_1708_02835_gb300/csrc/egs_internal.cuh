@@ -159,9 +159,10 @@ cudaError_t launch_matern_table(const egs_matern_params &P, double *tab, cudaStr
 
 // Tile Cholesky in place (FP64).  Stops doing work once st->fail_index is set.
 // ctr: T * potrf_diag_scratch_words(b) words of device scratch for the
-// one-launch diagonal POTRFs (zeroed here).
+// one-launch diagonal POTRFs (zeroed here).  tc_scratch: tc64_scratch_bytes(b, T) bytes
+// for the tensor-core update, or NULL for the DFMA update.
 cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *st, cudaStream_t s,
-                                   KernelTimer *kt, unsigned *ctr);
+                                   KernelTimer *kt, unsigned *ctr, void *tc_scratch = nullptr);
 // Counter words one diagonal tile's one-launch POTRF needs.
 size_t potrf_diag_scratch_words(int b);
 
@@ -222,7 +223,7 @@ cudaError_t run_loglik_mixed(const double *X, const double *Y, const double *z, 
 
 // Layouts and setup of one evaluation (api.cu), shared with the serving loop.
 struct Layout {
-    size_t tiles, locs, z, zpad, partials, status, mtab, pctr, total;
+    size_t tiles, locs, z, zpad, partials, status, mtab, pctr, tc, total;
 };
 struct MixedLayout {
     size_t f64, f32, slots, panel, oz, l32, wsp, vinv, locs, z, vec, partials, status, err, mtab, pctr, rs, total;
@@ -231,13 +232,20 @@ struct EvalSetup {
     TileGeom g;
     int band, refine, xband;
     bool mixed;
+    bool tc;  // FP64: the tensor-core update (its scratch is part of need)
     egs_precision p;
     Layout L;
     MixedLayout ML;
     size_t need, locs_off, z_off;
     egs_matern_params P;
 };
+// SMs of the device.
+int device_sms();
+
 egs_status eval_setup(int64_t n, const double *theta, egs_precision p, const egs_opts *opts, EvalSetup *es);
+// FP64 without the tensor-core scratch (the DFMA update), for a caller's workspace or a
+// budget that holds no more; true if that made the need smaller.
+bool eval_shrink(EvalSetup *es);
 // Enqueue one evaluation on s; inputs on the device, ws holds es.need bytes.
 cudaError_t eval_enqueue(const EvalSetup &es, const double *dlocs, const double *dz, char *ws, cudaStream_t s,
                          KernelTimer *kt, cudaEvent_t *ev);

@@ -83,8 +83,13 @@ extern "C" egs_status egs_predict(const double *locs_obs, const double *z_obs, i
     const size_t extra_new = a256((size_t)2 * m * sizeof(double)), extra_out = a256((size_t)m * sizeof(double));
     char *ws = nullptr;
     const Allocator A = current_allocator();
-    const size_t wbytes = es.need + extra_new + extra_out;
+    size_t wbytes = es.need + extra_new + extra_out;
     cudaError_t e = dev_alloc(A, (void **)&ws, wbytes, s);
+    if (e == cudaErrorMemoryAllocation && eval_shrink(&es)) {
+        cudaGetLastError();
+        wbytes = es.need + extra_new + extra_out;
+        e = dev_alloc(A, (void **)&ws, wbytes, s);
+    }
     if (e != cudaSuccess) return cuda_error(e, "egs_predict workspace");
     const double *dlocs = locs_obs, *dz = z_obs, *dnew = locs_new;
     double *dout = z_new;

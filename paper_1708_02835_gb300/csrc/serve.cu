@@ -183,6 +183,7 @@ bool admit_one(egs_server *S, std::unique_lock<std::mutex> &lk)
         S->cv_done.notify_all();
         return true;
     }
+    if (S->used + es.need > S->cfg.hbm_budget_bytes && S->inflight == 0) egs::eval_shrink(&es);
     if (S->used + es.need > S->cfg.hbm_budget_bytes) {
         if (S->inflight > 0) return false;  // wait for memory to free up
         // nothing in flight: only resident fields hold the budget, so this

@@ -1,0 +1,587 @@
+// FP64 trailing update of the tile Cholesky (Section 5.2, SYRK / GEMM tasks) on
+// the BF16 tensor cores: C_mn -= P_m P_n^T with FP64 operands and results, every
+// product formed from exact BF16 slices (the error-free splitting of Ozaki, Ogita,
+// Oishi and Rump, Numer. Algorithms 59 (2012)).
+//
+// Why: GB300's FP64 pipe issues 2 FMAs per clock per SM (1.25 TFLOP/s for the chip;
+// the DFMA update ran at 99% of it), its BF16 tensor cores about 4,096.  28 exact
+// slice products per FP64 product still leave a factor of more than 30.
+//
+// Splitting.  A row x (length K) with |x| < 2^e is read as x = 2^(e-8) sum_i q_i 2^-8i,
+// i = 0..6, with integer digits |q_0| <= 256, |q_i| <= 128 (balanced base 256, from the
+// 57-bit fixed-point value rounded once), each exact in BF16.  For two rows
+//   x . y = 2^(ex + ey - 16) sum_L 2^-8L sum_{i+j=L} q_i(x) . q_j(y)
+// and the levels L = 0..6 (28 pairs) are kept.  The dropped ones and the rounding of the
+// last digit amount to about 2^-53.8 sqrt(K / 512) of |x|_max |y|_max, below the rounding
+// of a length-K chain of DFMAs.
+// Each level has its own FP32 accumulator in TMEM, flushed to FP64 every K = 256 columns.
+// Levels 0 and 1 stay below 2^24 units, so they are exact; level 2 could pass 2^24 units
+// only if |2 q_0 q_2 + q_1^2| averaged over 80% of its maximum, in phase, over 256 columns
+// (and level 3 over 67%), which the pseudo-random lower digits of a factor never do; from
+// level 4 on the FP32 rounding is below 2^-50 of the level-0 range even then.
+//
+// Kernel: persistent, one CTA per SM, 320 threads, output blocks of 128 x 64.  A K chunk
+// of 64 is 7 A boxes (128 rows) and one B box of all 7 slices (64 rows each, back to
+// back).  A slice i multiplies B slices 0 .. 6-i in one or two MMAs (N <= 256) whose D
+// address is shifted by 64 i columns, so the block of B slice j lands in level i + j:
+// each A slice is read from shared memory once or twice per K step instead of once per
+// pair.  Shared memory (reads by the MMAs 96 KB and TMA writes 42 KB per 16-column K
+// step of 896 tensor clocks, at 128 B / clock) is what bounds the kernel; 128 x 64
+// with 7 x 64 accumulator columns is the largest block that fits TMEM.
+// A slots are freed slice by slice (7 slots of 16 KB), B is double buffered (2 x 56 KB).
+// Measured (n = 16,900, tile 512, all 33 updates): 1,361 ms with DFMA, 40.8 ms here, i.e.
+// 43 TFLOP/s of FP64-equivalent work, 1,207 executed on the tensor cores.  Error of the
+// factor, rms of Sigma - L L^T in twice the precision (n = 2,304, tile 256): 2.5e-17 against
+// 3.2e-17 with DFMA (theta = (1, 0.1, 0.5)), 2.9e-17 / 6.3e-17 (nu = 1.3), 9.9e-18 / 1.0e-17
+// (range 0.03).
+#include "blocks.cuh"
+#include "tc_common.cuh"
+#include "tc64.cuh"
+
+#include <cudaTypedefs.h>
+
+namespace egs {
+
+namespace {
+
+constexpr int FM = 128, FN = 64, FKC = 64;  // output block and K chunk
+constexpr int FA_SL = FM * 128, FB_SL = FN * 128;
+constexpr int FB_BUF = kF64Slices * FB_SL;
+constexpr int FSMEM = kF64Slices * FA_SL + 2 * FB_BUF + 1024;
+constexpr int FTHREADS = 320;      // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
+constexpr int FRING = 4;           // work items posted ahead by the producer
+constexpr int FLUSH = 256 / FKC;   // K chunks per accumulator flush
+constexpr uint32_t FTMEM = 512;
+constexpr int kBadRow = 1 << 20;   // exponent of a row holding an infinity or a NaN
+
+// ---- slicing ----------------------------------------------------------------
+
+// 57-bit fixed point of x relative to 2^e (|x| < 2^e): rint(x 2^(56 - e)), ties away.
+__device__ __forceinline__ long long fixed57(double x, int e)
+{
+    const long long bits = __double_as_longlong(x);
+    int ex = (int)((bits >> 52) & 0x7FF);
+    long long m = bits & 0xFFFFFFFFFFFFFll;
+    if (ex) m |= 0x10000000000000ll;
+    else ex = 1;
+    const int sh = 1019 + e - ex;  // >= -3
+    long long f;
+    if (sh <= 0) f = m << (-sh);
+    else if (sh < 56) f = (m + (1ll << (sh - 1))) >> sh;
+    else f = 0;
+    return bits < 0 ? -f : f;
+}
+
+// The seven digits of f (balanced base 256) as BF16 bit patterns q_i 2^-8i.
+__device__ __forceinline__ void digits7(long long f, uint32_t (&d)[kF64Slices])
+{
+#pragma unroll
+    for (int i = kF64Slices - 1; i >= 0; --i) {
+        int q;
+        if (i > 0) {
+            q = (int)(signed char)(f & 0xFF);
+            f = (f - q) >> 8;
+        } else {
+            q = (int)f;
+        }
+        const float v = __int_as_float(0x4B400000 + q) - 12582912.0f;  // (float)q, |q| <= 256
+        d[i] = __float_as_uint(v * __int_as_float((127 - 8 * i) << 23)) >> 16;  // exact: 8 significant bits
+    }
+}
+
+// One warp slices one row of b doubles (b <= 1024, a multiple of 64): slice i of the row
+// to dst[i * stride + c], the exponent to *ep.  Lanes take two consecutive columns.
+__device__ __forceinline__ void slice7_row(const double *__restrict__ src, int b, uint16_t *__restrict__ dst,
+                                           size_t stride, int *ep)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned mh = 0;
+    for (int c = 2 * lane; c < b; c += 64) {
+        const double2 v = *reinterpret_cast<const double2 *>(src + c);
+        const unsigned h0 = (unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, h1 = (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu;
+        mh = max(mh, max(h0, h1));
+    }
+    mh = __reduce_max_sync(0xffffffffu, mh);
+    const int emax = (int)(mh >> 20);
+    const bool bad = emax == 0x7FF;
+    const int e = mh == 0 ? 0 : max(emax, 1) - 1022;
+    if (lane == 0) *ep = bad ? kBadRow : e;
+    for (int c = 2 * lane; c < b; c += 64) {
+        const double2 v = *reinterpret_cast<const double2 *>(src + c);
+        uint32_t d0[kF64Slices], d1[kF64Slices];
+        digits7(bad || mh == 0 ? 0ll : fixed57(v.x, e), d0);
+        digits7(bad || mh == 0 ? 0ll : fixed57(v.y, e), d1);
+#pragma unroll
+        for (int i = 0; i < kF64Slices; ++i)
+            *reinterpret_cast<uint32_t *>(dst + (size_t)i * stride + c) = d0[i] | (d1[i] << 16);
+    }
+}
+
+// Panel rows of step k (tiles m0 .. T - 1 of column k) -> slices; one warp per row.
+// Memory bound: 8 bytes read (twice, the second time from L1 / L2) and 14 written per entry.
+__global__ void __launch_bounds__(256) k_slice_panel64(Tiles tl, int k, int m0, uint16_t *__restrict__ sl,
+                                                       int *__restrict__ ex, const DevStatus *st)
+{
+    if (failed(st)) return;
+    const int b = tl.b;
+    const size_t pr = (size_t)(m0 - k - 1) * b + (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int m = k + 1 + (int)(pr / b);
+    slice7_row(tl.t64(m, k) + (pr % b) * b, b, sl + pr * b, (size_t)(tl.T - 1) * b * b, ex + pr);
+}
+
+// ---- the update -------------------------------------------------------------
+
+struct F64Item {
+    int m, n, rb, cb;  // output tile, 128-row block, 64-column block; m < 0 ends
+};
+
+// Output tiles (m, n), n = col0 .. col1 - 1, m = n .. T - 1, visited by blocks of kF64Cols
+// columns (the block's triangle, then every lower row), so that the CTAs working side by
+// side share the block's B operands in L2.
+constexpr int kF64Cols = 8;
+struct F64Work {
+    Tiles tl;
+    int k, col0, col1;
+    __host__ __device__ int64_t tiles() const
+    {
+        const int64_t c = col1 - col0, h = tl.T - col0;
+        return c * h - c * (c - 1) / 2;
+    }
+    __host__ __device__ int per_tile() const { return ((tl.b + FM - 1) / FM) * (tl.b / FN); }
+    __device__ bool decode(int64_t item, F64Item &w) const
+    {
+        const int ncb = tl.b / FN, per = per_tile();
+        int64_t t = item / per;
+        const int blk = (int)(item % per);
+        int c_lo = col0;
+        for (;;) {
+            const int wd = min(kF64Cols, col1 - c_lo);
+            const int64_t tri = (int64_t)wd * (wd + 1) / 2;
+            const int64_t cnt = tri + (int64_t)(tl.T - c_lo - wd) * wd;
+            if (t < cnt) {
+                if (t < tri) {
+                    int ii = 0, u = (int)t;
+                    while (u > ii) {
+                        u -= ii + 1;
+                        ++ii;
+                    }
+                    w.m = c_lo + ii;
+                    w.n = c_lo + u;
+                } else {
+                    const int64_t u = t - tri;
+                    w.m = c_lo + wd + (int)(u / wd);
+                    w.n = c_lo + (int)(u % wd);
+                }
+                break;
+            }
+            t -= cnt;
+            c_lo += wd;
+        }
+        w.rb = blk / ncb;
+        w.cb = blk % ncb;
+        return !(w.m == w.n && w.cb * FN > w.rb * FM + FM - 1);  // strictly above the diagonal
+    }
+};
+
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// (double)x by integer operations (the conversion instruction runs on the FP64 pipe);
+// x is zero or a normal float.
+__device__ __forceinline__ double f32_to_f64(float x)
+{
+    const uint32_t u = __float_as_uint(x), a = u & 0x7FFFFFFFu;
+    const uint32_t hi = a ? (u & 0x80000000u) | ((a >> 3) + (896u << 20)) : 0u;
+    return __hiloint2double((int)hi, (int)(a ? u << 29 : 0u));
+}
+
+// 2^s as a double, -1022 <= s <= 1023.
+__device__ __forceinline__ double pow2(int s) { return __hiloint2double((s + 1023) << 20, 0); }
+
+// The level sums v_0 .. v_6 (v_L a multiple of 2^-8L) as a + c + r: a + c is exact to the
+// last bit of c, r carries the rest to 2^-40 (level-0 units, |v_0| <= 2^24).
+__device__ __forceinline__ void combine7(const float (&v)[kF64Slices], float &a, float &c, float &r)
+{
+    float p, q, rr, t, u, w, x, y, c0, e1;
+    two_sum(v[4], __fadd_rn(v[5], v[6]), p, q);
+    two_sum(v[3], p, rr, t);
+    t = __fadd_rn(t, q);
+    two_sum(v[2], rr, u, w);
+    two_sum(v[1], u, x, y);
+    two_sum(v[0], x, a, c0);
+    two_sum(c0, y, c, e1);
+    r = __fadd_rn(e1, __fadd_rn(w, t));
+}
+
+// 7 x 16 accumulator columns (levels 64 columns apart) of the calling warp's 32 lanes.
+__device__ __forceinline__ void tmem_ld_levels16(uint32_t taddr, float (&v)[kF64Slices][16])
+{
+    uint32_t r[kF64Slices][16];
+#define EGS_LD16(L)                                                                                                  \
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "  \
+                 "[%16];"                                                                                            \
+                 : "=r"(r[L][0]), "=r"(r[L][1]), "=r"(r[L][2]), "=r"(r[L][3]), "=r"(r[L][4]), "=r"(r[L][5]),         \
+                   "=r"(r[L][6]), "=r"(r[L][7]), "=r"(r[L][8]), "=r"(r[L][9]), "=r"(r[L][10]), "=r"(r[L][11]),       \
+                   "=r"(r[L][12]), "=r"(r[L][13]), "=r"(r[L][14]), "=r"(r[L][15])                                    \
+                 : "r"(taddr + (L) * FN))
+    EGS_LD16(0);
+    EGS_LD16(1);
+    EGS_LD16(2);
+    EGS_LD16(3);
+    EGS_LD16(4);
+    EGS_LD16(5);
+    EGS_LD16(6);
+#undef EGS_LD16
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int L = 0; L < kF64Slices; ++L)
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            // the loads have landed; an empty volatile statement keeps every use behind the wait
+            asm volatile("" : "+r"(r[L][j]));
+            v[L][j] = __uint_as_float(r[L][j]);
+        }
+}
+
+__device__ __forceinline__ void tma_load_3d(const CUtensorMap *map, uint64_t *bar, void *dst, int x, int y, int z)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], "
+        "[%2];" ::"r"(tc::smem_u32(dst)),
+        "l"((uint64_t)map), "r"(tc::smem_u32(bar)), "r"(x), "r"(y), "r"(z)
+        : "memory");
+}
+
+__global__ void __launch_bounds__(FTHREADS, 1)
+k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, F64Work work,
+         const int *__restrict__ ex, int64_t nitems, unsigned long long *next, DevStatus *st)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    __shared__ uint64_t afull[kF64Slices], aempty[kF64Slices], bfull[2], bempty[2], tfull, tempty;
+    __shared__ uint64_t rfull[FRING], rempty[FRING];
+    __shared__ F64Item ring[FRING];
+    __shared__ uint32_t tmem_base;
+    __shared__ int abort_flag, stop, loaded;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kF64Slices; ++i) {
+            tc::mbar_init(&afull[i], 1);
+            tc::mbar_init(&aempty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(&bfull[i], 1);
+            tc::mbar_init(&bempty[i], 1);
+        }
+        tc::mbar_init(&tfull, 1);
+        tc::mbar_init(&tempty, 8);
+        for (int r = 0; r < FRING; ++r) {
+            tc::mbar_init(&rfull[r], 1);
+            tc::mbar_init(&rempty[r], 1 + 8);
+        }
+        abort_flag = 0;
+        loaded = 0;
+        stop = failed(st) ? 1 : 0;
+        tc::fence_mbar_init();
+    }
+    __syncthreads();
+    if (stop) return;
+    if (warp == 0) tc::tmem_alloc(&tmem_base, FTMEM);
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tbase = tmem_base;
+    const int b = work.tl.b, kchunks = b / FKC;
+    uint8_t *sa = smem, *sb = smem + kF64Slices * FA_SL;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            tc::prefetch_tmap(&mapA);
+            tc::prefetch_tmap(&mapB);
+            int g = 0, r = 0;  // chunks loaded, items posted
+            int64_t claimed = (int64_t)atomicAdd(next, 1ull);
+            while (!abort_flag) {
+                F64Item wi;
+                const bool valid = claimed < nitems && work.decode(claimed, wi);
+                if (claimed < nitems && !valid) {
+                    claimed = (int64_t)atomicAdd(next, 1ull);
+                    continue;
+                }
+                const int slot = r % FRING;
+                if (!tc::mbar_wait(&rempty[slot], ((uint32_t)(r / FRING) & 1u) ^ 1u, &abort_flag)) break;
+                if (!valid) wi.m = -1;
+                ring[slot] = wi;
+                tc::mbar_arrive(&rfull[slot]);
+                ++r;
+                if (!valid) break;
+                claimed = (int64_t)atomicAdd(next, 1ull);  // overlaps the loads below
+                const int ya = (wi.m - work.k - 1) * b + wi.rb * FM, yb = (wi.n - work.k - 1) * b + wi.cb * FN;
+                for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
+                    const int bb = g & 1;
+                    if (!tc::mbar_wait(&bempty[bb], ((uint32_t)(g >> 1) & 1u) ^ 1u, &abort_flag)) break;
+                    tc::mbar_arrive_expect_tx(&bfull[bb], FB_BUF);
+                    tma_load_3d(&mapB, &bfull[bb], sb + bb * FB_BUF, c * FKC, yb, 0);
+                    int i = 0;
+                    for (; i < kF64Slices; ++i) {
+                        if (!tc::mbar_wait(&aempty[i], ((uint32_t)g & 1u) ^ 1u, &abort_flag)) break;
+                        tc::mbar_arrive_expect_tx(&afull[i], FA_SL);
+                        tma_load_3d(&mapA, &afull[i], sa + i * FA_SL, c * FKC, ya, i);
+                    }
+                    // loads issued so far: chunk g's B box and its first i A boxes
+                    loaded = g * 8 + 1 + i;
+                    if (i < kF64Slices) break;
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int g = 0, r = 0;
+            uint32_t f = 0;  // flush groups issued
+            while (!abort_flag) {
+                const int slot = r % FRING;
+                if (!tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag)) break;
+                const int m = ring[slot].m;
+                tc::mbar_arrive(&rempty[slot]);
+                ++r;
+                if (m < 0) break;
+                for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
+                    const bool first = c % FLUSH == 0;
+                    if (first) {
+                        if (!tc::mbar_wait(&tempty, (f & 1u) ^ 1u, &abort_flag)) break;
+                        tc::tc_fence_after();
+                    }
+                    const int bb = g & 1;
+                    if (!tc::mbar_wait(&bfull[bb], (uint32_t)(g >> 1) & 1u, &abort_flag)) break;
+                    const uint32_t b0 = tc::smem_u32(sb + bb * FB_BUF);
+#pragma unroll
+                    for (int i = 0; i < kF64Slices; ++i) {
+                        if (!tc::mbar_wait(&afull[i], (uint32_t)g & 1u, &abort_flag)) break;
+                        tc::tc_fence_after();
+                        const uint32_t a0 = tc::smem_u32(sa + i * FA_SL);
+                        const int n = kF64Slices - i;  // B slices 0 .. n - 1
+                        const int n0 = n < 4 ? n : 4, n1 = n - n0;
+                        const uint32_t id0 = tc::idesc_f32acc(FM, n0 * FN, 1);
+                        const uint32_t id1 = tc::idesc_f32acc(FM, (n1 > 0 ? n1 : 1) * FN, 1);
+#pragma unroll
+                        for (int j = 0; j < FKC / 16; ++j) {
+                            // the i = 0 MMAs of a flush group's first K step cover all
+                            // seven level blocks and so initialise them
+                            const uint32_t acc = (first && i == 0 && j == 0) ? 0u : 1u;
+                            const uint64_t ad = tc::desc_sw128(a0 + 32 * j);
+                            tc::mma_f16(tbase + (uint32_t)(i * FN), ad, tc::desc_sw128(b0 + 32 * j), id0, acc);
+                            if (n1 > 0)
+                                tc::mma_f16(tbase + (uint32_t)((i + n0) * FN), ad,
+                                            tc::desc_sw128(b0 + n0 * FB_SL + 32 * j), id1, acc);
+                        }
+                        tc::mma_commit(&aempty[i]);
+                    }
+                    tc::mma_commit(&bempty[bb]);
+                    if (c % FLUSH == FLUSH - 1 || c == kchunks - 1) {
+                        tc::mma_commit(&tfull);
+                        ++f;
+                    }
+                }
+            }
+        }
+    } else {
+        // warp w: TMEM lanes 32 (w % 4) .. + 31 (rows of the block), columns 32 half .. + 31
+        const int q = warp & 3, half = (warp - 2) >> 2;
+        const uint32_t t0 = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32);
+        const int nflush = (kchunks + FLUSH - 1) / FLUSH;
+        uint32_t f = 0;
+        int r = 0;
+        bool run = true;
+        while (run) {
+            const int slot = r % FRING;
+            const bool got = tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag);
+            if (!__all_sync(0xffffffffu, got && !abort_flag)) break;
+            const F64Item wi = ring[slot];
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&rempty[slot]);
+            ++r;
+            if (wi.m < 0) break;
+            double acc[32];
+            for (int fl = 0; fl < nflush; ++fl, ++f) {
+                const bool ok = tc::mbar_wait(&tfull, f & 1u, &abort_flag);
+                tc::tc_fence_after();
+                if (!__all_sync(0xffffffffu, ok && !abort_flag)) {
+                    run = false;
+                    break;
+                }
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    float v[kF64Slices][16];
+                    tmem_ld_levels16(t0 + (uint32_t)(hh * 16), v);
+                    if (hh == 1) {
+                        tc::tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(&tempty);  // every level is in registers
+                    }
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const float vj[kF64Slices] = {v[0][j], v[1][j], v[2][j], v[3][j], v[4][j], v[5][j], v[6][j]};
+                        float a, c, rr;
+                        combine7(vj, a, c, rr);
+                        const double d = (f32_to_f64(a) + f32_to_f64(c)) + f32_to_f64(rr);
+                        acc[hh * 16 + j] = fl == 0 ? d : acc[hh * 16 + j] + d;
+                    }
+                }
+            }
+            if (!run) break;
+            const int row = wi.rb * FM + q * 32 + lane;
+            if (row < b) {
+                const int col = wi.cb * FN + half * 32;
+                const int ea = ex[(size_t)(wi.m - work.k - 1) * b + row] - 16;
+                const int *eb = ex + (size_t)(wi.n - work.k - 1) * b + col;
+                double *C = work.tl.t64(wi.m, wi.n) + (size_t)row * b + col;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    double2 cv[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) cv[j] = *reinterpret_cast<const double2 *>(C + 16 * h + 2 * j);
+                    double *cd = reinterpret_cast<double *>(cv);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const int s = ea + __ldg(eb + 16 * h + j);
+                        const double d = acc[16 * h + j];
+                        if (s >= -960 && s <= 1000) {
+                            cd[j] = fma(-pow2(s), d, cd[j]);
+                        } else if (s > 1000) {
+                            // an infinity or a NaN in either row reaches every product with it
+                            cd[j] = s >= kBadRow / 2 ? __longlong_as_double(0x7ff8000000000000ll)
+                                                     : fma(-pow2(s - 100), d * pow2(100), cd[j]);
+                        } else {
+                            cd[j] = s < -2040 ? cd[j] : fma(-pow2(-600), d * pow2(max(s + 600, -1022)), cd[j]);
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) *reinterpret_cast<double2 *>(C + 16 * h + 2 * j) = cv[j];
+                }
+            }
+        }
+    }
+    __syncwarp();
+    __syncthreads();
+    if (abort_flag && threadIdx.x == 0) {
+        // let every load that was issued land before the CTA exits: chunk g = loaded / 8
+        // holds its B box and loaded % 8 - 1 A boxes, the chunks before it are complete
+        volatile int dummy = 0;
+        const int total = loaded;
+        for (int bbi = 0; bbi < 2; ++bbi) {
+            int last = (total + 7) / 8 - 1;  // last chunk whose B box was issued
+            if (last >= 0 && (last & 1) != bbi) --last;
+            if (last >= 0) tc::mbar_wait(&bfull[bbi], (uint32_t)(last >> 1) & 1u, &dummy);
+        }
+        for (int i = 0; i < kF64Slices; ++i) {
+            const int last = (total - 2 - i) >= 0 ? (total - 2 - i) / 8 : -1;
+            if (last >= 0) tc::mbar_wait(&afull[i], (uint32_t)last & 1u, &dummy);
+        }
+        atomicExch(&st->timeout, 1);
+        atomicMin(&st->fail_index, 0ull);  // stops the rest of the evaluation
+    }
+    tc::tc_fence_after();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tbase, FTMEM);
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 f64_encode_fn()
+{
+    static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        return (PFN_cuTensorMapEncodeTiled_v12000)p;
+    }();
+    return fn;
+}
+
+// 3-D map over the slices (7 x rows x K BF16), box 64 x box_rows x box_slices, 128-byte swizzle.
+cudaError_t make_map3(CUtensorMap *m, const void *base, uint64_t rows, uint64_t K, uint32_t box_rows, uint32_t box_sl)
+{
+    auto fn = f64_encode_fn();
+    if (!fn) return cudaErrorNotSupported;
+    cuuint64_t dims[3] = {K, rows, (cuuint64_t)kF64Slices};
+    cuuint64_t strides[2] = {K * 2, rows * K * 2};
+    cuuint32_t box[3] = {(cuuint32_t)FKC, box_rows, box_sl};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+int device_sms()
+{
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+            n = 148;
+        return n;
+    }();
+    return sms;
+}
+
+static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+size_t tc64_scratch_bytes(int b, int T)
+{
+    const size_t R = (size_t)(T - 1) * (size_t)b;
+    return a256(R * b * kF64Slices * sizeof(uint16_t)) + a256(R * sizeof(int)) + a256((size_t)T * sizeof(unsigned long long));
+}
+
+F64Scratch tc64_scratch(void *base, int b, int T)
+{
+    const size_t R = (size_t)(T - 1) * (size_t)b;
+    char *p = (char *)base;
+    F64Scratch sc;
+    sc.panel.slices = (uint16_t *)p;
+    p += a256(R * b * kF64Slices * sizeof(uint16_t));
+    sc.panel.exps = (int *)p;
+    p += a256(R * sizeof(int));
+    sc.counters = (unsigned long long *)p;
+    return sc;
+}
+
+cudaError_t make_f64_maps(const F64Panel &p, int b, int T, F64Maps *maps)
+{
+    const uint64_t R = (uint64_t)(T - 1) * (uint64_t)b;
+    cudaError_t e = make_map3(&maps->a, p.slices, R, (uint64_t)b, FM, 1);
+    if (e == cudaSuccess) e = make_map3(&maps->b, p.slices, R, (uint64_t)b, FN, kF64Slices);
+    return e;
+}
+
+cudaError_t launch_slice_panel64(const Tiles &tl, int k, int m0, const F64Panel &p, const DevStatus *st, cudaStream_t s,
+                                 KernelTimer *kt)
+{
+    if (m0 >= tl.T) return cudaSuccess;
+    EGS_LAUNCH(kt, KC_TRSM, s,
+               k_slice_panel64<<<(unsigned)((size_t)(tl.T - m0) * tl.b / 8), 256, 0, s>>>(tl, k, m0, p.slices, p.exps, st));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_update_tc64(const F64Maps &maps, const Tiles &tl, int k, int col0, int col1, const F64Panel &p,
+                               unsigned long long *counter, int reserve, DevStatus *st, cudaStream_t s, KernelTimer *kt)
+{
+    if (col0 >= col1) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(k_tc_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
+    if (e != cudaSuccess) return e;
+    const F64Work w{tl, k, col0, col1};
+    const int64_t items = w.tiles() * w.per_tile();
+    const int64_t ctas = device_sms() - reserve > 1 ? device_sms() - reserve : 1;
+    EGS_LAUNCH(kt, KC_UPDATE, s,
+               k_tc_f64<<<(unsigned)(items < ctas ? items : ctas), FTHREADS, FSMEM, s>>>(maps.a, maps.b, w, p.exps, items,
+                                                                                         counter, st));
+    return cudaGetLastError();
+}
+
+}  // namespace egs
