@@ -16,29 +16,38 @@ namespace egs {
 
 namespace {
 
-constexpr int PB = 32;       // new locations per CTA
-constexpr int GROUP = 8;     // threads per new location
 constexpr int OCHUNK = 256;  // observed locations staged per pass
 
-// z_new[i] = sum_j C(||s_i - s_j||) x_j for the PB new locations of this CTA.
-// Thread t handles new location t / GROUP and observed locations
-// t % GROUP + GROUP q of every staged chunk; the GROUP partial sums of a
-// location are combined by a fixed shuffle tree, so results are bitwise
-// reproducible.
+// z_new[i] = sum_j C(||s_i - s_j||) x_j, GROUP threads per new location and
+// 256 / GROUP locations per CTA.  Thread t handles new location t / GROUP and
+// the observed locations t % GROUP + GROUP q of every staged chunk; the GROUP
+// partial sums of a location are combined in a fixed order, so results are
+// bitwise reproducible.  FP64-pipe bound (the Matern evaluation).  tab: the
+// local polynomials of a general nu, built by the evaluation that made x:
+// 25 FP64 operations per entry instead of the direct method's 1,100, and
+// 6.4e7 entries of them took about 120 of the 168 ms of a kriging call from
+// 6,400 to 10,000 locations.
+template <int GROUP>
 __global__ void __launch_bounds__(256) k_predict(const double *__restrict__ Xn, const double *__restrict__ Yn,
                                                  int64_t m, const double *__restrict__ Xo,
                                                  const double *__restrict__ Yo, const double *__restrict__ x,
                                                  int64_t n, const __grid_constant__ egs_matern_params Pg,
-                                                 double *__restrict__ z_new, const DevStatus *st)
+                                                 const double *__restrict__ tab, double *__restrict__ z_new,
+                                                 const DevStatus *st)
 {
     if (*(volatile const unsigned long long *)&st->fail_index != kNoFail) return;
+    constexpr int PB = 256 / GROUP;  // new locations per CTA
     __shared__ egs_matern_params Ps;
+    __shared__ double T[EGS_MT_DOUBLES];
     __shared__ double sx[OCHUNK], sy[OCHUNK], sv[OCHUNK];
     {
         const double *s = reinterpret_cast<const double *>(&Pg);
         double *d = reinterpret_cast<double *>(&Ps);
         for (int i = threadIdx.x; i < (int)(sizeof(egs_matern_params) / sizeof(double)); i += blockDim.x) d[i] = s[i];
+        if (tab)
+            for (int i = threadIdx.x; i < EGS_MT_DOUBLES; i += blockDim.x) T[i] = tab[i];
     }
+    const double *Tab = tab ? T : nullptr;
     const int li = threadIdx.x / GROUP, g = threadIdx.x % GROUP;
     const int64_t i = (int64_t)blockIdx.x * PB + li;
     const double xi = i < m ? Xn[i] : 0.0, yi = i < m ? Yn[i] : 0.0;
@@ -54,13 +63,35 @@ __global__ void __launch_bounds__(256) k_predict(const double *__restrict__ Xn, 
         }
         __syncthreads();
         const int cnt = (n - j0 < OCHUNK) ? (int)(n - j0) : OCHUNK;
-        for (int t = g; t < cnt; t += GROUP) {
-            acc = fma(matern_eval(&Ps, loc_dist(&Ps, xi, yi, sx[t], sy[t]) * inv_th2), sv[t], acc);
-        }
+        for (int t = g; t < cnt; t += GROUP)
+            acc = fma(matern_eval(&Ps, loc_dist(&Ps, xi, yi, sx[t], sy[t]) * inv_th2, Tab), sv[t], acc);
     }
 #pragma unroll
-    for (int off = GROUP / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    for (int off = (GROUP < 32 ? GROUP : 32) / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    if (GROUP > 32) {
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) sx[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        acc = sx[0];
+        for (int w = 1; w < 8; ++w) acc += sx[w];
+    }
     if (g == 0 && i < m) z_new[i] = acc;
+}
+
+// A CTA per new location up to 304 of them, 8 threads per location (32 locations share the
+// staged observed ones) from 9,728 on, 32 threads in between: always two CTAs for every SM.
+cudaError_t launch_predict(const double *Xn, const double *Yn, int64_t m, const double *Xo, const double *Yo,
+                           const double *x, int64_t n, const egs_matern_params &P, const double *tab, double *z_new,
+                           const DevStatus *st, cudaStream_t s)
+{
+    const double *t = P.kind == EGS_MATERN_GENERAL ? tab : nullptr;
+    if (m >= 304 * 32)
+        k_predict<8><<<(unsigned)((m + 31) / 32), 256, 0, s>>>(Xn, Yn, m, Xo, Yo, x, n, P, t, z_new, st);
+    else if (m >= 304)
+        k_predict<32><<<(unsigned)((m + 7) / 8), 256, 0, s>>>(Xn, Yn, m, Xo, Yo, x, n, P, t, z_new, st);
+    else
+        k_predict<256><<<(unsigned)m, 256, 0, s>>>(Xn, Yn, m, Xo, Yo, x, n, P, t, z_new, st);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -113,10 +144,9 @@ extern "C" egs_status egs_predict(const double *locs_obs, const double *z_obs, i
     if (e == cudaSuccess) e = finish_solution(es, ws, s);
     // Algorithm 3, the product: Z_1 = Sigma_12 X, Sigma_12 formed on the fly
     if (e == cudaSuccess) {
-        k_predict<<<(unsigned)((m + PB - 1) / PB), 256, 0, s>>>(dnew, dnew + m, m, dlocs, dlocs + n,
-                                                               eval_solution(es, ws), n, es.P, dout,
-                                                               eval_status(es, ws));
-        e = cudaGetLastError();
+        const double *tab = (const double *)(ws + (es.mixed ? es.ML.mtab : es.L.mtab));
+        e = launch_predict(dnew, dnew + m, m, dlocs, dlocs + n, eval_solution(es, ws), n, es.P, tab, dout,
+                           eval_status(es, ws), s);
     }
     if (e == cudaSuccess && host_out) e = cudaMemcpyAsync(z_new, dout, (size_t)m * sizeof(double), cudaMemcpyDeviceToHost, s);
     DevStatus h;
