@@ -250,33 +250,29 @@ cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *
 {
     const int T = g.T;
     const Tiles tl{tiles, nullptr, g.b, T, T};
-    cudaError_t e0 = cudaMemsetAsync(ctr, 0, (size_t)T * potrf_diag_scratch_words(g.b) * sizeof(unsigned), s);
-    if (e0 != cudaSuccess) return e0;
-    F64Scratch sc{};
-    F64Maps maps;
+    cudaError_t e = cudaSuccess;
     if (tc_scratch) {
-        sc = tc64_scratch(tc_scratch, g.b, T);
-        e0 = make_f64_maps(sc.panel, g.b, T, &maps);
-        if (e0 == cudaSuccess) e0 = cudaMemsetAsync(sc.counters, 0, (size_t)T * sizeof(unsigned long long), s);
-        if (e0 != cudaSuccess) return e0;
-    }
-    for (int k = 0; k < T; ++k) {
-        if (kt) kt->step = k;
-        cudaError_t e = launch_potrf_diag(tl, k, st, s, kt, ctr + (size_t)k * potrf_diag_scratch_words(g.b));
-        if (e != cudaSuccess) return e;
-        if (k + 1 < T) {
-            e = launch_trsm_f64(tl, k, T - k - 1, st, s, kt);
-            if (e != cudaSuccess) return e;
-            if (tc_scratch) {
-                e = launch_slice_panel64(tl, k, k + 1, sc.panel, st, s, kt);
-                if (e == cudaSuccess)
-                    e = launch_update_tc64(maps, tl, k, k + 1, T, sc.panel, sc.counters + k, 0, st, s, kt);
-            } else {
-                e = launch_update_f64(tl, k, (int64_t)(T - k - 1) * (T - k) / 2, st, s, kt);
-            }
-            if (e != cudaSuccess) return e;
+        const F64Set set{nullptr, tc64_problem(tc_scratch, tl, st), 1, g.b, T};
+        F64Maps maps;
+        e = make_f64_maps(set.one.panel, set.one.inner, g.b, &maps);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(set.one.ctr, 0, tc64_counters(g.b, T) * sizeof(unsigned long long), s);
+        for (int k = 0; k < T && e == cudaSuccess; ++k) {
+            if (kt) kt->step = k;
+            e = launch_panel64(maps, set, k, s, kt);
+            if (e == cudaSuccess) e = launch_slice_panel64(set, k, s, kt);
+            if (e == cudaSuccess) e = launch_update_tc64(maps, set, k, 0, 0, s, kt);
+        }
+    } else {
+        e = cudaMemsetAsync(ctr, 0, (size_t)T * potrf_diag_scratch_words(g.b) * sizeof(unsigned), s);
+        for (int k = 0; k < T && e == cudaSuccess; ++k) {
+            if (kt) kt->step = k;
+            e = launch_potrf_diag(tl, k, st, s, kt, ctr + (size_t)k * potrf_diag_scratch_words(g.b));
+            if (e == cudaSuccess) e = launch_trsm_f64(tl, k, T - k - 1, st, s, kt);
+            if (e == cudaSuccess) e = launch_update_f64(tl, k, (int64_t)(T - k - 1) * (T - k) / 2, st, s, kt);
         }
     }
+    if (e != cudaSuccess) return e;
     if (kt) kt->step = -1;
     return cudaGetLastError();
 }

@@ -119,14 +119,142 @@ __device__ __forceinline__ void slice7_row(const double *__restrict__ src, int b
 
 // Panel rows of step k (tiles m0 .. T - 1 of column k) -> slices; one warp per row.
 // Memory bound: 8 bytes read (twice, the second time from L1 / L2) and 14 written per entry.
-__global__ void __launch_bounds__(256) k_slice_panel64(Tiles tl, int k, int m0, uint16_t *__restrict__ sl,
-                                                       int *__restrict__ ex, const DevStatus *st)
+__global__ void __launch_bounds__(256) k_slice_panel64(const __grid_constant__ F64Set set, int k)
 {
-    if (failed(st)) return;
+    const F64Prob &P = set.get(blockIdx.y);
+    const Tiles &tl = P.tl;
     const int b = tl.b;
-    const size_t pr = (size_t)(m0 - k - 1) * b + (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int m = k + 1 + (int)(pr / b);
-    slice7_row(tl.t64(m, k) + (pr % b) * b, b, sl + pr * b, (size_t)(tl.T - 1) * b * b, ex + pr);
+    const int64_t pr = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (pr >= (int64_t)(tl.T - 1 - k) * b || failed(P.st)) return;
+    const size_t r = P.panel.row0 + pr;
+    slice7_row(tl.t64(k + 1 + (int)(pr / b), k) + (pr % b) * b, b, P.panel.sl + r * b, P.panel.rows * b, P.panel.ex + r);
+}
+
+// ---- the panel ----------------------------------------------------------------
+//
+// Tile column k is factored in 64-column blocks, each in three launches:
+//   k_diag64    L_jj = chol of the 64 x 64 diagonal block and the inverses of its four
+//               16 x 16 diagonal blocks, one CTA;
+//   k_solve64   the rows below, in the tile and in every tile under it: X L_jj^T = A by
+//               16-column blocks, X_p = (A_p - sum_{i<p} X_i L_pi^T) L_pp^-T, and X's slices
+//               (K = 64, exponents of their own);
+//   k_tc_f64    the update of the panel's columns right of the block (inner work).
+// Why 64: the FP64 pipe does n^2 w / 2 FMAs in all solves of width w, 14.7 ms at
+// n = 16,900 for w = 64 and 118 ms for whole 512-column tiles, while each step costs three
+// launches and one 64 x 64 Cholesky of latency.  Measured (n = 16,900, tile 512): 36 ms of
+// diagonal tiles and 100 ms of whole-tile solves became 30 + 17 + 12 ms; the evaluation went
+// from 193 to 120 ms, that of n = 5,000 (tile 256) from 27.0 to 18.9 ms.
+constexpr int PW = kF64Panel;
+constexpr int PI = 16;       // inverted sub-blocks
+static_assert(kW16Doubles == (PW / PI) * PI * PI, "one inverse per 16 x 16 diagonal block");
+
+// One CTA per problem, 256 threads.  w16: the inverses W_pp, row-major, at 256 p.
+__global__ void __launch_bounds__(256) k_diag64(const __grid_constant__ F64Set set, int k, int j)
+{
+    __shared__ Potrf64Smem sm;
+    const F64Prob &P = set.get(blockIdx.y);
+    const Tiles &tl = P.tl;
+    DevStatus *st = P.st;
+    double *w16 = P.w16;
+    if (k >= tl.T || failed(st)) return;
+    const int b = tl.b, tid = threadIdx.x;
+    double *A = tl.t64(k, k) + (size_t)j * PW * (b + 1);
+    if (!potrf64_smem_s(sm, A, b, (int64_t)k * b + j * PW, st)) return;
+    const int right = b - (j + 1) * PW;
+    for (int e = tid; e < PW * right; e += 256) A[(size_t)(e / right) * b + PW + e % right] = 0.0;
+    // column c of W_pp by forward substitution, one thread each (the factor is still in sm)
+    if (tid < PW) {
+        const int p = tid / PI, c = tid % PI, q0 = p * PI;
+        double w[PI];
+#pragma unroll
+        for (int i = 0; i < PI; ++i) {
+            double v = i == c ? 1.0 : 0.0;
+#pragma unroll
+            for (int l = 0; l < i; ++l) v = fma(-sm.S[q0 + i][q0 + l], w[l], v);
+            w[i] = v * sm.rd[q0 + i];
+        }
+#pragma unroll
+        for (int i = 0; i < PI; ++i) w16[p * PI * PI + i * PI + c] = w[i];
+    }
+}
+
+// One warp slices the 64 entries of a row: lane's entries 2 lane, 2 lane + 1.
+__device__ __forceinline__ void slice7_row64(double x0, double x1, uint16_t *__restrict__ dst, size_t stride, int *ep)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned h0 = (unsigned)__double2hiint(x0) & 0x7FFFFFFFu, h1 = (unsigned)__double2hiint(x1) & 0x7FFFFFFFu;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, max(h0, h1));
+    const int emax = (int)(mh >> 20);
+    const bool bad = emax == 0x7FF;
+    const int e = mh == 0 ? 0 : max(emax, 1) - 1022;
+    if (lane == 0) *ep = bad ? kBadRow : e;
+    uint32_t d0[kF64Slices], d1[kF64Slices];
+    digits7(bad || mh == 0 ? 0ll : fixed57(x0, e), d0);
+    digits7(bad || mh == 0 ? 0ll : fixed57(x1, e), d1);
+#pragma unroll
+    for (int i = 0; i < kF64Slices; ++i)
+        *reinterpret_cast<uint32_t *>(dst + (size_t)i * stride + 2 * lane) = d0[i] | (d1[i] << 16);
+}
+
+// Panel rows (j + 1) 64 .. (T - k) b - 1, RB rows per CTA, 256 threads.  FP64-pipe bound
+// (RB 64 64 / 2 FMAs and the 16 x 16 products at 2 a clock per SM): RB = 16 while that
+// leaves SMs idle otherwise.
+template <int RB>
+__global__ void __launch_bounds__(256) k_solve64(const __grid_constant__ F64Set set, int k, int j)
+{
+    const F64Prob &P = set.get(blockIdx.y);
+    const Tiles &tl = P.tl;
+    const double *__restrict__ w16 = P.w16;
+    if ((int64_t)(j + 1) * PW + (int64_t)blockIdx.x * RB >= (int64_t)(tl.T - k) * tl.b || failed(P.st)) return;
+    constexpr int RT = RB / 16;  // rows per thread
+    // L below its 16 x 16 diagonal blocks: rows 16 .. 63, columns 0 .. 47
+    __shared__ double Ls[PW - PI][PW - PI + 1], Xs[RB][PW + 1], Ws[PW][PI + 1];
+    const int b = tl.b, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int pr0 = (j + 1) * PW + (int)blockIdx.x * RB;
+    double *X = tl.t64(k + pr0 / b, k) + (size_t)(pr0 % b) * b + j * PW;
+    const double *L = tl.t64(k, k) + (size_t)j * PW * (b + 1);
+    for (int e = tid; e < (PW - PI) * (PW - PI); e += 256)
+        Ls[e / (PW - PI)][e % (PW - PI)] = L[(size_t)(PI + e / (PW - PI)) * b + e % (PW - PI)];
+    for (int e = tid; e < RB * PW; e += 256) Xs[e >> 6][e & 63] = X[(size_t)(e >> 6) * b + (e & 63)];
+    for (int e = tid; e < (int)kW16Doubles; e += 256) Ws[e >> 4][e & 15] = w16[e];
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < PW / PI; ++p) {
+        double r[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) r[i] = Xs[ty + 16 * i][PI * p + tx];
+        for (int l = 0; l < PI * p; ++l) {
+            const double lv = Ls[PI * (p - 1) + tx][l];
+#pragma unroll
+            for (int i = 0; i < RT; ++i) r[i] = fma(-Xs[ty + 16 * i][l], lv, r[i]);
+        }
+        // a row's 16 entries belong to one half-warp
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < RT; ++i) Xs[ty + 16 * i][PI * p + tx] = r[i];
+        __syncwarp();
+        double x[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) x[i] = 0.0;
+#pragma unroll
+        for (int l = 0; l < PI; ++l) {
+            const double wv = Ws[PI * p + tx][l];
+#pragma unroll
+            for (int i = 0; i < RT; ++i) x[i] = fma(Xs[ty + 16 * i][PI * p + l], wv, x[i]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < RT; ++i) Xs[ty + 16 * i][PI * p + tx] = x[i];
+        __syncwarp();
+    }
+    __syncthreads();
+    const int lane = tid & 31;
+    for (int r = tid >> 5; r < RB; r += 8) {
+        const size_t sr = P.inner.row0 + pr0 + r;
+        const double x0 = Xs[r][2 * lane], x1 = Xs[r][2 * lane + 1];
+        *reinterpret_cast<double2 *>(X + (size_t)r * b + 2 * lane) = make_double2(x0, x1);
+        slice7_row64(x0, x1, P.inner.sl + sr * PW, P.inner.rows * PW, P.inner.ex + sr);
+    }
 }
 
 // ---- the update -------------------------------------------------------------
@@ -135,50 +263,67 @@ struct F64Item {
     int m, n, rb, cb;  // output tile, 128-row block, 64-column block; m < 0 ends
 };
 
-// Output tiles (m, n), n = col0 .. col1 - 1, m = n .. T - 1, visited by blocks of kF64Cols
-// columns (the block's triangle, then every lower row), so that the CTAs working side by
-// side share the block's B operands in L2.
+// Trailing update (inner = false): output tiles (m, n), n = col0 .. col1 - 1, m = n .. T - 1,
+// visited by blocks of kF64Cols columns (the block's triangle, then every lower row), so that
+// the CTAs working side by side share the block's B operands in L2.  Operand row r of tile m
+// is slice row (m - k - 1) b + r, K = b.
+// Inside a panel (inner = true): the 64-column blocks col0 .. col1 - 1 of tile column k, all
+// rows from each block's diagonal down; slice row (m - k) b + r, K = 64.
 constexpr int kF64Cols = 8;
 struct F64Work {
-    Tiles tl;
+    const Tiles &tl;
     int k, col0, col1;
-    __host__ __device__ int64_t tiles() const
+    bool inner;
+    __host__ __device__ int row_blocks() const { return (tl.b + FM - 1) / FM; }
+    __host__ __device__ int kchunks() const { return inner ? 1 : tl.b / FKC; }
+    __host__ __device__ int64_t items() const
     {
-        const int64_t c = col1 - col0, h = tl.T - col0;
-        return c * h - c * (c - 1) / 2;
+        const int64_t c = col1 - col0;
+        if (inner) return c * row_blocks() * (tl.T - k);
+        const int64_t h = tl.T - col0;
+        return (c * h - c * (c - 1) / 2) * row_blocks() * (tl.b / FN);
     }
-    __host__ __device__ int per_tile() const { return ((tl.b + FM - 1) / FM) * (tl.b / FN); }
+    __device__ size_t slice_row(int m) const { return (size_t)(m - k - (inner ? 0 : 1)) * tl.b; }
     __device__ bool decode(int64_t item, F64Item &w) const
     {
-        const int ncb = tl.b / FN, per = per_tile();
-        int64_t t = item / per;
-        const int blk = (int)(item % per);
-        int c_lo = col0;
-        for (;;) {
-            const int wd = min(kF64Cols, col1 - c_lo);
-            const int64_t tri = (int64_t)wd * (wd + 1) / 2;
-            const int64_t cnt = tri + (int64_t)(tl.T - c_lo - wd) * wd;
-            if (t < cnt) {
-                if (t < tri) {
-                    int ii = 0, u = (int)t;
-                    while (u > ii) {
-                        u -= ii + 1;
-                        ++ii;
+        if (inner) {
+            const int wd = col1 - col0, rbs = row_blocks();
+            const int64_t u = item / wd;
+            w.m = k + (int)(u / rbs);
+            w.n = k;
+            w.rb = (int)(u % rbs);
+            w.cb = col0 + (int)(item % wd);
+        } else {
+            const int ncb = tl.b / FN, per = row_blocks() * ncb;
+            int64_t t = item / per;
+            const int blk = (int)(item % per);
+            int c_lo = col0;
+            for (;;) {
+                const int wd = min(kF64Cols, col1 - c_lo);
+                const int64_t tri = (int64_t)wd * (wd + 1) / 2;
+                const int64_t cnt = tri + (int64_t)(tl.T - c_lo - wd) * wd;
+                if (t < cnt) {
+                    if (t < tri) {
+                        int ii = 0, u = (int)t;
+                        while (u > ii) {
+                            u -= ii + 1;
+                            ++ii;
+                        }
+                        w.m = c_lo + ii;
+                        w.n = c_lo + u;
+                    } else {
+                        const int64_t u = t - tri;
+                        w.m = c_lo + wd + (int)(u / wd);
+                        w.n = c_lo + (int)(u % wd);
                     }
-                    w.m = c_lo + ii;
-                    w.n = c_lo + u;
-                } else {
-                    const int64_t u = t - tri;
-                    w.m = c_lo + wd + (int)(u / wd);
-                    w.n = c_lo + (int)(u % wd);
+                    break;
                 }
-                break;
+                t -= cnt;
+                c_lo += wd;
             }
-            t -= cnt;
-            c_lo += wd;
+            w.rb = blk / ncb;
+            w.cb = blk % ncb;
         }
-        w.rb = blk / ncb;
-        w.cb = blk % ncb;
         return !(w.m == w.n && w.cb * FN > w.rb * FM + FM - 1);  // strictly above the diagonal
     }
 };
@@ -257,9 +402,21 @@ __device__ __forceinline__ void tma_load_3d(const CUtensorMap *map, uint64_t *ba
 }
 
 __global__ void __launch_bounds__(FTHREADS, 1)
-k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, F64Work work,
-         const int *__restrict__ ex, int64_t nitems, unsigned long long *next, DevStatus *st)
+k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+         const __grid_constant__ F64Set set, int k, int c0, int c1, int inner, int slot)
 {
+    const F64Prob &P = set.get(blockIdx.y);
+    if (P.tl.T <= k) return;
+    // trailing: columns k + c0 .. min(k + c1, T) - 1; inner: the blocks c0 .. c1 - 1 of column k
+    const F64Work work{P.tl, k, inner ? c0 : k + c0, inner ? c1 : min(k + c1, P.tl.T), inner != 0};
+    if (work.col0 >= work.col1) return;
+    const int64_t nitems = work.items();
+    if ((int64_t)blockIdx.x >= nitems) return;
+    unsigned long long *next = P.ctr + slot;
+    DevStatus *st = P.st;
+    const F64Rows &rows = inner ? P.inner : P.panel;
+    const int *__restrict__ ex = rows.ex + rows.row0;
+    const int yrow0 = (int)rows.row0;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     __shared__ uint64_t afull[kF64Slices], aempty[kF64Slices], bfull[2], bempty[2], tfull, tempty;
@@ -296,7 +453,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tbase = tmem_base;
-    const int b = work.tl.b, kchunks = b / FKC;
+    const int b = work.tl.b, kchunks = work.kchunks();
     uint8_t *sa = smem, *sb = smem + kF64Slices * FA_SL;
 
     if (warp == 0) {
@@ -320,7 +477,8 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                 ++r;
                 if (!valid) break;
                 claimed = (int64_t)atomicAdd(next, 1ull);  // overlaps the loads below
-                const int ya = (wi.m - work.k - 1) * b + wi.rb * FM, yb = (wi.n - work.k - 1) * b + wi.cb * FN;
+                const int ya = yrow0 + (int)work.slice_row(wi.m) + wi.rb * FM;
+                const int yb = yrow0 + (int)work.slice_row(wi.n) + wi.cb * FN;
                 for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
                     const int bb = g & 1;
                     if (!tc::mbar_wait(&bempty[bb], ((uint32_t)(g >> 1) & 1u) ^ 1u, &abort_flag)) break;
@@ -434,10 +592,12 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             }
             if (!run) break;
             const int row = wi.rb * FM + q * 32 + lane;
-            if (row < b) {
+            // rows of a diagonal tile above its column block are left alone: the factored blocks
+            // of the panel hold zeros there
+            if (row < b && !(wi.m == wi.n && row < wi.cb * FN)) {
                 const int col = wi.cb * FN + half * 32;
-                const int ea = ex[(size_t)(wi.m - work.k - 1) * b + row] - 16;
-                const int *eb = ex + (size_t)(wi.n - work.k - 1) * b + col;
+                const int ea = ex[work.slice_row(wi.m) + row] - 16;
+                const int *eb = ex + work.slice_row(wi.n) + col;
                 double *C = work.tl.t64(wi.m, wi.n) + (size_t)row * b + col;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -533,55 +693,107 @@ int device_sms()
 
 static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Slices and exponents of the panel (K = b) and of its 64-column blocks (K = 64, the
+// diagonal tile's rows too), the work counters, the 16 x 16 inverses.
 size_t tc64_scratch_bytes(int b, int T)
 {
-    const size_t R = (size_t)(T - 1) * (size_t)b;
-    return a256(R * b * kF64Slices * sizeof(uint16_t)) + a256(R * sizeof(int)) + a256((size_t)T * sizeof(unsigned long long));
+    const size_t R = (size_t)(T - 1) * (size_t)b, R1 = R + b;
+    return a256(R * b * kF64Slices * sizeof(uint16_t)) + a256(R * sizeof(int)) +
+           a256(R1 * PW * kF64Slices * sizeof(uint16_t)) + a256(R1 * sizeof(int)) +
+           a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(kW16Doubles * sizeof(double));
 }
 
-F64Scratch tc64_scratch(void *base, int b, int T)
+F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st)
 {
-    const size_t R = (size_t)(T - 1) * (size_t)b;
-    char *p = (char *)base;
-    F64Scratch sc;
-    sc.panel.slices = (uint16_t *)p;
-    p += a256(R * b * kF64Slices * sizeof(uint16_t));
-    sc.panel.exps = (int *)p;
-    p += a256(R * sizeof(int));
-    sc.counters = (unsigned long long *)p;
-    return sc;
+    const size_t R = (size_t)(tl.T - 1) * (size_t)tl.b, R1 = R + tl.b;
+    char *p = (char *)scratch;
+    auto take = [&p](size_t bytes) {
+        char *q = p;
+        p += a256(bytes);
+        return q;
+    };
+    F64Prob P;
+    P.tl = tl;
+    P.st = st;
+    P.panel.sl = (uint16_t *)take(R * tl.b * kF64Slices * sizeof(uint16_t));
+    P.panel.ex = (int *)take(R * sizeof(int));
+    P.panel.rows = R;
+    P.inner.sl = (uint16_t *)take(R1 * PW * kF64Slices * sizeof(uint16_t));
+    P.inner.ex = (int *)take(R1 * sizeof(int));
+    P.inner.rows = R1;
+    P.panel.row0 = P.inner.row0 = 0;
+    P.ctr = (unsigned long long *)take(tc64_counters(tl.b, tl.T) * sizeof(unsigned long long));
+    P.w16 = (double *)take(kW16Doubles * sizeof(double));
+    return P;
 }
 
-cudaError_t make_f64_maps(const F64Panel &p, int b, int T, F64Maps *maps)
+cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64Maps *maps)
 {
-    const uint64_t R = (uint64_t)(T - 1) * (uint64_t)b;
-    cudaError_t e = make_map3(&maps->a, p.slices, R, (uint64_t)b, FM, 1);
-    if (e == cudaSuccess) e = make_map3(&maps->b, p.slices, R, (uint64_t)b, FN, kF64Slices);
+    cudaError_t e = make_map3(&maps->a, panel.sl, panel.rows, (uint64_t)b, FM, 1);
+    if (e == cudaSuccess) e = make_map3(&maps->b, panel.sl, panel.rows, (uint64_t)b, FN, kF64Slices);
+    if (e == cudaSuccess) e = make_map3(&maps->ia, inner.sl, inner.rows, PW, FM, 1);
+    if (e == cudaSuccess) e = make_map3(&maps->ib, inner.sl, inner.rows, PW, FN, kF64Slices);
     return e;
 }
 
-cudaError_t launch_slice_panel64(const Tiles &tl, int k, int m0, const F64Panel &p, const DevStatus *st, cudaStream_t s,
-                                 KernelTimer *kt)
+// CTAs of a problem's update launch: the whole GPU for one problem, a share for each of many.
+static unsigned tc64_ctas(const F64Set &set, int64_t items, int reserve)
 {
-    if (m0 >= tl.T) return cudaSuccess;
-    EGS_LAUNCH(kt, KC_TRSM, s,
-               k_slice_panel64<<<(unsigned)((size_t)(tl.T - m0) * tl.b / 8), 256, 0, s>>>(tl, k, m0, p.slices, p.exps, st));
+    int64_t c = device_sms() - reserve;
+    if (set.count > 1) c = (c * 4 + set.count - 1) / set.count;
+    c = items < c ? items : c;
+    return (unsigned)(c > 1 ? c : 1);
+}
+
+static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, const F64Set &set, int k, int c0, int c1,
+                                 int inner, int slot, int reserve, cudaStream_t s, KernelTimer *kt)
+{
+    cudaError_t e = cudaFuncSetAttribute(k_tc_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
+    if (e != cudaSuccess) return e;
+    const Tiles tl{nullptr, nullptr, set.b, set.Tmax, set.Tmax};
+    const F64Work w{tl, k, inner ? c0 : k + c0, inner ? c1 : (k + c1 < set.Tmax ? k + c1 : set.Tmax), inner != 0};
+    if (w.col0 >= w.col1) return cudaSuccess;
+    const dim3 grid(tc64_ctas(set, w.items(), reserve), (unsigned)set.count);
+    EGS_LAUNCH(kt, KC_UPDATE, s, k_tc_f64<<<grid, FTHREADS, FSMEM, s>>>(a, b, set, k, c0, c1, inner, slot));
     return cudaGetLastError();
 }
 
-cudaError_t launch_update_tc64(const F64Maps &maps, const Tiles &tl, int k, int col0, int col1, const F64Panel &p,
-                               unsigned long long *counter, int reserve, DevStatus *st, cudaStream_t s, KernelTimer *kt)
+cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, cudaStream_t s, KernelTimer *kt)
 {
-    if (col0 >= col1) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_tc_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
-    if (e != cudaSuccess) return e;
-    const F64Work w{tl, k, col0, col1};
-    const int64_t items = w.tiles() * w.per_tile();
-    const int64_t ctas = device_sms() - reserve > 1 ? device_sms() - reserve : 1;
-    EGS_LAUNCH(kt, KC_UPDATE, s,
-               k_tc_f64<<<(unsigned)(items < ctas ? items : ctas), FTHREADS, FSMEM, s>>>(maps.a, maps.b, w, p.exps, items,
-                                                                                         counter, st));
+    const int nj = set.b / PW;
+    cudaError_t e = cudaSuccess;
+    for (int j = 0; j < nj && e == cudaSuccess; ++j) {
+        EGS_LAUNCH(kt, KC_POTRF, s, k_diag64<<<dim3(1, (unsigned)set.count), 256, 0, s>>>(set, k, j));
+        const int64_t rows = (int64_t)(set.Tmax - k) * set.b - (j + 1) * PW;
+        if (rows > 0) {
+            if (rows / 16 * set.count <= device_sms())
+                EGS_LAUNCH(kt, KC_TRSM, s,
+                           k_solve64<16><<<dim3((unsigned)(rows / 16), (unsigned)set.count), 256, 0, s>>>(set, k, j));
+            else
+                EGS_LAUNCH(kt, KC_TRSM, s,
+                           k_solve64<32><<<dim3((unsigned)(rows / 32), (unsigned)set.count), 256, 0, s>>>(set, k, j));
+        }
+        e = cudaGetLastError();
+        if (e == cudaSuccess && j + 1 < nj)
+            e = launch_tc_f64(maps.ia, maps.ib, set, k, j + 1, nj, 1, k * (2 + nj) + 2 + j, 0, s, kt);
+    }
+    return e;
+}
+
+cudaError_t launch_slice_panel64(const F64Set &set, int k, cudaStream_t s, KernelTimer *kt)
+{
+    if (k + 1 >= set.Tmax) return cudaSuccess;
+    EGS_LAUNCH(kt, KC_TRSM, s,
+               k_slice_panel64<<<dim3((unsigned)((size_t)(set.Tmax - k - 1) * set.b / 8), (unsigned)set.count), 256, 0,
+                                 s>>>(set, k));
     return cudaGetLastError();
+}
+
+cudaError_t launch_update_tc64(const F64Maps &maps, const F64Set &set, int k, int part, int reserve, cudaStream_t s,
+                               KernelTimer *kt)
+{
+    return launch_tc_f64(maps.a, maps.b, set, k, part == 2 ? 2 : 1, part == 1 ? 2 : set.Tmax, 0,
+                         k * (2 + set.b / PW) + (part == 2 ? 1 : 0), reserve, s, kt);
 }
 
 }  // namespace egs

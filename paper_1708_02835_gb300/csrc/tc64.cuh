@@ -1,20 +1,11 @@
-// Host interface of the FP64 trailing update on the tensor cores (tc64.cu).
+// Host interface of the FP64 factorisation on the tensor cores (tc64.cu).
 #pragma once
 #include "egs_internal.cuh"
 
 namespace egs {
 
 constexpr int kF64Slices = 7;
-
-// The sliced panel of one step: slice i of panel row r (row r of tiles k + 1 .. T - 1, in
-// order) at slices[(i R + r) b ..], R = (T - 1) b, and the row's exponent.
-struct F64Panel {
-    uint16_t *slices;
-    int *exps;
-};
-struct F64Maps {
-    CUtensorMap a, b;
-};
+constexpr int kF64Panel = 64;  // width of the blocks a tile column is factored in
 
 // FP64 factorisations take the tensor cores above this many rows.  Below it the chain of
 // diagonal tiles sets the time (n = 1,600: update 1.1 of 6.2 ms), and the persistent batch,
@@ -23,21 +14,54 @@ struct F64Maps {
 constexpr int64_t kTc64MinRows = 2049;
 inline bool tc64_applies(int64_t n, int b, int T) { return n >= kTc64MinRows && T > 1 && b % 64 == 0; }
 
-// Device scratch of one tensor-core FP64 factorisation.
-size_t tc64_scratch_bytes(int b, int T);
-struct F64Scratch {
-    F64Panel panel;
-    unsigned long long *counters;  // one work counter per launch
+// Slices of operand rows (slice i of row r at sl[(i rows + r) K ..], K = b or 64) and the
+// rows' exponents; several problems share one array, each from its own row0 on.
+struct F64Rows {
+    uint16_t *sl;
+    int *ex;
+    size_t rows, row0;
 };
-F64Scratch tc64_scratch(void *base, int b, int T);
 
-cudaError_t make_f64_maps(const F64Panel &p, int b, int T, F64Maps *maps);
-// Slices of the solved panel tiles (m0 .. T - 1, k).
-cudaError_t launch_slice_panel64(const Tiles &tl, int k, int m0, const F64Panel &p, const DevStatus *st, cudaStream_t s,
-                                 KernelTimer *kt);
-// C_mn -= P_m P_n^T for n = col0 .. col1 - 1, m = n .. T - 1.  counter: a zeroed word;
+// One problem as the kernels see it.
+struct F64Prob {
+    Tiles tl;
+    DevStatus *st;
+    F64Rows panel;            // K = b: row r of tile m at row0 + (m - k - 1) b + r
+    F64Rows inner;            // K = 64, the current 64-column block: row0 + (m - k) b + r
+    unsigned long long *ctr;  // tc64_counters(b, T) zeroed work counters
+    double *w16;              // inverses of the block's four 16 x 16 diagonal blocks
+};
+
+// The problems of a launch (one per grid row): one, or count of them in device memory with
+// Tmax tiles at most.
+struct F64Set {
+    const F64Prob *arr;
+    F64Prob one;
+    int count, b, Tmax;
+    __device__ const F64Prob &get(int i) const { return arr ? arr[i] : one; }
+};
+
+// Work counters of a problem: two trailing updates and b / 64 inner ones per step.
+inline size_t tc64_counters(int b, int T) { return (size_t)T * (2 + b / kF64Panel); }
+constexpr size_t kW16Doubles = 4 * 16 * 16;
+
+struct F64Maps {
+    CUtensorMap a, b, ia, ib;  // panel slices, inner slices
+};
+// Over slice arrays of rows (K = b) and irows (K = 64) rows.
+cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64Maps *maps);
+
+// Device scratch of one tensor-core FP64 factorisation, and the problem on it.
+size_t tc64_scratch_bytes(int b, int T);
+F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st);
+
+// POTRF of tile (k, k) and the solves of every tile below it, in 64-column blocks.
+cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, cudaStream_t s, KernelTimer *kt);
+// Slices of the solved panel tiles (k + 1 .. T - 1, k).
+cudaError_t launch_slice_panel64(const F64Set &set, int k, cudaStream_t s, KernelTimer *kt);
+// C_mn -= P_m P_n^T, m = n .. T - 1.  part 0: n = k + 1 .. T - 1; 1: n = k + 1; 2: the rest.
 // reserve: SMs left to other streams.
-cudaError_t launch_update_tc64(const F64Maps &maps, const Tiles &tl, int k, int col0, int col1, const F64Panel &p,
-                               unsigned long long *counter, int reserve, DevStatus *st, cudaStream_t s, KernelTimer *kt);
+cudaError_t launch_update_tc64(const F64Maps &maps, const F64Set &set, int k, int part, int reserve, cudaStream_t s,
+                               KernelTimer *kt);
 
 }  // namespace egs
