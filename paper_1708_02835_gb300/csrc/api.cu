@@ -151,8 +151,8 @@ static MixedLayout make_mixed_layout(const TileGeom &g, int band, egs_precision 
     off += 256;
     L.mtab = off;
     off += align256(EGS_MT_SCRATCH_DOUBLES * sizeof(double));
-    L.pctr = off;
-    off += align256((size_t)g.T * potrf_diag_scratch_words(g.b) * sizeof(unsigned));
+    L.dpan = off;
+    off += tc64_solo_bytes(g.b, g.T);
     L.rs = off;
     off += 2 * align256((size_t)(g.T > 1 ? g.T - 1 : 1) * g.b * sizeof(float));
     L.total = off;
@@ -261,7 +261,7 @@ cudaError_t eval_enqueue(const EvalSetup &es, const double *dlocs, const double 
         mb.partials = (double *)(ws + ML.partials);
         mb.err = (int *)(ws + ML.err);
         mb.mtab = (double *)(ws + ML.mtab);
-        mb.pctr = (unsigned *)(ws + ML.pctr);
+        mb.dpan = ws + ML.dpan;
         mb.xband = es.xband;
         for (int i = 0; i < 2; ++i)
             mb.rs[i] = (float *)(ws + ML.rs + i * align256((size_t)(g.T > 1 ? g.T - 1 : 1) * g.b * sizeof(float)));
@@ -283,15 +283,20 @@ cudaError_t eval_enqueue(const EvalSetup &es, const double *dlocs, const double 
     double *partials = (double *)(ws + es.L.partials);
     if (ev) cudaEventRecord(ev[0], s);
     cudaError_t e = launch_matern_tiles_f64(dlocs, dlocs + n, g, es.P, tiles, s, kt, (double *)(ws + es.L.mtab));
+    if (e == cudaSuccess && es.tc) e = launch_pad_vector(dz, n, zpad, (int64_t)g.T * g.b, s, kt);
     if (e == cudaSuccess) {
         if (ev) cudaEventRecord(ev[1], s);
-        e = launch_potrf_tiles_f64(tiles, g, st, s, kt, (unsigned *)(ws + es.L.pctr), es.tc ? ws + es.L.tc : nullptr);
+        e = launch_potrf_tiles_f64(tiles, g, st, s, kt, (unsigned *)(ws + es.L.pctr), es.tc ? ws + es.L.tc : nullptr,
+                                   zpad);
     }
-    if (e == cudaSuccess) {
-        if (ev) cudaEventRecord(ev[2], s);
-        e = launch_pad_vector(dz, n, zpad, (int64_t)g.T * g.b, s, kt);
+    if (e == cudaSuccess && ev) cudaEventRecord(ev[2], s);
+    if (es.tc) {
+        const Tiles tl{tiles, nullptr, g.b, g.T, g.T};
+        if (e == cudaSuccess) e = launch_logdet_quad(tl, n, zpad, partials, st, s, kt);
+    } else {
+        if (e == cudaSuccess) e = launch_pad_vector(dz, n, zpad, (int64_t)g.T * g.b, s, kt);
+        if (e == cudaSuccess) e = launch_trsv_tiles_f64(tiles, g, zpad, partials, st, s, kt);
     }
-    if (e == cudaSuccess) e = launch_trsv_tiles_f64(tiles, g, zpad, partials, st, s, kt);
     if (e == cudaSuccess && ev) cudaEventRecord(ev[3], s);
     return e;
 }

@@ -138,6 +138,145 @@ __device__ __forceinline__ bool potrf64_smem(double *A, int ld, int64_t row0, De
 }
 
 // ---------------------------------------------------------------------------
+// Cholesky of a 64 x 64 block by one CTA of 256 threads, with the right-hand side (z, may be
+// NULL) carried along as a 65th row, so that it leaves as y = L^-1 z.
+//
+// Bound by the FP64 pipe's issue rate within one SM: a warp-wide FP64 instruction occupies
+// its sub-partition for 64 clocks whether 1 or 32 lanes are active (measured; a dependent one
+// can follow at once), so what counts is the number of FP64 instructions on the longest
+// sub-partition, not latency:
+//  - L D L^T (no square root between pivots): with y ~ 1 / d from the hardware's approximation,
+//    e = 1 - d y, the column a / d = a y (1 + e + e^2) (Newton's iteration one order up) costs
+//    four instructions; the square roots are taken for all 64 columns at the end;
+//  - panels of 4 columns: warps 0 .. 2 each factor the 4 x 4 block in lanes 0 .. 3, redundantly
+//    (each has a sub-partition of its own), while lanes 4 .. 31 carry 28 rows below it, so that
+//    the rows below cost no instruction;
+//  - the 4-term updates of the entries right of the panel are spread over all lanes.
+// 64 pivots x 22 / 4 instructions of panels, about 400 of updates: 24 us (115 us with 16-column
+// panels, a thread per row below them and a square root per pivot).
+//
+// Leaves L (zero upper half), y in row 64 and 1 / L_jj in sm; false if a pivot is not positive
+// (its row is recorded as row0 + j).
+// ---------------------------------------------------------------------------
+struct Chol64Smem {
+    double S[65][65];
+    double W[65][5];  // a / d of the panel's columns
+    double rd[64];
+    int fail_j;
+};
+
+// 1 / sqrt(d) for normal d > 0: the hardware's approximation and one step of Householder's
+// third-order iteration.
+__device__ __forceinline__ double rsqrt_iter(double d)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-(d * y), y, 1.0);
+    return fma(fma(e, 0.375, 0.5), y * e, y);
+}
+
+__device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld, const double *z, int64_t row0,
+                                         DevStatus *st)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // a block far from 1 is scaled by 4^h, so that the reciprocals stay in range
+    const int e0 = ((__double2hiint(A[0]) >> 20) & 0x7FF) - 1023;
+    const int h = (e0 > 400 || e0 < -400) && e0 != 1024 ? -(e0 >> 1) : 0;
+    double v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        const int e = tid + 256 * q;
+        v[q] = (e & 63) <= (e >> 6) ? A[(size_t)(e >> 6) * ld + (e & 63)] : 0.0;
+    }
+    if (h != 0) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = scalbn(v[q], 2 * h);
+    }
+#pragma unroll
+    for (int q = 0; q < 16; ++q) sm.S[(tid + 256 * q) >> 6][tid & 63] = v[q];
+    if (z && tid < 64) sm.S[64][tid] = z[tid];
+    if (tid == 0) sm.fail_j = -1;
+    __syncthreads();
+    const int zr = z ? 1 : 0;
+#pragma unroll 1
+    for (int p0 = 0; p0 < 64; p0 += 4) {
+        const int q0 = p0 + 4, m = 64 - q0;  // rows and columns left
+        double a[4];
+        if (28 * warp < m + zr || warp == 0) {
+            const int t = 28 * warp + lane - 4;  // index among the rows below, z the last
+            const int i = lane < 4 ? p0 + lane : (t < m ? q0 + t : 64);
+            double w[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) a[c] = sm.S[i][p0 + c];
+            bool ok = true;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const double d = __shfl_sync(0xffffffffu, a[j], j);
+                if (ok && !(d > 0.0)) {
+                    ok = false;
+                    if (tid == 0) sm.fail_j = p0 + j;
+                }
+                double y;
+                asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+                const double e = fma(-d, y, 1.0);
+                const double ay = a[j] * y, u = fma(e, e, e);
+                w[j] = fma(ay, u, ay);
+#pragma unroll
+                for (int c = j + 1; c < 4; ++c) a[c] = fma(-a[j], __shfl_sync(0xffffffffu, w[j], c), a[c]);
+            }
+            if (lane >= 4 && t < m + zr) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    sm.S[i][p0 + c] = a[c];
+                    sm.W[i][c] = w[c];
+                }
+            }
+        }
+        __syncthreads();
+        if (tid < 4) {  // only now: every warp has read the block
+#pragma unroll
+            for (int c = 0; c < 4; ++c) sm.S[p0 + tid][p0 + c] = a[c];
+        }
+        if (sm.fail_j >= 0) {
+            if (tid == 0) atomicMin(&st->fail_index, (unsigned long long)(row0 + sm.fail_j));
+            return false;
+        }
+        // lower triangle of the rows and columns from q0 on, then the z row (the triangle's
+        // next row but for its last entry)
+        const int cnt = m * (m + 1) / 2 + (zr ? m : 0);
+        for (int e = tid; e < cnt; e += 256) {
+            int ii = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+            if (ii * (ii + 1) / 2 > e) --ii;
+            if ((ii + 1) * (ii + 2) / 2 <= e) ++ii;
+            const int i = ii < m ? q0 + ii : 64, c = q0 + e - ii * (ii + 1) / 2;
+            double acc = sm.S[i][c];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc = fma(-sm.S[i][p0 + j], sm.W[c][j], acc);
+            sm.S[i][c] = acc;
+        }
+        __syncthreads();
+    }
+    if (tid < 64) {
+        const double r = rsqrt_iter(sm.S[tid][tid]);
+        sm.rd[tid] = r;
+    }
+    __syncthreads();
+    const int jc = tid & 63;
+    const double rj = sm.rd[jc];
+    for (int i = tid >> 6; i < 64 + zr; i += 4) sm.S[i][jc] = jc <= i ? sm.S[i][jc] * rj : 0.0;
+    if (h != 0) {
+        __syncthreads();
+        for (int i = tid >> 6; i < 64; i += 4) sm.S[i][jc] = scalbn(sm.S[i][jc], -h);
+        if (tid < 64) {
+            sm.rd[tid] = scalbn(sm.rd[tid], h);
+            if (z) sm.S[64][tid] = scalbn(sm.S[64][tid], h);
+        }
+    }
+    __syncthreads();
+    return true;
+}
+
+// ---------------------------------------------------------------------------
 // C (32 x 32, row stride ldc) -= Am (32 x K) An (32 x K)^T; 2 x 2 outputs per
 // thread (rows ty + 16 i, columns tx + 16 j).  FP64 or FP32 operands, FP64
 // arithmetic.  256 threads.

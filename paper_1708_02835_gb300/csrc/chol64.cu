@@ -246,13 +246,13 @@ cudaError_t launch_update_f64(const Tiles &tl, int k, int64_t ntri, DevStatus *s
 }
 
 cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *st, cudaStream_t s, KernelTimer *kt,
-                                   unsigned *ctr, void *tc_scratch)
+                                   unsigned *ctr, void *tc_scratch, double *z)
 {
     const int T = g.T;
     const Tiles tl{tiles, nullptr, g.b, T, T};
     cudaError_t e = cudaSuccess;
     if (tc_scratch) {
-        const F64Set set{nullptr, tc64_problem(tc_scratch, tl, st), 1, g.b, T};
+        const F64Set set{nullptr, tc64_problem(tc_scratch, tl, st, z), 1, g.b, T, 0};
         F64Maps maps;
         e = make_f64_maps(set.one.panel, set.one.inner, g.b, &maps);
         if (e == cudaSuccess)

@@ -160,9 +160,10 @@ cudaError_t launch_matern_table(const egs_matern_params &P, double *tab, cudaStr
 // Tile Cholesky in place (FP64).  Stops doing work once st->fail_index is set.
 // ctr: T * potrf_diag_scratch_words(b) words of device scratch for the
 // one-launch diagonal POTRFs (zeroed here).  tc_scratch: tc64_scratch_bytes(b, T) bytes
-// for the tensor-core update, or NULL for the DFMA update.
+// for the tensor-core update, or NULL for the DFMA update.  With it, z (T b doubles, may be
+// NULL) is solved along: L^-1 z in place.
 cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *st, cudaStream_t s,
-                                   KernelTimer *kt, unsigned *ctr, void *tc_scratch = nullptr);
+                                   KernelTimer *kt, unsigned *ctr, void *tc_scratch = nullptr, double *z = nullptr);
 // Counter words one diagonal tile's one-launch POTRF needs.
 size_t potrf_diag_scratch_words(int b);
 
@@ -170,6 +171,10 @@ size_t potrf_diag_scratch_words(int b);
 // with per-tile log-det / dot partials and the final assembly into st->result.
 cudaError_t launch_trsv_tiles_f64(const double *tiles, const TileGeom &g, double *zpad, double *partials,
                                   DevStatus *st, cudaStream_t s, KernelTimer *kt = nullptr);
+
+// log|Sigma| and y . y from the factor's diagonal and y = L^-1 z, into st->result.
+cudaError_t launch_logdet_quad(const Tiles &tl, int64_t n, const double *y, double *partials, DevStatus *st,
+                               cudaStream_t s, KernelTimer *kt);
 
 // Sigma(theta) into any Tiles storage.  For
 // a mixed layout with the Euclidean distance the off-band tiles are evaluated
@@ -201,7 +206,7 @@ struct MixedBuffers {
     void *oz[2];      // FP32 mode: BF16 slices of the panel rows (ozaki_slices_bytes), step k uses k % 2
     double *ozs[2];   // FP32 mode: their row scales, (T-1) b doubles each
     double *mtab;     // EGS_MT_SCRATCH_DOUBLES: the generator's local polynomials (general nu)
-    unsigned *pctr;   // T * potrf_diag_scratch_words(b): counters of the one-launch diagonal POTRFs
+    void *dpan;       // tc64_solo_bytes(b, T): scratch of the diagonal tiles' POTRFs
     float *rs[2];     // FP32 mode: the power-of-two scales of the split-FP16 panel rows, (T-1) b each
     int xband;        // FP32 mode: tiles with i - j < xband get FP64-accurate updates (>= tl.band)
 };
@@ -226,7 +231,7 @@ struct Layout {
     size_t tiles, locs, z, zpad, partials, status, mtab, pctr, tc, total;
 };
 struct MixedLayout {
-    size_t f64, f32, slots, panel, oz, l32, wsp, vinv, locs, z, vec, partials, status, err, mtab, pctr, rs, total;
+    size_t f64, f32, slots, panel, oz, l32, wsp, vinv, locs, z, vec, partials, status, err, mtab, dpan, rs, total;
 };
 struct EvalSetup {
     TileGeom g;

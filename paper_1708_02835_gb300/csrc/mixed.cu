@@ -25,6 +25,7 @@
 // regenerated tile by tile (symv_regen.cu), x1 = x0 + L^-T L^-1 r, quad = Z^T x1.
 #include "blocks.cuh"
 #include "slices.cuh"
+#include "tc64.cuh"
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -658,8 +659,12 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_panel, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_col, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_diag, cudaEventDisableTiming);
-    if (e == cudaSuccess)  // the one-launch diagonal POTRFs' counters
-        e = cudaMemsetAsync(mb.pctr, 0, (size_t)T * potrf_diag_scratch_words(b) * sizeof(unsigned), s);
+    // POTRF of a diagonal tile: the FP64 path's 64-column blocks, on that tile alone (tile 512:
+    // OLD with the task graph of 32 x 32 blocks, NEW)
+    const F64Set diag{nullptr, tc64_problem(mb.dpan, tl, st, nullptr, true), 1, b, T, 1};
+    F64Maps dmaps;
+    if (e == cudaSuccess) e = make_f64_maps(diag.one.panel, diag.one.inner, b, &dmaps);
+    if (e == cudaSuccess) e = cudaMemsetAsync(diag.one.ctr, 0, tc64_counters(b, T) * sizeof(unsigned long long), s);
     if (e == cudaSuccess) e = cudaEventRecord(ev_col, s);  // the side stream starts after prior work on s
     KernelTimer *kts = kt;  // side-stream kernels are timed with events on the side stream
     for (int k = 0; k < T && e == cudaSuccess; ++k) {
@@ -677,7 +682,7 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
         // before the call (Sigma generation).
         if (k == 0) e = cudaStreamWaitEvent(side, ev_col, 0);
         if (e == cudaSuccess)
-            e = launch_potrf_diag(tl, k, st, side, kts, mb.pctr + (size_t)k * potrf_diag_scratch_words(b));
+            e = launch_panel64(dmaps, diag, k, side, kts);
         // FP32 mode: W = L_kk^-1 (and V_k = W^T for the solves) for the main
         // stream's off-band TRSM, off the main stream
         float *wsp = mb.wsp + (size_t)(k & 1) * 2 * tl.bb();

@@ -86,6 +86,35 @@ __global__ void k_finalize(const double *__restrict__ partials, int T, int64_t n
     }
 }
 
+// Partials of tile k = blockIdx.x for an already solved y: sum log L_ii and sum y_i^2.
+__global__ void __launch_bounds__(256) k_logdet_quad(Tiles tl, const double *__restrict__ y,
+                                                     double *__restrict__ partials, const DevStatus *st)
+{
+    if (failed_s(st)) return;
+    __shared__ double red[256];
+    const int b = tl.b, k = (int)blockIdx.x;
+    const double *L = tl.t64(k, k), *yk = y + (size_t)k * b;
+    double a = 0.0, q = 0.0;
+    for (int i = threadIdx.x; i < b; i += 256) {
+        a += log(L[(size_t)i * (b + 1)]);
+        q = fma(yk[i], yk[i], q);
+    }
+    const double lsum = block_sum(a, red);
+    __syncthreads();
+    const double qsum = block_sum(q, red);
+    if (threadIdx.x == 0) {
+        partials[k] = lsum;
+        partials[tl.T + k] = qsum;
+    }
+}
+
+cudaError_t launch_logdet_quad(const Tiles &tl, int64_t n, const double *y, double *partials, DevStatus *st,
+                               cudaStream_t s, KernelTimer *kt)
+{
+    EGS_LAUNCH(kt, KC_TRSV, s, k_logdet_quad<<<(unsigned)tl.T, 256, 0, s>>>(tl, y, partials, st));
+    return launch_finalize(partials, tl.T, n, st, s, kt);
+}
+
 // Z = L e over the lower tiles of L (Algorithm 1, dtrmm): out[i*b + r] =
 // sum_{j <= i} L_ij[r][:] . e_j, one warp per row, fixed shuffle tree.
 // Diagonal tiles hold L with a zero strict upper triangle.  grid = (T, b/8).

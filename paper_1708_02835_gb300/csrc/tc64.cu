@@ -133,10 +133,10 @@ __global__ void __launch_bounds__(256) k_slice_panel64(const __grid_constant__ F
 // ---- the panel ----------------------------------------------------------------
 //
 // Tile column k is factored in 64-column blocks, each in three launches:
-//   k_diag64    L_jj = chol of the 64 x 64 diagonal block and the inverses of its four
-//               16 x 16 diagonal blocks, one CTA;
+//   k_diag64    L_jj = chol of the 64 x 64 diagonal block and the inverses of its eight
+//               8 x 8 diagonal blocks, one CTA;
 //   k_solve64   the rows below, in the tile and in every tile under it: X L_jj^T = A by
-//               16-column blocks, X_p = (A_p - sum_{i<p} X_i L_pi^T) L_pp^-T, and X's slices
+//               8-column blocks, X_p = (A_p - sum_{i<p} X_i L_pi^T) L_pp^-T, and X's slices
 //               (K = 64, exponents of their own);
 //   k_tc_f64    the update of the panel's columns right of the block (inner work).
 // Why 64: the FP64 pipe does n^2 w / 2 FMAs in all solves of width w, 14.7 ms at
@@ -145,37 +145,41 @@ __global__ void __launch_bounds__(256) k_slice_panel64(const __grid_constant__ F
 // diagonal tiles and 100 ms of whole-tile solves became 30 + 17 + 12 ms; the evaluation went
 // from 193 to 120 ms, that of n = 5,000 (tile 256) from 27.0 to 18.9 ms.
 constexpr int PW = kF64Panel;
-constexpr int PI = 16;       // inverted sub-blocks
-static_assert(kW16Doubles == (PW / PI) * PI * PI, "one inverse per 16 x 16 diagonal block");
+constexpr int PI = 8;        // inverted sub-blocks
+static_assert(kWinvDoubles == (PW / PI) * PI * PI, "one inverse per 8 x 8 diagonal block");
 
-// One CTA per problem, 256 threads.  w16: the inverses W_pp, row-major, at 256 p.
+// One CTA per problem, 256 threads.  winv: the inverses W_pp, row-major, at 64 p.  The block
+// of the right-hand side becomes y_j.
 __global__ void __launch_bounds__(256) k_diag64(const __grid_constant__ F64Set set, int k, int j)
 {
-    __shared__ Potrf64Smem sm;
+    __shared__ Chol64Smem sm;
     const F64Prob &P = set.get(blockIdx.y);
     const Tiles &tl = P.tl;
-    DevStatus *st = P.st;
-    double *w16 = P.w16;
-    if (k >= tl.T || failed(st)) return;
+    if (k >= tl.T || failed(P.st)) return;
     const int b = tl.b, tid = threadIdx.x;
     double *A = tl.t64(k, k) + (size_t)j * PW * (b + 1);
-    if (!potrf64_smem_s(sm, A, b, (int64_t)k * b + j * PW, st)) return;
-    const int right = b - (j + 1) * PW;
-    for (int e = tid; e < PW * right; e += 256) A[(size_t)(e / right) * b + PW + e % right] = 0.0;
-    // column c of W_pp by forward substitution, one thread each (the factor is still in sm)
+    double *z = P.z ? P.z + (size_t)k * b + j * PW : nullptr;
+    if (!chol64_s(sm, A, b, z, (int64_t)k * b + j * PW, P.st)) return;
+    // column c of W_pp by forward substitution, one thread each
     if (tid < PW) {
         const int p = tid / PI, c = tid % PI, q0 = p * PI;
         double w[PI];
 #pragma unroll
-        for (int i = 0; i < PI; ++i) {
-            double v = i == c ? 1.0 : 0.0;
+        for (int i = 0; i < PI; ++i) w[i] = i == c ? 1.0 : 0.0;
 #pragma unroll
-            for (int l = 0; l < i; ++l) v = fma(-sm.S[q0 + i][q0 + l], w[l], v);
-            w[i] = v * sm.rd[q0 + i];
+        for (int i = 0; i < PI; ++i) {
+            w[i] *= sm.rd[q0 + i];
+#pragma unroll
+            for (int l = i + 1; l < PI; ++l) w[l] = fma(-sm.S[q0 + l][q0 + i], w[i], w[l]);
         }
 #pragma unroll
-        for (int i = 0; i < PI; ++i) w16[p * PI * PI + i * PI + c] = w[i];
+        for (int i = 0; i < PI; ++i) P.winv[p * PI * PI + i * PI + c] = w[i];
+        if (z) z[tid] = sm.S[64][tid];
     }
+    for (int e = tid; e < PW * PW; e += 256) A[(size_t)(e >> 6) * b + (e & 63)] = sm.S[e >> 6][e & 63];
+    const int right = b - (j + 1) * PW;
+    for (int r = tid >> 5; r < PW; r += 8)
+        for (int c = tid & 31; c < right; c += 32) A[(size_t)r * b + PW + c] = 0.0;
 }
 
 // One warp slices the 64 entries of a row: lane's entries 2 lane, 2 lane + 1.
@@ -196,64 +200,67 @@ __device__ __forceinline__ void slice7_row64(double x0, double x1, uint16_t *__r
         *reinterpret_cast<uint32_t *>(dst + (size_t)i * stride + 2 * lane) = d0[i] | (d1[i] << 16);
 }
 
-// Panel rows (j + 1) 64 .. (T - k) b - 1, RB rows per CTA, 256 threads.  FP64-pipe bound
-// (RB 64 64 / 2 FMAs and the 16 x 16 products at 2 a clock per SM): RB = 16 while that
-// leaves SMs idle otherwise.
+// Panel rows (j + 1) 64 .. (T - k) b - 1, RB rows and 8 RB threads per CTA: thread (row, c) has
+// column c of each 8-column block.  FP64-pipe bound: 288 FMAs a thread at 64 clocks a warp
+// and sub-partition, 9 us for one warp on each (RB = 16), 18 us for two; RB = 32 (the staged
+// block of L serves twice the rows) once RB = 16 fills the SMs.
 template <int RB>
-__global__ void __launch_bounds__(256) k_solve64(const __grid_constant__ F64Set set, int k, int j)
+__global__ void __launch_bounds__(8 * RB) k_solve64(const __grid_constant__ F64Set set, int k, int j)
 {
+    constexpr int NT = 8 * RB;
+    // L below its 8 x 8 diagonal blocks: rows 8 .. 63, columns 0 .. 55
+    __shared__ double Ls[PW - PI][PW - PI + 1], Xs[RB][PW + 1], Ws[PW][PI + 1];
     const F64Prob &P = set.get(blockIdx.y);
     const Tiles &tl = P.tl;
-    const double *__restrict__ w16 = P.w16;
-    if ((int64_t)(j + 1) * PW + (int64_t)blockIdx.x * RB >= (int64_t)(tl.T - k) * tl.b || failed(P.st)) return;
-    constexpr int RT = RB / 16;  // rows per thread
-    // L below its 16 x 16 diagonal blocks: rows 16 .. 63, columns 0 .. 47
-    __shared__ double Ls[PW - PI][PW - PI + 1], Xs[RB][PW + 1], Ws[PW][PI + 1];
-    const int b = tl.b, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int T = set.solo ? k + 1 : tl.T;
+    if ((int64_t)(j + 1) * PW + (int64_t)blockIdx.x * RB >= (int64_t)(T - k) * tl.b || failed(P.st)) return;
+    const int b = tl.b, tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
     const int pr0 = (j + 1) * PW + (int)blockIdx.x * RB;
     double *X = tl.t64(k + pr0 / b, k) + (size_t)(pr0 % b) * b + j * PW;
     const double *L = tl.t64(k, k) + (size_t)j * PW * (b + 1);
-    for (int e = tid; e < (PW - PI) * (PW - PI); e += 256)
-        Ls[e / (PW - PI)][e % (PW - PI)] = L[(size_t)(PI + e / (PW - PI)) * b + e % (PW - PI)];
-    for (int e = tid; e < RB * PW; e += 256) Xs[e >> 6][e & 63] = X[(size_t)(e >> 6) * b + (e & 63)];
-    for (int e = tid; e < (int)kW16Doubles; e += 256) Ws[e >> 4][e & 15] = w16[e];
+    for (int e = tid; e < RB * PW; e += NT) Xs[e >> 6][e & 63] = X[(size_t)(e >> 6) * b + (e & 63)];
+#pragma unroll 4
+    for (int e = tid; e < PW * PW; e += NT) {
+        const int r = e >> 6, c = e & 63;
+        if (r >= PI && c < PW - PI && c < r) Ls[r - PI][c] = L[(size_t)r * b + c];
+    }
+    for (int e = tid; e < (int)kWinvDoubles; e += NT) Ws[e >> 3][e & 7] = P.winv[e];
     __syncthreads();
 #pragma unroll
     for (int p = 0; p < PW / PI; ++p) {
-        double r[RT];
-#pragma unroll
-        for (int i = 0; i < RT; ++i) r[i] = Xs[ty + 16 * i][PI * p + tx];
-        for (int l = 0; l < PI * p; ++l) {
-            const double lv = Ls[PI * (p - 1) + tx][l];
-#pragma unroll
-            for (int i = 0; i < RT; ++i) r[i] = fma(-Xs[ty + 16 * i][l], lv, r[i]);
-        }
-        // a row's 16 entries belong to one half-warp
+        double r = Xs[ty][PI * p + tx];
+#pragma unroll 8
+        for (int l = 0; l < PI * p; ++l) r = fma(-Xs[ty][l], Ls[PI * (p - 1) + tx][l], r);
+        // a row's 8 entries belong to 8 lanes of one warp
         __syncwarp();
-#pragma unroll
-        for (int i = 0; i < RT; ++i) Xs[ty + 16 * i][PI * p + tx] = r[i];
+        Xs[ty][PI * p + tx] = r;
         __syncwarp();
-        double x[RT];
+        double x = 0.0;
 #pragma unroll
-        for (int i = 0; i < RT; ++i) x[i] = 0.0;
-#pragma unroll
-        for (int l = 0; l < PI; ++l) {
-            const double wv = Ws[PI * p + tx][l];
-#pragma unroll
-            for (int i = 0; i < RT; ++i) x[i] = fma(Xs[ty + 16 * i][PI * p + l], wv, x[i]);
-        }
+        for (int l = 0; l < PI; ++l) x = fma(Xs[ty][PI * p + l], Ws[PI * p + tx][l], x);
         __syncwarp();
-#pragma unroll
-        for (int i = 0; i < RT; ++i) Xs[ty + 16 * i][PI * p + tx] = x[i];
+        Xs[ty][PI * p + tx] = x;
         __syncwarp();
     }
     __syncthreads();
     const int lane = tid & 31;
-    for (int r = tid >> 5; r < RB; r += 8) {
+    // z_row -= X_row . y_j: the forward solve, while the rows are here
+    double y0 = 0.0, y1 = 0.0;
+    if (P.z) {
+        y0 = P.z[(size_t)k * b + j * PW + 2 * lane];
+        y1 = P.z[(size_t)k * b + j * PW + 2 * lane + 1];
+    }
+    for (int r = tid >> 5; r < RB; r += NT / 32) {
         const size_t sr = P.inner.row0 + pr0 + r;
         const double x0 = Xs[r][2 * lane], x1 = Xs[r][2 * lane + 1];
         *reinterpret_cast<double2 *>(X + (size_t)r * b + 2 * lane) = make_double2(x0, x1);
         slice7_row64(x0, x1, P.inner.sl + sr * PW, P.inner.rows * PW, P.inner.ex + sr);
+        if (P.z) {
+            double v = fma(x0, y0, x1 * y1);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            if (lane == 0) P.z[(size_t)k * b + pr0 + r] -= v;
+        }
     }
 }
 
@@ -272,15 +279,15 @@ struct F64Item {
 constexpr int kF64Cols = 8;
 struct F64Work {
     const Tiles &tl;
-    int k, col0, col1;
+    int T, k, col0, col1;
     bool inner;
     __host__ __device__ int row_blocks() const { return (tl.b + FM - 1) / FM; }
     __host__ __device__ int kchunks() const { return inner ? 1 : tl.b / FKC; }
     __host__ __device__ int64_t items() const
     {
         const int64_t c = col1 - col0;
-        if (inner) return c * row_blocks() * (tl.T - k);
-        const int64_t h = tl.T - col0;
+        if (inner) return c * row_blocks() * (T - k);
+        const int64_t h = T - col0;
         return (c * h - c * (c - 1) / 2) * row_blocks() * (tl.b / FN);
     }
     __device__ size_t slice_row(int m) const { return (size_t)(m - k - (inner ? 0 : 1)) * tl.b; }
@@ -301,7 +308,7 @@ struct F64Work {
             for (;;) {
                 const int wd = min(kF64Cols, col1 - c_lo);
                 const int64_t tri = (int64_t)wd * (wd + 1) / 2;
-                const int64_t cnt = tri + (int64_t)(tl.T - c_lo - wd) * wd;
+                const int64_t cnt = tri + (int64_t)(T - c_lo - wd) * wd;
                 if (t < cnt) {
                     if (t < tri) {
                         int ii = 0, u = (int)t;
@@ -406,9 +413,10 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
          const __grid_constant__ F64Set set, int k, int c0, int c1, int inner, int slot)
 {
     const F64Prob &P = set.get(blockIdx.y);
-    if (P.tl.T <= k) return;
+    const int T = set.solo ? k + 1 : P.tl.T;
+    if (T <= k) return;
     // trailing: columns k + c0 .. min(k + c1, T) - 1; inner: the blocks c0 .. c1 - 1 of column k
-    const F64Work work{P.tl, k, inner ? c0 : k + c0, inner ? c1 : min(k + c1, P.tl.T), inner != 0};
+    const F64Work work{P.tl, T, k, inner ? c0 : k + c0, inner ? c1 : min(k + c1, T), inner != 0};
     if (work.col0 >= work.col1) return;
     const int64_t nitems = work.items();
     if ((int64_t)blockIdx.x >= nitems) return;
@@ -694,18 +702,24 @@ int device_sms()
 static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Slices and exponents of the panel (K = b) and of its 64-column blocks (K = 64, the
-// diagonal tile's rows too), the work counters, the 16 x 16 inverses.
+// diagonal tile's rows too), the work counters, the 8 x 8 inverses.
+size_t tc64_solo_bytes(int b, int T)
+{
+    return a256((size_t)b * PW * kF64Slices * sizeof(uint16_t)) + a256((size_t)b * sizeof(int)) +
+           a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(kWinvDoubles * sizeof(double));
+}
+
 size_t tc64_scratch_bytes(int b, int T)
 {
     const size_t R = (size_t)(T - 1) * (size_t)b, R1 = R + b;
     return a256(R * b * kF64Slices * sizeof(uint16_t)) + a256(R * sizeof(int)) +
            a256(R1 * PW * kF64Slices * sizeof(uint16_t)) + a256(R1 * sizeof(int)) +
-           a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(kW16Doubles * sizeof(double));
+           a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(kWinvDoubles * sizeof(double));
 }
 
-F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st)
+F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st, double *z, bool solo)
 {
-    const size_t R = (size_t)(tl.T - 1) * (size_t)tl.b, R1 = R + tl.b;
+    const size_t R = solo ? 0 : (size_t)(tl.T - 1) * (size_t)tl.b, R1 = R + tl.b;
     char *p = (char *)scratch;
     auto take = [&p](size_t bytes) {
         char *q = p;
@@ -715,6 +729,7 @@ F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st)
     F64Prob P;
     P.tl = tl;
     P.st = st;
+    P.z = z;
     P.panel.sl = (uint16_t *)take(R * tl.b * kF64Slices * sizeof(uint16_t));
     P.panel.ex = (int *)take(R * sizeof(int));
     P.panel.rows = R;
@@ -723,14 +738,16 @@ F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st)
     P.inner.rows = R1;
     P.panel.row0 = P.inner.row0 = 0;
     P.ctr = (unsigned long long *)take(tc64_counters(tl.b, tl.T) * sizeof(unsigned long long));
-    P.w16 = (double *)take(kW16Doubles * sizeof(double));
+    P.winv = (double *)take(kWinvDoubles * sizeof(double));
     return P;
 }
 
 cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64Maps *maps)
 {
-    cudaError_t e = make_map3(&maps->a, panel.sl, panel.rows, (uint64_t)b, FM, 1);
-    if (e == cudaSuccess) e = make_map3(&maps->b, panel.sl, panel.rows, (uint64_t)b, FN, kF64Slices);
+    cudaError_t e = cudaSuccess;
+    if (panel.rows) e = make_map3(&maps->a, panel.sl, panel.rows, (uint64_t)b, FM, 1);
+    else maps->a = maps->b = CUtensorMap{};
+    if (e == cudaSuccess && panel.rows) e = make_map3(&maps->b, panel.sl, panel.rows, (uint64_t)b, FN, kF64Slices);
     if (e == cudaSuccess) e = make_map3(&maps->ia, inner.sl, inner.rows, PW, FM, 1);
     if (e == cudaSuccess) e = make_map3(&maps->ib, inner.sl, inner.rows, PW, FN, kF64Slices);
     return e;
@@ -750,8 +767,9 @@ static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, con
 {
     cudaError_t e = cudaFuncSetAttribute(k_tc_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
     if (e != cudaSuccess) return e;
-    const Tiles tl{nullptr, nullptr, set.b, set.Tmax, set.Tmax};
-    const F64Work w{tl, k, inner ? c0 : k + c0, inner ? c1 : (k + c1 < set.Tmax ? k + c1 : set.Tmax), inner != 0};
+    const int T = set.solo ? k + 1 : set.Tmax;
+    const Tiles tl{nullptr, nullptr, set.b, T, T};
+    const F64Work w{tl, T, k, inner ? c0 : k + c0, inner ? c1 : (k + c1 < T ? k + c1 : T), inner != 0};
     if (w.col0 >= w.col1) return cudaSuccess;
     const dim3 grid(tc64_ctas(set, w.items(), reserve), (unsigned)set.count);
     EGS_LAUNCH(kt, KC_UPDATE, s, k_tc_f64<<<grid, FTHREADS, FSMEM, s>>>(a, b, set, k, c0, c1, inner, slot));
@@ -764,11 +782,11 @@ cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, cudaSt
     cudaError_t e = cudaSuccess;
     for (int j = 0; j < nj && e == cudaSuccess; ++j) {
         EGS_LAUNCH(kt, KC_POTRF, s, k_diag64<<<dim3(1, (unsigned)set.count), 256, 0, s>>>(set, k, j));
-        const int64_t rows = (int64_t)(set.Tmax - k) * set.b - (j + 1) * PW;
+        const int64_t rows = (int64_t)(set.solo ? 1 : set.Tmax - k) * set.b - (j + 1) * PW;
         if (rows > 0) {
             if (rows / 16 * set.count <= device_sms())
                 EGS_LAUNCH(kt, KC_TRSM, s,
-                           k_solve64<16><<<dim3((unsigned)(rows / 16), (unsigned)set.count), 256, 0, s>>>(set, k, j));
+                           k_solve64<16><<<dim3((unsigned)(rows / 16), (unsigned)set.count), 128, 0, s>>>(set, k, j));
             else
                 EGS_LAUNCH(kt, KC_TRSM, s,
                            k_solve64<32><<<dim3((unsigned)(rows / 32), (unsigned)set.count), 256, 0, s>>>(set, k, j));

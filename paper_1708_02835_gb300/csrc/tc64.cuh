@@ -26,10 +26,11 @@ struct F64Rows {
 struct F64Prob {
     Tiles tl;
     DevStatus *st;
+    double *z;                // T b: the right-hand side, solved along (L^-1 z); NULL: none
     F64Rows panel;            // K = b: row r of tile m at row0 + (m - k - 1) b + r
     F64Rows inner;            // K = 64, the current 64-column block: row0 + (m - k) b + r
     unsigned long long *ctr;  // tc64_counters(b, T) zeroed work counters
-    double *w16;              // inverses of the block's four 16 x 16 diagonal blocks
+    double *winv;             // inverses of the block's eight 8 x 8 diagonal blocks
 };
 
 // The problems of a launch (one per grid row): one, or count of them in device memory with
@@ -38,12 +39,13 @@ struct F64Set {
     const F64Prob *arr;
     F64Prob one;
     int count, b, Tmax;
+    int solo;  // 1: only the diagonal tile of a step (POTRF of one tile; launch_panel64 alone)
     __device__ const F64Prob &get(int i) const { return arr ? arr[i] : one; }
 };
 
 // Work counters of a problem: two trailing updates and b / 64 inner ones per step.
 inline size_t tc64_counters(int b, int T) { return (size_t)T * (2 + b / kF64Panel); }
-constexpr size_t kW16Doubles = 4 * 16 * 16;
+constexpr size_t kWinvDoubles = 8 * 8 * 8;
 
 struct F64Maps {
     CUtensorMap a, b, ia, ib;  // panel slices, inner slices
@@ -53,7 +55,8 @@ cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64
 
 // Device scratch of one tensor-core FP64 factorisation, and the problem on it.
 size_t tc64_scratch_bytes(int b, int T);
-F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st);
+size_t tc64_solo_bytes(int b, int T);  // of the POTRFs of T diagonal tiles
+F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st, double *z, bool solo = false);
 
 // POTRF of tile (k, k) and the solves of every tile below it, in 64-column blocks.
 cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, cudaStream_t s, KernelTimer *kt);
