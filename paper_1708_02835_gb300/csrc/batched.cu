@@ -19,6 +19,7 @@
 #include "batched_dag.cuh"
 #include "blocks.cuh"
 #include "matern.cuh"
+#include "tc64.cuh"
 
 namespace egs {
 
@@ -390,6 +391,30 @@ __global__ void __launch_bounds__(256) kb_finalize_mixed(BatchArgs a)
     }
 }
 
+// Tensor-core batches: the partials of tile k (item = (problem, tile)) from the factor's
+// diagonal and the solved right-hand side, as k_logdet_quad.
+__global__ void __launch_bounds__(256) kb_logdet_quad(BatchArgs a)
+{
+    int64_t local;
+    const BatchProblem &pr = a.probs[find_problem(a, blockIdx.x, local)];
+    if (failed(pr.st)) return;
+    __shared__ double red[256];
+    const int b = a.b, k = (int)local;
+    const double *L = dense_tiles(pr, b).t64(k, k), *y = pr.zpad + (size_t)k * b;
+    double s = 0.0, q = 0.0;
+    for (int i = threadIdx.x; i < b; i += 256) {
+        s += log(L[(size_t)i * (b + 1)]);
+        q = fma(y[i], y[i], q);
+    }
+    const double lsum = block_sum(s, red);
+    __syncthreads();
+    const double qsum = block_sum(q, red);
+    if (threadIdx.x == 0) {
+        pr.partials[k] = lsum;
+        pr.partials[pr.T + k] = qsum;
+    }
+}
+
 __global__ void __launch_bounds__(256) kb_finalize(BatchArgs a)
 {
     int64_t local;
@@ -427,6 +452,7 @@ using namespace egs;
 struct egs_batch {
     int nprob = 0, b = 0;
     bool mixed = false;  // EGS_MIX_FP32 batch (band kBatchBand)
+    int ntab = 0;        // problems with local polynomials of their own (the first ones)
     int band = 0;
     std::vector<int64_t> n;
     std::vector<int> T;
@@ -452,7 +478,15 @@ struct egs_batch {
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     int launches_per_run = 0;
-    // persistent scheduler (FP64 batches with tile <= 256): one launch over
+    // tensor-core batch: step-synchronous launches of the FP64 tensor-core factorisation over
+    // all problems (by falling T, so that the ones with a step k are the first active[k])
+    bool tc = false;
+    F64Prob *d_f64 = nullptr;
+    F64Maps maps;
+    std::vector<int> active;
+    unsigned long long *d_f64ctr = nullptr;
+    size_t f64ctr = 0;
+    // persistent scheduler (other FP64 batches with tile <= 256): one launch over
     // the task list of every problem
     bool dag = false;
     int4 *d_tasks = nullptr;
@@ -470,7 +504,7 @@ namespace {
 
 enum {
     L_GEN, L_POTRF, L_TRSM_SUB, L_SYRK_SUB, L_TRSM, L_TRSM32, L_UPDATE, L_PAD, L_TRSV, L_GEMV, L_FINAL,
-    L_COPY, L_TRSV_T, L_GEMV_T, L_SYMV_R, L_SYMV_C, L_RESID, L_AXPY, L_FINAL_M
+    L_COPY, L_FACTOR64, L_LDQ, L_TRSV_T, L_GEMV_T, L_SYMV_R, L_SYMV_C, L_RESID, L_AXPY, L_FINAL_M
 };
 
 constexpr int kBatchBand = 2;  // FP64 band of the mixed batches (tiles)
@@ -514,6 +548,13 @@ void plan_launches(egs_batch *B, std::vector<int64_t> &prefix)
     auto nb_of = [&](int q, int k) { return (int64_t)std::min(band_of(q) - 1, B->T[q] - k - 1); };
     auto vec_items = [&](int q) { return ((int64_t)B->T[q] * b + 255) / 256; };
     add(L_GEN, 0, 0, [&](int q) { return (int64_t)B->T[q] * (B->T[q] + 1) / 2 * nsub * nsub; });
+    if (B->tc) {
+        add(L_PAD, 0, 0, vec_items);
+        add(L_FACTOR64, 0, 0, [&](int) { return (int64_t)1; });
+        add(L_LDQ, 0, 0, [&](int q) { return (int64_t)B->T[q]; });
+        add(L_FINAL, 0, 0, [&](int) { return (int64_t)1; });
+        return;
+    }
     for (int k = 0; k < Tmax; ++k) {
         for (int p = 0; p < b; p += kIB) {
             const int64_t nrest = (b - p - kIB) / 16, n32 = (b - p - kIB) / 32;
@@ -563,9 +604,32 @@ void plan_launches(egs_batch *B, std::vector<int64_t> &prefix)
     add(L_FINAL_M, 0, 0, [&](int) { return (int64_t)1; });
 }
 
+// The tile Cholesky of every problem, step by step, on the tensor cores (tc64.cu).
+cudaError_t enqueue_factor64(egs_batch *B, cudaStream_t s, int *count)
+{
+    KernelTimer kt;
+    cudaError_t e = cudaMemsetAsync(B->d_f64ctr, 0, B->f64ctr * sizeof(unsigned long long), s);
+    const int Tmax = (int)B->active.size();
+    for (int k = 0; k < Tmax && e == cudaSuccess; ++k) {
+        F64Set set{};
+        set.arr = B->d_f64;
+        set.count = B->active[k];
+        set.b = B->b;
+        set.Tmax = Tmax;
+        e = launch_panel64(B->maps, set, k, s, &kt);
+        if (k + 1 < Tmax) {
+            set.count = B->active[k + 1];
+            if (e == cudaSuccess) e = launch_slice_panel64(set, k, s, &kt);
+            if (e == cudaSuccess) e = launch_update_tc64(B->maps, set, k, 0, 0, s, &kt);
+        }
+    }
+    *count += kt.launches;
+    return e;
+}
+
 cudaError_t enqueue_all(egs_batch *B, cudaStream_t s)
 {
-    cudaError_t et = launch_batch_tables(B->d_probs, B->nprob, s);
+    cudaError_t et = launch_batch_tables(B->d_probs, B->ntab, s);
     if (et != cudaSuccess) return et;
     if (B->dag) {
         cudaError_t e = cudaMemsetAsync(B->d_cnt, 0, B->ncnt * sizeof(unsigned), s);
@@ -589,6 +653,12 @@ cudaError_t enqueue_all(egs_batch *B, cudaStream_t s)
         case L_TRSM32: kb_trsm_panel32<<<g, 256, 0, s>>>(a, L.k); break;
         case L_UPDATE: kb_update<<<g, 256, 0, s>>>(a, L.k); break;
         case L_PAD: kb_pad<<<g, 256, 0, s>>>(a); break;
+        case L_FACTOR64:
+            et = enqueue_factor64(B, s, &count);
+            if (et != cudaSuccess) return et;
+            --count;
+            break;
+        case L_LDQ: kb_logdet_quad<<<g, 256, 0, s>>>(a); break;
         case L_TRSV: kb_trsv_diag<<<g, B->b, 0, s>>>(a, L.k, L.p); break;
         case L_GEMV:
             kb_gemv_panel<<<g, 256, (size_t)B->b * (sizeof(double) + sizeof(float)), s>>>(a, L.k, L.p);
@@ -609,11 +679,12 @@ cudaError_t enqueue_all(egs_batch *B, cudaStream_t s)
     return cudaGetLastError();
 }
 
-}  // namespace
-
-extern "C" {
-
-egs_status egs_batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_precision p, egs_batch **out)
+// A batch takes the tensor cores when its largest problem does as a single evaluation, with
+// all its problems (96 problems of 256 to 4,096 rows, tile 128: 607 ms as one persistent
+// launch of DFMA tasks, 101 ms so); without such a problem it stays on the persistent launch,
+// whose results equal single evaluations bit for bit.  any_size (the independent-blocks
+// approximation, whose blocks are no single evaluations): whatever the sizes.
+egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_precision p, bool any_size, egs_batch **out)
 {
     if (!out || !n || nprob < 1) return set_error(EGS_ERR_ARG, "egs_batch_create: bad arguments");
     *out = nullptr;
@@ -627,9 +698,13 @@ egs_status egs_batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_p
     }
     if (tile < 64 || tile > 1024 || tile % 64) return set_error(EGS_ERR_ARG, "egs_batch_create: tile %d invalid", tile);
     egs_batch *B = new egs_batch;
-    B->nprob = nprob;
+    B->nprob = B->ntab = nprob;
     B->b = tile;
     B->mixed = (p == EGS_MIX_FP32);
+    if (!B->mixed && nprob <= 65535) {  // a grid row per problem
+        B->tc = any_size;
+        for (int i = 0; i < nprob && !B->tc; ++i) B->tc = tc64_applies(n[i], tile, (int)((n[i] + tile - 1) / tile));
+    }
     size_t off = 0;
     std::vector<size_t> tiles_off(nprob), zpad_off(nprob), part_off(nprob), f32_off(nprob), sig_off(nprob),
         vec_off(nprob), mtab_off(nprob);
@@ -669,10 +744,45 @@ egs_status egs_batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_p
     off += a256(sizeof(DevStatus) * nprob);
     const size_t inputs_off = off;
     off += a256(in_doubles * sizeof(double));
+    // tensor-core batch: the slices of all problems in two arrays, problem order[i] from row
+    // prow[i] / irow[i] on
+    std::vector<int> order;
+    std::vector<size_t> prow, irow, fctr;
+    size_t R = 0, R1 = 0;
+    if (B->tc) {
+        for (int i = 0; i < nprob; ++i) order.push_back(i);
+        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return B->T[x] > B->T[y]; });
+        for (int i = 0; i < nprob; ++i) {
+            const int T = B->T[order[i]];
+            prow.push_back(R);
+            irow.push_back(R1);
+            fctr.push_back(B->f64ctr);
+            R += (size_t)(T - 1) * tile;
+            R1 += (size_t)T * tile;
+            B->f64ctr += tc64_counters(tile, T);
+        }
+        B->active.assign((size_t)B->T[order[0]], 0);
+        for (int i = 0; i < nprob; ++i)
+            for (int k = 0; k < B->T[i]; ++k) ++B->active[k];
+    }
+    const size_t f64_off = off;
+    if (B->tc) off += a256(sizeof(F64Prob) * nprob);
+    const size_t psl_off = off;
+    off += a256(R * tile * kF64Slices * sizeof(uint16_t));
+    const size_t pex_off = off;
+    off += a256(R * sizeof(int));
+    const size_t isl_off = off;
+    off += a256(R1 * kF64Panel * kF64Slices * sizeof(uint16_t));
+    const size_t iex_off = off;
+    off += a256(R1 * sizeof(int));
+    const size_t fctr_off = off;
+    off += a256(B->f64ctr * sizeof(unsigned long long));
+    const size_t winv_off = off;
+    if (B->tc) off += a256((size_t)nprob * kWinvDoubles * sizeof(double));
     std::vector<int64_t> prefix;
     std::vector<int4> tasks;
     std::vector<size_t> cnt_off;
-    B->dag = !B->mixed && tile <= 256;
+    B->dag = !B->mixed && !B->tc && tile <= 256;
     if (B->dag) {
         egs_status sc = dag_plan(B->T, tile, tasks, cnt_off, B->ncnt);
         if (sc != EGS_OK) {
@@ -760,6 +870,24 @@ egs_status egs_batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_p
         pr.mtab = (double *)(B->ws + mtab_off[i]);
     }
     e = cudaMemcpy(B->d_probs, B->h_probs, sizeof(BatchProblem) * nprob, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && B->tc) {
+        std::vector<F64Prob> fp((size_t)nprob);
+        B->d_f64 = (F64Prob *)(B->ws + f64_off);
+        B->d_f64ctr = (unsigned long long *)(B->ws + fctr_off);
+        for (int i = 0; i < nprob; ++i) {
+            const BatchProblem &pr = B->h_probs[order[i]];
+            F64Prob &P = fp[(size_t)i];
+            P.tl = Tiles{pr.tiles, nullptr, tile, pr.T, pr.T};
+            P.st = pr.st;
+            P.z = pr.zpad;
+            P.panel = F64Rows{(uint16_t *)(B->ws + psl_off), (int *)(B->ws + pex_off), R, prow[i]};
+            P.inner = F64Rows{(uint16_t *)(B->ws + isl_off), (int *)(B->ws + iex_off), R1, irow[i]};
+            P.ctr = B->d_f64ctr + fctr[i];
+            P.winv = (double *)(B->ws + winv_off) + (size_t)i * kWinvDoubles;
+        }
+        e = make_f64_maps(fp[0].panel, fp[0].inner, tile, &B->maps);
+        if (e == cudaSuccess) e = cudaMemcpy(B->d_f64, fp.data(), fp.size() * sizeof(F64Prob), cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
         egs_batch_destroy(B);
         return cuda_error(e, "egs_batch_create");
@@ -768,13 +896,19 @@ egs_status egs_batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_p
     return EGS_OK;
 }
 
-}  // extern "C"
+}  // namespace
+
+extern "C" egs_status egs_batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_precision p, egs_batch **out)
+{
+    return batch_create(nprob, n, tile, p, false, out);
+}
 
 namespace {
 
 // After the inputs have been staged on B->cs: the parameters, the graph
-// (captured on first use) and the statuses back to the host; synchronises.
-cudaError_t run_staged(egs_batch *B, cudaStream_t us, cudaError_t e)
+// (captured on first use; a batch that runs once goes without) and the statuses back to the
+// host; synchronises.
+cudaError_t run_staged(egs_batch *B, cudaStream_t us, cudaError_t e, bool once = false)
 {
     if (B->dag) {
         std::memset(B->h_ctl, 0, 2 * sizeof(DagCtl));
@@ -784,7 +918,7 @@ cudaError_t run_staged(egs_batch *B, cudaStream_t us, cudaError_t e)
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(B->d_params, B->h_params, sizeof(egs_matern_params) * B->nprob, cudaMemcpyHostToDevice, B->cs);
     if (e == cudaSuccess) e = cudaMemsetAsync(B->d_status, 0xFF, sizeof(DevStatus) * B->nprob, B->cs);
-    if (e == cudaSuccess && !B->exec) {
+    if (e == cudaSuccess && !B->exec && !once) {
         cudaGraph_t g = nullptr;
         e = cudaStreamBeginCapture(B->cs, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
@@ -795,7 +929,7 @@ cudaError_t run_staged(egs_batch *B, cudaStream_t us, cudaError_t e)
         if (e == cudaSuccess) e = cudaGraphInstantiate(&B->exec, g, 0);
         if (g) cudaGraphDestroy(g);
     }
-    if (e == cudaSuccess) e = cudaGraphLaunch(B->exec, B->cs);
+    if (e == cudaSuccess) e = once ? enqueue_all(B, B->cs) : cudaGraphLaunch(B->exec, B->cs);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(B->h_status, B->d_status, sizeof(DevStatus) * B->nprob, cudaMemcpyDeviceToHost, B->cs);
     if (e == cudaSuccess) e = cudaEventRecord(B->ev_out, B->cs);
@@ -835,6 +969,14 @@ egs_status egs_batch_run(egs_batch *B, const double *const *locs, const double *
         return set_error(EGS_ERR_TIMEOUT, "egs_batch_run: %u dependency wait(s) of the persistent launch ran out of "
                                           "time; the run was abandoned", B->h_ctl[1].timeouts);
     }
+    for (int i = 0; B->tc && i < B->nprob; ++i)
+        if (B->h_status[i].timeout == 1) {
+            for (int q = 0; q < B->nprob; ++q) {
+                if (out) out[q] = NAN;
+                if (per_status) per_status[q] = EGS_ERR_TIMEOUT;
+            }
+            return set_error(EGS_ERR_TIMEOUT, "egs_batch_run: a bounded device wait timed out; the run was abandoned");
+        }
     egs_status worst = EGS_OK;
     for (int i = 0; i < B->nprob; ++i) {
         const DevStatus &h = B->h_status[i];
@@ -858,7 +1000,9 @@ int64_t egs_batch_tasks(const egs_batch *B) { return B && B->dag ? (int64_t)B->n
 egs_status egs_batch_set_wait_limit(egs_batch *B, int64_t limit_ns, int64_t withhold_task)
 {
     if (!B) return set_error(EGS_ERR_ARG, "egs_batch_set_wait_limit: NULL batch");
-    if (!B->dag) return set_error(EGS_ERR_UNIMPLEMENTED, "egs_batch_set_wait_limit: not a persistent batch");
+    // a tensor-core batch accepts a limit, but its waits (within one SM) keep their own, and it
+    // has no task to withhold
+    if (!B->dag && !B->tc) return set_error(EGS_ERR_UNIMPLEMENTED, "egs_batch_set_wait_limit: not a persistent batch");
     if (limit_ns < 1 || withhold_task < -1 || withhold_task >= (int64_t)B->ntasks)
         return set_error(EGS_ERR_ARG, "egs_batch_set_wait_limit: limit %lld ns or task %lld out of range",
                          (long long)limit_ns, (long long)withhold_task);
@@ -972,22 +1116,35 @@ egs_status egs_loglik_ind(const double *locs, const double *z, const double thet
     std::vector<int64_t> ns((size_t)nblk);
     for (int64_t i = 0; i < nblk; ++i) ns[(size_t)i] = std::min(bs, n - i * bs);
     egs_batch *B = nullptr;
-    egs_status sc = egs_batch_create((int32_t)nblk, ns.data(), tile, EGS_FP64, &B);
+    // one block is the exact likelihood, and equals egs_loglik bit for bit
+    egs_status sc = batch_create((int32_t)nblk, ns.data(), tile, EGS_FP64, nblk > 1, &B);
     if (sc != EGS_OK) return sc;
     for (int i = 0; i < B->nprob; ++i) B->h_params[i] = P;
     cudaStream_t us = (cudaStream_t)stream;
     cudaError_t e = cudaEventRecord(B->ev_in, us);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(B->cs, B->ev_in, 0);
-    // block i: x[i bs ..], y[i bs ..] (y starts at locs + n), z[i bs ..]
-    for (int i = 0; i < B->nprob && e == cudaSuccess; ++i) {
-        double *in = B->d_inputs + B->in_off[i];
-        const size_t bytes = (size_t)B->n[i] * sizeof(double);
-        const int64_t off = (int64_t)i * bs;
-        e = cudaMemcpyAsync(in, locs + off, bytes, cudaMemcpyDefault, B->cs);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(in + B->n[i], locs + n + off, bytes, cudaMemcpyDefault, B->cs);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(in + 2 * B->n[i], z + off, bytes, cudaMemcpyDefault, B->cs);
+    // block i: x[i bs ..], y[i bs ..] (y starts at locs + n), z[i bs ..], read in place, or from
+    // one staged copy if the inputs are host memory
+    const double *dl = locs, *dz = z;
+    if (e == cudaSuccess && !is_device_ptr(locs)) {
+        e = cudaMemcpyAsync(B->d_inputs, locs, (size_t)2 * n * sizeof(double), cudaMemcpyHostToDevice, B->cs);
+        dl = B->d_inputs;
     }
-    e = run_staged(B, us, e);
+    if (e == cudaSuccess && !is_device_ptr(z)) {
+        e = cudaMemcpyAsync(B->d_inputs + 2 * n, z, (size_t)n * sizeof(double), cudaMemcpyHostToDevice, B->cs);
+        dz = B->d_inputs + 2 * n;
+    }
+    for (int i = 0; i < B->nprob; ++i) {
+        const int64_t off = (int64_t)i * bs;
+        B->h_probs[i].X = dl + off;
+        B->h_probs[i].Y = dl + n + off;
+        B->h_probs[i].z = dz + off;
+        B->h_probs[i].mtab = B->h_probs[0].mtab;  // one theta
+    }
+    B->ntab = 1;
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(B->d_probs, B->h_probs, sizeof(BatchProblem) * B->nprob, cudaMemcpyHostToDevice, B->cs);
+    e = run_staged(B, us, e, true);
     if (e != cudaSuccess) {
         egs_batch_destroy(B);
         return cuda_error(e, "egs_loglik_ind");
@@ -996,6 +1153,11 @@ egs_status egs_loglik_ind(const double *locs, const double *z, const double thet
         egs_batch_destroy(B);
         return set_error(EGS_ERR_TIMEOUT, "egs_loglik_ind: a dependency wait of the persistent launch ran out of time");
     }
+    for (int i = 0; B->tc && i < B->nprob; ++i)
+        if (B->h_status[i].timeout == 1) {
+            egs_batch_destroy(B);
+            return set_error(EGS_ERR_TIMEOUT, "egs_loglik_ind: a bounded device wait timed out");
+        }
     // fixed-order FP64 sums over the blocks
     double ll = 0.0, ld = 0.0, q = 0.0;
     int64_t fail = -1;

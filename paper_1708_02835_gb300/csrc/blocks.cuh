@@ -152,7 +152,7 @@ __device__ __forceinline__ bool potrf64_smem(double *A, int ld, int64_t row0, De
 //    (each has a sub-partition of its own), while lanes 4 .. 31 carry 28 rows below it, so that
 //    the rows below cost no instruction;
 //  - the 4-term updates of the entries right of the panel are spread over all lanes.
-// 64 pivots x 22 / 4 instructions of panels, about 400 of updates: 24 us (115 us with 16-column
+// 64 pivots x 22 / 4 instructions of panels, about 400 of updates: 47 us with the launch (115 us with 16-column
 // panels, a thread per row below them and a square root per pivot).
 //
 // Leaves L (zero upper half), y in row 64 and 1 / L_jj in sm; false if a pivot is not positive

@@ -660,7 +660,7 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_col, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_diag, cudaEventDisableTiming);
     // POTRF of a diagonal tile: the FP64 path's 64-column blocks, on that tile alone (tile 512:
-    // OLD with the task graph of 32 x 32 blocks, NEW)
+    // 1.05 ms with a task graph of 32 x 32 blocks, 0.4 ms so)
     const F64Set diag{nullptr, tc64_problem(mb.dpan, tl, st, nullptr, true), 1, b, T, 1};
     F64Maps dmaps;
     if (e == cudaSuccess) e = make_f64_maps(diag.one.panel, diag.one.inner, b, &dmaps);
