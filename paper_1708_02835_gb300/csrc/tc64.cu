@@ -29,9 +29,9 @@
 // step of 896 tensor clocks, at 128 B / clock) is what bounds the kernel; 128 x 64
 // with 7 x 64 accumulator columns is the largest block that fits TMEM.
 // A slots are freed slice by slice (7 slots of 16 KB), B is double buffered (2 x 56 KB).
-// Measured (n = 16,900, tile 512, all 33 updates): 1,361 ms with DFMA, 40.8 ms here, i.e.
-// 43 TFLOP/s of FP64-equivalent work, 1,207 executed on the tensor cores.  Error of the
-// factor, rms of Sigma - L L^T in twice the precision (n = 2,304, tile 256): 2.5e-17 against
+// Measured (n = 16,900, tile 512, all 33 updates): 1,361 ms with DFMA, 40.8 ms here with FP64
+// additions in the epilogue, 33 ms with integer ones, i.e. 53 TFLOP/s of FP64-equivalent work,
+// 1,490 executed on the tensor cores.  Error of the factor, rms of Sigma - L L^T in twice the precision (n = 2,304, tile 256): 2.5e-17 against
 // 3.2e-17 with DFMA (theta = (1, 0.1, 0.5)), 2.9e-17 / 6.3e-17 (nu = 1.3), 9.9e-18 / 1.0e-17
 // (range 0.03).
 #include "blocks.cuh"
@@ -335,39 +335,32 @@ struct F64Work {
     }
 };
 
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+// The level sums v_0 .. v_6 of one flush (v_L a multiple of 2^-8L, |v_0| <= 2^24) as fixed
+// point in units of 2^-37, all but the last exactly: the FP64 pipe, at 64 clocks a warp-wide
+// instruction, took longer over two additions and the conversions (an epilogue of 250 clocks
+// an entry against 75) than the tensor cores over the products.
+__device__ __forceinline__ long long fixed_sum7(const float (&v)[kF64Slices])
 {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    const int u0 = __float2int_rn(v[0]), u1 = __float2int_rn(v[1] * 0x1p8f), u2 = __float2int_rn(v[2] * 0x1p16f);
+    const int u3 = __float2int_rn(v[3] * 0x1p24f), u4 = __float2int_rn(v[4] * 0x1p32f);
+    const int w = __float2int_rn(__fadd_rn(v[5], v[6]) * 0x1p37f);
+    const long long hi = (long long)u0 * 256 + u1, lo = (long long)u2 * 256 + u3;
+    return hi * (1ll << 29) + lo * (1ll << 13) + ((long long)u4 * 32 + w);
 }
 
-// (double)x by integer operations (the conversion instruction runs on the FP64 pipe);
-// x is zero or a normal float.
-__device__ __forceinline__ double f32_to_f64(float x)
+// f 2^-(37 - up) as a double, rounded once, by integer operations.
+__device__ __forceinline__ double fixed_to_f64(long long f, int up)
 {
-    const uint32_t u = __float_as_uint(x), a = u & 0x7FFFFFFFu;
-    const uint32_t hi = a ? (u & 0x80000000u) | ((a >> 3) + (896u << 20)) : 0u;
-    return __hiloint2double((int)hi, (int)(a ? u << 29 : 0u));
+    const unsigned long long m = f < 0 ? 0ull - (unsigned long long)f : (unsigned long long)f;
+    if (m == 0) return 0.0;
+    const int lz = __clzll((long long)m);
+    const unsigned long long n = m << lz, r = (n >> 11) + ((n >> 10) & 1);
+    const unsigned long long bits = ((unsigned long long)(1022 + 63 - lz - 37 + up) << 52) + r;
+    return __longlong_as_double((long long)(bits | (f < 0 ? 1ull << 63 : 0ull)));
 }
 
 // 2^s as a double, -1022 <= s <= 1023.
 __device__ __forceinline__ double pow2(int s) { return __hiloint2double((s + 1023) << 20, 0); }
-
-// The level sums v_0 .. v_6 (v_L a multiple of 2^-8L) as a + c + r: a + c is exact to the
-// last bit of c, r carries the rest to 2^-40 (level-0 units, |v_0| <= 2^24).
-__device__ __forceinline__ void combine7(const float (&v)[kF64Slices], float &a, float &c, float &r)
-{
-    float p, q, rr, t, u, w, x, y, c0, e1;
-    two_sum(v[4], __fadd_rn(v[5], v[6]), p, q);
-    two_sum(v[3], p, rr, t);
-    t = __fadd_rn(t, q);
-    two_sum(v[2], rr, u, w);
-    two_sum(v[1], u, x, y);
-    two_sum(v[0], x, a, c0);
-    two_sum(c0, y, c, e1);
-    r = __fadd_rn(e1, __fadd_rn(w, t));
-}
 
 // 7 x 16 accumulator columns (levels 64 columns apart) of the calling warp's 32 lanes.
 __device__ __forceinline__ void tmem_ld_levels16(uint32_t taddr, float (&v)[kF64Slices][16])
@@ -559,6 +552,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
         const int q = warp & 3, half = (warp - 2) >> 2;
         const uint32_t t0 = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32);
         const int nflush = (kchunks + FLUSH - 1) / FLUSH;
+        const int up = nflush > 2 ? 1 : 0;  // the sum over the flushes stays below 2^63
         uint32_t f = 0;
         int r = 0;
         bool run = true;
@@ -571,7 +565,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             if (lane == 0) tc::mbar_arrive(&rempty[slot]);
             ++r;
             if (wi.m < 0) break;
-            double acc[32];
+            long long acc[32];
             for (int fl = 0; fl < nflush; ++fl, ++f) {
                 const bool ok = tc::mbar_wait(&tfull, f & 1u, &abort_flag);
                 tc::tc_fence_after();
@@ -591,9 +585,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const float vj[kF64Slices] = {v[0][j], v[1][j], v[2][j], v[3][j], v[4][j], v[5][j], v[6][j]};
-                        float a, c, rr;
-                        combine7(vj, a, c, rr);
-                        const double d = (f32_to_f64(a) + f32_to_f64(c)) + f32_to_f64(rr);
+                        const long long d = fixed_sum7(vj) >> up;
                         acc[hh * 16 + j] = fl == 0 ? d : acc[hh * 16 + j] + d;
                     }
                 }
@@ -616,7 +608,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const int s = ea + __ldg(eb + 16 * h + j);
-                        const double d = acc[16 * h + j];
+                        const double d = fixed_to_f64(acc[16 * h + j], up);
                         if (s >= -960 && s <= 1000) {
                             cd[j] = fma(-pow2(s), d, cd[j]);
                         } else if (s > 1000) {
