@@ -101,7 +101,7 @@ static Layout make_layout(const TileGeom &g, bool tc)
     L.status = off;
     off += align256(sizeof(DevStatus));
     L.mtab = off;
-    off += align256(EGS_MT_DOUBLES * sizeof(double));
+    off += align256(EGS_MT_SCRATCH_DOUBLES * sizeof(double));
     L.pctr = off;
     off += align256((size_t)g.T * potrf_diag_scratch_words(g.b) * sizeof(unsigned));
     L.tc = off;

@@ -57,23 +57,23 @@ __device__ __forceinline__ int band_rows(const BatchProblem &p, int k)
 }
 
 // Local polynomials of the general-nu problems (blockIdx.y = problem).
-__global__ void __launch_bounds__(256) kb_table(const BatchProblem *probs)
+__global__ void __launch_bounds__(128) kb_table(const BatchProblem *probs)
 {
     const BatchProblem &pr = probs[blockIdx.y];
     __shared__ egs_matern_params Ps;
-    __shared__ double vals[8][EGS_MT_NC];
+    __shared__ double vals[4][EGS_MT_NC];
     const double *s = reinterpret_cast<const double *>(pr.P);
     double *d = reinterpret_cast<double *>(&Ps);
     for (int i = threadIdx.x; i < (int)(sizeof(egs_matern_params) / sizeof(double)); i += blockDim.x) d[i] = s[i];
     __syncthreads();
     if (Ps.kind != EGS_MATERN_GENERAL) return;
-    const int w = threadIdx.x >> 5, iv = (int)blockIdx.x * 8 + w;
+    const int w = threadIdx.x >> 5, iv = (int)blockIdx.x * 4 + w;
     if (iv < EGS_MT_OCT * EGS_MT_SUB) matern_table_interval(&Ps, iv, pr.mtab, vals[w]);
 }
 
 cudaError_t launch_batch_tables(const BatchProblem *probs, int nprob, cudaStream_t s)
 {
-    kb_table<<<dim3((EGS_MT_OCT * EGS_MT_SUB + 7) / 8, (unsigned)nprob), 256, 0, s>>>(probs);
+    kb_table<<<dim3((EGS_MT_OCT * EGS_MT_SUB + 3) / 4, (unsigned)nprob), 128, 0, s>>>(probs);
     return cudaGetLastError();
 }
 
@@ -83,19 +83,15 @@ __global__ void __launch_bounds__(256) kb_gen(BatchArgs a)
     int64_t local;
     const BatchProblem &pr = a.probs[find_problem(a, blockIdx.x, local)];
     __shared__ egs_matern_params Ps;
-    __shared__ double Ts[EGS_MT_DOUBLES];
+    __shared__ double Ts[EGS_MT_INTS];
     {
         const double *s = reinterpret_cast<const double *>(pr.P);
         double *d = reinterpret_cast<double *>(&Ps);
         for (int i = threadIdx.x; i < (int)(sizeof(egs_matern_params) / sizeof(double)); i += blockDim.x) d[i] = s[i];
         __syncthreads();
     }
-    const bool general = Ps.kind == EGS_MATERN_GENERAL;
-    if (general) {
-        for (int i = threadIdx.x; i < EGS_MT_DOUBLES; i += blockDim.x) Ts[i] = pr.mtab[i];
-        __syncthreads();
-    }
-    const double *Tab = general ? Ts : nullptr;
+    const double *Tab = stage_table(&Ps, pr.mtab, Ts);
+    __syncthreads();
     const int b = a.b, nsub = b >> 6;
     const int64_t t = local / (nsub * nsub);
     const int sub = (int)(local % (nsub * nsub));
@@ -118,7 +114,7 @@ __global__ void __launch_bounds__(256) kb_gen(BatchArgs a)
         if (gi >= n || gj >= n) v = (gi == gj) ? 1.0 : 0.0;
         else if (gi == gj) v = Ps.th1;
         else {
-            v = matern_eval(&Ps, loc_dist(&Ps, pr.X[gi], pr.Y[gi], xj, yj) * Ps.inv_th2, Tab);
+            v = matern_pair(&Ps, Tab, pr.X[gi], pr.Y[gi], xj, yj);
         }
         const size_t off = (size_t)r * b + sc * 64 + tx;
         if (is64) tile[off] = v;
@@ -732,7 +728,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
         part_off[i] = off;
         off += a256((size_t)2 * T * sizeof(double));
         mtab_off[i] = off;
-        off += a256(EGS_MT_DOUBLES * sizeof(double));
+        off += a256(EGS_MT_SCRATCH_DOUBLES * sizeof(double));
         B->in_off.push_back(in_doubles);
         in_doubles += (size_t)3 * n[i];
     }

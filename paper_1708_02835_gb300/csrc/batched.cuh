@@ -19,7 +19,7 @@ struct BatchProblem {
     DevStatus *st;
     const egs_matern_params *P;
     unsigned *cnt;     // persistent scheduler: T(T+1)/2 tile counters, then T vector-block counters
-    double *mtab;      // EGS_MT_DOUBLES: the generator's local polynomials (general nu)
+    double *mtab;      // EGS_MT_SCRATCH_DOUBLES: the generator's local polynomials (general nu)
 };
 
 // The local polynomials of every general-nu problem of a batch: grid =

@@ -57,7 +57,7 @@ struct TrsvSmem {
 // The tasks' shared memory, overlaid: one task runs at a time in a CTA.
 struct GenSmem {
     egs_matern_params P;
-    double T[EGS_MT_DOUBLES];
+    double T[EGS_MT_INTS];
 };
 
 union DagSmem {
@@ -192,12 +192,8 @@ __device__ void task_gen(GenSmem &gs, const BatchProblem &pr, int b, int ti, int
         for (int i = threadIdx.x; i < (int)(sizeof(egs_matern_params) / sizeof(double)); i += blockDim.x) d[i] = s[i];
         __syncthreads();
     }
-    const bool general = Ps.kind == EGS_MATERN_GENERAL;
-    if (general) {
-        for (int i = threadIdx.x; i < EGS_MT_DOUBLES; i += blockDim.x) gs.T[i] = pr.mtab[i];
-        __syncthreads();
-    }
-    const double *Tab = general ? gs.T : nullptr;
+    const double *Tab = stage_table(&Ps, pr.mtab, gs.T);
+    __syncthreads();
     const int nsub = b >> 6, tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
     const int64_t n = pr.n;
     double *tile = pr.tiles + (size_t)tile_linear(ti, tj) * b * b;
@@ -211,7 +207,7 @@ __device__ void task_gen(GenSmem &gs, const BatchProblem &pr, int b, int ti, int
             double v;
             if (gi >= n || gj >= n) v = (gi == gj) ? 1.0 : 0.0;
             else if (gi == gj) v = Ps.th1;
-            else v = matern_eval(&Ps, loc_dist(&Ps, pr.X[gi], pr.Y[gi], xj, yj) * Ps.inv_th2, Tab);
+            else v = matern_pair(&Ps, Tab, pr.X[gi], pr.Y[gi], xj, yj);
             tile[(size_t)r * b + sc * 64 + tx] = v;
         }
     }

@@ -148,13 +148,13 @@ egs_status set_error(egs_status code, const char *fmt, ...);
 egs_status cuda_error(cudaError_t e, const char *what);
 
 // ---- launchers (stream-ordered, no synchronisation) ----
-// Sigma(theta) into FP64 lower tiles.  tab: EGS_MT_DOUBLES doubles of device
+// Sigma(theta) into FP64 lower tiles.  tab: EGS_MT_SCRATCH_DOUBLES doubles of device
 // scratch for the local polynomials of a general nu (built first on s), or
 // NULL to evaluate every entry directly.
 cudaError_t launch_matern_tiles_f64(const double *X, const double *Y, const TileGeom &g,
                                     const egs_matern_params &P, double *tiles, cudaStream_t s,
                                     KernelTimer *kt = nullptr, double *tab = nullptr);
-// The local polynomials of a general nu into tab (EGS_MT_DOUBLES doubles).
+// The local polynomials of a general nu into tab (EGS_MT_SCRATCH_DOUBLES doubles).
 cudaError_t launch_matern_table(const egs_matern_params &P, double *tab, cudaStream_t s, KernelTimer *kt = nullptr);
 
 // Tile Cholesky in place (FP64).  Stops doing work once st->fail_index is set.

@@ -3,8 +3,8 @@
 // (genDistanceMatrix) is never stored: each entry's distance is formed in
 // registers from the SoA coordinates.
 //
-// One CTA writes a 64 x 64 sub-block of one tile; a warp writes 32 consecutive
-// columns of one row (256 contiguous bytes), so stores are fully coalesced.
+// A warp writes 32 consecutive columns of one row (256 contiguous bytes), so
+// stores are fully coalesced.
 #include "egs_internal.cuh"
 #include "matern.cuh"
 #include "matern_df.cuh"
@@ -33,23 +33,26 @@ __device__ __forceinline__ void tile_decode(int64_t t, int &i, int &j)
 }
 
 // Writes tile blockIdx.x (lower-tile order) of Sigma into tl: as double when
-// the tile is FP64 in tl, else rounded to float.
+// the tile is FP64 in tl, else rounded to float.  A CTA covers 64 columns and
+// `rows` rows of the tile (all of them once there are enough CTAs, so that the
+// staged constants serve more entries).
 // tab: the local polynomials of a general nu (built by k_matern_table before
 // this launch), staged in shared memory; NULL for the closed forms.
 // band_only: blockIdx.x enumerates only the FP64 band tiles of a mixed
 // layout, as i * band + (i - j) (slots with j < 0 exit at once).
-__global__ void __launch_bounds__(256)
+// Bound by instruction issue (about 250 integer instructions and 4 FP64 ones
+// an entry, about 780 clocks a warp and sub-partition; 2,870 with FP64 arithmetic):
+// n = 25,600, nu = 1.3: 25.9 ms in FP64, 7.1 ms.
+__global__ void __launch_bounds__(256, 3)
 k_matern_tiles(const double *__restrict__ X, const double *__restrict__ Y, int64_t n, Tiles tl,
                const __grid_constant__ egs_matern_params Pg, const double *__restrict__ tab,
-               int band_only)
+               int band_only, int rows)
 {
     const int b = tl.b;
     __shared__ egs_matern_params Ps;
-    __shared__ double Ts[EGS_MT_DOUBLES];
-    if (tab)
-        for (int i = threadIdx.x; i < EGS_MT_DOUBLES; i += blockDim.x) Ts[i] = tab[i];
+    __shared__ double Ts[EGS_MT_INTS];
+    const double *T = stage_table(&Pg, tab, Ts);
     stage_params(&Pg, &Ps);
-    const double *T = tab ? Ts : nullptr;
     const egs_matern_params *P = &Ps;
     int ti, tj;
     if (band_only) {
@@ -59,34 +62,34 @@ k_matern_tiles(const double *__restrict__ X, const double *__restrict__ Y, int64
     } else {
         tile_decode((int64_t)blockIdx.x, ti, tj);
     }
-    const int nsub = b >> 6;
-    const int sr = (int)blockIdx.y / nsub, sc = (int)blockIdx.y % nsub;
-    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
-    const int64_t gj = (int64_t)tj * b + sc * 64 + tx;
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6, c = (int)blockIdx.y * 64 + tx;
+    const int64_t gj = (int64_t)tj * b + c;
     double xj = 0.0, yj = 0.0;
     if (gj < n) {
         xj = X[gj];
         yj = Y[gj];
     }
-    const double inv_th2 = P->inv_th2;
     const bool is64 = tl.is64(ti, tj);
     double *t64 = is64 ? tl.t64(ti, tj) : nullptr;
     float *t32 = is64 ? nullptr : tl.t32(ti, tj);
-    for (int rr = 0; rr < 16; ++rr) {
-        const int r = sr * 64 + ty + 4 * rr;
+    const int r0 = (int)blockIdx.z * rows;
+    for (int r = r0 + ty; r < r0 + rows; r += 4) {
         const int64_t gi = (int64_t)ti * b + r;
         double v;
-        if (gi >= n || gj >= n) {
-            v = (gi == gj) ? 1.0 : 0.0;
-        } else if (gi == gj) {
-            v = P->th1;
-        } else {
-            v = matern_eval(P, loc_dist(P, X[gi], Y[gi], xj, yj) * inv_th2, T);
-        }
-        const size_t off = (size_t)r * b + sc * 64 + tx;
+        if (gi >= n || gj >= n) v = (gi == gj) ? 1.0 : 0.0;
+        else if (gi == gj) v = P->th1;
+        else v = matern_pair(P, T, X[gi], Y[gi], xj, yj);
+        const size_t off = (size_t)r * b + c;
         if (is64) t64[off] = v;
         else t32[off] = (float)v;
     }
+}
+
+// Rows a CTA covers: all b once that makes 8 CTAs for every SM.
+static dim3 tiles_grid(size_t ntiles, int b, int *rows)
+{
+    *rows = ntiles * (size_t)(b / 64) >= 8 * 152 ? b : 64;
+    return dim3((unsigned)ntiles, (unsigned)(b / 64), (unsigned)(b / *rows));
 }
 
 // Split a double into a float pair h + l (48 of its 53 bits).
@@ -151,14 +154,16 @@ __global__ void k_split_table(const double *__restrict__ tab, float2 *__restrict
     }
 }
 
-// The local polynomials of a general nu: one warp per sub-interval.
-__global__ void __launch_bounds__(256) k_matern_table(const __grid_constant__ egs_matern_params Pg, double *tab)
+// The local polynomials of a general nu: one warp per sub-interval, four to a
+// CTA, so that each has the FP64 unit of an SM sub-partition to itself (0.35 ms
+// with eight and one lane forming the coefficients, 0.08 ms now).
+__global__ void __launch_bounds__(128) k_matern_table(const __grid_constant__ egs_matern_params Pg, double *tab)
 {
     __shared__ egs_matern_params Ps;
-    __shared__ double vals[8][EGS_MT_NC];
+    __shared__ double vals[4][EGS_MT_NC];
     stage_params(&Pg, &Ps);
     const int w = threadIdx.x >> 5;
-    const int iv = (int)blockIdx.x * 8 + w;
+    const int iv = (int)blockIdx.x * 4 + w;
     if (iv < EGS_MT_OCT * EGS_MT_SUB) matern_table_interval(&Ps, iv, tab, vals[w]);
 }
 
@@ -173,8 +178,8 @@ float2 *matern_df_table(double *tab) { return reinterpret_cast<float2 *>(tab + E
 
 cudaError_t launch_matern_table(const egs_matern_params &P, double *tab, cudaStream_t s, KernelTimer *kt)
 {
-    constexpr int blocks = (EGS_MT_OCT * EGS_MT_SUB + 7) / 8;
-    EGS_LAUNCH(kt, KC_GEN, s, k_matern_table<<<blocks, 256, 0, s>>>(P, tab));
+    constexpr int blocks = (EGS_MT_OCT * EGS_MT_SUB + 3) / 4;
+    EGS_LAUNCH(kt, KC_GEN, s, k_matern_table<<<blocks, 128, 0, s>>>(P, tab));
     return cudaGetLastError();
 }
 
@@ -187,13 +192,13 @@ cudaError_t launch_matern_tiles(const double *X, const double *Y, int64_t n, con
         if (e != cudaSuccess) return e;
         t = tab;
     }
-    const unsigned nsub = (unsigned)((tl.b / 64) * (tl.b / 64));
+    int rows;
     egs_matern_df D;
     if (!tl.dense() && matern_df_applies(P, tab != nullptr, &D)) {
         // mixed layout: FP64 band tiles directly, the FP32 off-band tiles in
         // double-float
-        EGS_LAUNCH(kt, KC_GEN, s,
-                   k_matern_tiles<<<dim3((unsigned)(tl.T * tl.band), nsub), 256, 0, s>>>(X, Y, n, tl, P, t, 1));
+        const dim3 bgrid = tiles_grid((size_t)tl.T * tl.band, tl.b, &rows);
+        EGS_LAUNCH(kt, KC_GEN, s, k_matern_tiles<<<bgrid, 256, 0, s>>>(X, Y, n, tl, P, t, 1, rows));
         const dim3 grid((unsigned)Tiles::f32_tiles(tl.T, tl.band), (unsigned)(tl.b / 64));
         if (P.kind == EGS_MATERN_GENERAL) {
             float2 *ctab = matern_df_table(tab);
@@ -205,7 +210,8 @@ cudaError_t launch_matern_tiles(const double *X, const double *Y, int64_t n, con
         return cudaGetLastError();
     }
     const size_t ntiles = (size_t)tl.T * (tl.T + 1) / 2;
-    EGS_LAUNCH(kt, KC_GEN, s, k_matern_tiles<<<dim3((unsigned)ntiles, nsub), 256, 0, s>>>(X, Y, n, tl, P, t, 0));
+    const dim3 grid = tiles_grid(ntiles, tl.b, &rows);
+    EGS_LAUNCH(kt, KC_GEN, s, k_matern_tiles<<<grid, 256, 0, s>>>(X, Y, n, tl, P, t, 0, rows));
     return cudaGetLastError();
 }
 

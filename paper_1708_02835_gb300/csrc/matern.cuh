@@ -15,6 +15,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "matern_int.cuh"
 #include "matern_params.h"
 
 namespace egs {
@@ -225,48 +226,106 @@ __device__ __forceinline__ double matern_eval(const egs_matern_params *__restric
     }
 }
 
+// The staged polynomials of a general nu: EGS_MT_INTS words of shared memory, the integer ones
+// for planar distances (matern_int.cuh), the FP64 ones for great-circle distances.  tab: the
+// generator scratch (EGS_MT_SCRATCH_DOUBLES), or NULL.  Whole CTA, no barrier.
+__device__ __forceinline__ const double *stage_table(const egs_matern_params *__restrict__ Pp, const double *tab,
+                                                     double *T)
+{
+    if (!tab || Pp->kind != EGS_MATERN_GENERAL) return nullptr;
+    const bool plane = Pp->metric == EGS_DIST_EUCLIDEAN;
+    const double *src = plane ? tab + 2 * EGS_MT_DOUBLES : tab;
+    for (int i = threadIdx.x; i < (plane ? EGS_MT_INTS : EGS_MT_DOUBLES); i += blockDim.x) T[i] = src[i];
+    return T;
+}
+
+// The FP64 evaluation where the integer one does not reach, kept out of its registers.
+static __device__ __noinline__ double matern_rest(const egs_matern_params *Pp, double q)
+{
+    return matern_eval(Pp, sqrt(q) * Pp->inv_th2);
+}
+
+// The covariance of two locations; tab: what stage_table staged (or NULL).
+__device__ __forceinline__ double matern_pair(const egs_matern_params *__restrict__ Pp, const double *__restrict__ tab,
+                                              double xi, double yi, double xj, double yj)
+{
+    if (Pp->metric == EGS_DIST_EUCLIDEAN) {
+        const double dx = xi - xj, dy = yi - yj, q = fma(dx, dx, dy * dy);
+        double v;
+        if ((tab || Pp->kind != EGS_MATERN_GENERAL) &&
+            mi::matern_int(Pp, reinterpret_cast<const int64_t *>(tab), q, &v))
+            return v;
+        return matern_rest(Pp, q);
+    }
+    return matern_eval(Pp, loc_dist(Pp, xi, yi, xj, yj) * Pp->inv_th2, tab);
+}
+
+// cos(pi m / 24), m = 0 .. 47, and the coefficients of the Chebyshev polynomials T_0 .. T_11.
+static_assert(EGS_MT_NC == 12, "the tables below are for 12 points");
+__device__ constexpr double kMtCos[48] = {
+    1.0, 0.9914448613738104, 0.9659258262890683, 0.9238795325112867,
+    0.8660254037844386, 0.7933533402912352, 0.7071067811865476, 0.6087614290087207,
+    0.5, 0.3826834323650898, 0.25881904510252074, 0.1305261922200516,
+    0.0, -0.1305261922200516, -0.25881904510252074, -0.3826834323650898,
+    -0.5, -0.6087614290087207, -0.7071067811865476, -0.7933533402912352,
+    -0.8660254037844386, -0.9238795325112867, -0.9659258262890683, -0.9914448613738104,
+    -1.0, -0.9914448613738104, -0.9659258262890683, -0.9238795325112867,
+    -0.8660254037844386, -0.7933533402912352, -0.7071067811865476, -0.6087614290087207,
+    -0.5, -0.3826834323650898, -0.25881904510252074, -0.1305261922200516,
+    0.0, 0.1305261922200516, 0.25881904510252074, 0.3826834323650898,
+    0.5, 0.6087614290087207, 0.7071067811865476, 0.7933533402912352,
+    0.8660254037844386, 0.9238795325112867, 0.9659258262890683, 0.9914448613738104};
+__device__ constexpr short kMtCheb[12][12] = {
+    {1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0},
+    {0, 1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0},
+    {-1, 0, 2, 0, 0, 0, 0, 0, 0, 0, 0, 0},
+    {0, -3, 0, 4, 0, 0, 0, 0, 0, 0, 0, 0},
+    {1, 0, -8, 0, 8, 0, 0, 0, 0, 0, 0, 0},
+    {0, 5, 0, -20, 0, 16, 0, 0, 0, 0, 0, 0},
+    {-1, 0, 18, 0, -48, 0, 32, 0, 0, 0, 0, 0},
+    {0, -7, 0, 56, 0, -112, 0, 64, 0, 0, 0, 0},
+    {1, 0, -32, 0, 160, 0, -256, 0, 128, 0, 0, 0},
+    {0, 9, 0, -120, 0, 432, 0, -576, 0, 256, 0, 0},
+    {-1, 0, 50, 0, -400, 0, 1120, 0, -1280, 0, 512, 0},
+    {0, -11, 0, 220, 0, -1232, 0, 2816, 0, -2816, 0, 1024}};
+
 // One warp builds the local polynomial of sub-interval iv (0 <= iv <
 // EGS_MT_OCT * EGS_MT_SUB): lanes 0..NC-1 evaluate g = theta1^-1 e^x C(x) at
-// the NC Chebyshev points of the interval with the direct method, lane 0
-// forms the Chebyshev coefficients c_k = (2 / NC) sum_i g_i cos(pi k (i + 1/2) / NC)
-// (c_0 halved) and converts sum_k c_k T_k(s) to monomials in s (T_{k+1} =
-// 2 s T_k - T_{k-1}).  vals: NC doubles of shared memory for this warp.
+// the NC Chebyshev points of the interval with the direct method and form the
+// Chebyshev coefficients c_k = (2 / NC) sum_i g_i cos(pi k (i + 1/2) / NC)
+// (c_0 halved), then the monomials' sum_k c_k T_k(s), a lane per coefficient,
+// in FP64 and as the integers of matern_int.cuh (tab: the generator scratch).
+// vals: NC doubles of shared memory for this warp.
 __device__ __forceinline__ void matern_table_interval(const egs_matern_params *__restrict__ Pp, int iv, double *tab,
                                                       double *vals)
 {
     const int lane = threadIdx.x & 31;
     const int oct = iv / EGS_MT_SUB, sub = iv % EGS_MT_SUB;
     if (lane < EGS_MT_NC) {
-        const double t = cospi((2.0 * lane + 1.0) / (2.0 * EGS_MT_NC));  // Chebyshev point in s
+        const double t = kMtCos[2 * lane + 1];  // Chebyshev point in s
         const double y = ldexp(1.0 + (sub + 0.5 * (1.0 + t)) / EGS_MT_SUB, oct + EGS_MT_E0);
         const double x = 1.25 * y;
         vals[lane] = matern_general(Pp, x, true) / Pp->th1;
     }
     __syncwarp();
-    if (lane == 0) {
-        double c[EGS_MT_NC], a[EGS_MT_NC], tkm[EGS_MT_NC], tk[EGS_MT_NC], tn[EGS_MT_NC];
-        for (int k = 0; k < EGS_MT_NC; ++k) {
-            double acc = 0.0;
-            for (int i = 0; i < EGS_MT_NC; ++i) acc = fma(vals[i], cospi(k * (2.0 * i + 1.0) / (2.0 * EGS_MT_NC)), acc);
-            c[k] = acc * (k == 0 ? 1.0 : 2.0) / EGS_MT_NC;
-            a[k] = 0.0;
-            tkm[k] = tk[k] = 0.0;
-        }
-        tkm[0] = 1.0;  // T_0
-        tk[1] = 1.0;   // T_1
-        a[0] = c[0];
-        a[1] = c[1];
-        for (int k = 1; k + 1 < EGS_MT_NC; ++k) {
-            // T_{k+1} = 2 s T_k - T_{k-1}
-            for (int j = 0; j < EGS_MT_NC; ++j) tn[j] = (j > 0 ? 2.0 * tk[j - 1] : 0.0) - tkm[j];
-            for (int j = 0; j < EGS_MT_NC; ++j) {
-                a[j] = fma(c[k + 1], tn[j], a[j]);
-                tkm[j] = tk[j];
-                tk[j] = tn[j];
-            }
-        }
-        for (int j = 0; j < EGS_MT_NC; ++j) tab[iv * EGS_MT_NC + j] = a[j];
+    // lane k: c_k; then lane j: the coefficient of s^j, sum_k c_k [s^j] T_k
+    double c = 0.0, a = 0.0;
+    if (lane < EGS_MT_NC) {
+        for (int i = 0; i < EGS_MT_NC; ++i) c = fma(vals[i], kMtCos[lane * (2 * i + 1) % (4 * EGS_MT_NC)], c);
+        c *= (lane == 0 ? 1.0 : 2.0) / EGS_MT_NC;
     }
+    for (int k = 0; k < EGS_MT_NC; ++k) {
+        const double ck = __shfl_sync(0xffffffffu, c, k);
+        if (lane < EGS_MT_NC) a = fma(ck, (double)kMtCheb[k][lane], a);
+    }
+    __syncwarp();
+    if (lane < EGS_MT_NC) {
+        tab[iv * EGS_MT_NC + lane] = a;
+        vals[lane] = a;
+    }
+    __syncwarp();
+    if (lane == 0)
+        mi::scale_interval(vals, reinterpret_cast<int64_t *>(tab + 2 * EGS_MT_DOUBLES) + iv * (EGS_MT_NC + 1));
     __syncwarp();
 }
 

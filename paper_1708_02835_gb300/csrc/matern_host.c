@@ -95,6 +95,19 @@ int egs_matern_params_init(const double theta[3], egs_matern_params *P)
     /* theta1 2^(-j/64) for the table-driven exponential of the half-integer kinds */
     for (int j = 0; j < EGS_EXP_TAB; ++j)
         P->exp_tab[j] = (double)((q_t)theta[0] * exp2f128(-(q_t)j / (q_t)EGS_EXP_TAB));
+    /* 64-bit mantissas of the integer evaluation */
+    int e = 0;
+    q_t m = frexpf128(0.8f128 / (q_t)theta[1], &e) * 2.0f128;
+    P->iy_m = (uint64_t)rintf128(ldexpf128(m, 63));
+    P->iy_e = e - 1;
+    if (P->iy_m == 0) { /* rounded up to 2 */
+        P->iy_m = (uint64_t)1 << 63;
+        P->iy_e += 1;
+    }
+    m = frexpf128((q_t)theta[0], &e) * 2.0f128;
+    P->th1_e = e - 1;
+    for (int j = 0; j < 256; ++j)
+        P->exp2_tab[j] = (uint64_t)rintf128(ldexpf128(m * exp2f128(-(q_t)j / 256.0f128), 63));
     return 0;
 }
 

@@ -6,6 +6,8 @@
 #ifndef EGS_MATERN_PARAMS_H
 #define EGS_MATERN_PARAMS_H
 
+#include <stdint.h>
+
 #define EGS_TEMME_MAX 24 /* terms of Temme's series (x <= 1.25) */
 #define EGS_CF_MAX 140   /* depth of the backward recurrence (x > 1.25) */
 #define EGS_EXP_TAB 64   /* entries of the exponential's table (2^(j/64)) */
@@ -19,9 +21,11 @@
 #define EGS_MT_NC 12
 #define EGS_MT_E0 (-12)
 #define EGS_MT_DOUBLES (EGS_MT_OCT * EGS_MT_SUB * EGS_MT_NC)
-/* device scratch of a mixed-precision evaluation's generator: the FP64
- * polynomials, then the same split into float pairs */
-#define EGS_MT_SCRATCH_DOUBLES (2 * EGS_MT_DOUBLES)
+/* the same as 64-bit integers, a scale exponent per sub-interval (matern_int.cuh) */
+#define EGS_MT_INTS (EGS_MT_OCT * EGS_MT_SUB * (EGS_MT_NC + 1))
+/* device scratch of an evaluation's generator: the FP64 polynomials, the same
+ * split into float pairs, the integers */
+#define EGS_MT_SCRATCH_DOUBLES (2 * EGS_MT_DOUBLES + EGS_MT_INTS)
 
 /* distance between two locations */
 #define EGS_DIST_EUCLIDEAN 0    /* (x, y) in the plane */
@@ -56,6 +60,11 @@ typedef struct {
     double cf_c[EGS_CF_MAX + 2];    /* C_k = prod_{j=1..k} ((j - 1/2)^2 - mu^2) / j, C_0 = 1 */
     double cf_ic[EGS_CF_MAX + 2];   /* 1 / C_k (unused when half_mu) */
     double exp_tab[EGS_EXP_TAB];    /* theta1 2^(-j/64), j = 0..63: the table of theta1 e^-x */
+    /* the integer evaluation (matern_int.cuh): 0.8 / theta2 = iy_m 2^(iy_e - 63) and
+     * theta1 2^(-j/256) = exp2_tab[j] 2^(th1_e - 63), iy_m and exp2_tab[0] in [2^63, 2^64) */
+    int iy_e, th1_e;
+    uint64_t iy_m;
+    uint64_t exp2_tab[256];
 } egs_matern_params;
 
 /* Constants of the double-float evaluation of the closed-form kinds

@@ -22,11 +22,10 @@ constexpr int OCHUNK = 256;  // observed locations staged per pass
 // 256 / GROUP locations per CTA.  Thread t handles new location t / GROUP and
 // the observed locations t % GROUP + GROUP q of every staged chunk; the GROUP
 // partial sums of a location are combined in a fixed order, so results are
-// bitwise reproducible.  FP64-pipe bound (the Matern evaluation).  tab: the
-// local polynomials of a general nu, built by the evaluation that made x:
-// 25 FP64 operations per entry instead of the direct method's 1,100, and
-// 6.4e7 entries of them took about 120 of the 168 ms of a kriging call from
-// 6,400 to 10,000 locations.
+// bitwise reproducible.  Bound by the Matern evaluation.  tab: the local
+// polynomials of a general nu, built by the evaluation that made x; the direct
+// method (1,100 FP64 operations an entry, 6.4e7 entries) took about 120 of the
+// 168 ms of a kriging call from 6,400 to 10,000 locations.
 template <int GROUP>
 __global__ void __launch_bounds__(256) k_predict(const double *__restrict__ Xn, const double *__restrict__ Yn,
                                                  int64_t m, const double *__restrict__ Xo,
@@ -38,20 +37,17 @@ __global__ void __launch_bounds__(256) k_predict(const double *__restrict__ Xn, 
     if (*(volatile const unsigned long long *)&st->fail_index != kNoFail) return;
     constexpr int PB = 256 / GROUP;  // new locations per CTA
     __shared__ egs_matern_params Ps;
-    __shared__ double T[EGS_MT_DOUBLES];
+    __shared__ double T[EGS_MT_INTS];
     __shared__ double sx[OCHUNK], sy[OCHUNK], sv[OCHUNK];
     {
         const double *s = reinterpret_cast<const double *>(&Pg);
         double *d = reinterpret_cast<double *>(&Ps);
         for (int i = threadIdx.x; i < (int)(sizeof(egs_matern_params) / sizeof(double)); i += blockDim.x) d[i] = s[i];
-        if (tab)
-            for (int i = threadIdx.x; i < EGS_MT_DOUBLES; i += blockDim.x) T[i] = tab[i];
     }
-    const double *Tab = tab ? T : nullptr;
+    const double *Tab = stage_table(&Pg, tab, T);
     const int li = threadIdx.x / GROUP, g = threadIdx.x % GROUP;
     const int64_t i = (int64_t)blockIdx.x * PB + li;
     const double xi = i < m ? Xn[i] : 0.0, yi = i < m ? Yn[i] : 0.0;
-    const double inv_th2 = Pg.inv_th2;
     double acc = 0.0;
     for (int64_t j0 = 0; j0 < n; j0 += OCHUNK) {
         __syncthreads();
@@ -64,7 +60,7 @@ __global__ void __launch_bounds__(256) k_predict(const double *__restrict__ Xn, 
         __syncthreads();
         const int cnt = (n - j0 < OCHUNK) ? (int)(n - j0) : OCHUNK;
         for (int t = g; t < cnt; t += GROUP)
-            acc = fma(matern_eval(&Ps, loc_dist(&Ps, xi, yi, sx[t], sy[t]) * inv_th2, Tab), sv[t], acc);
+            acc = fma(matern_pair(&Ps, Tab, xi, yi, sx[t], sy[t]), sv[t], acc);
     }
 #pragma unroll
     for (int off = (GROUP < 32 ? GROUP : 32) / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
