@@ -102,8 +102,8 @@ static Layout make_layout(const TileGeom &g, bool tc)
     off += align256(sizeof(DevStatus));
     L.mtab = off;
     off += align256(EGS_MT_SCRATCH_DOUBLES * sizeof(double));
-    L.pctr = off;
-    off += align256((size_t)g.T * potrf_diag_scratch_words(g.b) * sizeof(unsigned));
+    L.winv = off;
+    off += align256(kWinvDoubles * sizeof(double));
     L.tc = off;
     if (tc) off += tc64_scratch_bytes(g.b, g.T);
     L.total = off;
@@ -283,20 +283,14 @@ cudaError_t eval_enqueue(const EvalSetup &es, const double *dlocs, const double 
     double *partials = (double *)(ws + es.L.partials);
     if (ev) cudaEventRecord(ev[0], s);
     cudaError_t e = launch_matern_tiles_f64(dlocs, dlocs + n, g, es.P, tiles, s, kt, (double *)(ws + es.L.mtab));
-    if (e == cudaSuccess && es.tc) e = launch_pad_vector(dz, n, zpad, (int64_t)g.T * g.b, s, kt);
+    if (e == cudaSuccess) e = launch_pad_vector(dz, n, zpad, (int64_t)g.T * g.b, s, kt);
     if (e == cudaSuccess) {
         if (ev) cudaEventRecord(ev[1], s);
-        e = launch_potrf_tiles_f64(tiles, g, st, s, kt, (unsigned *)(ws + es.L.pctr), es.tc ? ws + es.L.tc : nullptr,
-                                   zpad);
+        // the forward solve runs along with the factorisation
+        e = launch_potrf_tiles_f64(tiles, g, st, s, kt, (double *)(ws + es.L.winv), es.tc ? ws + es.L.tc : nullptr, zpad);
     }
     if (e == cudaSuccess && ev) cudaEventRecord(ev[2], s);
-    if (es.tc) {
-        const Tiles tl{tiles, nullptr, g.b, g.T, g.T};
-        if (e == cudaSuccess) e = launch_logdet_quad(tl, n, zpad, partials, st, s, kt);
-    } else {
-        if (e == cudaSuccess) e = launch_pad_vector(dz, n, zpad, (int64_t)g.T * g.b, s, kt);
-        if (e == cudaSuccess) e = launch_trsv_tiles_f64(tiles, g, zpad, partials, st, s, kt);
-    }
+    if (e == cudaSuccess) e = launch_logdet_quad(Tiles{tiles, nullptr, g.b, g.T, g.T}, n, zpad, partials, st, s, kt);
     if (e == cudaSuccess && ev) cudaEventRecord(ev[3], s);
     return e;
 }
@@ -443,7 +437,7 @@ egs_status egs_potrf_tiles(void *tiles, int64_t n, int32_t tile, int64_t *fail_i
     DevStatus *st = nullptr;
     const size_t sbytes = align256(sizeof(DevStatus));
     const Allocator A = current_allocator();
-    const size_t cbytes = align256(sbytes + (size_t)g.T * potrf_diag_scratch_words(g.b) * sizeof(unsigned));
+    const size_t cbytes = align256(sbytes + kWinvDoubles * sizeof(double));
     bool tc = tc64_applies(n, tile, g.T);
     size_t wbytes = cbytes + (tc ? tc64_scratch_bytes(g.b, g.T) : 0);
     cudaError_t e = dev_alloc(A, (void **)&st, wbytes, s);
@@ -455,14 +449,14 @@ egs_status egs_potrf_tiles(void *tiles, int64_t n, int32_t tile, int64_t *fail_i
     }
     if (e != cudaSuccess) return cuda_error(e, "egs_potrf_tiles workspace");
     status_init(st, s);
-    e = launch_potrf_tiles_f64((double *)tiles, g, st, s, nullptr, (unsigned *)((char *)st + sbytes),
-                               tc ? (char *)st + cbytes : nullptr);
+    e = launch_potrf_tiles_f64((double *)tiles, g, st, s, nullptr, (double *)((char *)st + sbytes),
+                               tc ? (char *)st + cbytes : nullptr, nullptr);
     DevStatus h;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s);
     dev_free(A, st, wbytes, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(e, "egs_potrf_tiles");
-    if (h.timeout) return set_error(EGS_ERR_TIMEOUT, "egs_potrf_tiles: a dependency wait of the diagonal POTRF timed out");
+    if (h.timeout) return set_error(EGS_ERR_TIMEOUT, "egs_potrf_tiles: a bounded device wait timed out");
     const int64_t fi = (h.fail_index == kNoFail) ? -1 : (int64_t)h.fail_index;
     if (fail_index) *fail_index = fi;
     if (fi >= 0) return set_error(EGS_ERR_NOT_PD, "not positive definite at row %lld", (long long)fi);
@@ -632,8 +626,8 @@ egs_status egs_simulate(const double *locs, const double *e, const double theta[
         err = launch_matern_tiles_f64(dlocs, dlocs + n, g, es.P, tiles, s, nullptr, (double *)(ws + es.L.mtab));
     }
     if (err == cudaSuccess)
-        err = launch_potrf_tiles_f64(tiles, g, st, s, nullptr, (unsigned *)(ws + es.L.pctr),
-                                     es.tc ? ws + es.L.tc : nullptr);
+        err = launch_potrf_tiles_f64(tiles, g, st, s, nullptr, (double *)(ws + es.L.winv),
+                                     es.tc ? ws + es.L.tc : nullptr, nullptr);
     if (err == cudaSuccess) err = launch_pad_vector(de, n, epad, (int64_t)g.T * g.b, s);
     if (err == cudaSuccess) err = launch_trmv_lower(tiles, g, epad, zfull, st, s);
     if (err == cudaSuccess) err = cudaMemcpyAsync(z, zfull, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, s);

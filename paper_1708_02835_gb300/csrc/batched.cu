@@ -395,20 +395,8 @@ __global__ void __launch_bounds__(256) kb_logdet_quad(BatchArgs a)
     const BatchProblem &pr = a.probs[find_problem(a, blockIdx.x, local)];
     if (failed(pr.st)) return;
     __shared__ double red[256];
-    const int b = a.b, k = (int)local;
-    const double *L = dense_tiles(pr, b).t64(k, k), *y = pr.zpad + (size_t)k * b;
-    double s = 0.0, q = 0.0;
-    for (int i = threadIdx.x; i < b; i += 256) {
-        s += log(L[(size_t)i * (b + 1)]);
-        q = fma(y[i], y[i], q);
-    }
-    const double lsum = block_sum(s, red);
-    __syncthreads();
-    const double qsum = block_sum(q, red);
-    if (threadIdx.x == 0) {
-        pr.partials[k] = lsum;
-        pr.partials[pr.T + k] = qsum;
-    }
+    const int k = (int)local;
+    logdet_quad_tile(dense_tiles(pr, a.b).t64(k, k), a.b, pr.zpad + (size_t)k * a.b, red, pr.partials + k, (size_t)pr.T);
 }
 
 __global__ void __launch_bounds__(256) kb_finalize(BatchArgs a)
@@ -703,7 +691,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     }
     size_t off = 0;
     std::vector<size_t> tiles_off(nprob), zpad_off(nprob), part_off(nprob), f32_off(nprob), sig_off(nprob),
-        vec_off(nprob), mtab_off(nprob);
+        vec_off(nprob), mtab_off(nprob), winv_offs(nprob);
     size_t in_doubles = 0;
     for (int i = 0; i < nprob; ++i) {
         if (n[i] < 1) {
@@ -727,6 +715,8 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
         off += a256(npad * sizeof(double));
         part_off[i] = off;
         off += a256((size_t)2 * T * sizeof(double));
+        winv_offs[i] = off;
+        if (!B->mixed && !B->tc) off += a256((size_t)T * (tile / 64) * kWinvDoubles * sizeof(double));
         mtab_off[i] = off;
         off += a256(EGS_MT_SCRATCH_DOUBLES * sizeof(double));
         B->in_off.push_back(in_doubles);
@@ -864,6 +854,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
         pr.P = B->d_params + i;
         pr.cnt = B->dag ? B->d_cnt + cnt_off[i] : nullptr;
         pr.mtab = (double *)(B->ws + mtab_off[i]);
+        pr.winv = (double *)(B->ws + winv_offs[i]);
     }
     e = cudaMemcpy(B->d_probs, B->h_probs, sizeof(BatchProblem) * nprob, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && B->tc) {

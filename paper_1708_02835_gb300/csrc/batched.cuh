@@ -18,7 +18,8 @@ struct BatchProblem {
     double *partials;  // 2T
     DevStatus *st;
     const egs_matern_params *P;
-    unsigned *cnt;     // persistent scheduler: T(T+1)/2 tile counters, then T vector-block counters
+    unsigned *cnt;     // persistent scheduler: T(T+1)/2 tile counters
+    double *winv;      // persistent scheduler: inverses of the 8 x 8 diagonal blocks, kWinvDoubles per 64 columns
     double *mtab;      // EGS_MT_SCRATCH_DOUBLES: the generator's local polynomials (general nu)
 };
 

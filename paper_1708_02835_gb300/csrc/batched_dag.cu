@@ -7,17 +7,17 @@
 // reached the values the task needs:
 //
 //   GEN(i, j)       tile (i, j) of Sigma; GEN(i, i) also copies z block i
-//   POTRF(k)        needs the k updates of tile (k, k)
-//   TRSM(m, k)      needs POTRF(k) and the k updates of tile (m, k)
+//   POTRF(k)        needs the k updates of tile (k, k); also solves z block k and
+//                   forms the tile's log-determinant and dot product
+//   TRSM(m, k)      needs POTRF(k), the k updates of tile (m, k) and GEN(m, m) (z
+//                   block m); also takes tile (m, k)'s product with y_k off z block m
 //   UPDATE(m, n, k) needs TRSM(m, k), TRSM(n, k) and updates 0..k-1 of (m, n)
 //                   (so the updates of a tile are applied in step order)
-//   TRSV(k)         needs POTRF(k) and the k panel products into z block k
-//   GEMV(m, k)      needs TRSV(k), TRSM(m, k) and the earlier products into m
-//   FINAL           needs TRSV(T - 1); assembles l (Eq. 1)
+//   FINAL           needs POTRF(T - 1); assembles l (Eq. 1)
 //
 // Tile counter (i, j) counts 1 for its generation, 1 per update applied and 1
-// when it is final (after POTRF or TRSM); vector counter k counts 1 for its
-// initial copy, 1 per panel product and 1 when the block solve is done.
+// when it is final (after POTRF or TRSM).  The products into z block m need no
+// counter: TRSM(m, k + 1) waits for an update that waits for TRSM(m, k).
 //
 // The list is built on the host in a topological order (checked on the host
 // by replaying it sequentially), so the lowest unfinished task always has its
@@ -45,14 +45,7 @@ namespace egs {
 
 namespace {
 
-enum DagType { D_GEN = 0, D_POTRF, D_TRSM, D_UPDATE, D_TRSV, D_GEMV, D_FINAL };
-
-struct TrsvSmem {
-    double yv[256];
-    double red[256];
-    double D[32][33];
-    double ldq[2];
-};
+enum DagType { D_GEN = 0, D_POTRF, D_TRSM, D_UPDATE, D_FINAL };
 
 // The tasks' shared memory, overlaid: one task runs at a time in a CTA.
 struct GenSmem {
@@ -61,12 +54,9 @@ struct GenSmem {
 };
 
 union DagSmem {
-    TrsmSmem<64, double> trsm;
-    Trsm32Smem trsm32;
-    PotrfSmem<32> potrf32;
+    Chol64Smem chol;
+    Solve64Smem<32> solve;
     GemmSmem<double> gemm;
-    Gemm32Smem gemm32;
-    TrsvSmem trsv;
     GenSmem gen;
     double vec[256];
 };
@@ -117,72 +107,6 @@ __device__ __forceinline__ unsigned *tile_cnt(const BatchProblem &p, int i, int 
     return p.cnt + tile_linear(i, j);
 }
 
-__device__ __forceinline__ unsigned *vec_cnt(const BatchProblem &p, int k)
-{
-    return p.cnt + (size_t)p.T * (p.T + 1) / 2 + k;
-}
-
-// Forward substitution on one diagonal tile, as trsv_fwd_tile but for a CTA
-// of 256 threads and b <= 256 (threads >= b own no row; their zeros enter the
-// fixed-order trees as exact additions, so the sums are those of a CTA of b
-// threads).  Reads go through plain (coherent) loads: the tile and the vector
-// were written earlier in the same launch.
-__device__ void dag_trsv_fwd(TrsvSmem &sm, const double *L, int b, double *v, double *ld_q)
-{
-    double(&yv)[256] = sm.yv;
-    double(&D)[32][33] = sm.D;
-    double *red = sm.red;
-    const int i = threadIdx.x, lane = i & 31, w = i >> 5;
-    const bool own = i < b;
-    const double *Li = L + (size_t)(own ? i : 0) * b;
-    double r = own ? v[i] : 0.0;
-    for (int cb = 0; cb < b / 32; ++cb) {
-        const int c0 = cb * 32;
-        for (int e = i; e < 32 * 32; e += 256) D[e >> 5][e & 31] = L[(size_t)(c0 + (e >> 5)) * b + c0 + (e & 31)];
-        __syncthreads();
-        if (w == cb) {
-            for (int jj = 0; jj < 32; ++jj) {
-                const double yj = __shfl_sync(0xffffffffu, r, jj) / D[jj][jj];
-                if (lane == jj) yv[c0 + jj] = yj;
-                if (lane > jj) r = fma(-D[lane][jj], yj, r);
-            }
-        }
-        __syncthreads();
-        if (own && i >= c0 + 32) {
-            double s = 0.0;
-#pragma unroll 8
-            for (int jj = 0; jj < 32; ++jj) s = fma(Li[c0 + jj], yv[c0 + jj], s);
-            r -= s;
-        }
-    }
-    __syncthreads();
-    const double y = own ? yv[i] : 0.0;
-    if (own) v[i] = y;
-    const double ld = block_sum(own ? log(Li[i]) : 0.0, red);
-    __syncthreads();
-    const double q = block_sum(y * y, red);
-    if (i == 0) {
-        ld_q[0] = ld;
-        ld_q[1] = q;
-    }
-    __syncthreads();
-}
-
-// out[r] -= L[r][:] . ys for the 64 rows r0..r0+63 (as gemv_rows, plain loads).
-__device__ __forceinline__ void dag_gemv_rows(const double *A, int b, int r0, const double *ys, double *out)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int rr = 0; rr < 8; ++rr) {
-        const int r = r0 + warp * 8 + rr;
-        const double *row = A + (size_t)r * b;
-        double s = 0.0;
-        for (int c = lane; c < b; c += 32) s = fma(row[c], ys[c], s);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) out[r] -= s;
-    }
-}
-
 __device__ void task_gen(GenSmem &gs, const BatchProblem &pr, int b, int ti, int tj)
 {
     egs_matern_params &Ps = gs.P;
@@ -218,39 +142,74 @@ __device__ void task_gen(GenSmem &gs, const BatchProblem &pr, int b, int ti, int
         }
 }
 
-// POTRF of diagonal tile k in one CTA: the 32 x 32 block operations of the
-// single-problem diagonal POTRF (chol64.cu) run in its task order -- for each
-// block column p, POTRF of block (p, p) (and the zeros right of it), the
-// 32-row solves below it, then the updates of the trailing blocks -- so every
-// element sees the same operations in the same order and the factor is the
-// single evaluation's bit for bit.
-__device__ void task_potrf(DagSmem &sm, const BatchProblem &pr, int b, int k)
+// The rows below a 64-column block j of tile column k in one tile, 32 at a time: X and the
+// products with y off z (the block of z those rows belong to), as k_solve64.
+__device__ __forceinline__ void solve_tile_rows(Solve64Smem<32> &sm, const BatchProblem &pr, double *tile, int b, int k,
+                                                int j, int row0, double *z)
 {
-    double *A = pr.tiles + (size_t)tile_linear(k, k) * b * b;
-    const int nb = b >> 5;
-    for (int p = 0; p < nb; ++p) {
-        double *Ap = A + (size_t)p * 32 * b + p * 32;
-        if (!potrf_smem_s<32>(sm.potrf32, Ap, b, (int64_t)k * b + p * 32, pr.st)) return;
-        for (int e = threadIdx.x; e < 32 * (b - p * 32 - 32); e += 256) {
-            const int r = e / (b - p * 32 - 32), c = e % (b - p * 32 - 32);
-            Ap[(size_t)r * b + 32 + c] = 0.0;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const double *L = pr.tiles + (size_t)tile_linear(k, k) * b * b + (size_t)j * 64 * (b + 1);
+    const double *y = pr.zpad + (size_t)k * b + j * 64;
+    __syncthreads();
+    solve64_stage(sm, L, b, pr.winv + ((size_t)k * (b / 64) + j) * kWinvDoubles);
+    const double y0 = y[2 * lane], y1 = y[2 * lane + 1];
+    for (int r0 = row0; r0 < b; r0 += 32) {
+        double *X = tile + (size_t)r0 * b + j * 64;
+        for (int e = tid; e < 32 * 64; e += 256) sm.Xs[e >> 6][e & 63] = X[(size_t)(e >> 6) * b + (e & 63)];
+        __syncthreads();
+        solve64_rows(sm);
+        __syncthreads();
+        for (int r = tid >> 5; r < 32; r += 8) {
+            const double x0 = sm.Xs[r][2 * lane], x1 = sm.Xs[r][2 * lane + 1];
+            X[(size_t)r * b + 2 * lane] = x0;
+            X[(size_t)r * b + 2 * lane + 1] = x1;
+            const double v = dot64(x0, x1, y0, y1);
+            if (lane == 0) z[r0 + r] -= v;
         }
         __syncthreads();
-        for (int m = p + 1; m < nb; ++m) trsm32_s(sm.trsm32, Ap, b, A + (size_t)m * 32 * b + p * 32, b);
-        for (int m = p + 1; m < nb; ++m)
-            for (int n = p + 1; n <= m; ++n) {
-                gemm_sub32_s(sm.gemm32, A + (size_t)m * 32 * b + p * 32, b, A + (size_t)n * 32 * b + p * 32, b, 32,
-                             A + (size_t)m * 32 * b + n * 32, b);
-                __syncthreads();
-            }
     }
+}
+
+// The update of a tile's columns right of block j by its solved columns (K = 64), as
+// k_inner_f64; diag: the diagonal tile itself, blocks from its diagonal down.
+__device__ __forceinline__ void inner_update(GemmSmem<double> &sm, double *tile, const double *diag_tile, int b, int j,
+                                             bool diag)
+{
+    const int nj = b >> 6;
+    for (int c = j + 1; c < nj; ++c)
+        for (int r = diag ? c : 0; r < nj; ++r)
+            gemm_sub64_s(sm, tile + (size_t)r * 64 * b + j * 64, b, diag_tile + (size_t)c * 64 * b + j * 64, b, 64,
+                         tile + (size_t)r * 64 * b + c * 64, b);
+    __syncthreads();
+}
+
+// POTRF of diagonal tile k in one CTA, by the single evaluation's 64-column blocks: the same
+// operations on every element in the same order, so factors are equal bit for bit.
+__device__ void task_potrf(DagSmem &sm, const BatchProblem &pr, int b, int k)
+{
+    double *A = pr.tiles + (size_t)tile_linear(k, k) * b * b, *z = pr.zpad + (size_t)k * b;
+    for (int j = 0; j < b / 64; ++j) {
+        if (!diag64_block(sm.chol, A + (size_t)j * 64 * (b + 1), b, b - (j + 1) * 64, z + j * 64,
+                          pr.winv + ((size_t)k * (b / 64) + j) * kWinvDoubles, (int64_t)k * b + j * 64, pr.st))
+            return;
+        __syncthreads();
+        if ((j + 1) * 64 < b) {
+            solve_tile_rows(sm.solve, pr, A, b, k, j, (j + 1) * 64, z);
+            inner_update(sm.gemm, A, A, b, j, true);
+        }
+    }
+    __syncthreads();
+    logdet_quad_tile(A, b, z, sm.vec, pr.partials + k, (size_t)pr.T);
 }
 
 __device__ void task_trsm(DagSmem &sm, const BatchProblem &pr, int b, int m, int k)
 {
     const double *Lkk = pr.tiles + (size_t)tile_linear(k, k) * b * b;
     double *X = pr.tiles + (size_t)tile_linear(m, k) * b * b;
-    for (int r0 = 0; r0 < b; r0 += 64) trsm_rows_s<64>(sm.trsm, Lkk, b, X + (size_t)r0 * b, b, b);
+    for (int j = 0; j < b / 64; ++j) {
+        solve_tile_rows(sm.solve, pr, X, b, k, j, 0, pr.zpad + (size_t)m * b);
+        inner_update(sm.gemm, X, Lkk, b, j, false);
+    }
 }
 
 __device__ void task_update(DagSmem &sm, const BatchProblem &pr, int b, int m, int nc, int k)
@@ -266,25 +225,6 @@ __device__ void task_update(DagSmem &sm, const BatchProblem &pr, int b, int m, i
             gemm_sub64_s(sm.gemm, Am + (size_t)sr * 64 * b, b, An + (size_t)sc * 64 * b, b, b,
                          C + (size_t)sr * 64 * b + sc * 64, b);
         }
-}
-
-__device__ void task_trsv(DagSmem &sm, const BatchProblem &pr, int b, int k)
-{
-    double *ldq = sm.trsv.ldq;
-    dag_trsv_fwd(sm.trsv, pr.tiles + (size_t)tile_linear(k, k) * b * b, b, pr.zpad + (size_t)k * b, ldq);
-    if (threadIdx.x == 0) {
-        pr.partials[k] = ldq[0];
-        pr.partials[pr.T + k] = ldq[1];
-    }
-}
-
-__device__ void task_gemv(DagSmem &sm, const BatchProblem &pr, int b, int m, int k)
-{
-    double *ys = sm.vec;
-    for (int c = threadIdx.x; c < b; c += 256) ys[c] = pr.zpad[(size_t)k * b + c];
-    __syncthreads();
-    const double *A = pr.tiles + (size_t)tile_linear(m, k) * b * b;
-    for (int r0 = 0; r0 < b; r0 += 64) dag_gemv_rows(A, b, r0, ys, pr.zpad + (size_t)m * b);
 }
 
 // l from the log-det and dot partials (as k_finalize / kb_finalize).
@@ -318,17 +258,13 @@ __device__ bool task_wait(int type, int i, int j, int k, const BatchProblem &pr,
 {
     switch (type) {
     case D_POTRF: return dag_wait(tile_cnt(pr, k, k), (unsigned)k + 1, ctl);
-    case D_TRSM:
-        return dag_wait(tile_cnt(pr, k, k), (unsigned)k + 2, ctl) && dag_wait(tile_cnt(pr, i, k), (unsigned)k + 1, ctl);
+    case D_TRSM:  // (i, i) generated: z block i is there
+        return dag_wait(tile_cnt(pr, k, k), (unsigned)k + 2, ctl) && dag_wait(tile_cnt(pr, i, k), (unsigned)k + 1, ctl) &&
+               dag_wait(tile_cnt(pr, i, i), 1u, ctl);
     case D_UPDATE:
         return dag_wait(tile_cnt(pr, i, k), (unsigned)k + 2, ctl) && dag_wait(tile_cnt(pr, j, k), (unsigned)k + 2, ctl) &&
                dag_wait(tile_cnt(pr, i, j), (unsigned)k + 1, ctl);
-    case D_TRSV:
-        return dag_wait(tile_cnt(pr, k, k), (unsigned)k + 2, ctl) && dag_wait(vec_cnt(pr, k), (unsigned)k + 1, ctl);
-    case D_GEMV:
-        return dag_wait(vec_cnt(pr, k), (unsigned)k + 2, ctl) && dag_wait(tile_cnt(pr, i, k), (unsigned)k + 2, ctl) &&
-               dag_wait(vec_cnt(pr, i), (unsigned)k + 1, ctl);
-    case D_FINAL: return dag_wait(vec_cnt(pr, pr.T - 1), (unsigned)pr.T + 1, ctl);
+    case D_FINAL: return dag_wait(tile_cnt(pr, pr.T - 1, pr.T - 1), (unsigned)pr.T + 1, ctl);
     default: return true;  // D_GEN
     }
 }
@@ -338,15 +274,10 @@ __device__ void task_signal(int type, int i, int j, int k, const BatchProblem &p
 {
     __threadfence();
     switch (type) {
-    case D_GEN:
-        atomicAdd(tile_cnt(pr, i, j), 1u);
-        if (i == j) atomicAdd(vec_cnt(pr, i), 1u);
-        break;
+    case D_GEN: atomicAdd(tile_cnt(pr, i, j), 1u); break;
     case D_POTRF: atomicAdd(tile_cnt(pr, k, k), 1u); break;
     case D_TRSM: atomicAdd(tile_cnt(pr, i, k), 1u); break;
     case D_UPDATE: atomicAdd(tile_cnt(pr, i, j), 1u); break;
-    case D_TRSV: atomicAdd(vec_cnt(pr, k), 1u); break;
-    case D_GEMV: atomicAdd(vec_cnt(pr, i), 1u); break;
     default: break;
     }
 }
@@ -388,8 +319,6 @@ __global__ void __launch_bounds__(256, 2) kb_dag(DagArgs a)
             case D_POTRF: task_potrf(sm, pr, a.b, k); break;
             case D_TRSM: task_trsm(sm, pr, a.b, i, k); break;
             case D_UPDATE: task_update(sm, pr, a.b, i, j, k); break;
-            case D_TRSV: task_trsv(sm, pr, a.b, k); break;
-            case D_GEMV: task_gemv(sm, pr, a.b, i, k); break;
             case D_FINAL: task_final(sm, pr); break;
             }
         }
@@ -414,11 +343,11 @@ egs_status dag_plan(const std::vector<int> &T, int b, std::vector<int4> &tasks, 
         if (T[p] > 32767) return set_error(EGS_ERR_ARG, "persistent batch: %d tiles per side is too many", T[p]);
         Tmax = std::max(Tmax, T[p]);
         cnt_off[p] = ncounters;
-        ncounters += (size_t)T[p] * (T[p] + 1) / 2 + T[p];
+        ncounters += (size_t)T[p] * (T[p] + 1) / 2;
     }
     tasks.clear();
     // position key = k + Tmax - T_p; generation at key - 1.  Within a key:
-    // POTRF, TRSM, UPDATE, TRSV, GEMV, FINAL, each over all problems.
+    // POTRF, TRSM, UPDATE, FINAL, each over all problems.
     for (int key = -1; key < Tmax; ++key) {
         for (int p = 0; p < np; ++p) {
             const int k = key - (Tmax - T[p]) + 1;  // generation precedes step 0
@@ -426,7 +355,7 @@ egs_status dag_plan(const std::vector<int> &T, int b, std::vector<int4> &tasks, 
                 for (int i = 0; i < T[p]; ++i)
                     for (int j = 0; j <= i; ++j) tasks.push_back(pack(p, D_GEN, i, j, 0));
         }
-        for (int rank = 0; rank < 6; ++rank)
+        for (int rank = 0; rank < 4; ++rank)
             for (int p = 0; p < np; ++p) {
                 const int k = key - (Tmax - T[p]);
                 if (k < 0 || k >= T[p]) continue;
@@ -440,11 +369,7 @@ egs_status dag_plan(const std::vector<int> &T, int b, std::vector<int4> &tasks, 
                     for (int m = k + 1; m < Tp; ++m)
                         for (int n = k + 1; n <= m; ++n) tasks.push_back(pack(p, D_UPDATE, m, n, k));
                     break;
-                case 3: tasks.push_back(pack(p, D_TRSV, k, k, k)); break;
-                case 4:
-                    for (int m = k + 1; m < Tp; ++m) tasks.push_back(pack(p, D_GEMV, m, k, k));
-                    break;
-                case 5:
+                case 3:
                     if (k == Tp - 1) tasks.push_back(pack(p, D_FINAL, 0, 0, 0));
                     break;
                 }
@@ -455,32 +380,30 @@ egs_status dag_plan(const std::vector<int> &T, int b, std::vector<int4> &tasks, 
     // counter must end at its final value.
     std::vector<unsigned> c(ncounters, 0);
     auto tc = [&](int p, int i, int j) -> unsigned & { return c[cnt_off[p] + (size_t)i * (i + 1) / 2 + j]; };
-    auto vc = [&](int p, int k) -> unsigned & { return c[cnt_off[p] + (size_t)T[p] * (T[p] + 1) / 2 + k]; };
     for (size_t t = 0; t < tasks.size(); ++t) {
         const int4 tk = tasks[t];
         const int p = tk.x, type = tk.y & 0xFFFF, i = tk.y >> 16, j = tk.z & 0xFFFF, k = tk.z >> 16;
         const unsigned uk = (unsigned)k;
         bool ok = true;
         switch (type) {
-        case D_GEN: ++tc(p, i, j); if (i == j) ++vc(p, i); break;
+        case D_GEN: ++tc(p, i, j); break;
         case D_POTRF: ok = tc(p, k, k) >= uk + 1; ++tc(p, k, k); break;
-        case D_TRSM: ok = tc(p, k, k) >= uk + 2 && tc(p, i, k) >= uk + 1; ++tc(p, i, k); break;
+        case D_TRSM:
+            ok = tc(p, k, k) >= uk + 2 && tc(p, i, k) >= uk + 1 && tc(p, i, i) >= 1;
+            ++tc(p, i, k);
+            break;
         case D_UPDATE:
             ok = tc(p, i, k) >= uk + 2 && tc(p, j, k) >= uk + 2 && tc(p, i, j) >= uk + 1;
             ++tc(p, i, j);
             break;
-        case D_TRSV: ok = tc(p, k, k) >= uk + 2 && vc(p, k) >= uk + 1; ++vc(p, k); break;
-        case D_GEMV: ok = vc(p, k) >= uk + 2 && tc(p, i, k) >= uk + 2 && vc(p, i) >= uk + 1; ++vc(p, i); break;
-        case D_FINAL: ok = vc(p, T[p] - 1) >= (unsigned)T[p] + 1; break;
+        case D_FINAL: ok = tc(p, T[p] - 1, T[p] - 1) >= (unsigned)T[p] + 1; break;
         }
         if (!ok) return set_error(EGS_ERR_ARG, "persistent batch: task %zu of the plan is not in dependency order", t);
     }
     for (int p = 0; p < np; ++p)
-        for (int i = 0; i < T[p]; ++i) {
-            if (vc(p, i) != (unsigned)i + 2) return set_error(EGS_ERR_ARG, "persistent batch: incomplete solve plan");
+        for (int i = 0; i < T[p]; ++i)
             for (int j = 0; j <= i; ++j)
                 if (tc(p, i, j) != (unsigned)j + 2) return set_error(EGS_ERR_ARG, "persistent batch: incomplete plan");
-        }
     return EGS_OK;
 }
 

@@ -212,7 +212,8 @@ __device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const double d = __shfl_sync(0xffffffffu, a[j], j);
-                if (ok && !(d > 0.0)) {
+                // normal and positive by its high word, the rest by an FP64 comparison
+                if ((unsigned)__double2hiint(d) - 0x00100000u >= 0x7FE00000u && ok && !(d > 0.0)) {
                     ok = false;
                     if (tid == 0) sm.fail_j = p0 + j;
                 }
@@ -274,6 +275,98 @@ __device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld
     }
     __syncthreads();
     return true;
+}
+
+// The inverses of L's eight 8 x 8 diagonal blocks into winv (row-major, 64 p on), column c of
+// block p by thread 8 p + c (forward substitution); sm as chol64_s left it.
+constexpr int kWinvDoubles = 8 * 8 * 8;
+__device__ __forceinline__ void inv8_blocks(const Chol64Smem &sm, double *winv)
+{
+    const int tid = threadIdx.x;
+    if (tid >= 64) return;
+    const int p = tid >> 3, c = tid & 7, q0 = 8 * p;
+    double w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = i == c ? 1.0 : 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        w[i] *= sm.rd[q0 + i];
+#pragma unroll
+        for (int l = i + 1; l < 8; ++l) w[l] = fma(-sm.S[q0 + l][q0 + i], w[i], w[l]);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) winv[p * 64 + i * 8 + c] = w[i];
+}
+
+// Diagonal block j of a tile (A: its corner, row stride ld; `right` columns of the tile to its
+// right, zeroed): chol64_s and the write-back of L, y and the inverses.  256 threads.
+__device__ __forceinline__ bool diag64_block(Chol64Smem &sm, double *A, int ld, int right, double *z, double *winv,
+                                             int64_t row0, DevStatus *st)
+{
+    const int tid = threadIdx.x;
+    if (!chol64_s(sm, A, ld, z, row0, st)) return false;
+    inv8_blocks(sm, winv);
+    if (z && tid < 64) z[tid] = sm.S[64][tid];
+    for (int e = tid; e < 64 * 64; e += 256) A[(size_t)(e >> 6) * ld + (e & 63)] = sm.S[e >> 6][e & 63];
+    for (int r = tid >> 5; r < 64; r += 8)
+        for (int c = tid & 31; c < right; c += 32) A[(size_t)r * ld + 64 + c] = 0.0;
+    return true;
+}
+
+// X L^T = A for RB rows of 64 columns by 8 RB threads, L a 64 x 64 diagonal block: thread (row, c)
+// has column c of each 8-column block, X_p = (A_p - sum_{i<p} X_i L_pi^T) W_p^T with the
+// inverses W_p of L's 8 x 8 diagonal blocks.  FP64-pipe bound: 288 FMAs a thread at 64 clocks a
+// warp and sub-partition, 9 us for one warp on each (RB = 16), 18 us for two.
+template <int RB>
+struct Solve64Smem {
+    double Ls[56][57];  // L below its 8 x 8 diagonal blocks: rows 8 .. 63, columns 0 .. 55
+    double Xs[RB][65];
+    double Ws[64][9];
+};
+
+template <int RB>
+__device__ __forceinline__ void solve64_stage(Solve64Smem<RB> &sm, const double *L, int ld, const double *winv)
+{
+    constexpr int NT = 8 * RB;
+    const int tid = threadIdx.x;
+#pragma unroll 16
+    for (int e = tid; e < 64 * 64; e += NT) {
+        const int r = e >> 6, c = e & 63;
+        if (r >= 8 && c < 56 && c < r) sm.Ls[r - 8][c] = L[(size_t)r * ld + c];
+    }
+    for (int e = tid; e < kWinvDoubles; e += NT) sm.Ws[e >> 3][e & 7] = winv[e];
+}
+
+// Xs holds A on entry and X on return; barriers around it are the caller's.
+template <int RB>
+__device__ __forceinline__ void solve64_rows(Solve64Smem<RB> &sm)
+{
+    const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        double r = sm.Xs[ty][8 * p + tx];
+#pragma unroll 8
+        for (int l = 0; l < 8 * p; ++l) r = fma(-sm.Xs[ty][l], sm.Ls[8 * (p - 1) + tx][l], r);
+        // a row's 8 entries belong to 8 lanes of one warp
+        __syncwarp();
+        sm.Xs[ty][8 * p + tx] = r;
+        __syncwarp();
+        double x = 0.0;
+#pragma unroll
+        for (int l = 0; l < 8; ++l) x = fma(sm.Xs[ty][8 * p + l], sm.Ws[8 * p + tx][l], x);
+        __syncwarp();
+        sm.Xs[ty][8 * p + tx] = x;
+        __syncwarp();
+    }
+}
+
+// X_row . y over 64 columns, two per lane (y0, y1: the lane's entries of y); the sum in lane 0.
+__device__ __forceinline__ double dot64(double x0, double x1, double y0, double y1)
+{
+    double v = fma(x0, y0, x1 * y1);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
 }
 
 // ---------------------------------------------------------------------------
@@ -402,49 +495,6 @@ __device__ __forceinline__ void trsm_rows(const double *Lp, int ldl, TX *Xp, int
 }
 
 // ---------------------------------------------------------------------------
-// X L^T = A for one 32 x 32 block (the TRSM tasks of the diagonal-tile task
-// graphs): X and A at Xp (row stride ldx, solved in place), L lower at Lp
-// (row stride ldl).  Four threads per row split each dot product over the
-// solved columns (l = q mod 4) and combine it with two shuffles in a fixed
-// order, so 4 warps (one per SM sub-partition) share the substitution and
-// the row's chain per column is about j / 4 FMAs, two additions and a
-// multiplication by 1 / L_jj.  256 threads (warps 4-7 only stage the block).
-// ---------------------------------------------------------------------------
-struct Trsm32Smem {
-    double X[32][33];
-    double L[32][33];
-    double rd[32];
-};
-
-__device__ __forceinline__ void trsm32_s(Trsm32Smem &sm, const double *Lp, int ldl, double *Xp, int ldx)
-{
-    const int tid = threadIdx.x;
-    for (int e = tid; e < 32 * 32; e += 256) {
-        const int r = e >> 5, c = e & 31;
-        sm.X[r][c] = Xp[(size_t)r * ldx + c];
-        sm.L[r][c] = c <= r ? Lp[(size_t)r * ldl + c] : 0.0;
-    }
-    if (tid < 32) sm.rd[tid] = 1.0 / Lp[(size_t)tid * ldl + tid];
-    __syncthreads();
-    if (tid < 128) {
-        const int r = tid >> 2, q = tid & 3;
-        for (int j = 0; j < 32; ++j) {
-            double part = 0.0;
-            for (int l = q; l < j; l += 4) part = fma(sm.X[r][l], sm.L[j][l], part);
-            part += __shfl_xor_sync(0xffffffffu, part, 1);
-            part += __shfl_xor_sync(0xffffffffu, part, 2);
-            const double x = (sm.X[r][j] - part) * sm.rd[j];
-            __syncwarp();
-            if (q == 0) sm.X[r][j] = x;
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-    for (int e = tid; e < 32 * 32; e += 256) Xp[(size_t)(e >> 5) * ldx + (e & 31)] = sm.X[e >> 5][e & 31];
-    __syncthreads();  // sm is free for the next block
-}
-
-// ---------------------------------------------------------------------------
 // C (64 x 64, row stride ldc) -= Am (64 x K) An (64 x K)^T with row strides
 // lda, ldb; the operands may be FP64 or FP32 and are converted to the
 // accumulation type TC on staging (TC = double: FP64 products and sums of
@@ -522,6 +572,24 @@ __device__ __forceinline__ double block_sum(double v, double *red)
         __syncthreads();
     }
     return red[0];
+}
+
+// A tile's sums of log L_ii and y_i^2 into out[0] and out[stride]; red: 256 doubles, 256 threads.
+__device__ __forceinline__ void logdet_quad_tile(const double *L, int b, const double *y, double *red, double *out,
+                                                 size_t stride)
+{
+    double a = 0.0, q = 0.0;
+    for (int i = threadIdx.x; i < b; i += 256) {
+        a += log(L[(size_t)i * (b + 1)]);
+        q = fma(y[i], y[i], q);
+    }
+    const double lsum = block_sum(a, red);
+    __syncthreads();
+    const double qsum = block_sum(q, red);
+    if (threadIdx.x == 0) {
+        out[0] = lsum;
+        out[stride] = qsum;
+    }
 }
 
 // Forward substitution on one diagonal tile: y = L^-1 r in place on v

@@ -158,14 +158,11 @@ cudaError_t launch_matern_tiles_f64(const double *X, const double *Y, const Tile
 cudaError_t launch_matern_table(const egs_matern_params &P, double *tab, cudaStream_t s, KernelTimer *kt = nullptr);
 
 // Tile Cholesky in place (FP64).  Stops doing work once st->fail_index is set.
-// ctr: T * potrf_diag_scratch_words(b) words of device scratch for the
-// one-launch diagonal POTRFs (zeroed here).  tc_scratch: tc64_scratch_bytes(b, T) bytes
-// for the tensor-core update, or NULL for the DFMA update.  With it, z (T b doubles, may be
-// NULL) is solved along: L^-1 z in place.
+// z (T b doubles, may be NULL) is solved along: L^-1 z in place.  tc_scratch:
+// tc64_scratch_bytes(b, T) bytes for the tensor-core update, or NULL for the DFMA
+// update, which needs winv (kWinvDoubles doubles of scratch).
 cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *st, cudaStream_t s,
-                                   KernelTimer *kt, unsigned *ctr, void *tc_scratch = nullptr, double *z = nullptr);
-// Counter words one diagonal tile's one-launch POTRF needs.
-size_t potrf_diag_scratch_words(int b);
+                                   KernelTimer *kt, double *winv, void *tc_scratch, double *z);
 
 // Forward solve L y = z in place on zpad (T*b doubles, padded with zeros),
 // with per-tile log-det / dot partials and the final assembly into st->result.
@@ -228,7 +225,7 @@ cudaError_t run_loglik_mixed(const double *X, const double *Y, const double *z, 
 
 // Layouts and setup of one evaluation (api.cu), shared with the serving loop.
 struct Layout {
-    size_t tiles, locs, z, zpad, partials, status, mtab, pctr, tc, total;
+    size_t tiles, locs, z, zpad, partials, status, mtab, winv, tc, total;
 };
 struct MixedLayout {
     size_t f64, f32, slots, panel, oz, l32, wsp, vinv, locs, z, vec, partials, status, err, mtab, dpan, rs, total;
@@ -271,10 +268,6 @@ bool mixed_result_ok(const EvalSetup &es, const DevStatus &h);
 int32_t default_tile(int64_t n, egs_precision p);
 
 // Building blocks shared by the FP64 and mixed drivers.
-// POTRF of diagonal tile k: one launch over the task graph of its 32 x 32
-// blocks; ctr: zeroed potrf_diag_scratch_words(b) words for its counters.
-cudaError_t launch_potrf_diag(const Tiles &tl, int k, DevStatus *st, cudaStream_t s, KernelTimer *kt, unsigned *ctr);
-cudaError_t launch_trsm_f64(const Tiles &tl, int k, int nrows, DevStatus *st, cudaStream_t s, KernelTimer *kt);
 // FP64 update of the first ntri tiles of step k's trailing triangle (row order).
 cudaError_t launch_update_f64(const Tiles &tl, int k, int64_t ntri, DevStatus *st, cudaStream_t s, KernelTimer *kt,
                               int cls = KC_UPDATE);

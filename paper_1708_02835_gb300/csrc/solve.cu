@@ -92,20 +92,8 @@ __global__ void __launch_bounds__(256) k_logdet_quad(Tiles tl, const double *__r
 {
     if (failed_s(st)) return;
     __shared__ double red[256];
-    const int b = tl.b, k = (int)blockIdx.x;
-    const double *L = tl.t64(k, k), *yk = y + (size_t)k * b;
-    double a = 0.0, q = 0.0;
-    for (int i = threadIdx.x; i < b; i += 256) {
-        a += log(L[(size_t)i * (b + 1)]);
-        q = fma(yk[i], yk[i], q);
-    }
-    const double lsum = block_sum(a, red);
-    __syncthreads();
-    const double qsum = block_sum(q, red);
-    if (threadIdx.x == 0) {
-        partials[k] = lsum;
-        partials[tl.T + k] = qsum;
-    }
+    const int k = (int)blockIdx.x;
+    logdet_quad_tile(tl.t64(k, k), tl.b, y + (size_t)k * tl.b, red, partials + k, (size_t)tl.T);
 }
 
 cudaError_t launch_logdet_quad(const Tiles &tl, int64_t n, const double *y, double *partials, DevStatus *st,

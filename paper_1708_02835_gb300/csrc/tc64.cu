@@ -145,41 +145,18 @@ __global__ void __launch_bounds__(256) k_slice_panel64(const __grid_constant__ F
 // diagonal tiles and 100 ms of whole-tile solves became 30 + 17 + 12 ms; the evaluation went
 // from 193 to 120 ms, that of n = 5,000 (tile 256) from 27.0 to 18.9 ms.
 constexpr int PW = kF64Panel;
-constexpr int PI = 8;        // inverted sub-blocks
-static_assert(kWinvDoubles == (PW / PI) * PI * PI, "one inverse per 8 x 8 diagonal block");
+static_assert(PW == 64, "the block routines' size");
 
-// One CTA per problem, 256 threads.  winv: the inverses W_pp, row-major, at 64 p.  The block
-// of the right-hand side becomes y_j.
+// One CTA per problem, 256 threads.  The block of the right-hand side becomes y_j.
 __global__ void __launch_bounds__(256) k_diag64(const __grid_constant__ F64Set set, int k, int j)
 {
     __shared__ Chol64Smem sm;
     const F64Prob &P = set.get(blockIdx.y);
     const Tiles &tl = P.tl;
     if (k >= tl.T || failed(P.st)) return;
-    const int b = tl.b, tid = threadIdx.x;
-    double *A = tl.t64(k, k) + (size_t)j * PW * (b + 1);
-    double *z = P.z ? P.z + (size_t)k * b + j * PW : nullptr;
-    if (!chol64_s(sm, A, b, z, (int64_t)k * b + j * PW, P.st)) return;
-    // column c of W_pp by forward substitution, one thread each
-    if (tid < PW) {
-        const int p = tid / PI, c = tid % PI, q0 = p * PI;
-        double w[PI];
-#pragma unroll
-        for (int i = 0; i < PI; ++i) w[i] = i == c ? 1.0 : 0.0;
-#pragma unroll
-        for (int i = 0; i < PI; ++i) {
-            w[i] *= sm.rd[q0 + i];
-#pragma unroll
-            for (int l = i + 1; l < PI; ++l) w[l] = fma(-sm.S[q0 + l][q0 + i], w[i], w[l]);
-        }
-#pragma unroll
-        for (int i = 0; i < PI; ++i) P.winv[p * PI * PI + i * PI + c] = w[i];
-        if (z) z[tid] = sm.S[64][tid];
-    }
-    for (int e = tid; e < PW * PW; e += 256) A[(size_t)(e >> 6) * b + (e & 63)] = sm.S[e >> 6][e & 63];
-    const int right = b - (j + 1) * PW;
-    for (int r = tid >> 5; r < PW; r += 8)
-        for (int c = tid & 31; c < right; c += 32) A[(size_t)r * b + PW + c] = 0.0;
+    const int b = tl.b;
+    diag64_block(sm, tl.t64(k, k) + (size_t)j * PW * (b + 1), b, b - (j + 1) * PW,
+                 P.z ? P.z + (size_t)k * b + j * PW : nullptr, P.winv, (int64_t)k * b + j * PW, P.st);
 }
 
 // One warp slices the 64 entries of a row: lane's entries 2 lane, 2 lane + 1.
@@ -200,65 +177,39 @@ __device__ __forceinline__ void slice7_row64(double x0, double x1, uint16_t *__r
         *reinterpret_cast<uint32_t *>(dst + (size_t)i * stride + 2 * lane) = d0[i] | (d1[i] << 16);
 }
 
-// Panel rows (j + 1) 64 .. (T - k) b - 1, RB rows and 8 RB threads per CTA: thread (row, c) has
-// column c of each 8-column block.  FP64-pipe bound: 288 FMAs a thread at 64 clocks a warp
-// and sub-partition, 9 us for one warp on each (RB = 16), 18 us for two; RB = 32 (the staged
+// Panel rows (j + 1) 64 .. (T - k) b - 1, RB rows and 8 RB threads per CTA.  RB = 32 (the staged
 // block of L serves twice the rows) once RB = 16 fills the SMs.
 template <int RB>
 __global__ void __launch_bounds__(8 * RB) k_solve64(const __grid_constant__ F64Set set, int k, int j)
 {
     constexpr int NT = 8 * RB;
-    // L below its 8 x 8 diagonal blocks: rows 8 .. 63, columns 0 .. 55
-    __shared__ double Ls[PW - PI][PW - PI + 1], Xs[RB][PW + 1], Ws[PW][PI + 1];
+    __shared__ Solve64Smem<RB> sm;
     const F64Prob &P = set.get(blockIdx.y);
     const Tiles &tl = P.tl;
     const int T = set.solo ? k + 1 : tl.T;
     if ((int64_t)(j + 1) * PW + (int64_t)blockIdx.x * RB >= (int64_t)(T - k) * tl.b || failed(P.st)) return;
-    const int b = tl.b, tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int b = tl.b, tid = threadIdx.x, lane = tid & 31;
     const int pr0 = (j + 1) * PW + (int)blockIdx.x * RB;
     double *X = tl.t64(k + pr0 / b, k) + (size_t)(pr0 % b) * b + j * PW;
-    const double *L = tl.t64(k, k) + (size_t)j * PW * (b + 1);
-    for (int e = tid; e < RB * PW; e += NT) Xs[e >> 6][e & 63] = X[(size_t)(e >> 6) * b + (e & 63)];
-#pragma unroll 4
-    for (int e = tid; e < PW * PW; e += NT) {
-        const int r = e >> 6, c = e & 63;
-        if (r >= PI && c < PW - PI && c < r) Ls[r - PI][c] = L[(size_t)r * b + c];
-    }
-    for (int e = tid; e < (int)kWinvDoubles; e += NT) Ws[e >> 3][e & 7] = P.winv[e];
-    __syncthreads();
 #pragma unroll
-    for (int p = 0; p < PW / PI; ++p) {
-        double r = Xs[ty][PI * p + tx];
-#pragma unroll 8
-        for (int l = 0; l < PI * p; ++l) r = fma(-Xs[ty][l], Ls[PI * (p - 1) + tx][l], r);
-        // a row's 8 entries belong to 8 lanes of one warp
-        __syncwarp();
-        Xs[ty][PI * p + tx] = r;
-        __syncwarp();
-        double x = 0.0;
-#pragma unroll
-        for (int l = 0; l < PI; ++l) x = fma(Xs[ty][PI * p + l], Ws[PI * p + tx][l], x);
-        __syncwarp();
-        Xs[ty][PI * p + tx] = x;
-        __syncwarp();
-    }
-    __syncthreads();
-    const int lane = tid & 31;
+    for (int e = tid; e < RB * PW; e += NT) sm.Xs[e >> 6][e & 63] = X[(size_t)(e >> 6) * b + (e & 63)];
+    solve64_stage(sm, tl.t64(k, k) + (size_t)j * PW * (b + 1), b, P.winv);
     // z_row -= X_row . y_j: the forward solve, while the rows are here
     double y0 = 0.0, y1 = 0.0;
     if (P.z) {
         y0 = P.z[(size_t)k * b + j * PW + 2 * lane];
         y1 = P.z[(size_t)k * b + j * PW + 2 * lane + 1];
     }
+    __syncthreads();
+    solve64_rows(sm);
+    __syncthreads();
     for (int r = tid >> 5; r < RB; r += NT / 32) {
         const size_t sr = P.inner.row0 + pr0 + r;
-        const double x0 = Xs[r][2 * lane], x1 = Xs[r][2 * lane + 1];
+        const double x0 = sm.Xs[r][2 * lane], x1 = sm.Xs[r][2 * lane + 1];
         *reinterpret_cast<double2 *>(X + (size_t)r * b + 2 * lane) = make_double2(x0, x1);
-        slice7_row64(x0, x1, P.inner.sl + sr * PW, P.inner.rows * PW, P.inner.ex + sr);
+        if (P.inner.sl) slice7_row64(x0, x1, P.inner.sl + sr * PW, P.inner.rows * PW, P.inner.ex + sr);
         if (P.z) {
-            double v = fma(x0, y0, x1 * y1);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            const double v = dot64(x0, x1, y0, y1);
             if (lane == 0) P.z[(size_t)k * b + pr0 + r] -= v;
         }
     }
@@ -768,22 +719,37 @@ static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, con
     return cudaGetLastError();
 }
 
+cudaError_t launch_diag_solve64(const F64Set &set, int k, int j, cudaStream_t s, KernelTimer *kt)
+{
+    EGS_LAUNCH(kt, KC_POTRF, s, k_diag64<<<dim3(1, (unsigned)set.count), 256, 0, s>>>(set, k, j));
+    const int64_t rows = (int64_t)(set.solo ? 1 : set.Tmax - k) * set.b - (j + 1) * PW;
+    if (rows > 0) {
+        if (rows / 16 * set.count <= device_sms())
+            EGS_LAUNCH(kt, KC_TRSM, s,
+                       k_solve64<16><<<dim3((unsigned)(rows / 16), (unsigned)set.count), 128, 0, s>>>(set, k, j));
+        else
+            EGS_LAUNCH(kt, KC_TRSM, s,
+                       k_solve64<32><<<dim3((unsigned)(rows / 32), (unsigned)set.count), 256, 0, s>>>(set, k, j));
+    }
+    return cudaGetLastError();
+}
+
+F64Prob dfma_problem(double *winv, const Tiles &tl, DevStatus *st, double *z)
+{
+    F64Prob P{};
+    P.tl = tl;
+    P.st = st;
+    P.z = z;
+    P.winv = winv;
+    return P;
+}
+
 cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, cudaStream_t s, KernelTimer *kt)
 {
     const int nj = set.b / PW;
     cudaError_t e = cudaSuccess;
     for (int j = 0; j < nj && e == cudaSuccess; ++j) {
-        EGS_LAUNCH(kt, KC_POTRF, s, k_diag64<<<dim3(1, (unsigned)set.count), 256, 0, s>>>(set, k, j));
-        const int64_t rows = (int64_t)(set.solo ? 1 : set.Tmax - k) * set.b - (j + 1) * PW;
-        if (rows > 0) {
-            if (rows / 16 * set.count <= device_sms())
-                EGS_LAUNCH(kt, KC_TRSM, s,
-                           k_solve64<16><<<dim3((unsigned)(rows / 16), (unsigned)set.count), 128, 0, s>>>(set, k, j));
-            else
-                EGS_LAUNCH(kt, KC_TRSM, s,
-                           k_solve64<32><<<dim3((unsigned)(rows / 32), (unsigned)set.count), 256, 0, s>>>(set, k, j));
-        }
-        e = cudaGetLastError();
+        e = launch_diag_solve64(set, k, j, s, kt);
         if (e == cudaSuccess && j + 1 < nj)
             e = launch_tc_f64(maps.ia, maps.ib, set, k, j + 1, nj, 1, k * (2 + nj) + 2 + j, 0, s, kt);
     }

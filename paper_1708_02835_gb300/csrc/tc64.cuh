@@ -1,5 +1,6 @@
 // Host interface of the FP64 factorisation on the tensor cores (tc64.cu).
 #pragma once
+#include "blocks.cuh"
 #include "egs_internal.cuh"
 
 namespace egs {
@@ -28,7 +29,7 @@ struct F64Prob {
     DevStatus *st;
     double *z;                // T b: the right-hand side, solved along (L^-1 z); NULL: none
     F64Rows panel;            // K = b: row r of tile m at row0 + (m - k - 1) b + r
-    F64Rows inner;            // K = 64, the current 64-column block: row0 + (m - k) b + r
+    F64Rows inner;            // K = 64, the current 64-column block: row0 + (m - k) b + r; sl NULL: no slices
     unsigned long long *ctr;  // tc64_counters(b, T) zeroed work counters
     double *winv;             // inverses of the block's eight 8 x 8 diagonal blocks
 };
@@ -45,7 +46,6 @@ struct F64Set {
 
 // Work counters of a problem: two trailing updates and b / 64 inner ones per step.
 inline size_t tc64_counters(int b, int T) { return (size_t)T * (2 + b / kF64Panel); }
-constexpr size_t kWinvDoubles = 8 * 8 * 8;
 
 struct F64Maps {
     CUtensorMap a, b, ia, ib;  // panel slices, inner slices
@@ -57,6 +57,11 @@ cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64
 size_t tc64_scratch_bytes(int b, int T);
 size_t tc64_solo_bytes(int b, int T);  // of the POTRFs of T diagonal tiles
 F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st, double *z, bool solo = false);
+
+// The same without slices, for the DFMA updates; winv: kWinvDoubles of scratch.
+F64Prob dfma_problem(double *winv, const Tiles &tl, DevStatus *st, double *z);
+// Diagonal block j of step k; the solves of the rows below it (launch_panel64's first two parts).
+cudaError_t launch_diag_solve64(const F64Set &set, int k, int j, cudaStream_t s, KernelTimer *kt);
 
 // POTRF of tile (k, k) and the solves of every tile below it, in 64-column blocks.
 cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, cudaStream_t s, KernelTimer *kt);
