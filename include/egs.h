@@ -160,8 +160,9 @@ egs_status egs_trace_last(egs_trace_rec *out, int64_t cap, int64_t *count);
  * egs_set_allocator - the device memory of the library's calls (per-call
  * workspaces, serving slots and fields, batch plans) from the caller's
  * allocator, for example a framework's caching allocator, instead of
- * cudaMallocAsync / cudaFreeAsync on the call's stream.  The paper has no
- * counterpart: this is the boundary's memory-management convention.
+ * the library's own stream-ordered pool (which keeps up to 4 GiB between
+ * calls).  The paper has no counterpart: this is the boundary's
+ * memory-management convention.
  *   alloc(bytes, stream, ctx)   returns device memory of at least bytes
  *                               bytes, usable in stream order on stream
  *                               (a cudaStream_t), aligned to 256 bytes; NULL
@@ -171,7 +172,7 @@ egs_status egs_trace_last(egs_trace_rec *out, int64_t cap, int64_t *count);
  *                               stream may still use ptr, so the allocator
  *                               must not hand it out to another stream
  *                               before that work has finished
- * Both NULL restores cudaMallocAsync / cudaFreeAsync; one NULL is
+ * Both NULL restores the library's pool; one NULL is
  * EGS_ERR_ARG.  Memory is always returned to the allocator that provided it,
  * also when the allocator is replaced in the meantime.  The library may call
  * the hooks from its serving thread, with its internal locks held: a hook
@@ -304,14 +305,16 @@ egs_status egs_loglik_ex(const double *locs, const double *z, const double theta
  * Batched evaluation (independent problems: uneven n, own theta each).
  *
  * Each problem is Eq. 1 evaluated by Algorithm 2 exactly as egs_loglik does
- * in EGS_FP64.  EGS_FP64 batches with tile <= 256 run as ONE persistent
+ * in EGS_FP64.  An EGS_FP64 batch with a problem of more than 2048 rows runs
+ * as step-synchronous launches on the tensor cores, each covering one step of
+ * every problem.  Other EGS_FP64 batches with tile <= 256 run as ONE persistent
  * kernel launch: the tile tasks of every problem (Matern tiles, the POTRF /
  * TRSM / SYRK-GEMM tasks of the tile Cholesky of Section 5.2 -- the DAG of
  * its tile algorithm -- and the forward-solve tasks) form one list in a
  * dependency order checked when the plan is made, and each CTA claims the
  * next task and waits on per-tile device counters until its inputs are final
- * (every wait bounded: EGS_ERR_TIMEOUT if one runs out).  Every l of a problem
- * with n <= 2048 is bitwise equal to egs_loglik_ex's with the same tile.  Other batches (EGS_MIX_FP32,
+ * (every wait bounded: EGS_ERR_TIMEOUT if one runs out).  Every l is then bitwise
+ * equal to egs_loglik_ex's with the same tile.  Other batches (EGS_MIX_FP32,
  * or tiles above 256) run as step-synchronous launches, each covering one
  * step of every problem.  Either way the run is captured into a CUDA graph on
  * the first egs_batch_run and replayed afterwards.
@@ -371,7 +374,9 @@ int64_t egs_batch_tasks(const egs_batch *batch);
  * NaN) with the batch still usable.  withhold_task in [0, egs_batch_tasks)
  * makes the launch never signal that task's completion, so that the waits
  * on it run out (for tests of this path); -1 signals every task.  Applies to
- * the following runs.  EGS_ERR_UNIMPLEMENTED for a step-synchronous batch.
+ * the following runs.  A tensor-core batch has no tasks: it accepts a limit,
+ * and its waits keep their own of 2 s.  EGS_ERR_UNIMPLEMENTED for another
+ * step-synchronous batch.
  */
 egs_status egs_batch_set_wait_limit(egs_batch *batch, int64_t limit_ns, int64_t withhold_task);
 

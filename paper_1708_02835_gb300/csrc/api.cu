@@ -42,9 +42,58 @@ Allocator current_allocator()
     return g_alloc;
 }
 
+// The library's memory pool of the current device.  The default pool gives its memory back to
+// the system at every synchronisation, so that each call mapped its workspace anew: 0.44 ms of
+// the 2.0 ms of an n = 777 evaluation, 4 ms at n = 16,900 (1.4 GB).  This one keeps up to
+// kPoolKeep bytes between calls; beyond that it gives back, and all of it when an allocation
+// fails.  Streams do not wait for one another's memory.
+constexpr uint64_t kPoolKeep = 4ull << 30;
+constexpr int kMaxDevices = 64;
+
+static cudaError_t lib_pool(cudaMemPool_t *pool)
+{
+    static std::mutex mu;
+    static cudaMemPool_t pools[kMaxDevices] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= kMaxDevices) return cudaDeviceGetDefaultMemPool(pool, dev);
+    std::lock_guard<std::mutex> lk(mu);
+    if (!pools[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t q = nullptr;
+        e = cudaMemPoolCreate(&q, &props);
+        uint64_t keep = kPoolKeep;
+        int no = 0;
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(q, cudaMemPoolReuseAllowInternalDependencies, &no);
+        if (e != cudaSuccess) {
+            if (q) cudaMemPoolDestroy(q);
+            return e;
+        }
+        pools[dev] = q;
+    }
+    *pool = pools[dev];
+    return cudaSuccess;
+}
+
 cudaError_t dev_alloc(const Allocator &A, void **p, size_t bytes, cudaStream_t s)
 {
-    if (!A.alloc) return cudaMallocAsync(p, bytes, s);
+    if (!A.alloc) {
+        cudaMemPool_t pool = nullptr;
+        cudaError_t e = lib_pool(&pool);
+        if (e != cudaSuccess) return e;
+        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+        if (e == cudaErrorMemoryAllocation) {  // what earlier calls left mapped may not fit this one
+            cudaGetLastError();
+            cudaMemPoolTrimTo(pool, 0);
+            e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+        }
+        return e;
+    }
     *p = A.alloc(bytes, (void *)s, A.ctx);
     if (!*p) return cudaErrorMemoryAllocation;
     if (((uintptr_t)*p & 255) != 0) {  // the layouts need 256-byte alignment

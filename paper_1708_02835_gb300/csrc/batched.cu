@@ -11,6 +11,7 @@
 // the whole sequence is captured once into a CUDA graph and replayed.
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -443,6 +444,8 @@ struct egs_batch {
     char *ws = nullptr;
     size_t ws_bytes = 0;
     Allocator alloc{};  // the allocator that provided ws
+    bool once = false;    // lives for one call: no graph, pageable staging
+    bool pooled = false;  // ws from dev_alloc, not cudaMalloc
     BatchProblem *d_probs = nullptr;
     egs_matern_params *d_params = nullptr;
     DevStatus *d_status = nullptr;
@@ -667,8 +670,10 @@ cudaError_t enqueue_all(egs_batch *B, cudaStream_t s)
 // all its problems (96 problems of 256 to 4,096 rows, tile 128: 607 ms as one persistent
 // launch of DFMA tasks, 101 ms so); without such a problem it stays on the persistent launch,
 // whose results equal single evaluations bit for bit.  any_size (the independent-blocks
-// approximation, whose blocks are no single evaluations): whatever the sizes.
-egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_precision p, bool any_size, egs_batch **out)
+// approximation, whose blocks are no single evaluations): whatever the sizes.  once: the batch
+// lives for one call, its memory comes from the pool.
+egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_precision p, bool any_size, bool once,
+                        egs_batch **out)
 {
     if (!out || !n || nprob < 1) return set_error(EGS_ERR_ARG, "egs_batch_create: bad arguments");
     *out = nullptr;
@@ -789,10 +794,12 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     off += a256(sizeof(DagCtl));
     B->ws_bytes = off;
     B->alloc = current_allocator();
+    B->once = once;
+    B->pooled = B->alloc.alloc || once;
     cudaError_t e;
-    if (!B->alloc.alloc) {
+    if (!B->pooled) {
         e = cudaMalloc((void **)&B->ws, off);
-    } else {  // the caller's hook, on the legacy stream (the batch outlives any call's stream)
+    } else {  // the caller's hook or the pool, on the legacy stream (the batch outlives any call's stream)
         e = dev_alloc(B->alloc, (void **)&B->ws, off, nullptr);
         if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     }
@@ -805,9 +812,14 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     B->d_status = (DevStatus *)(B->ws + status_off);
     B->d_inputs = (double *)(B->ws + inputs_off);
     B->d_prefix = (int64_t *)(B->ws + prefix_off);
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&B->h_probs, sizeof(BatchProblem) * nprob);
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&B->h_params, sizeof(egs_matern_params) * nprob);
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&B->h_status, sizeof(DevStatus) * nprob);
+    auto host = [&](void **p, size_t bytes) {
+        if (!once) return cudaMallocHost(p, bytes);
+        *p = std::calloc(1, bytes);
+        return *p ? cudaSuccess : cudaErrorMemoryAllocation;
+    };
+    if (e == cudaSuccess) e = host((void **)&B->h_probs, sizeof(BatchProblem) * nprob);
+    if (e == cudaSuccess) e = host((void **)&B->h_params, sizeof(egs_matern_params) * nprob);
+    if (e == cudaSuccess) e = host((void **)&B->h_status, sizeof(DevStatus) * nprob);
     if (e == cudaSuccess && !prefix.empty())
         e = cudaMemcpy(B->d_prefix, prefix.data(), prefix.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
     if (B->dag) {
@@ -816,7 +828,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
         B->d_ctl = (DagCtl *)(B->ws + ctl_off);
         B->grid = dag_grid();
         if (B->grid < 1) e = cudaErrorInvalidConfiguration;
-        if (e == cudaSuccess) e = cudaMallocHost((void **)&B->h_ctl, 2 * sizeof(DagCtl));
+        if (e == cudaSuccess) e = host((void **)&B->h_ctl, 2 * sizeof(DagCtl));
         if (e == cudaSuccess)
             e = cudaMemcpy(B->d_tasks, tasks.data(), tasks.size() * sizeof(int4), cudaMemcpyHostToDevice);
     }
@@ -887,7 +899,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
 
 extern "C" egs_status egs_batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_precision p, egs_batch **out)
 {
-    return batch_create(nprob, n, tile, p, false, out);
+    return batch_create(nprob, n, tile, p, false, false, out);
 }
 
 namespace {
@@ -895,7 +907,7 @@ namespace {
 // After the inputs have been staged on B->cs: the parameters, the graph
 // (captured on first use; a batch that runs once goes without) and the statuses back to the
 // host; synchronises.
-cudaError_t run_staged(egs_batch *B, cudaStream_t us, cudaError_t e, bool once = false)
+cudaError_t run_staged(egs_batch *B, cudaStream_t us, cudaError_t e)
 {
     if (B->dag) {
         std::memset(B->h_ctl, 0, 2 * sizeof(DagCtl));
@@ -905,7 +917,7 @@ cudaError_t run_staged(egs_batch *B, cudaStream_t us, cudaError_t e, bool once =
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(B->d_params, B->h_params, sizeof(egs_matern_params) * B->nprob, cudaMemcpyHostToDevice, B->cs);
     if (e == cudaSuccess) e = cudaMemsetAsync(B->d_status, 0xFF, sizeof(DevStatus) * B->nprob, B->cs);
-    if (e == cudaSuccess && !B->exec && !once) {
+    if (e == cudaSuccess && !B->exec && !B->once) {
         cudaGraph_t g = nullptr;
         e = cudaStreamBeginCapture(B->cs, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
@@ -916,7 +928,7 @@ cudaError_t run_staged(egs_batch *B, cudaStream_t us, cudaError_t e, bool once =
         if (e == cudaSuccess) e = cudaGraphInstantiate(&B->exec, g, 0);
         if (g) cudaGraphDestroy(g);
     }
-    if (e == cudaSuccess) e = once ? enqueue_all(B, B->cs) : cudaGraphLaunch(B->exec, B->cs);
+    if (e == cudaSuccess) e = B->once ? enqueue_all(B, B->cs) : cudaGraphLaunch(B->exec, B->cs);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(B->h_status, B->d_status, sizeof(DevStatus) * B->nprob, cudaMemcpyDeviceToHost, B->cs);
     if (e == cudaSuccess) e = cudaEventRecord(B->ev_out, B->cs);
@@ -1059,13 +1071,13 @@ egs_status egs_batch_destroy(egs_batch *B)
     if (B->ev_out) cudaEventDestroy(B->ev_out);
     if (B->cs) cudaStreamDestroy(B->cs);
     if (B->ws) {
-        if (!B->alloc.alloc) cudaFree(B->ws);
+        if (!B->pooled) cudaFree(B->ws);
         else dev_free(B->alloc, B->ws, B->ws_bytes, nullptr);
     }
-    if (B->h_probs) cudaFreeHost(B->h_probs);
-    if (B->h_params) cudaFreeHost(B->h_params);
-    if (B->h_status) cudaFreeHost(B->h_status);
-    if (B->h_ctl) cudaFreeHost(B->h_ctl);
+    for (void *p : {(void *)B->h_probs, (void *)B->h_params, (void *)B->h_status, (void *)B->h_ctl}) {
+        if (B->once) std::free(p);
+        else if (p) cudaFreeHost(p);
+    }
     delete B;
     return EGS_OK;
 }
@@ -1074,7 +1086,7 @@ egs_status egs_loglik_batched(int32_t nprob, const int64_t *n, const double *con
                               const double *theta, egs_precision p, double *out, egs_status *per_status, void *stream)
 {
     egs_batch *B = nullptr;
-    egs_status st = egs_batch_create(nprob, n, 0, p, &B);
+    egs_status st = batch_create(nprob, n, 0, p, false, true, &B);
     if (st != EGS_OK) return st;
     st = egs_batch_run(B, locs, z, theta, out, per_status, stream);
     egs_batch_destroy(B);
@@ -1104,7 +1116,7 @@ egs_status egs_loglik_ind(const double *locs, const double *z, const double thet
     for (int64_t i = 0; i < nblk; ++i) ns[(size_t)i] = std::min(bs, n - i * bs);
     egs_batch *B = nullptr;
     // one block is the exact likelihood, and equals egs_loglik bit for bit
-    egs_status sc = batch_create((int32_t)nblk, ns.data(), tile, EGS_FP64, nblk > 1, &B);
+    egs_status sc = batch_create((int32_t)nblk, ns.data(), tile, EGS_FP64, nblk > 1, true, &B);
     if (sc != EGS_OK) return sc;
     for (int i = 0; i < B->nprob; ++i) B->h_params[i] = P;
     cudaStream_t us = (cudaStream_t)stream;
@@ -1131,7 +1143,7 @@ egs_status egs_loglik_ind(const double *locs, const double *z, const double thet
     B->ntab = 1;
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(B->d_probs, B->h_probs, sizeof(BatchProblem) * B->nprob, cudaMemcpyHostToDevice, B->cs);
-    e = run_staged(B, us, e, true);
+    e = run_staged(B, us, e);
     if (e != cudaSuccess) {
         egs_batch_destroy(B);
         return cuda_error(e, "egs_loglik_ind");

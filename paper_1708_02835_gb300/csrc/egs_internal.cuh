@@ -127,10 +127,10 @@ void store_trace(const KernelTimer &kt, cudaEvent_t origin);
     } while (0)
 
 // Device memory of the library's calls: the caller's hooks (egs_set_allocator)
-// or cudaMallocAsync / cudaFreeAsync.  An allocation is freed with the
+// or the library's own stream-ordered pool (api.cu).  An allocation is freed with the
 // Allocator value that made it.
 struct Allocator {
-    egs_alloc_fn alloc;  // NULL: cudaMallocAsync
+    egs_alloc_fn alloc;  // NULL: the pool
     egs_free_fn free;
     void *ctx;
 };
