@@ -54,6 +54,9 @@ struct Tiles {
     }
 };
 
+// FP64 tiles below a diagonal tile of a mixed layout.
+inline int band_tiles(const Tiles &tl) { return (tl.band < tl.T ? tl.band : tl.T) - 1; }
+
 // Geometry of a lower-tile matrix.
 struct TileGeom {
     int64_t n;
@@ -196,14 +199,13 @@ struct MixedBuffers {
     double *partials; // 2T
     int *err;
     float *l32;       // b x b: L_kk rounded to FP32 for the off-band TRSM of step k (TF32 / BF16 modes)
-    double *lt;       // b x b, the same region: L_kk^T of step k (FP32 mode, for the inversion)
     float *wsp;       // FP32 mode: W = L_kk^-1 in split-TF32 layout, b rows of [hi | lo] (2b); two such
                       // buffers of 2 b^2 floats, step k uses k % 2
     double *vinv;     // T b x b: V_k = L_kk^-T (upper triangular) for the solves
     void *oz[2];      // FP32 mode: BF16 slices of the panel rows (ozaki_slices_bytes), step k uses k % 2
     double *ozs[2];   // FP32 mode: their row scales, (T-1) b doubles each
     double *mtab;     // EGS_MT_SCRATCH_DOUBLES: the generator's local polynomials (general nu)
-    void *dpan;       // tc64_solo_bytes(b, T): scratch of the diagonal tiles' POTRFs
+    void *dpan;       // tc64_solo_bytes(b, T, band_tiles(tl)): scratch of the diagonal tiles' POTRFs and band solves
     float *rs[2];     // FP32 mode: the power-of-two scales of the split-FP16 panel rows, (T-1) b each
     int xband;        // FP32 mode: tiles with i - j < xband get FP64-accurate updates (>= tl.band)
 };

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) k_panel_from_f32_split(Tiles tl, int k, i
     const size_t pr = (size_t)(m0 - k - 1) * b + (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);  // panel row
     const int m = k + 1 + (int)(pr / b);
     const float *x = tl.t32(m, k) + (pr % b) * b;
-    const int e = slice_row_f32(x, b, oz + pr * b, (size_t)(tl.T - 1) * b * b, ozs + pr);
+    const int e = slice_row(x, b, oz + pr * b, (size_t)(tl.T - 1) * b * b, ozs + pr);
     panel_row_f16(x, b, e, reinterpret_cast<__half *>(panel), rs, pr);
 }
 
@@ -144,110 +144,6 @@ __global__ void __launch_bounds__(256) k_presplit_a(Tiles tl, int k, int m0, flo
     }
 }
 
-// W = L_kk^-1 column by column, in FP64: warp w of CTA c solves L w_j = e_j
-// for column j = c + gridDim.x w by column-oriented forward substitution:
-// with p = e_j, for i = j .. b-1: w_i = p_i / L_ii, then p_r -= L_ri w_i for
-// every r > i.  Lane l keeps p_r of the rows r = l + 32 t in registers, so a
-// step's critical chain is one shuffle (w_i from its owner lane), one
-// multiply and the owner's update of row i + 1; the other rows' updates
-// overlap it.  Column i of L_kk is read as row i of LT = L_kk^T, one
-// contiguous 256-byte load per 32 rows (reading L_kk itself by columns cost
-// 32 cache lines per load).  Each p_r receives its terms in the order of i, so results are
-// bitwise reproducible.  Outputs: V_k = W^T (row j of V_k is w_j, the
-// upper-triangular inverse the solves use) and W in the split-TF32 layout
-// of the tensor-core TRSM (row c: [hi | lo] of (float) W[c][.]).
-// NT = b / 32 rows per lane.  Shared memory: (1 + warps) b doubles.
-template <int NT>
-__global__ void __launch_bounds__(128) k_inv_cols(Tiles tl, int k, const double *__restrict__ LT,
-                                                  double *__restrict__ V, float *__restrict__ wsp, const DevStatus *st)
-{
-    if (mfailed(st)) return;
-    extern __shared__ double inv_sm[];
-    const int b = tl.b, lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
-    const double *L = tl.t64(k, k);
-    double *rinv = inv_sm, *xs = inv_sm + (size_t)(1 + wq) * b;
-    for (int i = threadIdx.x; i < b; i += blockDim.x) rinv[i] = 1.0 / L[(size_t)i * b + i];
-    for (int i = lane; i < b; i += 32) xs[i] = 0.0;
-    __syncthreads();
-    const int j = (int)blockIdx.x + (int)gridDim.x * wq;
-    double p[NT];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) p[t] = (lane + 32 * t == j) ? 1.0 : 0.0;
-    // rows i .. i + D - 1 of LT in registers: a row is loaded D steps before
-    // its use, which hides the L2 latency behind D steps of FMAs
-    constexpr int D = NT <= 16 ? 4 : (NT <= 24 ? 2 : 1);
-    double ring[D][NT];
-#pragma unroll
-    for (int d = 0; d < D; ++d)
-#pragma unroll
-        for (int t = 0; t < NT; ++t) ring[d][t] = (j + d < b) ? LT[(size_t)(j + d) * b + lane + 32 * t] : 0.0;
-#pragma unroll
-    for (int s = 0; s < NT; ++s) {
-        if (32 * s + 31 < j) continue;  // rows of this slot lie above j: w = 0 there
-        const int ii0 = j > 32 * s ? j - 32 * s : 0;
-        for (int ii = ii0; ii < 32; ++ii) {
-            const int i = 32 * s + ii;
-            double nx[NT];  // row i + D
-#pragma unroll
-            for (int t = s; t < NT; ++t) nx[t] = (i + D < b) ? LT[(size_t)(i + D) * b + lane + 32 * t] : 0.0;
-            const double wi = __shfl_sync(0xffffffffu, p[s], ii) * rinv[i];
-            if (lane == 0) xs[i] = wi;
-#pragma unroll
-            for (int t = s; t < NT; ++t)
-                if (lane + 32 * t > i) p[t] = fma(-ring[0][t], wi, p[t]);
-#pragma unroll
-            for (int t = s; t < NT; ++t) {
-#pragma unroll
-                for (int d = 0; d + 1 < D; ++d) ring[d][t] = ring[d + 1][t];
-                ring[D - 1][t] = nx[t];
-            }
-        }
-    }
-    __syncwarp();
-    double *Vj = V + (size_t)k * tl.bb() + (size_t)j * b;
-    const size_t ld2 = 2 * (size_t)b;
-    for (int c = lane; c < b; c += 32) {
-        const double x = xs[c];
-        Vj[c] = x;
-        const float v = (float)x, hi = to_tf32(v), lo = to_tf32(v - hi);
-        float *pw = wsp + (size_t)c * ld2 + j;
-        pw[0] = hi;
-        pw[b] = lo;
-    }
-}
-
-// LT = L_kk^T (32 x 32 blocks through shared memory), so that the inversion
-// reads a column of L_kk as one contiguous row.
-__global__ void __launch_bounds__(256) k_transpose_diag(Tiles tl, int k, double *__restrict__ LT, const DevStatus *st)
-{
-    __shared__ double blk[32][33];
-    if (mfailed(st)) return;
-    const int b = tl.b, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int r0 = 32 * (int)blockIdx.y, c0 = 32 * (int)blockIdx.x;
-    const double *L = tl.t64(k, k);
-    for (int r = ty; r < 32; r += 8) blk[r][tx] = L[(size_t)(r0 + r) * b + c0 + tx];
-    __syncthreads();
-    for (int r = ty; r < 32; r += 8) LT[(size_t)(c0 + r) * b + r0 + tx] = blk[tx][r];
-}
-
-cudaError_t launch_inv_cols(const Tiles &tl, int k, double *LT, double *V, float *wsp, const DevStatus *st,
-                            cudaStream_t s, KernelTimer *kt)
-{
-    const int b = tl.b;
-    EGS_LAUNCH(kt, KC_TRSM, s,
-               k_transpose_diag<<<dim3((unsigned)(b / 32), (unsigned)(b / 32)), 256, 0, s>>>(tl, k, LT, st));
-    const unsigned grid = (unsigned)(b / 4);
-    const size_t sm = (size_t)5 * b * sizeof(double);
-    switch (b / 32) {
-    case 8: EGS_LAUNCH(kt, KC_TRSM, s, k_inv_cols<8><<<grid, 128, sm, s>>>(tl, k, LT, V, wsp, st)); break;
-    case 16: EGS_LAUNCH(kt, KC_TRSM, s, k_inv_cols<16><<<grid, 128, sm, s>>>(tl, k, LT, V, wsp, st)); break;
-    case 24: EGS_LAUNCH(kt, KC_TRSM, s, k_inv_cols<24><<<grid, 128, sm, s>>>(tl, k, LT, V, wsp, st)); break;
-    case 32: EGS_LAUNCH(kt, KC_TRSM, s, k_inv_cols<32><<<grid, 128, sm, s>>>(tl, k, LT, V, wsp, st)); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
 // FP64 band panel tiles (m = k+1..k+nrows) -> operand format.
 template <int FMT>
 __global__ void __launch_bounds__(256) k_panel_from_f64(Tiles tl, int k, int nrows, void *panel, const DevStatus *st)
@@ -262,92 +158,6 @@ __global__ void __launch_bounds__(256) k_panel_from_f64(Tiles tl, int k, int nro
         panel_store<FMT>(panel, tl, (size_t)(m - k - 1) * tl.b + off / tl.b, (int)(off % tl.b),
                          (float)tl.t64(m, k)[off]);
     }
-}
-
-// FP64 TRSM of the band rows of step k (tiles (k+1 .. k+nb, k)): X L_kk^T = A,
-// solved in place.  A CTA keeps kTbR rows of one tile in shared memory and
-// sweeps the 32-column blocks of L_kk: block j first subtracts the solved
-// columns, X[:, 0:32j] L[32j:32j+32, 0:32j]^T, one 32 x 32 chunk of L at a
-// time (staged transposed in shared memory while the next chunk is loaded
-// into registers; two warps per row, each over half of a chunk), then one
-// warp per row solves the 32 x 32 diagonal block by column-oriented
-// substitution (a shuffle, a multiplication by 1 / L_ii and an FMA per
-// column).  b / kTbR CTAs per tile spread the b^3 / 2 FMA of a tile over the
-// GPU; the chain of the FP64 band is latency-bound, and this solve sits on it
-// once per step.
-constexpr int kTbR = 4;
-static_assert(kTbR * 64 == 256, "two warps per row of the CTA");
-__global__ void __launch_bounds__(256) k_trsm_band_f64(Tiles tl, int k, const DevStatus *st)
-{
-    extern __shared__ double tb_xs[];  // kTbR x b: the CTA's rows
-    __shared__ double LcT[2][32][33];  // chunk (j, i) transposed: LcT[cc][cr] = L[32j + cr][32i + cc]
-    __shared__ double part[2][kTbR][32];
-    __shared__ double rdg[1024];  // 1 / L_ii
-    if (mfailed(st)) return;
-    const int b = tl.b, nblk = b >> 5, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int r = tid >> 6, h = (tid >> 5) & 1;  // row of the CTA, half of a chunk
-    double *X = tl.t64(k + 1 + (int)blockIdx.y, k) + (size_t)blockIdx.x * kTbR * b;
-    const double *L = tl.t64(k, k);
-    for (int e = tid; e < kTbR * b; e += 256) tb_xs[e] = X[e];
-    for (int e = tid; e < b; e += 256) rdg[e] = 1.0 / L[(size_t)e * b + e];
-    double reg[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) reg[q] = L[(size_t)((tid >> 5) + 8 * q) * b + lane];  // chunk (0, 0)
-    double acc = 0.0;
-    int j = 0, i = 0, buf = 0;
-    for (;;) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) LcT[buf][lane][(tid >> 5) + 8 * q] = reg[q];
-        int jn = j, in = i + 1;
-        if (in > jn) {
-            ++jn;
-            in = 0;
-        }
-        if (jn < nblk) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) reg[q] = L[(size_t)(32 * jn + (tid >> 5) + 8 * q) * b + 32 * in + lane];
-        }
-        __syncthreads();
-        if (i < j) {
-            const double *xr = tb_xs + (size_t)r * b + 32 * i + 16 * h;
-#pragma unroll
-            for (int l = 0; l < 16; ++l) acc = fma(xr[l], LcT[buf][16 * h + l][lane], acc);
-        } else {
-            part[h][r][lane] = acc;
-            acc = 0.0;
-            __syncthreads();
-            if (warp < kTbR) {
-                double *xj = tb_xs + (size_t)warp * b + 32 * j;
-                double v = xj[lane] - (part[0][warp][lane] + part[1][warp][lane]);
-                for (int l = 0; l < 32; ++l) {
-                    // every lane forms x_l (a warp-wide FP64 instruction costs
-                    // the same with one lane active or all 32)
-                    const double x = __shfl_sync(0xffffffffu, v, l) * rdg[32 * j + l];
-                    const double u = fma(-x, LcT[buf][l][lane], v);
-                    v = lane > l ? u : (lane == l ? x : v);
-                }
-                xj[lane] = v;
-            }
-        }
-        j = jn;
-        i = in;
-        buf ^= 1;
-        if (j >= nblk) break;
-    }
-    __syncthreads();
-    for (int e = tid; e < kTbR * b; e += 256) X[e] = tb_xs[e];
-}
-
-cudaError_t launch_trsm_band_f64(const Tiles &tl, int k, int nb, const DevStatus *st, cudaStream_t s, KernelTimer *kt)
-{
-    if (nb <= 0) return cudaSuccess;
-    cudaError_t e =
-        cudaFuncSetAttribute(k_trsm_band_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, kTbR * 1024 * (int)sizeof(double));
-    if (e != cudaSuccess) return e;
-    EGS_LAUNCH(kt, KC_TRSM, s,
-               k_trsm_band_f64<<<dim3((unsigned)(tl.b / kTbR), (unsigned)nb), 256, (size_t)kTbR * tl.b * sizeof(double),
-                                 s>>>(tl, k, st));
-    return cudaGetLastError();
 }
 
 // L_kk rounded to FP32 once per step for the FP32 TRSM of the TF32 / BF16
@@ -447,7 +257,7 @@ __global__ void __launch_bounds__(256, 3) k_trsm_panel_f32(Tiles tl, int k, int 
         // (re-read from L1/L2; one warp per row)
         const size_t R = (size_t)(tl.T - 1) * b;
         for (int rr = tid >> 5; rr < 64; rr += 8)
-            slice_row_f32(A + (size_t)rr * b, b, oz + (prow0 + rr) * b, R * b, ozs + prow0 + rr);
+            slice_row(A + (size_t)rr * b, b, oz + (prow0 + rr) * b, R * b, ozs + prow0 + rr);
     }
 }
 
@@ -466,21 +276,10 @@ __global__ void __launch_bounds__(256) k_gemv_T(Tiles tl, int k, const double *x
     gemv_T_cols(tl, k, (int)blockIdx.x, (int)blockIdx.y * 64, xsrc + (size_t)k * tl.b, v + (size_t)blockIdx.x * tl.b);
 }
 
-// V_k = L_kk^-T for every diagonal tile k = blockIdx.x: 16 rows of V_k per
-// CTA, each the solution of x L_kk^T = e_r (trsm_rows on identity rows; the
-// columns before the row's 32-column block are zero and skipped).  V_k is
-// upper triangular, so y = L_kk^-1 r = V_k^T r and x = L_kk^-T r = V_k r
-// become matrix-vector products spread over many SMs instead of a serial
+// V_k = L_kk^-T for every diagonal tile k (from the factorisation) is upper
+// triangular, so y = L_kk^-1 r = V_k^T r and x = L_kk^-T r = V_k r are
+// matrix-vector products spread over many SMs instead of a serial
 // substitution on one.
-__global__ void __launch_bounds__(256) k_inv_diag(Tiles tl, double *__restrict__ V, const DevStatus *st)
-{
-    if (mfailed(st)) return;
-    const int b = tl.b, k = (int)blockIdx.x, r0 = (int)blockIdx.y * 16;
-    double *X = V + (size_t)k * tl.bb() + (size_t)r0 * b;
-    for (int e = threadIdx.x; e < 16 * b; e += 256) X[e] = (e / b + r0 == e % b) ? 1.0 : 0.0;
-    __syncthreads();
-    trsm_rows<16>(tl.t64(k, k), b, X, b, b, (r0 / 32) * 32);
-}
 
 // partials[k] = sum_i log L_kk[i][i] (fixed-order tree).
 __global__ void __launch_bounds__(256) k_logdet_tiles(Tiles tl, double *__restrict__ partials, const DevStatus *st)
@@ -659,12 +458,14 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_panel, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_col, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_diag, cudaEventDisableTiming);
-    // POTRF of a diagonal tile: the FP64 path's 64-column blocks, on that tile alone (tile 512:
-    // 1.05 ms with a task graph of 32 x 32 blocks, 0.4 ms so)
-    const F64Set diag{nullptr, tc64_problem(mb.dpan, tl, st, nullptr, true), 1, b, T, 1};
+    // POTRF of a diagonal tile and its inverse V_k = L_kk^-T: the FP64 path's 64-column blocks on
+    // that tile alone with V_k's rows below it; the band rows by multiplication with W = V_k^T on
+    // the tensor cores (tc64.cu).  Tile 512: 1.05 ms of POTRF, 0.32 of inversion and 0.22 of band
+    // solve as task graph, column and row substitutions; 0.85 and 0.05 ms so
+    const F64Set diag{nullptr, tc64_solo_problem(mb.dpan, tl, st, mb.vinv, band_tiles(tl)), 1, b, T, 1};
     F64Maps dmaps;
-    if (e == cudaSuccess) e = make_f64_maps(diag.one.panel, diag.one.inner, b, &dmaps);
-    if (e == cudaSuccess) e = cudaMemsetAsync(diag.one.ctr, 0, tc64_counters(b, T) * sizeof(unsigned long long), s);
+    if (e == cudaSuccess) e = make_f64_solo_maps(diag.one, &dmaps);
+    if (e == cudaSuccess) e = launch_solo_init(diag, s, kt);
     if (e == cudaSuccess) e = cudaEventRecord(ev_col, s);  // the side stream starts after prior work on s
     KernelTimer *kts = kt;  // side-stream kernels are timed with events on the side stream
     for (int k = 0; k < T && e == cudaSuccess; ++k) {
@@ -683,10 +484,10 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
         if (k == 0) e = cudaStreamWaitEvent(side, ev_col, 0);
         if (e == cudaSuccess)
             e = launch_panel64(dmaps, diag, k, side, kts);
-        // FP32 mode: W = L_kk^-1 (and V_k = W^T for the solves) for the main
-        // stream's off-band TRSM, off the main stream
+        // the rows of W for the band solve and (FP32 mode, split TF32) for the main stream's
+        // off-band TRSM
         float *wsp = mb.wsp + (size_t)(k & 1) * 2 * tl.bb();
-        if (e == cudaSuccess && FMT == 3) e = launch_inv_cols(tl, k, mb.lt, mb.vinv, wsp, st, side, kts);
+        if (e == cudaSuccess && k + 1 < T) e = launch_winv(diag, k, FMT == 3 ? wsp : nullptr, side, kts);
         if (e == cudaSuccess) e = cudaEventRecord(ev_diag, side);
         if (e == cudaSuccess && k > 0) e = cudaStreamWaitEvent(side, ev_col, 0);
         if (e == cudaSuccess && k + 1 < T) {
@@ -694,7 +495,7 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
                 EGS_LAUNCH(kts, KC_TRSM, side,
                            k_l32_from_f64<<<(unsigned)((tl.bb() + 255) / 256 < 1024 ? (tl.bb() + 255) / 256 : 1024), 256,
                                             0, side>>>(tl, k, mb.l32, st));
-            e = launch_trsm_band_f64(tl, k, nb, st, side, kts);
+            e = launch_band_solve(dmaps, diag, k, nb, side, kts);
             if (e == cudaSuccess && nb > 0) {
                 if (FMT == 3) {
                     EGS_LAUNCH(kts, KC_TRSM, side,
@@ -835,11 +636,7 @@ cudaError_t run_loglik_mixed(const double *X, const double *Y, const double *z, 
     else e = factor_mixed<1>(mb, ma, mbm, ma3, mc, moz, nullptr, st, s, kt);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[2], s);
-    // V_k = L_kk^-T for every diagonal tile (FP32 mode: computed during the
-    // factorisation) and the log-det partials, then res = L^-1 z (kept for
-    // y.y), x = L^-T res
-    if (fmt != 3)
-        EGS_LAUNCH(kt, KC_TRSV, s, k_inv_diag<<<dim3((unsigned)T, (unsigned)(b / 16)), 256, 0, s>>>(tl, mb.vinv, st));
+    // the log-det partials, then res = L^-1 z (kept for y.y), x = L^-T res
     EGS_LAUNCH(kt, KC_TRSV, s, k_logdet_tiles<<<(unsigned)T, 256, 0, s>>>(tl, mb.partials, st));
     e = launch_pad_vector(z, n, mb.zp, npad, s, kt);
     if (e != cudaSuccess) return e;

@@ -97,7 +97,7 @@ __device__ __forceinline__ void slice7_row(const double *__restrict__ src, int b
     const int lane = threadIdx.x & 31;
     unsigned mh = 0;
     for (int c = 2 * lane; c < b; c += 64) {
-        const double2 v = *reinterpret_cast<const double2 *>(src + c);
+        const double2 v = make_double2(src[c], src[c + 1]);
         const unsigned h0 = (unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, h1 = (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu;
         mh = max(mh, max(h0, h1));
     }
@@ -107,7 +107,7 @@ __device__ __forceinline__ void slice7_row(const double *__restrict__ src, int b
     const int e = mh == 0 ? 0 : max(emax, 1) - 1022;
     if (lane == 0) *ep = bad ? kBadRow : e;
     for (int c = 2 * lane; c < b; c += 64) {
-        const double2 v = *reinterpret_cast<const double2 *>(src + c);
+        const double2 v = make_double2(src[c], src[c + 1]);
         uint32_t d0[kF64Slices], d1[kF64Slices];
         digits7(bad || mh == 0 ? 0ll : fixed57(v.x, e), d0);
         digits7(bad || mh == 0 ? 0ll : fixed57(v.y, e), d1);
@@ -186,11 +186,12 @@ __global__ void __launch_bounds__(8 * RB) k_solve64(const __grid_constant__ F64S
     __shared__ Solve64Smem<RB> sm;
     const F64Prob &P = set.get(blockIdx.y);
     const Tiles &tl = P.tl;
-    const int T = set.solo ? k + 1 : tl.T;
-    if ((int64_t)(j + 1) * PW + (int64_t)blockIdx.x * RB >= (int64_t)(T - k) * tl.b || failed(P.st)) return;
     const int b = tl.b, tid = threadIdx.x, lane = tid & 31;
-    const int pr0 = (j + 1) * PW + (int)blockIdx.x * RB;
-    double *X = tl.t64(k + pr0 / b, k) + (size_t)(pr0 % b) * b + j * PW;
+    const int64_t below = (int64_t)((set.solo ? k + 1 : tl.T) - k) * b - (j + 1) * PW, i0 = (int64_t)blockIdx.x * RB;
+    if (i0 >= below + (P.vinv ? (j + 1) * PW : 0) || failed(P.st)) return;
+    // the rows below, then V's rows 0 .. 64 (j + 1) - 1 (the later ones are zero in these columns)
+    const int pr0 = i0 < below ? (j + 1) * PW + (int)i0 : b + (int)(i0 - below);
+    double *X = (i0 < below ? tl.t64(k + pr0 / b, k) : P.vinv + (size_t)k * tl.bb()) + (size_t)(pr0 % b) * b + j * PW;
 #pragma unroll
     for (int e = tid; e < RB * PW; e += NT) sm.Xs[e >> 6][e & 63] = X[(size_t)(e >> 6) * b + (e & 63)];
     solve64_stage(sm, tl.t64(k, k) + (size_t)j * PW * (b + 1), b, P.winv);
@@ -215,74 +216,127 @@ __global__ void __launch_bounds__(8 * RB) k_solve64(const __grid_constant__ F64S
     }
 }
 
+// V_k = identity for every tile; grid = (T, b / 64).
+__global__ void __launch_bounds__(256) k_identity_tiles(double *__restrict__ V, int b)
+{
+    double *t = V + (size_t)blockIdx.x * b * b;
+    for (int r = (int)blockIdx.y * 64; r < (int)blockIdx.y * 64 + 64; ++r)
+        for (int c = threadIdx.x; c < b; c += 256) t[(size_t)r * b + c] = r == c ? 1.0 : 0.0;
+}
+
+__device__ __forceinline__ float tf32_rna(float x)
+{
+    uint32_t r;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+    return __uint_as_float(r);
+}
+
+// Rows c0 .. c0 + 7 of W = V_k^T through shared memory (8 columns of V_k, 64-byte segments), one
+// warp each: the slices, and the split-TF32 layout if wsp is given.  Shared: 8 (b + 1) doubles.
+__global__ void __launch_bounds__(256) k_winv_rows(const __grid_constant__ F64Set set, int k, float *__restrict__ wsp)
+{
+    extern __shared__ double wrow[];
+    const F64Prob &P = set.one;
+    if (failed(P.st)) return;
+    const int b = P.tl.b, c0 = (int)blockIdx.x * 8, ld = b + 1;
+    const double *V = P.vinv + (size_t)k * P.tl.bb();
+    for (int e = threadIdx.x; e < 8 * b; e += 256) wrow[(e & 7) * ld + (e >> 3)] = V[(size_t)(e >> 3) * b + c0 + (e & 7)];
+    __syncthreads();
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, c = c0 + w;
+    const double *row = wrow + w * ld;
+    slice7_row(row, b, P.w.sl + (size_t)c * b, (size_t)b * b, P.w.ex + c);
+    if (!wsp) return;
+    float *out = wsp + (size_t)c * 2 * b;
+    for (int i = lane; i < b; i += 32) {
+        const float v = (float)row[i], hi = tf32_rna(v);
+        out[i] = hi;
+        out[b + i] = tf32_rna(v - hi);
+    }
+}
+
 // ---- the update -------------------------------------------------------------
 
 struct F64Item {
     int m, n, rb, cb;  // output tile, 128-row block, 64-column block; m < 0 ends
 };
 
-// Trailing update (inner = false): output tiles (m, n), n = col0 .. col1 - 1, m = n .. T - 1,
-// visited by blocks of kF64Cols columns (the block's triangle, then every lower row), so that
-// the CTAs working side by side share the block's B operands in L2.  Operand row r of tile m
-// is slice row (m - k - 1) b + r, K = b.
-// Inside a panel (inner = true): the 64-column blocks col0 .. col1 - 1 of tile column k, all
-// rows from each block's diagonal down; slice row (m - k) b + r, K = 64.
+// F64_TRAIL: output tiles (m, n), n = col0 .. col1 - 1, m = n .. T - 1, visited by blocks of
+// kF64Cols columns (the block's triangle, then every lower row), so that the CTAs working side
+// by side share the block's B operands in L2.  Operand row r of tile m is slice row
+// (m - k - 1) b + r, K = b.
+// F64_INNER, inside a panel: the 64-column blocks col0 .. col1 - 1 of tile column k, all rows
+// from each block's diagonal down; slice row (m - k) b + r, K = 64.  Tile k + 1 of a diagonal
+// tile alone is V_k, its rows below 64 col0 as far as they are nonzero.
+// F64_BAND: the tiles k + 1 .. col1 - 1 of column k times W^T (B operand: the rows of W; lower
+// triangular, so column block c needs K = 64 (c + 1) only), stored in their place.
+enum F64Mode { F64_TRAIL = 0, F64_INNER, F64_BAND };
 constexpr int kF64Cols = 8;
 struct F64Work {
     const Tiles &tl;
-    int T, k, col0, col1;
-    bool inner;
+    int T, k, col0, col1, mode;
     __host__ __device__ int row_blocks() const { return (tl.b + FM - 1) / FM; }
-    __host__ __device__ int kchunks() const { return inner ? 1 : tl.b / FKC; }
+    __device__ int kchunks(int cb) const { return mode == F64_INNER ? 1 : (mode == F64_BAND ? cb + 1 : tl.b / FKC); }
     __host__ __device__ int64_t items() const
     {
         const int64_t c = col1 - col0;
-        if (inner) return c * row_blocks() * (T - k);
+        if (mode == F64_INNER) return c * row_blocks() * (T - k);
+        if (mode == F64_BAND) return c * row_blocks() * (tl.b / FN);
         const int64_t h = T - col0;
         return (c * h - c * (c - 1) / 2) * row_blocks() * (tl.b / FN);
     }
-    __device__ size_t slice_row(int m) const { return (size_t)(m - k - (inner ? 0 : 1)) * tl.b; }
+    __device__ size_t slice_row(int m) const { return (size_t)(m - k - (mode == F64_INNER ? 0 : 1)) * tl.b; }
     __device__ bool decode(int64_t item, F64Item &w) const
     {
-        if (inner) {
+        if (mode == F64_INNER) {
             const int wd = col1 - col0, rbs = row_blocks();
             const int64_t u = item / wd;
             w.m = k + (int)(u / rbs);
             w.n = k;
             w.rb = (int)(u % rbs);
             w.cb = col0 + (int)(item % wd);
-        } else {
-            const int ncb = tl.b / FN, per = row_blocks() * ncb;
-            int64_t t = item / per;
-            const int blk = (int)(item % per);
-            int c_lo = col0;
-            for (;;) {
-                const int wd = min(kF64Cols, col1 - c_lo);
-                const int64_t tri = (int64_t)wd * (wd + 1) / 2;
-                const int64_t cnt = tri + (int64_t)(T - c_lo - wd) * wd;
-                if (t < cnt) {
-                    if (t < tri) {
-                        int ii = 0, u = (int)t;
-                        while (u > ii) {
-                            u -= ii + 1;
-                            ++ii;
-                        }
-                        w.m = c_lo + ii;
-                        w.n = c_lo + u;
-                    } else {
-                        const int64_t u = t - tri;
-                        w.m = c_lo + wd + (int)(u / wd);
-                        w.n = c_lo + (int)(u % wd);
-                    }
-                    break;
-                }
-                t -= cnt;
-                c_lo += wd;
-            }
-            w.rb = blk / ncb;
-            w.cb = blk % ncb;
+            return true;
         }
-        return !(w.m == w.n && w.cb * FN > w.rb * FM + FM - 1);  // strictly above the diagonal
+        const int ncb = tl.b / FN, per = row_blocks() * ncb;
+        int64_t t = item / per;
+        const int blk = (int)(item % per);
+        w.rb = blk / ncb;
+        w.cb = blk % ncb;
+        if (mode == F64_BAND) {
+            w.m = col0 + (int)t;
+            w.n = k;
+            return true;
+        }
+        int c_lo = col0;
+        for (;;) {
+            const int wd = min(kF64Cols, col1 - c_lo);
+            const int64_t tri = (int64_t)wd * (wd + 1) / 2;
+            const int64_t cnt = tri + (int64_t)(T - c_lo - wd) * wd;
+            if (t < cnt) {
+                if (t < tri) {
+                    int ii = 0, u = (int)t;
+                    while (u > ii) {
+                        u -= ii + 1;
+                        ++ii;
+                    }
+                    w.m = c_lo + ii;
+                    w.n = c_lo + u;
+                } else {
+                    const int64_t u = t - tri;
+                    w.m = c_lo + wd + (int)(u / wd);
+                    w.n = c_lo + (int)(u % wd);
+                }
+                return true;
+            }
+            t -= cnt;
+            c_lo += wd;
+        }
+    }
+    // Rows of the item's block that are outputs: r0 <= row < r1 of tile m.  On the diagonal tile
+    // from the column block's diagonal down (the factored blocks hold zeros above it).
+    __device__ int r0(const F64Item &w) const { return w.m == w.n ? w.cb * FN : 0; }
+    __device__ int r1(const F64Item &w, bool solo) const
+    {
+        return mode == F64_INNER && solo && w.m == k + 1 ? col0 * FN : tl.b;
     }
 };
 
@@ -354,21 +408,22 @@ __device__ __forceinline__ void tma_load_3d(const CUtensorMap *map, uint64_t *ba
 
 __global__ void __launch_bounds__(FTHREADS, 1)
 k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-         const __grid_constant__ F64Set set, int k, int c0, int c1, int inner, int slot)
+         const __grid_constant__ F64Set set, int k, int c0, int c1, int mode, int slot)
 {
     const F64Prob &P = set.get(blockIdx.y);
-    const int T = set.solo ? k + 1 : P.tl.T;
-    if (T <= k) return;
-    // trailing: columns k + c0 .. min(k + c1, T) - 1; inner: the blocks c0 .. c1 - 1 of column k
-    const F64Work work{P.tl, T, k, inner ? c0 : k + c0, inner ? c1 : min(k + c1, T), inner != 0};
+    const bool solo = set.solo != 0;
+    if (P.tl.T <= k) return;
+    const int T = solo && mode == F64_INNER ? k + 1 + (P.vinv ? 1 : 0) : P.tl.T;
+    // columns k + c0 .. min(k + c1, T) - 1; inside a panel the blocks c0 .. c1 - 1 of column k
+    const F64Work work{P.tl, T, k, mode == F64_INNER ? c0 : k + c0, mode == F64_INNER ? c1 : min(k + c1, T), mode};
     if (work.col0 >= work.col1) return;
     const int64_t nitems = work.items();
     if ((int64_t)blockIdx.x >= nitems) return;
     unsigned long long *next = P.ctr + slot;
     DevStatus *st = P.st;
-    const F64Rows &rows = inner ? P.inner : P.panel;
-    const int *__restrict__ ex = rows.ex + rows.row0;
-    const int yrow0 = (int)rows.row0;
+    const F64Rows &rows = mode == F64_INNER ? P.inner : P.panel, &brows = mode == F64_BAND ? P.w : rows;
+    const int *__restrict__ ex = rows.ex + rows.row0, *__restrict__ exb = brows.ex + brows.row0;
+    const int yrow0 = (int)rows.row0, ybrow0 = (int)brows.row0;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     __shared__ uint64_t afull[kF64Slices], aempty[kF64Slices], bfull[2], bempty[2], tfull, tempty;
@@ -405,7 +460,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tbase = tmem_base;
-    const int b = work.tl.b, kchunks = work.kchunks();
+    const int b = work.tl.b;
     uint8_t *sa = smem, *sb = smem + kF64Slices * FA_SL;
 
     if (warp == 0) {
@@ -416,7 +471,8 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             int64_t claimed = (int64_t)atomicAdd(next, 1ull);
             while (!abort_flag) {
                 F64Item wi;
-                const bool valid = claimed < nitems && work.decode(claimed, wi);
+                const bool valid = claimed < nitems && work.decode(claimed, wi) && wi.rb * FM + FM > work.r0(wi) &&
+                                   wi.rb * FM < work.r1(wi, solo);
                 if (claimed < nitems && !valid) {
                     claimed = (int64_t)atomicAdd(next, 1ull);
                     continue;
@@ -430,7 +486,8 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                 if (!valid) break;
                 claimed = (int64_t)atomicAdd(next, 1ull);  // overlaps the loads below
                 const int ya = yrow0 + (int)work.slice_row(wi.m) + wi.rb * FM;
-                const int yb = yrow0 + (int)work.slice_row(wi.n) + wi.cb * FN;
+                const int yb = ybrow0 + (mode == F64_BAND ? 0 : (int)work.slice_row(wi.n)) + wi.cb * FN;
+                const int kchunks = work.kchunks(wi.cb);
                 for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
                     const int bb = g & 1;
                     if (!tc::mbar_wait(&bempty[bb], ((uint32_t)(g >> 1) & 1u) ^ 1u, &abort_flag)) break;
@@ -455,7 +512,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             while (!abort_flag) {
                 const int slot = r % FRING;
                 if (!tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag)) break;
-                const int m = ring[slot].m;
+                const int m = ring[slot].m, kchunks = work.kchunks(ring[slot].cb);
                 tc::mbar_arrive(&rempty[slot]);
                 ++r;
                 if (m < 0) break;
@@ -502,8 +559,6 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
         // warp w: TMEM lanes 32 (w % 4) .. + 31 (rows of the block), columns 32 half .. + 31
         const int q = warp & 3, half = (warp - 2) >> 2;
         const uint32_t t0 = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32);
-        const int nflush = (kchunks + FLUSH - 1) / FLUSH;
-        const int up = nflush > 2 ? 1 : 0;  // the sum over the flushes stays below 2^63
         uint32_t f = 0;
         int r = 0;
         bool run = true;
@@ -516,6 +571,8 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             if (lane == 0) tc::mbar_arrive(&rempty[slot]);
             ++r;
             if (wi.m < 0) break;
+            const int nflush = (work.kchunks(wi.cb) + FLUSH - 1) / FLUSH;
+            const int up = nflush > 2 ? 1 : 0;  // the sum over the flushes stays below 2^63
             long long acc[32];
             for (int fl = 0; fl < nflush; ++fl, ++f) {
                 const bool ok = tc::mbar_wait(&tfull, f & 1u, &abort_flag);
@@ -543,23 +600,24 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             }
             if (!run) break;
             const int row = wi.rb * FM + q * 32 + lane;
-            // rows of a diagonal tile above its column block are left alone: the factored blocks
-            // of the panel hold zeros there
-            if (row < b && !(wi.m == wi.n && row < wi.cb * FN)) {
+            if (row >= work.r0(wi) && row < work.r1(wi, solo)) {
                 const int col = wi.cb * FN + half * 32;
                 const int ea = ex[work.slice_row(wi.m) + row] - 16;
-                const int *eb = ex + work.slice_row(wi.n) + col;
-                double *C = work.tl.t64(wi.m, wi.n) + (size_t)row * b + col;
+                const int *eb = exb + (mode == F64_BAND ? 0 : work.slice_row(wi.n)) + col;
+                double *C = (solo && mode == F64_INNER && wi.m > k ? P.vinv + (size_t)k * work.tl.bb()
+                                                                   : work.tl.t64(wi.m, wi.n)) + (size_t)row * b + col;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     double2 cv[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) cv[j] = *reinterpret_cast<const double2 *>(C + 16 * h + 2 * j);
+                    for (int j = 0; j < 8; ++j)
+                        cv[j] = mode == F64_BAND ? make_double2(0.0, 0.0)
+                                                 : *reinterpret_cast<const double2 *>(C + 16 * h + 2 * j);
                     double *cd = reinterpret_cast<double *>(cv);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const int s = ea + __ldg(eb + 16 * h + j);
-                        const double d = fixed_to_f64(acc[16 * h + j], up);
+                        const double d = fixed_to_f64(mode == F64_BAND ? -acc[16 * h + j] : acc[16 * h + j], up);
                         if (s >= -960 && s <= 1000) {
                             cd[j] = fma(-pow2(s), d, cd[j]);
                         } else if (s > 1000) {
@@ -646,12 +704,6 @@ static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Slices and exponents of the panel (K = b) and of its 64-column blocks (K = 64, the
 // diagonal tile's rows too), the work counters, the 8 x 8 inverses.
-size_t tc64_solo_bytes(int b, int T)
-{
-    return a256((size_t)b * PW * kF64Slices * sizeof(uint16_t)) + a256((size_t)b * sizeof(int)) +
-           a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(kWinvDoubles * sizeof(double));
-}
-
 size_t tc64_scratch_bytes(int b, int T)
 {
     const size_t R = (size_t)(T - 1) * (size_t)b, R1 = R + b;
@@ -660,16 +712,16 @@ size_t tc64_scratch_bytes(int b, int T)
            a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(kWinvDoubles * sizeof(double));
 }
 
-F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st, double *z, bool solo)
+F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st, double *z)
 {
-    const size_t R = solo ? 0 : (size_t)(tl.T - 1) * (size_t)tl.b, R1 = R + tl.b;
+    const size_t R = (size_t)(tl.T - 1) * (size_t)tl.b, R1 = R + tl.b;
     char *p = (char *)scratch;
     auto take = [&p](size_t bytes) {
         char *q = p;
         p += a256(bytes);
         return q;
     };
-    F64Prob P;
+    F64Prob P{};
     P.tl = tl;
     P.st = st;
     P.z = z;
@@ -696,6 +748,55 @@ cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64
     return e;
 }
 
+size_t tc64_solo_bytes(int b, int T, int nb)
+{
+    const size_t bb = (size_t)b * b;
+    return a256((size_t)nb * bb * kF64Slices * sizeof(uint16_t)) + a256((size_t)nb * b * sizeof(int)) +
+           a256((size_t)2 * b * PW * kF64Slices * sizeof(uint16_t)) + a256((size_t)2 * b * sizeof(int)) +
+           a256(bb * kF64Slices * sizeof(uint16_t)) + a256((size_t)b * sizeof(int)) +
+           a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(kWinvDoubles * sizeof(double));
+}
+
+F64Prob tc64_solo_problem(void *scratch, const Tiles &tl, DevStatus *st, double *vinv, int nb)
+{
+    const size_t b = (size_t)tl.b;
+    char *p = (char *)scratch;
+    auto take = [&p](size_t bytes) {
+        char *q = p;
+        p += a256(bytes);
+        return q;
+    };
+    auto rows = [&](size_t n, size_t K) {
+        F64Rows r{};
+        r.sl = (uint16_t *)take(n * K * kF64Slices * sizeof(uint16_t));
+        r.ex = (int *)take(n * sizeof(int));
+        r.rows = n;
+        return r;
+    };
+    F64Prob P{};
+    P.tl = tl;
+    P.st = st;
+    P.vinv = vinv;
+    P.panel = rows((size_t)nb * b, b);
+    P.inner = rows(2 * b, PW);
+    P.w = rows(b, b);
+    P.ctr = (unsigned long long *)take(tc64_counters(tl.b, tl.T) * sizeof(unsigned long long));
+    P.winv = (double *)take(kWinvDoubles * sizeof(double));
+    return P;
+}
+
+cudaError_t make_f64_solo_maps(const F64Prob &P, F64Maps *maps)
+{
+    const uint64_t b = (uint64_t)P.tl.b;
+    cudaError_t e = cudaSuccess;
+    maps->a = CUtensorMap{};
+    if (P.panel.rows) e = make_map3(&maps->a, P.panel.sl, P.panel.rows, b, FM, 1);
+    if (e == cudaSuccess) e = make_map3(&maps->b, P.w.sl, P.w.rows, b, FN, kF64Slices);
+    if (e == cudaSuccess) e = make_map3(&maps->ia, P.inner.sl, P.inner.rows, PW, FM, 1);
+    if (e == cudaSuccess) e = make_map3(&maps->ib, P.inner.sl, P.inner.rows, PW, FN, kF64Slices);
+    return e;
+}
+
 // CTAs of a problem's update launch: the whole GPU for one problem, a share for each of many.
 static unsigned tc64_ctas(const F64Set &set, int64_t items, int reserve)
 {
@@ -706,23 +807,27 @@ static unsigned tc64_ctas(const F64Set &set, int64_t items, int reserve)
 }
 
 static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, const F64Set &set, int k, int c0, int c1,
-                                 int inner, int slot, int reserve, cudaStream_t s, KernelTimer *kt)
+                                 int mode, int slot, int reserve, cudaStream_t s, KernelTimer *kt)
 {
     cudaError_t e = cudaFuncSetAttribute(k_tc_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
     if (e != cudaSuccess) return e;
-    const int T = set.solo ? k + 1 : set.Tmax;
+    // of the largest problem, as in the kernel
+    const int T = set.solo && mode == F64_INNER ? k + 1 + (set.one.vinv ? 1 : 0) : set.Tmax;
     const Tiles tl{nullptr, nullptr, set.b, T, T};
-    const F64Work w{tl, T, k, inner ? c0 : k + c0, inner ? c1 : (k + c1 < T ? k + c1 : T), inner != 0};
+    const bool in = mode == F64_INNER;
+    const F64Work w{tl, T, k, in ? c0 : k + c0, in ? c1 : (k + c1 < T ? k + c1 : T), mode};
     if (w.col0 >= w.col1) return cudaSuccess;
     const dim3 grid(tc64_ctas(set, w.items(), reserve), (unsigned)set.count);
-    EGS_LAUNCH(kt, KC_UPDATE, s, k_tc_f64<<<grid, FTHREADS, FSMEM, s>>>(a, b, set, k, c0, c1, inner, slot));
+    EGS_LAUNCH(kt, mode == F64_BAND ? KC_TRSM : KC_UPDATE, s,
+               k_tc_f64<<<grid, FTHREADS, FSMEM, s>>>(a, b, set, k, c0, c1, mode, slot));
     return cudaGetLastError();
 }
 
 cudaError_t launch_diag_solve64(const F64Set &set, int k, int j, cudaStream_t s, KernelTimer *kt)
 {
     EGS_LAUNCH(kt, KC_POTRF, s, k_diag64<<<dim3(1, (unsigned)set.count), 256, 0, s>>>(set, k, j));
-    const int64_t rows = (int64_t)(set.solo ? 1 : set.Tmax - k) * set.b - (j + 1) * PW;
+    const int64_t rows = set.solo && set.one.vinv ? set.b
+                                                  : (int64_t)(set.solo ? 1 : set.Tmax - k) * set.b - (j + 1) * PW;
     if (rows > 0) {
         if (rows / 16 * set.count <= device_sms())
             EGS_LAUNCH(kt, KC_TRSM, s,
@@ -751,7 +856,7 @@ cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, cudaSt
     for (int j = 0; j < nj && e == cudaSuccess; ++j) {
         e = launch_diag_solve64(set, k, j, s, kt);
         if (e == cudaSuccess && j + 1 < nj)
-            e = launch_tc_f64(maps.ia, maps.ib, set, k, j + 1, nj, 1, k * (2 + nj) + 2 + j, 0, s, kt);
+            e = launch_tc_f64(maps.ia, maps.ib, set, k, j + 1, nj, F64_INNER, k * (2 + nj) + 2 + j, 0, s, kt);
     }
     return e;
 }
@@ -768,8 +873,35 @@ cudaError_t launch_slice_panel64(const F64Set &set, int k, cudaStream_t s, Kerne
 cudaError_t launch_update_tc64(const F64Maps &maps, const F64Set &set, int k, int part, int reserve, cudaStream_t s,
                                KernelTimer *kt)
 {
-    return launch_tc_f64(maps.a, maps.b, set, k, part == 2 ? 2 : 1, part == 1 ? 2 : set.Tmax, 0,
+    return launch_tc_f64(maps.a, maps.b, set, k, part == 2 ? 2 : 1, part == 1 ? 2 : set.Tmax, F64_TRAIL,
                          k * (2 + set.b / PW) + (part == 2 ? 1 : 0), reserve, s, kt);
+}
+
+cudaError_t launch_solo_init(const F64Set &set, cudaStream_t s, KernelTimer *kt)
+{
+    cudaError_t e = cudaMemsetAsync(set.one.ctr, 0, tc64_counters(set.b, set.Tmax) * sizeof(unsigned long long), s);
+    if (e != cudaSuccess) return e;
+    EGS_LAUNCH(kt, KC_OTHER, s,
+               k_identity_tiles<<<dim3((unsigned)set.Tmax, (unsigned)(set.b / 64)), 256, 0, s>>>(set.one.vinv, set.b));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_winv(const F64Set &set, int k, float *wsp, cudaStream_t s, KernelTimer *kt)
+{
+    const size_t sm = (size_t)8 * (set.b + 1) * sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(k_winv_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * 1025 * sizeof(double));
+    if (e != cudaSuccess) return e;
+    EGS_LAUNCH(kt, KC_TRSM, s, k_winv_rows<<<(unsigned)(set.b / 8), 256, sm, s>>>(set, k, wsp));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_band_solve(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt)
+{
+    if (nb <= 0) return cudaSuccess;
+    EGS_LAUNCH(kt, KC_TRSM, s, k_slice_panel64<<<dim3((unsigned)((size_t)nb * set.b / 8), 1), 256, 0, s>>>(set, k));
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_tc_f64(maps.a, maps.b, set, k, 1, 1 + nb, F64_BAND, k * (2 + set.b / PW), 0, s, kt);
 }
 
 }  // namespace egs

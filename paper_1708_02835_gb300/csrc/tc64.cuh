@@ -28,8 +28,10 @@ struct F64Prob {
     Tiles tl;
     DevStatus *st;
     double *z;                // T b: the right-hand side, solved along (L^-1 z); NULL: none
+    double *vinv;             // diagonal tiles alone: V_k = L_kk^-T (T b x b, identities before), or NULL
     F64Rows panel;            // K = b: row r of tile m at row0 + (m - k - 1) b + r
     F64Rows inner;            // K = 64, the current 64-column block: row0 + (m - k) b + r; sl NULL: no slices
+    F64Rows w;                // diagonal tiles alone: K = b, the rows of L_kk^-1
     unsigned long long *ctr;  // tc64_counters(b, T) zeroed work counters
     double *winv;             // inverses of the block's eight 8 x 8 diagonal blocks
 };
@@ -40,7 +42,8 @@ struct F64Set {
     const F64Prob *arr;
     F64Prob one;
     int count, b, Tmax;
-    int solo;  // 1: only the diagonal tile of a step (POTRF of one tile; launch_panel64 alone)
+    int solo;  // 1: the diagonal tile of a step alone (launch_panel64 is its POTRF and, with vinv, its
+               // inverse: V_k as further rows of the panel, row r at inner slice row b + r)
     __device__ const F64Prob &get(int i) const { return arr ? arr[i] : one; }
 };
 
@@ -55,8 +58,21 @@ cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64
 
 // Device scratch of one tensor-core FP64 factorisation, and the problem on it.
 size_t tc64_scratch_bytes(int b, int T);
-size_t tc64_solo_bytes(int b, int T);  // of the POTRFs of T diagonal tiles
-F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st, double *z, bool solo = false);
+F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st, double *z);
+
+// The same for the diagonal tiles of a mixed factorisation and the solves of nb tiles below
+// each (the FP64 band): launch_solo_init once, then per step launch_panel64, launch_winv and
+// launch_band_solve.
+size_t tc64_solo_bytes(int b, int T, int nb);
+F64Prob tc64_solo_problem(void *scratch, const Tiles &tl, DevStatus *st, double *vinv, int nb);
+cudaError_t make_f64_solo_maps(const F64Prob &p, F64Maps *maps);
+// Identities into V, the counters.
+cudaError_t launch_solo_init(const F64Set &set, cudaStream_t s, KernelTimer *kt);
+// The rows of W = L_kk^-1 = V_k^T: slices, and (wsp not NULL) the split-TF32 layout of the
+// off-band solve, row c: [hi | lo] of (float)W[c][.].
+cudaError_t launch_winv(const F64Set &set, int k, float *wsp, cudaStream_t s, KernelTimer *kt);
+// Tiles (k + 1 .. k + nb, k): X = A W^T, in place.
+cudaError_t launch_band_solve(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt);
 
 // The same without slices, for the DFMA updates; winv: kWinvDoubles of scratch.
 F64Prob dfma_problem(double *winv, const Tiles &tl, DevStatus *st, double *z);
