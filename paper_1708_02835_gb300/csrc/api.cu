@@ -152,7 +152,7 @@ static Layout make_layout(const TileGeom &g, bool tc)
     L.mtab = off;
     off += align256(EGS_MT_SCRATCH_DOUBLES * sizeof(double));
     L.winv = off;
-    off += align256(kWinvDoubles * sizeof(double));
+    off += align256(2 * kWinvDoubles * sizeof(double));
     L.tc = off;
     if (tc) off += tc64_scratch_bytes(g.b, g.T);
     L.total = off;
@@ -485,7 +485,7 @@ egs_status egs_potrf_tiles(void *tiles, int64_t n, int32_t tile, int64_t *fail_i
     DevStatus *st = nullptr;
     const size_t sbytes = align256(sizeof(DevStatus));
     const Allocator A = current_allocator();
-    const size_t cbytes = align256(sbytes + kWinvDoubles * sizeof(double));
+    const size_t cbytes = align256(sbytes + 2 * kWinvDoubles * sizeof(double));
     bool tc = tc64_applies(n, tile, g.T);
     size_t wbytes = cbytes + (tc ? tc64_scratch_bytes(g.b, g.T) : 0);
     cudaError_t e = dev_alloc(A, (void **)&st, wbytes, s);

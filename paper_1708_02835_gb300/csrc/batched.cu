@@ -603,7 +603,7 @@ cudaError_t enqueue_factor64(egs_batch *B, cudaStream_t s, int *count)
         set.count = B->active[k];
         set.b = B->b;
         set.Tmax = Tmax;
-        e = launch_panel64(B->maps, set, k, s, &kt);
+        e = launch_panel64(B->maps, set, k, nullptr, s, &kt);
         if (k + 1 < Tmax) {
             set.count = B->active[k + 1];
             if (e == cudaSuccess) e = launch_slice_panel64(set, k, s, &kt);
@@ -769,7 +769,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     const size_t fctr_off = off;
     off += a256(B->f64ctr * sizeof(unsigned long long));
     const size_t winv_off = off;
-    if (B->tc) off += a256((size_t)nprob * kWinvDoubles * sizeof(double));
+    if (B->tc) off += a256((size_t)nprob * 2 * kWinvDoubles * sizeof(double));
     std::vector<int64_t> prefix;
     std::vector<int4> tasks;
     std::vector<size_t> cnt_off;
@@ -882,7 +882,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
             P.panel = F64Rows{(uint16_t *)(B->ws + psl_off), (int *)(B->ws + pex_off), R, prow[i]};
             P.inner = F64Rows{(uint16_t *)(B->ws + isl_off), (int *)(B->ws + iex_off), R1, irow[i]};
             P.ctr = B->d_f64ctr + fctr[i];
-            P.winv = (double *)(B->ws + winv_off) + (size_t)i * kWinvDoubles;
+            P.winv = (double *)(B->ws + winv_off) + (size_t)i * 2 * kWinvDoubles;
         }
         e = make_f64_maps(fp[0].panel, fp[0].inner, tile, &B->maps);
         if (e == cudaSuccess) e = cudaMemcpy(B->d_f64, fp.data(), fp.size() * sizeof(F64Prob), cudaMemcpyHostToDevice);

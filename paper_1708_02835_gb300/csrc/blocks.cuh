@@ -360,6 +360,26 @@ __device__ __forceinline__ void solve64_rows(Solve64Smem<RB> &sm)
     }
 }
 
+// A 16 x 16 sub-block of a panel's update by its 64-column block j (K = 64), one entry a thread of
+// 256: columns c0 .. c0 + 15 of the rows at `row` minus X_row X_col^T, X in columns 64 j .. 64 j + 63 of
+// the rows at `row` and `col` (row stride b).  4.3 us of FP64 pipe.
+__device__ __forceinline__ void inner16(double (&As)[16][65], double (&Bs)[16][65], double *row, const double *col, int b,
+                                        int j, int c0)
+{
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    for (int e = tid; e < 16 * 64; e += 256) {
+        As[e >> 6][e & 63] = row[(size_t)(e >> 6) * b + j * 64 + (e & 63)];
+        Bs[e >> 6][e & 63] = col[(size_t)(e >> 6) * b + j * 64 + (e & 63)];
+    }
+    double *C = row + (size_t)ty * b + c0 + tx;
+    const double c = *C;
+    __syncthreads();
+    double acc = 0.0;
+#pragma unroll 8
+    for (int l = 0; l < 64; ++l) acc = fma(As[ty][l], Bs[tx][l], acc);
+    *C = c - acc;
+}
+
 // X_row . y over 64 columns, two per lane (y0, y1: the lane's entries of y); the sum in lane 0.
 __device__ __forceinline__ double dot64(double x0, double x1, double y0, double y1)
 {

@@ -41,31 +41,16 @@ __global__ void __launch_bounds__(256) k_update_f64(Tiles tl, int k, DevStatus *
                tl.t64(m, nc) + (size_t)sr * 64 * b + sc * 64, b);
 }
 
-// The update inside a panel by its 64-column block j: C -= X_rows X_cols^T (K = 64) for the
-// rows and columns of tile column k right of and below the block, one 16 x 16 sub-block per CTA
-// (one entry a thread: 4.3 us; blocks on the diagonal or below it).  grid = (row sub-blocks,
-// column sub-blocks).
+// The update inside a panel by its 64-column block j for the rows and columns of tile column k
+// right of and below the block, one 16 x 16 sub-block per CTA (blocks on the diagonal or below
+// it).  grid = (row sub-blocks, column sub-blocks).
 __global__ void __launch_bounds__(256) k_inner_f64(Tiles tl, int k, int j, const DevStatus *st)
 {
     if (failed(st)) return;
     __shared__ double As[16][65], Bs[16][65];
-    const int b = tl.b, tid = threadIdx.x, c0 = (j + 1) * 64 + (int)blockIdx.y * 16;
-    const int pr0 = (j + 1) * 64 + (int)blockIdx.x * 16;
+    const int b = tl.b, c0 = (j + 1) * 64 + (int)blockIdx.y * 16, pr0 = (j + 1) * 64 + (int)blockIdx.x * 16;
     if (pr0 < c0) return;
-    double *row = tl.t64(k + pr0 / b, k) + (size_t)(pr0 % b) * b;
-    const double *col = tl.t64(k, k) + (size_t)c0 * b + j * 64;
-    for (int e = tid; e < 16 * 64; e += 256) {
-        As[e >> 6][e & 63] = row[(size_t)(e >> 6) * b + j * 64 + (e & 63)];
-        Bs[e >> 6][e & 63] = col[(size_t)(e >> 6) * b + (e & 63)];
-    }
-    const int tx = tid & 15, ty = tid >> 4;
-    double *C = row + (size_t)ty * b + c0 + tx;
-    const double c = *C;
-    __syncthreads();
-    double acc = 0.0;
-#pragma unroll 8
-    for (int l = 0; l < 64; ++l) acc = fma(As[ty][l], Bs[tx][l], acc);
-    *C = c - acc;
+    inner16(As, Bs, tl.t64(k + pr0 / b, k) + (size_t)(pr0 % b) * b, tl.t64(k, k) + (size_t)c0 * b, b, j, c0);
 }
 
 // The same update in 32 x 32 sub-blocks, for launches too small to fill the
@@ -108,11 +93,13 @@ cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *
         const F64Set set{nullptr, tc64_problem(tc_scratch, tl, st, z), 1, g.b, T, 0};
         F64Maps maps;
         e = make_f64_maps(set.one.panel, set.one.inner, g.b, &maps);
+        F64Fork fork;
+        if (e == cudaSuccess) e = fork.create(false);
         if (e == cudaSuccess)
             e = cudaMemsetAsync(set.one.ctr, 0, tc64_counters(g.b, T) * sizeof(unsigned long long), s);
         for (int k = 0; k < T && e == cudaSuccess; ++k) {
             if (kt) kt->step = k;
-            e = launch_panel64(maps, set, k, s, kt);
+            e = launch_panel64(maps, set, k, &fork, s, kt);
             if (e == cudaSuccess) e = launch_slice_panel64(set, k, s, kt);
             if (e == cudaSuccess) e = launch_update_tc64(maps, set, k, 0, 0, s, kt);
         }

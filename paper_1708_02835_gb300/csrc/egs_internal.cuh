@@ -163,7 +163,7 @@ cudaError_t launch_matern_table(const egs_matern_params &P, double *tab, cudaStr
 // Tile Cholesky in place (FP64).  Stops doing work once st->fail_index is set.
 // z (T b doubles, may be NULL) is solved along: L^-1 z in place.  tc_scratch:
 // tc64_scratch_bytes(b, T) bytes for the tensor-core update, or NULL for the DFMA
-// update, which needs winv (kWinvDoubles doubles of scratch).
+// update, which needs winv (2 kWinvDoubles doubles of scratch).
 cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *st, cudaStream_t s,
                                    KernelTimer *kt, double *winv, void *tc_scratch, double *z);
 

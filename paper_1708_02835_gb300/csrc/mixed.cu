@@ -464,6 +464,8 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
     // solve as task graph, column and row substitutions; 0.85 and 0.05 ms so
     const F64Set diag{nullptr, tc64_solo_problem(mb.dpan, tl, st, mb.vinv, band_tiles(tl)), 1, b, T, 1};
     F64Maps dmaps;
+    F64Fork fork;
+    if (e == cudaSuccess) e = fork.create(true);
     if (e == cudaSuccess) e = make_f64_solo_maps(diag.one, &dmaps);
     if (e == cudaSuccess) e = launch_solo_init(diag, s, kt);
     if (e == cudaSuccess) e = cudaEventRecord(ev_col, s);  // the side stream starts after prior work on s
@@ -483,7 +485,7 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
         // before the call (Sigma generation).
         if (k == 0) e = cudaStreamWaitEvent(side, ev_col, 0);
         if (e == cudaSuccess)
-            e = launch_panel64(dmaps, diag, k, side, kts);
+            e = launch_panel64(dmaps, diag, k, &fork, side, kts);
         // the rows of W for the band solve and (FP32 mode, split TF32) for the main stream's
         // off-band TRSM
         float *wsp = mb.wsp + (size_t)(k & 1) * 2 * tl.bb();

@@ -33,7 +33,7 @@ struct F64Prob {
     F64Rows inner;            // K = 64, the current 64-column block: row0 + (m - k) b + r; sl NULL: no slices
     F64Rows w;                // diagonal tiles alone: K = b, the rows of L_kk^-1
     unsigned long long *ctr;  // tc64_counters(b, T) zeroed work counters
-    double *winv;             // inverses of the block's eight 8 x 8 diagonal blocks
+    double *winv;             // inverses of the block's eight 8 x 8 diagonal blocks, two of kWinvDoubles (j & 1)
 };
 
 // The problems of a launch (one per grid row): one, or count of them in device memory with
@@ -74,13 +74,22 @@ cudaError_t launch_winv(const F64Set &set, int k, float *wsp, cudaStream_t s, Ke
 // Tiles (k + 1 .. k + nb, k): X = A W^T, in place.
 cudaError_t launch_band_solve(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt);
 
-// The same without slices, for the DFMA updates; winv: kWinvDoubles of scratch.
+// The same without slices, for the DFMA updates; winv: 2 kWinvDoubles of scratch.
 F64Prob dfma_problem(double *winv, const Tiles &tl, DevStatus *st, double *z);
 // Diagonal block j of step k; the solves of the rows below it (launch_panel64's first two parts).
 cudaError_t launch_diag_solve64(const F64Set &set, int k, int j, cudaStream_t s, KernelTimer *kt);
 
-// POTRF of tile (k, k) and the solves of every tile below it, in 64-column blocks.
-cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, cudaStream_t s, KernelTimer *kt);
+// A second stream for the panels of one factorisation.
+struct F64Fork {
+    cudaStream_t aux = nullptr;
+    cudaEvent_t diag = nullptr, next = nullptr, bulk = nullptr;
+    cudaError_t create(bool high_priority);
+    ~F64Fork();
+};
+
+// POTRF of tile (k, k) and the solves of every tile below it, in 64-column blocks; fork may be NULL.
+cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, F64Fork *fork, cudaStream_t s,
+                           KernelTimer *kt);
 // Slices of the solved panel tiles (k + 1 .. T - 1, k).
 cudaError_t launch_slice_panel64(const F64Set &set, int k, cudaStream_t s, KernelTimer *kt);
 // C_mn -= P_m P_n^T, m = n .. T - 1.  part 0: n = k + 1 .. T - 1; 1: n = k + 1; 2: the rest.
