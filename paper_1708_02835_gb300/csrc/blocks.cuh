@@ -151,18 +151,19 @@ __device__ __forceinline__ bool potrf64_smem(double *A, int ld, int64_t row0, De
 //  - panels of 4 columns: warps 0 .. 2 each factor the 4 x 4 block in lanes 0 .. 3, redundantly
 //    (each has a sub-partition of its own), while lanes 4 .. 31 carry 28 rows below it, so that
 //    the rows below cost no instruction;
-//  - the 4-term updates of the entries right of the panel are spread over all lanes.
-// 64 pivots x 22 / 4 instructions of panels, about 400 of updates: 47 us with the launch (115 us with 16-column
-// panels, a thread per row below them and a square root per pivot).
+//  - the 4-term updates of the entries right of the panel are spread over all lanes, those of
+//    the next panel's columns at once, the others while the next panel is factored.
+// 64 pivots x 22 / 4 instructions of panels, about 400 of updates: 43 us with the launch (115 us
+// with 16-column panels, a thread per row below them and a square root per pivot).
 //
 // Leaves L (zero upper half), y in row 64 and 1 / L_jj in sm; false if a pivot is not positive
 // (its row is recorded as row0 + j).
 // ---------------------------------------------------------------------------
 struct Chol64Smem {
     double S[65][65];
-    double W[65][5];  // a / d of the panel's columns
+    double W[2][65][5];  // a / d of the columns of this panel and the one before
     double rd[64];
-    int fail_j;
+    int fail_j, claim;
 };
 
 // 1 / sqrt(d) for normal d > 0: the hardware's approximation and one step of Householder's
@@ -195,11 +196,16 @@ __device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld
 #pragma unroll
     for (int q = 0; q < 16; ++q) sm.S[(tid + 256 * q) >> 6][tid & 63] = v[q];
     if (z && tid < 64) sm.S[64][tid] = z[tid];
-    if (tid == 0) sm.fail_j = -1;
+    if (tid == 0) {
+        sm.fail_j = -1;
+        sm.claim = 0;
+    }
     __syncthreads();
     const int zr = z ? 1 : 0;
 #pragma unroll 1
     for (int p0 = 0; p0 < 64; p0 += 4) {
+        double(&W)[65][5] = sm.W[(p0 >> 2) & 1];
+        const double(&Wp)[65][5] = sm.W[((p0 >> 2) & 1) ^ 1];
         const int q0 = p0 + 4, m = 64 - q0;  // rows and columns left
         double a[4];
         if (28 * warp < m + zr || warp == 0) {
@@ -229,7 +235,33 @@ __device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     sm.S[i][p0 + c] = a[c];
-                    sm.W[i][c] = w[c];
+                    W[i][c] = w[c];
+                }
+            }
+        }
+        // the columns right of this panel by the panel before, 64 entries at a time to whichever
+        // warp is free: lower triangle from q0 on, then the z row (the triangle's next row but for
+        // its last entry)
+        if (p0 > 0) {
+            const int cnt = m * (m + 1) / 2 + (zr ? m : 0);
+            for (;;) {
+                int base = 0;
+                if (lane == 0) base = atomicAdd(&sm.claim, 64);
+                base = __shfl_sync(0xffffffffu, base, 0);
+                if (base >= cnt) break;
+#pragma unroll
+                for (int h2 = 0; h2 < 2; ++h2) {
+                    const int e = base + 32 * h2 + lane;
+                    if (e < cnt) {
+                        int ii = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+                        if (ii * (ii + 1) / 2 > e) --ii;
+                        if ((ii + 1) * (ii + 2) / 2 <= e) ++ii;
+                        const int i = ii < m ? q0 + ii : 64, c = q0 + e - ii * (ii + 1) / 2;
+                        double acc = sm.S[i][c];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) acc = fma(-sm.S[i][p0 - 4 + j], Wp[c][j], acc);
+                        sm.S[i][c] = acc;
+                    }
                 }
             }
         }
@@ -242,17 +274,13 @@ __device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld
             if (tid == 0) atomicMin(&st->fail_index, (unsigned long long)(row0 + sm.fail_j));
             return false;
         }
-        // lower triangle of the rows and columns from q0 on, then the z row (the triangle's
-        // next row but for its last entry)
-        const int cnt = m * (m + 1) / 2 + (zr ? m : 0);
-        for (int e = tid; e < cnt; e += 256) {
-            int ii = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-            if (ii * (ii + 1) / 2 > e) --ii;
-            if ((ii + 1) * (ii + 2) / 2 <= e) ++ii;
-            const int i = ii < m ? q0 + ii : 64, c = q0 + e - ii * (ii + 1) / 2;
+        // the next panel's four columns by this one
+        if (tid == 0) sm.claim = 0;
+        const int ri = tid >> 2, c = q0 + (tid & 3), i = ri < m ? q0 + ri : 64;
+        if (m > 0 && ri < m + zr && i >= c) {
             double acc = sm.S[i][c];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc = fma(-sm.S[i][p0 + j], sm.W[c][j], acc);
+            for (int j = 0; j < 4; ++j) acc = fma(-sm.S[i][p0 + j], W[c][j], acc);
             sm.S[i][c] = acc;
         }
         __syncthreads();

@@ -10,7 +10,7 @@
 //          panel buffer in the tensor-core operand format (TF32-rounded FP32,
 //          split TF32 hi/lo pairs, or BF16);
 //   UPDATE C_mn -= P_m P_n^T: when both P_m and P_n are FP64 band tiles the
-//          update runs in FP64 (DFMA) on the unrounded values.  TF32 / BF16:
+//          update is FP64-accurate, on the unrounded values (tc64.cu).  TF32 / BF16:
 //          every other update runs on tcgen05 with FP32 accumulation
 //          (tc_gemm.cu) and is subtracted in FP64 from band tiles and in FP32
 //          from the others.  FP32 mode (split TF32): each update takes the
@@ -515,13 +515,13 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
         if (e == cudaSuccess) e = cudaEventRecord(ev_panel, side);
         // updates whose two operands are FP64 band tiles stay FP64-accurate
         // (they carry the nearest-neighbour entries that set the diagonal
-        // pivots): on DFMA, or in the FP32 mode as exact slice products;
+        // pivots): as exact slice products (in the FP32 mode of 35 bits);
         // their outputs are read by nothing else at this step
         if (e == cudaSuccess && k + 1 < T) {
             if (FMT == 3)  // FP32 mode: from the band rows' exact slices on tcgen05
                 e = launch_band_band_ozaki(moz[k & 1][0], moz[k & 1][1], tl, k, nb, ozs, mb.err, side, kts);
             else
-                e = launch_update_f64(tl, k, (int64_t)nb * (nb + 1) / 2, st, side, kts, KC_UPDATE64);
+                e = launch_band_update(dmaps, diag, k, nb, side, kts);  // 84 us by DFMA at tile 256
         }
         if (k + 1 == T || e != cudaSuccess) break;
         // ---- step k on the main stream: the off-band TRSM (whole GPU),

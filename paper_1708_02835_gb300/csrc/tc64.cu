@@ -434,7 +434,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
     const F64Prob &P = set.get(blockIdx.y);
     const bool solo = set.solo != 0;
     if (P.tl.T <= k) return;
-    const int T = solo && mode == F64_INNER ? k + 1 + (P.vinv ? 1 : 0) : P.tl.T;
+    const int T = !solo ? P.tl.T : (mode == F64_INNER ? k + 1 + (P.vinv ? 1 : 0) : k + c1);
     // columns k + c0 .. min(k + c1, T) - 1; inside a panel the blocks c0 .. c1 - 1 of column k
     const F64Work work{P.tl, T, k, mode == F64_INNER ? c0 : k + c0, mode == F64_INNER ? c1 : min(k + c1, T), mode};
     if (work.col0 >= work.col1) return;
@@ -812,6 +812,7 @@ cudaError_t make_f64_solo_maps(const F64Prob &P, F64Maps *maps)
     cudaError_t e = cudaSuccess;
     maps->a = CUtensorMap{};
     if (P.panel.rows) e = make_map3(&maps->a, P.panel.sl, P.panel.rows, b, FM, 1);
+    if (e == cudaSuccess && P.panel.rows) e = make_map3(&maps->pb, P.panel.sl, P.panel.rows, b, FN, kF64Slices);
     if (e == cudaSuccess) e = make_map3(&maps->b, P.w.sl, P.w.rows, b, FN, kF64Slices);
     if (e == cudaSuccess) e = make_map3(&maps->ia, P.inner.sl, P.inner.rows, PW, FM, 1);
     if (e == cudaSuccess) e = make_map3(&maps->ib, P.inner.sl, P.inner.rows, PW, FN, kF64Slices);
@@ -833,13 +834,15 @@ static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, con
     cudaError_t e = cudaFuncSetAttribute(k_tc_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
     if (e != cudaSuccess) return e;
     // of the largest problem, as in the kernel
-    const int T = set.solo && mode == F64_INNER ? k + 1 + (set.one.vinv ? 1 : 0) : set.Tmax;
+    const int T = !set.solo ? set.Tmax : (mode == F64_INNER ? k + 1 + (set.one.vinv ? 1 : 0) : k + c1);
     const Tiles tl{nullptr, nullptr, set.b, T, T};
     const bool in = mode == F64_INNER;
     const F64Work w{tl, T, k, in ? c0 : k + c0, in ? c1 : (k + c1 < T ? k + c1 : T), mode};
     if (w.col0 >= w.col1) return cudaSuccess;
     const dim3 grid(tc64_ctas(set, w.items(), reserve), (unsigned)set.count);
-    EGS_LAUNCH(kt, mode == F64_BAND ? KC_TRSM : KC_UPDATE, s,
+    // of a mixed factorisation's diagonal tile: part of its POTRF; its band: the FP64 update class
+    const int cls = mode == F64_BAND ? KC_TRSM : (!set.solo ? KC_UPDATE : (in ? KC_POTRF : KC_UPDATE64));
+    EGS_LAUNCH(kt, cls, s,
                k_tc_f64<<<grid, FTHREADS, FSMEM, s>>>(a, b, set, k, c0, c1, mode, slot));
     return cudaGetLastError();
 }
@@ -926,7 +929,8 @@ cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, F64For
         }
         if (e != cudaSuccess) break;
         if (more) {
-            EGS_LAUNCH(kt, KC_UPDATE, s, k_next64<<<dim3(10, (unsigned)set.count), 256, 0, s>>>(set, k, j));
+            EGS_LAUNCH(kt, set.solo ? KC_POTRF : KC_UPDATE, s,
+                       k_next64<<<dim3(10, (unsigned)set.count), 256, 0, s>>>(set, k, j));
             e = cudaGetLastError();
             if (fork && e == cudaSuccess) e = cudaStreamWaitEvent(bs, fork->next, 0);
             if (e == cudaSuccess)
@@ -979,6 +983,15 @@ cudaError_t launch_band_solve(const F64Maps &maps, const F64Set &set, int k, int
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_tc_f64(maps.a, maps.b, set, k, 1, 1 + nb, F64_BAND, k * (2 + set.b / PW), 0, s, kt);
+}
+
+cudaError_t launch_band_update(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt)
+{
+    if (nb <= 0) return cudaSuccess;
+    EGS_LAUNCH(kt, KC_TRSM, s, k_slice_panel64<<<dim3((unsigned)((size_t)nb * set.b / 8), 1), 256, 0, s>>>(set, k));
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_tc_f64(maps.a, maps.pb, set, k, 1, 1 + nb, F64_TRAIL, k * (2 + set.b / PW) + 1, 0, s, kt);
 }
 
 }  // namespace egs

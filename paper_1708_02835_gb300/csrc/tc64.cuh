@@ -51,7 +51,8 @@ struct F64Set {
 inline size_t tc64_counters(int b, int T) { return (size_t)T * (2 + b / kF64Panel); }
 
 struct F64Maps {
-    CUtensorMap a, b, ia, ib;  // panel slices, inner slices
+    CUtensorMap a, b, ia, ib;  // panel slices, inner slices; diagonal tiles alone: b is W's, pb the panel's
+    CUtensorMap pb;
 };
 // Over slice arrays of rows (K = b) and irows (K = 64) rows.
 cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64Maps *maps);
@@ -90,6 +91,8 @@ struct F64Fork {
 // POTRF of tile (k, k) and the solves of every tile below it, in 64-column blocks; fork may be NULL.
 cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, F64Fork *fork, cudaStream_t s,
                            KernelTimer *kt);
+// C_mn -= X_m X_n^T for the FP64 band tiles k < n <= m <= k + nb, from the solved band rows.
+cudaError_t launch_band_update(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt);
 // Slices of the solved panel tiles (k + 1 .. T - 1, k).
 cudaError_t launch_slice_panel64(const F64Set &set, int k, cudaStream_t s, KernelTimer *kt);
 // C_mn -= P_m P_n^T, m = n .. T - 1.  part 0: n = k + 1 .. T - 1; 1: n = k + 1; 2: the rest.
