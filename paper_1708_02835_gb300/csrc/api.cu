@@ -489,7 +489,7 @@ egs_status egs_potrf_tiles(void *tiles, int64_t n, int32_t tile, int64_t *fail_i
     bool tc = tc64_applies(n, tile, g.T);
     size_t wbytes = cbytes + (tc ? tc64_scratch_bytes(g.b, g.T) : 0);
     cudaError_t e = dev_alloc(A, (void **)&st, wbytes, s);
-    if (e == cudaErrorMemoryAllocation && tc) {  // no room for the slices: the DFMA update
+    if (e == cudaErrorMemoryAllocation && tc && !A.alloc) {  // no room for the slices: the DFMA update
         cudaGetLastError();
         tc = false;
         wbytes = cbytes;
@@ -572,7 +572,7 @@ egs_status egs_loglik_ex(const double *locs, const double *z, const double theta
         ws = (char *)opts->workspace;
     } else {
         e = dev_alloc(A, (void **)&ws, es.need, s);
-        if (e == cudaErrorMemoryAllocation && eval_shrink(&es)) {
+        if (e == cudaErrorMemoryAllocation && !A.alloc && eval_shrink(&es)) {  // a hook is asked once
             cudaGetLastError();
             e = dev_alloc(A, (void **)&ws, es.need, s);
         }
@@ -649,7 +649,7 @@ egs_status egs_simulate(const double *locs, const double *e, const double theta[
     char *ws = nullptr;
     const Allocator A = current_allocator();
     cudaError_t err = dev_alloc(A, (void **)&ws, es.need, s);
-    if (err == cudaErrorMemoryAllocation && eval_shrink(&es)) {
+    if (err == cudaErrorMemoryAllocation && !A.alloc && eval_shrink(&es)) {  // a hook is asked once
         cudaGetLastError();
         err = dev_alloc(A, (void **)&ws, es.need, s);
     }

@@ -112,7 +112,7 @@ extern "C" egs_status egs_predict(const double *locs_obs, const double *z_obs, i
     const Allocator A = current_allocator();
     size_t wbytes = es.need + extra_new + extra_out;
     cudaError_t e = dev_alloc(A, (void **)&ws, wbytes, s);
-    if (e == cudaErrorMemoryAllocation && eval_shrink(&es)) {
+    if (e == cudaErrorMemoryAllocation && !A.alloc && eval_shrink(&es)) {  // a hook is asked once
         cudaGetLastError();
         wbytes = es.need + extra_new + extra_out;
         e = dev_alloc(A, (void **)&ws, wbytes, s);
