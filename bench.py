@@ -188,6 +188,16 @@ def tensor_peak(precision: str, sustained: bool = False) -> dict:
     return {"tflops": bf16, "source": src}
 
 
+F64_KERNEL = ("k_tc_f64 (SYRK/GEMM trailing update, 28 exact BF16 slice products per FP64 product on tcgen05; the "
+              "event time includes the updates inside the panels)")
+
+
+def f64_tensor_peak() -> dict:
+    """FP64-equivalent rate of 28 BF16 products per FP64 product at the sustained BF16 rate."""
+    p = tensor_peak("bf16", sustained=True)
+    return {"tflops": p["tflops"] / 28.0, "source": p["source"] + " / 28 (slice products per FP64 product)"}
+
+
 class ClockSampler:
     """nvidia-smi clock / throttle sampling during the timed region."""
 
@@ -515,11 +525,10 @@ def fp64_leg(a, egs, dlocs, dz, theta, stream) -> dict:
             "phase_ms": {"generate": info["ms_generate"], "factor": info["ms_factor"], "solve": info["ms_solve"]},
             "kernel_class_ms": {k: info["ms_" + k] for k in ("update", "potrf", "trsm", "trsv")},
             "gpu_launches": info["launches"], "clocks": clocks,
-            "roofline": {"bound": "alu", "kernel": "k_update_f64 (SYRK/GEMM trailing update, DFMA)",
-                         "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                         "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
-                         "peak_source": "derived: 152 SMs x 2 DFMA/clk x 2 flop x 2070 MHz (FP64 pipe; no FP64 "
-                                        "tensor-core path is used)",
+            "roofline": {"bound": "tensor", "kernel": F64_KERNEL,
+                         "achieved": achieved, "peak": f64_tensor_peak()["tflops"], "unit": "TFLOP/s",
+                         "frac": achieved / f64_tensor_peak()["tflops"], "traffic": None,
+                         "peak_source": f64_tensor_peak()["source"],
                          "launches": nlaunch, "flops_per_launch": fc["update"] / nlaunch,
                          "ms_per_launch": upd / nlaunch},
             "note": "one evaluation, CUDA events on the launching stream, same inputs as the timed mixed steps"}
@@ -642,9 +651,10 @@ def main():
                            "stream include time spent waiting for SMs")
         if a.precision == "fp64":
             achieved = fc["update"] / (upd_ms / 1e3) / 1e12 if upd_ms > 0 else 0.0
-            roof = {"bound": "alu", "kernel": "k_update_f64 (SYRK/GEMM trailing update)", "achieved": achieved,
-                    "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
-                    "peak_source": "derived: 152 SMs x 2 DFMA/clk x 2 flop x 2070 MHz (FP64 pipe, no tensor path)",
+            peak = f64_tensor_peak()
+            roof = {"bound": "tensor", "kernel": F64_KERNEL, "achieved": achieved,
+                    "peak": peak["tflops"], "unit": "TFLOP/s", "frac": achieved / peak["tflops"], "traffic": None,
+                    "peak_source": peak["source"],
                     "launches_per_step": launches_update,
                     "flops_per_launch": fc["update"] / launches_update, "ms_per_launch": upd_ms / launches_update}
         else:
@@ -688,9 +698,9 @@ def main():
             upd64 = info2["ms_update_f64"]
             if upd64 > 0:
                 a64 = f64_flops / (upd64 / 1e3) / 1e12
-                kern = "k_update_f64 (band x band, DFMA)"
+                kern = "k_tc_f64 (band x band, 28 exact BF16 slice products on tcgen05)"
                 if a.precision == "fp32":
-                    kern += " + k_tc_ozaki (other band outputs, 15 exact BF16 slice products on tcgen05)"
+                    kern = "k_tc_ozaki (band outputs, 15 exact BF16 slice products on tcgen05)"
                 roof["fp64_accurate_updates"] = {
                     "kernel": kern, "achieved_fp64_equivalent": a64, "fp64_peak": FP64_PEAK_TFLOPS,
                     "unit": "TFLOP/s", "vs_fp64_peak": a64 / FP64_PEAK_TFLOPS, "flops_per_step": f64_flops,
