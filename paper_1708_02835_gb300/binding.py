@@ -208,7 +208,7 @@ def egs_set_allocator(alloc=None, free=None):
     alloc(nbytes, stream) returns a device pointer (an int; 0 when it cannot),
     usable in stream order on stream (a cudaStream_t as an int, 0 = legacy);
     free(ptr, nbytes, stream) returns it.  Both None restores the library's
-    own cudaMallocAsync.  The library may call them from its serving thread,
+    own memory pool.  The library may call them from its serving thread,
     and servers and batches keep the hooks they were created with (the
     callbacks are therefore never released)."""
     lib = load_library()

@@ -9,9 +9,9 @@ constexpr int kF64Slices = 7;
 constexpr int kF64Panel = 64;  // width of the blocks a tile column is factored in
 
 // FP64 factorisations take the tensor cores above this many rows.  Below it the chain of
-// diagonal tiles sets the time (n = 1,600: update 1.1 of 6.2 ms), and the persistent batch,
-// which runs the DFMA routines, stays bit for bit equal to a single evaluation; above it the
-// update does (n = 5,000: 36.4 of 57 ms with DFMA, 1.6 here).
+// diagonal blocks sets the time (n = 1,600: DFMA trailing updates 1.1 of 3.6 ms), and the
+// persistent batch, which runs the DFMA routines, stays bit for bit equal to a single evaluation;
+// above it the updates do (n = 5,000: 36.4 ms by DFMA, 2.5 here).
 constexpr int64_t kTc64MinRows = 2049;
 inline bool tc64_applies(int64_t n, int b, int T) { return n >= kTc64MinRows && T > 1 && b % 64 == 0; }
 
