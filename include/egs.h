@@ -508,7 +508,7 @@ egs_status egs_tc_gemm_test_withhold(const void *A, const void *B, int32_t M, in
  *   A  device, M x K row-major FP64;  B  device, N x K row-major FP64
  *   C  device, M x N row-major FP64, written
  * M % 128 == 0, N % 32 == 0, K % 64 == 0, K <= 512.  Synchronises stream;
- * allocates its slices with cudaMallocAsync on stream.
+ * allocates its slices in stream order on stream.
  */
 egs_status egs_ozaki_gemm_test(const double *A, const double *B, int32_t M, int32_t N, int32_t K, double *C,
                                void *stream);

@@ -395,7 +395,7 @@ egs_status egs_set_allocator(egs_alloc_fn alloc, egs_free_fn free_fn, void *ctx)
 {
     g_err[0] = 0;
     if ((alloc == nullptr) != (free_fn == nullptr))
-        return set_error(EGS_ERR_ARG, "egs_set_allocator: give both hooks, or neither to restore cudaMallocAsync");
+        return set_error(EGS_ERR_ARG, "egs_set_allocator: give both hooks, or neither to restore the library's pool");
     std::lock_guard<std::mutex> lk(g_alloc_mu);
     g_alloc = Allocator{alloc, free_fn, alloc ? ctx : nullptr};
     return EGS_OK;
