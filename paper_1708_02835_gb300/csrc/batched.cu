@@ -668,7 +668,7 @@ cudaError_t enqueue_all(egs_batch *B, cudaStream_t s)
 
 // A batch takes the tensor cores when its largest problem does as a single evaluation, with
 // all its problems (96 problems of 256 to 4,096 rows, tile 128: 607 ms as one persistent
-// launch of DFMA tasks, 101 ms so); without such a problem it stays on the persistent launch,
+// launch of DFMA tasks, 76 ms so); without such a problem it stays on the persistent launch,
 // whose results equal single evaluations bit for bit.  any_size (the independent-blocks
 // approximation, whose blocks are no single evaluations): whatever the sizes.  once: the batch
 // lives for one call, its memory comes from the pool.

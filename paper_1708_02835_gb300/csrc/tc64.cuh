@@ -9,7 +9,7 @@ constexpr int kF64Slices = 7;
 constexpr int kF64Panel = 64;  // width of the blocks a tile column is factored in
 
 // FP64 factorisations take the tensor cores above this many rows.  Below it the chain of
-// diagonal blocks sets the time (n = 1,600: DFMA trailing updates 1.1 of 3.6 ms), and the
+// diagonal blocks sets the time (n = 1,600: DFMA trailing updates 1.1 of 3.4 ms), and the
 // persistent batch, which runs the DFMA routines, stays bit for bit equal to a single evaluation;
 // above it the updates do (n = 5,000: 36.4 ms by DFMA, 2.5 here).
 constexpr int64_t kTc64MinRows = 2049;
