@@ -278,15 +278,11 @@ cudaError_t launch_update_f64(const Tiles &tl, int k, int64_t ntri, DevStatus *s
 // (ozaki.cu).  The TRSM stage writes the slices of every panel row.
 size_t ozaki_slices_bytes(int b, int T);
 cudaError_t make_ozaki_maps(const void *oz, int b, int T, CUtensorMap *mapA, CUtensorMap *mapB);
-// Band tiles of columns col0 .. col0 + ncols - 1 at step k.
-// xband >= tl.band: outputs m = n .. n + xband - 1 (those with m - n >= band
-// are FP32 tiles, updated in FP64 and rounded once).
-cudaError_t launch_band_out_ozaki(const CUtensorMap &mapA, const CUtensorMap &mapB, const Tiles &tl, int xband, int k,
-                                  int col0, int ncols, const double *scale, int *err, cudaStream_t s, KernelTimer *kt);
-// The band x band update of step k (tiles (m, n), k < n <= m <= k + nb) from
-// the slices of the FP64 band rows.
-cudaError_t launch_band_band_ozaki(const CUtensorMap &mapA, const CUtensorMap &mapB, const Tiles &tl, int k, int nb,
-                                   const double *scale, int *err, cudaStream_t s, KernelTimer *kt);
+// One part (mixed_order.cuh) of step k.  xband >= tl.band: kColumn and kRest write the outputs with
+// m - n < xband (those with m - n >= band are FP32 tiles, updated in FP64 and rounded once);
+// kBandBand the tiles (m, n), k < n <= m < k + band, from the slices of the FP64 band rows.
+cudaError_t launch_band_ozaki(const CUtensorMap &mapA, const CUtensorMap &mapB, const Tiles &tl, int xband, int k,
+                              int part, const double *scale, int *err, cudaStream_t s, KernelTimer *kt);
 cudaError_t launch_forward_solve(const Tiles &tl, double *zpad, double *partials, DevStatus *st, cudaStream_t s,
                                  KernelTimer *kt);
 // z_m -= L_mk y_k for m > k, y_k read from ysrc (may equal zpad).
@@ -316,7 +312,7 @@ size_t panel_buffer_bytes(int b, int T, int fmt);
 cudaError_t make_panel_maps(const void *panel, int fmt, int b, int T, CUtensorMap *mapA, CUtensorMap *mapB);
 // Map for the epilogue's TMA reduce into the off-band FP32 tiles.
 cudaError_t make_offband_map(const float *f32, int b, size_t ntiles, CUtensorMap *mapC);
-// part 0: all trailing tiles of step k; 1: column k + 1; 2: columns k + 2 onwards.
+// part: mixed_order.cuh, kColumn or kRest.
 // fmt 3 updates only the off-band outputs (m - n >= band); the band outputs
 // are left to the FP64 kernels.
 // FP32 mode: the off-band panel TRSM of step k (tiles m0 .. T - 1) on the
@@ -330,7 +326,7 @@ cudaError_t launch_trsm_tc(const CUtensorMap &mapA, const CUtensorMap &mapW, con
 // scale of every panel row (panel_f16_scales); NULL otherwise.
 // xband (fmt >= 3): outputs with m - n < xband are left to the FP64-accurate kernels.
 cudaError_t launch_update_tc(const CUtensorMap &mapA, const CUtensorMap &mapB, const CUtensorMap &mapC, int fmt,
-                             const Tiles &tl, int k, int *err, cudaStream_t s, KernelTimer *kt, int part = 0,
-                             const float *rs = nullptr, int xband = 0);
+                             const Tiles &tl, int k, int *err, cudaStream_t s, KernelTimer *kt, int part,
+                             const float *rs, int xband);
 
 }  // namespace egs

@@ -24,6 +24,7 @@
 // iterative refinement: x0 = L^-T L^-1 Z, r = Z - Sigma x0 with Sigma
 // regenerated tile by tile (symv_regen.cu), x1 = x0 + L^-T L^-1 r, quad = Z^T x1.
 #include "blocks.cuh"
+#include "mixed_order.cuh"
 #include "slices.cuh"
 #include "tc64.cuh"
 
@@ -428,13 +429,16 @@ namespace {
 // The factorisation with one step of lookahead.  The FP64 chain of step k
 // (POTRF, the band TRSM, the band rows' operands, then the FP64 band x band
 // update) runs on a side stream; the main stream runs the TRSM of the
-// off-band panel on the whole GPU and the tensor-core update of column k + 1,
-// signals the side stream, and updates the rest of the trailing matrix
-// (leaving a few SMs free) while the next chain runs.  Diagonal tile k + 1
-// is final once the chain's own band x band update of step k is done (every
-// other update of column k + 1 writes tiles below it), so POTRF(k + 1) does
-// not wait for the main stream: only the band TRSM of step k + 1, whose rows
-// column k + 1's other updates write, waits for its signal.  In the FP32 mode
+// off-band panel on the whole GPU and the tensor-core update of column k + 1
+// and of the corner (the tiles of row k + band that the next chain's band x
+// band update writes too, mixed_order.cuh), signals the side stream, and
+// updates the rest of the trailing matrix (leaving a few SMs free) while the
+// next chain runs.  With a band of two tiles or more, diagonal tile k + 1 is
+// final once the chain's own band x band update of step k is done: its other
+// updates are the corner's of step k - 1 and earlier ones, ahead of the signal
+// that chain k waited for.  So POTRF(k + 1) does not wait for the main stream:
+// only the band TRSM of step k + 1, whose rows column k + 1's other updates
+// write, waits for its signal.  In the FP32 mode
 // the chain also inverts L_kk right after POTRF(k) (a latency-bound kernel
 // kept off the main stream), and the main stream's off-band TRSM through
 // L_kk^-1 starts once that is done, beside the chain's band TRSM.  Panels,
@@ -483,7 +487,7 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
         // band rows' operands; then (after signalling the main stream) the
         // FP64 band x band update.  At k = 0 ev_col marks the work on s
         // before the call (Sigma generation).
-        if (k == 0) e = cudaStreamWaitEvent(side, ev_col, 0);
+        if (k == 0 || order::potrf_waits_for_column(tl.band)) e = cudaStreamWaitEvent(side, ev_col, 0);
         if (e == cudaSuccess)
             e = launch_panel64(dmaps, diag, k, &fork, side, kts);
         // the rows of W for the band solve and (FP32 mode, split TF32) for the main stream's
@@ -519,13 +523,14 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
         // their outputs are read by nothing else at this step
         if (e == cudaSuccess && k + 1 < T) {
             if (FMT == 3)  // FP32 mode: from the band rows' exact slices on tcgen05
-                e = launch_band_band_ozaki(moz[k & 1][0], moz[k & 1][1], tl, k, nb, ozs, mb.err, side, kts);
+                e = launch_band_ozaki(moz[k & 1][0], moz[k & 1][1], tl, mb.xband, k, order::kBandBand, ozs, mb.err, side,
+                                      kts);
             else
                 e = launch_band_update(dmaps, diag, k, nb, side, kts);  // 84 us by DFMA at tile 256
         }
         if (k + 1 == T || e != cudaSuccess) break;
         // ---- step k on the main stream: the off-band TRSM (whole GPU),
-        // column k + 1, signal, then the rest
+        // column k + 1 and the corner, signal, then the rest
         e = cudaStreamWaitEvent(s, FMT == 3 ? ev_diag : ev_panel, 0);
         if (FMT == 3) {
             // X = A W^T on the tensor cores with W = L_kk^-1 from the chain
@@ -554,18 +559,18 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
         if (e == cudaSuccess && FMT == 3) e = cudaStreamWaitEvent(s, ev_panel, 0);
         // FP32 mode: band outputs with an FP32 operand by exact slices
         if (e == cudaSuccess && FMT == 3)
-            e = launch_band_out_ozaki(moz[k & 1][0], moz[k & 1][1], tl, mb.xband, k, k + 1, 1, ozs, mb.err, s, kt);
+            e = launch_band_ozaki(moz[k & 1][0], moz[k & 1][1], tl, mb.xband, k, order::kColumn, ozs, mb.err, s, kt);
         // FP32 mode: the off-band update in split FP16 (fmt 4) from the scaled rows
         const int ufmt = FMT == 3 ? 4 : FMT;
         const float *urs = FMT == 3 ? mb.rs[k & 1] : nullptr;
         if (e == cudaSuccess)
-            e = launch_update_tc(ma[k & 1], mbm[k & 1], mc, ufmt, tl, k, mb.err, s, kt, 1, urs, mb.xband);
+            e = launch_update_tc(ma[k & 1], mbm[k & 1], mc, ufmt, tl, k, mb.err, s, kt, order::kColumn, urs,
+                                 mb.xband);
         if (e == cudaSuccess) e = cudaEventRecord(ev_col, s);
         if (e == cudaSuccess && FMT == 3)
-            e = launch_band_out_ozaki(moz[k & 1][0], moz[k & 1][1], tl, mb.xband, k, k + 2, T - k - 2, ozs, mb.err, s,
-                                      kt);
+            e = launch_band_ozaki(moz[k & 1][0], moz[k & 1][1], tl, mb.xband, k, order::kRest, ozs, mb.err, s, kt);
         if (e == cudaSuccess)
-            e = launch_update_tc(ma[k & 1], mbm[k & 1], mc, ufmt, tl, k, mb.err, s, kt, 2, urs, mb.xband);
+            e = launch_update_tc(ma[k & 1], mbm[k & 1], mc, ufmt, tl, k, mb.err, s, kt, order::kRest, urs, mb.xband);
     }
     if (kt) kt->step = -1;
     if (e == cudaSuccess) e = cudaEventRecord(ev_panel, side);

@@ -42,6 +42,7 @@
 // warps 2-5 read the accumulators with tcgen05.ld and apply the FP64
 // epilogue.
 #include "egs_internal.cuh"
+#include "mixed_order.cuh"
 #include "slices.cuh"
 #include "tc_common.cuh"
 
@@ -105,25 +106,19 @@ struct OzItem {
     int ya, yb;  // operand rows (within one slice) of the A and B boxes
 };
 
-// FP64-accurate outputs of step k not covered by the FP64 band x band
-// update: tiles (m, n), n = col0 .. col0 + ncols - 1, m = n .. n + xband - 1
-// < T, with m - k >= band (an FP32 panel operand).  C_mn -= P_m P_n^T in
-// FP64; tiles with m - n >= band are FP32 and take the FP64 result rounded
-// once.  With band_band set, the items are instead the band x band update
-// itself (m - k < band: both operands FP64 band tiles).
+// FP64-accurate outputs of step k (part: mixed_order.cuh): the band x band update, or the tiles
+// within xband of the diagonal with an FP32 panel operand.  C_mn -= P_m P_n^T in FP64; tiles
+// with m - n >= band are FP32 and take the FP64 result rounded once.
 struct OzBandWork {
     Tiles tl;
-    int k, col0, xband, band_band;
+    int k, part, xband;
     __device__ bool decode(int64_t item, OzItem &w) const
     {
         const int nrb = tl.b / OBM, ncb = tl.b / OBN, per = nrb * ncb;
-        const int64_t t = item / per;
         const int blk = (int)(item % per);
-        w.n = col0 + (int)(t / xband);
-        w.m = w.n + (int)(t % xband);
+        if (!order::band_tile(part, k, tl.band, xband, tl.T, item / per, w.m, w.n)) return false;
         w.rb = blk / ncb;
         w.cb = blk % ncb;
-        if (w.m >= tl.T || (w.m - k < tl.band) != (band_band != 0)) return false;
         if (w.m == w.n && w.cb * OBN > w.rb * OBM + OBM - 1) return false;  // strictly above the diagonal
         w.ya = (w.m - k - 1) * tl.b + w.rb * OBM;
         w.yb = (w.n - k - 1) * tl.b + w.cb * OBN;
@@ -418,30 +413,15 @@ cudaError_t make_ozaki_maps(const void *oz, int b, int T, CUtensorMap *mapA, CUt
     return e;
 }
 
-cudaError_t launch_band_out_ozaki(const CUtensorMap &mapA, const CUtensorMap &mapB, const Tiles &tl, int xband, int k,
-                                  int col0, int ncols, const double *scale, int *err, cudaStream_t s, KernelTimer *kt)
+cudaError_t launch_band_ozaki(const CUtensorMap &mapA, const CUtensorMap &mapB, const Tiles &tl, int xband, int k,
+                              int part, const double *scale, int *err, cudaStream_t s, KernelTimer *kt)
 {
-    if (ncols <= 0) return cudaSuccess;
     if (xband < tl.band) xband = tl.band;
     const int64_t per = (int64_t)(tl.b / OBM) * (tl.b / OBN);
-    const int64_t items = (int64_t)ncols * xband * per;
+    const int64_t items = order::band_tiles_of(part, k, tl.band, xband, tl.T) * per;
+    if (items <= 0) return cudaSuccess;
     const int R = (tl.T - 1) * tl.b;
-    OzBandWork w{tl, k, col0, xband, 0};
-    cudaError_t e;
-    if (kt) kt->begin(KC_UPDATE64, s);
-    e = launch_ozaki(mapA, mapB, w, scale, scale, R, R, items, tl.b / OKC, err, s);
-    if (kt) kt->end(KC_UPDATE64, s);
-    return e;
-}
-
-cudaError_t launch_band_band_ozaki(const CUtensorMap &mapA, const CUtensorMap &mapB, const Tiles &tl, int k, int nb,
-                                   const double *scale, int *err, cudaStream_t s, KernelTimer *kt)
-{
-    if (nb <= 0) return cudaSuccess;
-    const int64_t per = (int64_t)(tl.b / OBM) * (tl.b / OBN);
-    const int64_t items = (int64_t)nb * nb * per;
-    const int R = (tl.T - 1) * tl.b;
-    OzBandWork w{tl, k, k + 1, nb, 1};
+    OzBandWork w{tl, k, part, xband};
     cudaError_t e;
     if (kt) kt->begin(KC_UPDATE64, s);
     e = launch_ozaki(mapA, mapB, w, scale, scale, R, R, items, tl.b / OKC, err, s);

@@ -14,6 +14,7 @@
 // FP32 tiles, by a read-modify-write in FP64 for band tiles.  No cluster
 // multicast is used.
 #include "egs_internal.cuh"
+#include "mixed_order.cuh"
 #include "tc_common.cuh"
 
 #include <cudaTypedefs.h>
@@ -59,9 +60,9 @@ struct WorkItem {
 };
 
 // Trailing update of step k over the lower-tile storage: the output tiles
-// (m, n) with m >= n >= col0 (one_col: only n = col0).  Panel tile m of
+// (m, n) of one part of it (mixed_order.cuh).  Panel tile m of
 // step k is operand row block m - k - 1.  skip_band: leave every band output
-// (m - n < band) to the FP64 kernels (split-TF32 mode).
+// (m - n < band) to the FP64 kernels (FP32 mode).
 //
 // Tiles are visited by blocks of kColBlock columns: for each block, its
 // triangle (rows inside the block) then every lower row, kColBlock tiles per
@@ -74,8 +75,7 @@ constexpr int kColBlock = 16;
 struct UpdateWork {
     Tiles tl;
     int k;
-    int col0;
-    int one_col;
+    int part;
     int skip_band;
     const float *rs;  // split FP16: the power-of-two scale of every panel row
     int xband;        // skip_band: outputs with m - n < xband are done by the FP64-accurate kernels
@@ -85,13 +85,14 @@ struct UpdateWork {
         const int nrb = tl.b / BM, ncb = tl.b / BN, per = nrb * ncb;
         int64_t t = bid / per;
         const int blk = (int)(bid % per);
-        if (one_col) {
-            w.m = col0 + (int)t;
-            w.n = col0;
+        if (part == order::kColumn) {
+            w.m = k + 1 + (int)t;
+            w.n = k + 1;
+            if (w.m >= tl.T) order::update_corner(k, tl.band, tl.T, t, w.m, w.n);
         } else {
             // column block c_lo .. c_lo + wd - 1: wd (wd + 1) / 2 triangle tiles,
             // then (T - c_lo - wd) rows of wd tiles
-            int c_lo = col0;
+            int c_lo = k + 2;
             while (true) {
                 const int wd = min(kColBlock, tl.T - c_lo);
                 if (wd <= 0) return false;  // past the last tile (not reached for valid items)
@@ -117,8 +118,7 @@ struct UpdateWork {
         }
         w.rb = blk / ncb;
         w.cb = blk % ncb;
-        if (w.m - k < tl.band && w.n - k < tl.band) return false;         // FP64 band x band: done in FP64
-        if (skip_band && w.m - w.n < xband) return false;                // FP64-accurate output: done elsewhere
+        if (!order::update_tile(part, k, tl.band, w.m, w.n, skip_band, xband)) return false;
         if (w.m == w.n && w.cb * BN > w.rb * BM + BM - 1) return false;  // strictly above the diagonal
         w.ya = (w.m - k - 1) * tl.b + w.rb * BM;
         w.yb = (w.n - k - 1) * tl.b + w.cb * BN;
@@ -646,25 +646,15 @@ cudaError_t launch_update_tc(const CUtensorMap &mapA, const CUtensorMap &mapB, c
                              const Tiles &tl, int k, int *err, cudaStream_t s, KernelTimer *kt, int part,
                              const float *rs, int xband)
 {
-    // part 0: every trailing tile; 1: column k + 1 only; 2: columns k + 2 .. T - 1
-    const int64_t r = tl.T - k - 1;
-    int64_t ntiles = 0;
-    UpdateWork w{tl, k, k + 1, 0, fmt >= 3 ? 1 : 0, rs, xband > tl.band ? xband : tl.band};
-    if (part == 0) ntiles = r * (r + 1) / 2;
-    else if (part == 1) {
-        ntiles = r;
-        w.one_col = 1;
-    } else {
-        ntiles = (r - 1) * r / 2;
-        w.col0 = k + 2;
-    }
+    const UpdateWork w{tl, k, part, fmt >= 3 ? 1 : 0, rs, xband > tl.band ? xband : tl.band};
+    const int64_t ntiles = order::update_tiles_of(part, k, tl.band, w.skip_band, tl.T);
     if (ntiles <= 0) return cudaSuccess;
     const int64_t blocks = ntiles * (tl.b / BM) * (tl.b / BN);
     // split TF32 / FP16 (fmt 3 / 4): three products per K slice of the [hi | lo] rows
     const int kchunks = tl.b / ((fmt == 1 || fmt == 4) ? 64 : 32);
     cudaError_t e;
     if (kt) kt->begin(KC_UPDATE, s);
-    const int reserve = (part != 2) ? 0 : (blocks >= kLongBulkItems ? kReserveSmsLong : kReserveSms);
+    const int reserve = part != order::kRest ? 0 : (blocks >= kLongBulkItems ? kReserveSmsLong : kReserveSms);
     if (fmt == 4) e = launch_gemm<4>(mapA, mapB, mapC, w, blocks, kchunks, err, s, reserve);
     else if (fmt == 3) e = launch_gemm<3>(mapA, mapB, mapC, w, blocks, kchunks, err, s, reserve);
     else if (fmt == 2) e = launch_gemm<2>(mapA, mapB, mapC, w, blocks, kchunks, err, s, reserve);
