@@ -225,7 +225,9 @@ egs_status egs_matern_tiles(const double *locs, int64_t n, const double theta[3]
  * egs_potrf_tiles - tile Cholesky Sigma = L L^T in place (Algorithm 2,
  * dpotrf; the right-looking tile algorithm of Section 5.2: POTRF on the
  * diagonal tile, TRSM on the panel, SYRK/GEMM on the trailing tiles).
- *   tiles       device, lower tiles of Sigma in EGS_FP64 layout; on return L
+ *   tiles       device, lower tiles of Sigma in EGS_FP64 layout; on return L.
+ *               Above 2048 rows the tensor-core update needs a 16-byte
+ *               boundary; tiles without it take the slower FP64-pipe update
  *   fail_index  host; first failing row or -1.  The call synchronises stream.
  * EGS_ERR_ARG if tiles is not device memory.
  */

@@ -486,7 +486,7 @@ egs_status egs_potrf_tiles(void *tiles, int64_t n, int32_t tile, int64_t *fail_i
     const size_t sbytes = align256(sizeof(DevStatus));
     const Allocator A = current_allocator();
     const size_t cbytes = align256(sbytes + 2 * kWinvDoubles * sizeof(double));
-    bool tc = tc64_applies(n, tile, g.T);
+    bool tc = tc64_applies(n, tile, g.T) && tc64_aligned(tiles);
     size_t wbytes = cbytes + (tc ? tc64_scratch_bytes(g.b, g.T) : 0);
     cudaError_t e = dev_alloc(A, (void **)&st, wbytes, s);
     if (e == cudaErrorMemoryAllocation && tc && !A.alloc) {  // no room for the slices: the DFMA update
@@ -566,7 +566,7 @@ egs_status egs_loglik_ex(const double *locs, const double *z, const double theta
     cudaError_t e = cudaSuccess;
     const Allocator A = current_allocator();
     if (opts && opts->workspace) {
-        if (opts->workspace_bytes < es.need) eval_shrink(&es);
+        if (opts->workspace_bytes < es.need || !tc64_aligned(opts->workspace)) eval_shrink(&es);
         if (opts->workspace_bytes < es.need)
             return set_error(EGS_ERR_ARG, "workspace of %zu bytes < %zu needed", opts->workspace_bytes, es.need);
         ws = (char *)opts->workspace;

@@ -210,7 +210,9 @@ __global__ void __launch_bounds__(8 * RB) k_solve64(const __grid_constant__ F64S
     for (int r = tid >> 5; r < RB; r += NT / 32) {
         const size_t sr = P.inner.row0 + pr0 + r;
         const double x0 = sm.Xs[r][2 * lane], x1 = sm.Xs[r][2 * lane + 1];
-        *reinterpret_cast<double2 *>(X + (size_t)r * b + 2 * lane) = make_double2(x0, x1);
+        // two 8-byte stores: a caller's tiles may start at any double
+        X[(size_t)r * b + lane] = sm.Xs[r][lane];
+        X[(size_t)r * b + 32 + lane] = sm.Xs[r][32 + lane];
         if (P.inner.sl) slice7_row64(x0, x1, P.inner.sl + sr * PW, P.inner.rows * PW, P.inner.ex + sr);
         if (P.z) {
             const double v = dot64(x0, x1, y0, y1);

@@ -13,6 +13,9 @@ constexpr int kF64Panel = 64;  // width of the blocks a tile column is factored 
 // persistent batch, which runs the DFMA routines, stays bit for bit equal to a single evaluation;
 // above it the updates do (n = 5,000: 36.4 ms by DFMA, 2.5 here).
 constexpr int64_t kTc64MinRows = 2049;
+// They also need memory that starts on a 16-byte boundary (tc64_aligned: TMA boxes, pairs of doubles
+// in the update's epilogue); a caller's tiles or workspace without that take the DFMA update.
+inline bool tc64_aligned(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 inline bool tc64_applies(int64_t n, int b, int T) { return n >= kTc64MinRows && T > 1 && b % 64 == 0; }
 
 // Slices of operand rows (slice i of row r at sl[(i rows + r) K ..], K = b or 64) and the
