@@ -502,7 +502,8 @@ egs_status egs_potrf_tiles(void *tiles, int64_t n, int32_t tile, int64_t *fail_i
     DevStatus h;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s);
     dev_free(A, st, wbytes, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    const cudaError_t sync = cudaStreamSynchronize(s);  // after an error too: the tiles are the caller's
+    if (e == cudaSuccess) e = sync;
     if (e != cudaSuccess) return cuda_error(e, "egs_potrf_tiles");
     if (h.timeout) return set_error(EGS_ERR_TIMEOUT, "egs_potrf_tiles: a bounded device wait timed out");
     const int64_t fi = (h.fail_index == kNoFail) ? -1 : (int64_t)h.fail_index;
@@ -597,7 +598,8 @@ egs_status egs_loglik_ex(const double *locs, const double *z, const double theta
     if (e == cudaSuccess && es.mixed) e = cudaMemcpyAsync(&herr, ws + es.ML.err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, eval_status(es, ws), sizeof(h), cudaMemcpyDeviceToHost, s);
     if (own) dev_free(A, ws, es.need, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    const cudaError_t sync = cudaStreamSynchronize(s);  // after an error too: the workspace may be the caller's
+    if (e == cudaSuccess) e = sync;
     float ms[3] = {0, 0, 0};
     if (timing) {
         if (e == cudaSuccess)

@@ -94,7 +94,7 @@ cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *
         F64Maps maps;
         e = make_f64_maps(set.one.panel, set.one.inner, g.b, &maps);
         F64Fork fork;
-        if (e == cudaSuccess) e = fork.create(false);
+        if (e == cudaSuccess) e = fork.create(s, false);
         if (e == cudaSuccess)
             e = cudaMemsetAsync(set.one.ctr, 0, tc64_counters(g.b, T) * sizeof(unsigned long long), s);
         for (int k = 0; k < T && e == cudaSuccess; ++k) {

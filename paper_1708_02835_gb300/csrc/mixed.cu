@@ -450,29 +450,28 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
 {
     const Tiles &tl = mb.tl;
     const int T = tl.T, b = tl.b;
-    cudaStream_t side = nullptr;
     cudaEvent_t ev_panel = nullptr, ev_col = nullptr, ev_diag = nullptr;
     // The chain gates the next step, so its kernels take the SMs that the
     // main stream's kernels free first: the side stream runs at the highest
     // priority (otherwise each step's POTRF waits for the whole slice-product
     // launch ahead of it to drain).
-    int prio_least = 0, prio_greatest = 0;
-    cudaError_t e = cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, prio_greatest);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_panel, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_col, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_diag, cudaEventDisableTiming);
+    SideStream chain;
+    cudaError_t e = chain.create(s, true);
+    cudaStream_t side = chain.st;
+    for (cudaEvent_t *ev : {&ev_panel, &ev_col, &ev_diag})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     // POTRF of a diagonal tile and its inverse V_k = L_kk^-T: the FP64 path's 64-column blocks on
     // that tile alone with V_k's rows below it; the band rows by multiplication with W = V_k^T on
     // the tensor cores (tc64.cu).  Tile 512: 1.05 ms of POTRF, 0.32 of inversion and 0.22 of band
     // solve as task graph, column and row substitutions; 0.85 and 0.05 ms so
     const F64Set diag{nullptr, tc64_solo_problem(mb.dpan, tl, st, mb.vinv, band_tiles(tl)), 1, b, T, 1};
     F64Maps dmaps;
-    F64Fork fork;
-    if (e == cudaSuccess) e = fork.create(true);
+    F64Fork fork;  // joined to the chain's stream, which is joined to s
+    if (e == cudaSuccess) e = fork.create(side, true);
     if (e == cudaSuccess) e = make_f64_solo_maps(diag.one, &dmaps);
     if (e == cudaSuccess) e = launch_solo_init(diag, s, kt);
     if (e == cudaSuccess) e = cudaEventRecord(ev_col, s);  // the side stream starts after prior work on s
+    chain.open = e == cudaSuccess;
     KernelTimer *kts = kt;  // side-stream kernels are timed with events on the side stream
     for (int k = 0; k < T && e == cudaSuccess; ++k) {
         if (kt) kt->step = k;
@@ -573,15 +572,11 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
             e = launch_update_tc(ma[k & 1], mbm[k & 1], mc, ufmt, tl, k, mb.err, s, kt, order::kRest, urs, mb.xband);
     }
     if (kt) kt->step = -1;
-    if (e == cudaSuccess) e = cudaEventRecord(ev_panel, side);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev_panel, 0);  // join the side stream
-    // destroying a stream or event with work still pending is legal: the
-    // resources are released once that work completes, and s already waits
-    // for it through ev_panel
-    if (side) cudaStreamDestroy(side);
-    if (ev_panel) cudaEventDestroy(ev_panel);
-    if (ev_col) cudaEventDestroy(ev_col);
-    if (ev_diag) cudaEventDestroy(ev_diag);
+    // on any way out: the fork's stream first, then the chain's
+    const cudaError_t ej = fork.aux.join(), ec = chain.join();
+    if (e == cudaSuccess) e = ej != cudaSuccess ? ej : ec;
+    for (cudaEvent_t ev : {ev_panel, ev_col, ev_diag})
+        if (ev) cudaEventDestroy(ev);
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

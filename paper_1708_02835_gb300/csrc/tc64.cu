@@ -876,21 +876,17 @@ cudaError_t launch_diag_solve64(const F64Set &set, int k, int j, cudaStream_t s,
     return e == cudaSuccess ? launch_solve64(set, k, j, 0, false, s, kt) : e;
 }
 
-cudaError_t F64Fork::create(bool high_priority)
+cudaError_t F64Fork::create(cudaStream_t s, bool high_priority)
 {
-    int least = 0, greatest = 0;
-    cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&aux, cudaStreamNonBlocking, high_priority ? greatest : least);
-    for (cudaEvent_t *ev : {&diag, &next, &bulk})
+    cudaError_t e = aux.create(s, high_priority);
+    for (cudaEvent_t *ev : {&diag, &next})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     return e;
 }
 
-// Streams and events with work pending are released once it completes.
 F64Fork::~F64Fork()
 {
-    if (aux) cudaStreamDestroy(aux);
-    for (cudaEvent_t ev : {diag, next, bulk})
+    for (cudaEvent_t ev : {diag, next})
         if (ev) cudaEventDestroy(ev);
 }
 
@@ -911,8 +907,9 @@ cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, F64For
 {
     const int nj = set.b / PW;
     if (kt && kt->on) fork = nullptr;  // per-launch times and traces: one stream, launches in order
-    cudaStream_t bs = fork ? fork->aux : s;
+    cudaStream_t bs = fork ? fork->aux.st : s;
     cudaError_t e = cudaSuccess;
+    if (fork) fork->aux.open = true;  // until s waits for it below; otherwise its owner does at the end
     for (int j = 0; j < nj && e == cudaSuccess; ++j) {
         const bool more = j + 1 < nj;
         e = launch_diag64(set, k, j, s, kt);
@@ -923,7 +920,7 @@ cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, F64For
             if (e == cudaSuccess) e = cudaStreamWaitEvent(bs, fork->diag, 0);
             if (e == cudaSuccess && more) {
                 // the next block's rows carry block j - 1's update of column j
-                if (j > 0) e = cudaStreamWaitEvent(s, fork->bulk, 0);
+                if (j > 0) e = cudaStreamWaitEvent(s, fork->aux.done, 0);
                 if (e == cudaSuccess) e = launch_solve64(set, k, j, 0, true, s, kt);
                 if (e == cudaSuccess) e = cudaEventRecord(fork->next, s);
             }
@@ -938,9 +935,10 @@ cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, F64For
             if (e == cudaSuccess)
                 e = launch_tc_f64(maps.ia, maps.ib, set, k, j + 1, nj, F64_INNER, k * (2 + nj) + 2 + j, 0, bs, kt);
         }
-        if (fork && e == cudaSuccess) e = cudaEventRecord(fork->bulk, bs);
+        if (fork && e == cudaSuccess) e = cudaEventRecord(fork->aux.done, bs);
     }
-    if (fork && e == cudaSuccess) e = cudaStreamWaitEvent(s, fork->bulk, 0);
+    if (fork && e == cudaSuccess) e = cudaStreamWaitEvent(s, fork->aux.done, 0);
+    if (fork && e == cudaSuccess) fork->aux.open = false;
     return e;
 }
 

@@ -2,6 +2,7 @@
 #pragma once
 #include "blocks.cuh"
 #include "egs_internal.cuh"
+#include "side_stream.cuh"
 
 namespace egs {
 
@@ -83,11 +84,11 @@ F64Prob dfma_problem(double *winv, const Tiles &tl, DevStatus *st, double *z);
 // Diagonal block j of step k; the solves of the rows below it (launch_panel64's first two parts).
 cudaError_t launch_diag_solve64(const F64Set &set, int k, int j, cudaStream_t s, KernelTimer *kt);
 
-// A second stream for the panels of one factorisation.
+// A second stream for the panels of one factorisation on stream s.
 struct F64Fork {
-    cudaStream_t aux = nullptr;
-    cudaEvent_t diag = nullptr, next = nullptr, bulk = nullptr;
-    cudaError_t create(bool high_priority);
+    SideStream aux;  // aux.done: the panel's bulk
+    cudaEvent_t diag = nullptr, next = nullptr;
+    cudaError_t create(cudaStream_t s, bool high_priority);
     ~F64Fork();
 };
 
