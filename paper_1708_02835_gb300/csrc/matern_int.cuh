@@ -186,7 +186,8 @@ EGS_HD bool matern_int(const egs_matern_params *P, const int64_t *itab, double q
     int ey = k + P->iy_e;
     if (Y >> 63) ++ey;
     else Y <<= 1;
-    if (ey > 8 || ey < (P->kind == EGS_MATERN_GENERAL ? EGS_MT_E0 : -60)) return false;
+    const bool general = P->kind == EGS_MATERN_GENERAL;
+    if (ey > (general ? EGS_MT_E0 + EGS_MT_OCT - 1 : 8) || ey < (general ? EGS_MT_E0 : -60)) return false;
     // theta1 e^-x = Er 2^(th1_e - n - 63)
     const uint64_t Z = mulhi_exact(Y, 0xE6D4C9F3B31DECEBull);  // 1.25 / ln 2 in units of 2^-63
     const int sh = ey + 2;
