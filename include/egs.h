@@ -439,7 +439,10 @@ egs_status egs_loglik_ind(const double *locs, const double *z, const double thet
  *                       if the request's workspace does not fit in the budget
  *                       beside the resident fields even with nothing else in
  *                       flight (it is failed at the head of the queue instead
- *                       of blocking it).  A ticket is
+ *                       of blocking it), or cannot be allocated within 2 s of
+ *                       nothing being in flight.  An FP64 request that does
+ *                       not fit with the tensor-core update's scratch takes
+ *                       the FP64 pipe's update.  A ticket is
  *                       consumed by the successful or failed wait that
  *                       returns its result.
  *   egs_serve_stats     p50 / p99 / mean latency, throughput, counters.

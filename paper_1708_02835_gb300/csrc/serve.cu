@@ -83,6 +83,8 @@ struct egs_server {
     int inflight = 0, inflight_peak = 0;
     clk::time_point first_submit{}, last_done{};
     bool any_submit = false;
+    int64_t starved = 0;  // ticket at the head whose workspace could not be allocated
+    clk::time_point starved_since{};
 };
 
 namespace {
@@ -154,6 +156,21 @@ void finish_slot(egs_server *S, Slot &sl)
     release_slot(S, sl);
 }
 
+// The head of the queue is answered without a run (S->mu held).
+void reject_head(egs_server *S, egs_status status)
+{
+    Result &r = S->results[S->queue.front().ticket];
+    r.done = true;
+    r.status = status;
+    r.loglik = NAN;
+    ++S->rejected;
+    S->queue.pop_front();
+    S->cv_done.notify_all();
+}
+
+// How long a request whose workspace cannot be allocated with nothing in flight is tried again.
+constexpr std::chrono::seconds kAllocPatience{2};
+
 bool admit_one(egs_server *S, std::unique_lock<std::mutex> &lk)
 {
     // called with S->mu held; admits the head of the queue if possible.  The
@@ -174,13 +191,7 @@ bool admit_one(egs_server *S, std::unique_lock<std::mutex> &lk)
     if (rq.p == EGS_MIX_FP32 && S->cfg.xband > S->cfg.band) o.xband = S->cfg.xband;
     egs::EvalSetup es;
     if (egs::eval_setup(f.n, rq.theta, rq.p, &o, &es) != EGS_OK) {
-        Result &r = S->results[rq.ticket];
-        r.done = true;
-        r.status = EGS_ERR_ARG;
-        r.loglik = NAN;
-        ++S->rejected;
-        S->queue.pop_front();
-        S->cv_done.notify_all();
+        reject_head(S, EGS_ERR_ARG);
         return true;
     }
     if (S->used + es.need > S->cfg.hbm_budget_bytes && S->inflight == 0) egs::eval_shrink(&es);
@@ -188,21 +199,27 @@ bool admit_one(egs_server *S, std::unique_lock<std::mutex> &lk)
         if (S->inflight > 0) return false;  // wait for memory to free up
         // nothing in flight: only resident fields hold the budget, so this
         // request can never be admitted; fail it rather than block the queue
-        Result &r = S->results[rq.ticket];
-        r.done = true;
-        r.status = EGS_ERR_OOM;
-        r.loglik = NAN;
-        ++S->rejected;
-        S->queue.pop_front();
-        S->cv_done.notify_all();
+        reject_head(S, EGS_ERR_OOM);
         return true;
     }
     Slot &sl = *free_slot;
     char *ws = nullptr;
     cudaError_t e = egs::dev_alloc(S->alloc, (void **)&ws, es.need, sl.stream);
+    if (e != cudaSuccess && S->inflight == 0 && egs::eval_shrink(&es)) {
+        cudaGetLastError();
+        e = egs::dev_alloc(S->alloc, (void **)&ws, es.need, sl.stream);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        if (S->inflight > 0) return false;  // memory comes back when those end
+        // nothing of this server's gives memory back; others' may, for a while
+        if (S->starved != rq.ticket) {
+            S->starved = rq.ticket;
+            S->starved_since = clk::now();
+        }
+        if (clk::now() - S->starved_since < kAllocPatience) return false;
+        reject_head(S, EGS_ERR_OOM);
+        return true;
     }
     sl.busy = true;
     sl.req = rq;
@@ -359,8 +376,8 @@ egs_status egs_serve_wait(egs_server *S, int64_t ticket, int32_t timeout_ms, dou
     if (out_loglik) *out_loglik = r.loglik;
     if (info) *info = r.info;
     if (r.status == EGS_ERR_OOM)
-        return set_error(r.status, "egs_serve_wait: request %lld needs more workspace than the budget leaves beside "
-                                   "the resident fields",
+        return set_error(r.status, "egs_serve_wait: request %lld needs more workspace than the budget, or the device, "
+                                   "leaves beside the resident fields",
                          (long long)ticket);
     if (r.status != EGS_OK) return set_error(r.status, "egs_serve_wait: request %lld failed", (long long)ticket);
     return EGS_OK;
