@@ -173,7 +173,9 @@ egs_status egs_trace_last(egs_trace_rec *out, int64_t cap, int64_t *count);
  *                               must not hand it out to another stream
  *                               before that work has finished
  * Both NULL restores the library's pool; one NULL is
- * EGS_ERR_ARG.  Memory is always returned to the allocator that provided it,
+ * EGS_ERR_ARG.  Every call also returns what the pool holds unused to the
+ * system (as egs_serve_destroy does, and the library by itself when an
+ * allocation from the pool fails).  Memory is always returned to the allocator that provided it,
  * also when the allocator is replaced in the meantime.  The library may call
  * the hooks from its serving thread, with its internal locks held: a hook
  * must not call back into the library.  A server or batch keeps the
@@ -422,7 +424,8 @@ egs_status egs_loglik_ind(const double *locs, const double *z, const double thet
  * resident.  Requests (field, theta, precision) enter a FIFO queue; a
  * scheduler thread admits the head request as soon as an execution slot is
  * free and its workspace fits in the HBM budget (resident fields plus
- * workspaces in flight <= hbm_budget_bytes), and enqueues it on the slot's own
+ * workspaces in flight <= hbm_budget_bytes; what the library's pool keeps
+ * unused, at most 4 GiB, is not part of it), and enqueues it on the slot's own
  * stream, so requests that arrive while others run overlap with them on the
  * GPU.  Each evaluation is exactly egs_loglik's (deterministic kernels), so a
  * result is the same alone and in the mix.  Latency is measured from submit

@@ -140,6 +140,8 @@ struct Allocator {
 Allocator current_allocator();
 cudaError_t dev_alloc(const Allocator &A, void **p, size_t bytes, cudaStream_t s);
 void dev_free(const Allocator &A, void *p, size_t bytes, cudaStream_t s);
+// What the pool holds unused goes back to the system.
+void dev_trim();
 
 // True for device (or managed) memory; host pointers are staged by the calls.
 bool is_device_ptr(const void *p);

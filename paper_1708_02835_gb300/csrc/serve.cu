@@ -438,6 +438,7 @@ egs_status egs_serve_destroy(egs_server *S)
         field_free(S->alloc, f.z, (size_t)f.n * sizeof(double));
     }
     delete S;
+    egs::dev_trim();
     return EGS_OK;
 }
 
