@@ -309,19 +309,19 @@ egs_status egs_loglik_ex(const double *locs, const double *z, const double theta
  * Batched evaluation (independent problems: uneven n, own theta each).
  *
  * Each problem is Eq. 1 evaluated by Algorithm 2 exactly as egs_loglik does
- * in EGS_FP64.  An EGS_FP64 batch with a problem of more than 2048 rows runs
- * as step-synchronous launches on the tensor cores, each covering one step of
- * every problem.  Other EGS_FP64 batches with tile <= 256 run as ONE persistent
- * kernel launch: the tile tasks of every problem (Matern tiles, the POTRF /
+ * in EGS_FP64.  In an EGS_FP64 batch with tile <= 256 every l is bitwise
+ * equal to egs_loglik_ex's with the same tile, whatever the other problems:
+ * those of more than 2048 rows run as step-synchronous launches on the tensor
+ * cores, each covering one step of every such problem, and the others as ONE
+ * persistent kernel launch: their tile tasks (Matern tiles, the POTRF /
  * TRSM / SYRK-GEMM tasks of the tile Cholesky of Section 5.2 -- the DAG of
  * its tile algorithm -- and the forward-solve tasks) form one list in a
  * dependency order checked when the plan is made, and each CTA claims the
  * next task and waits on per-tile device counters until its inputs are final
- * (every wait bounded: EGS_ERR_TIMEOUT if one runs out).  Every l is then bitwise
- * equal to egs_loglik_ex's with the same tile.  Other batches (EGS_MIX_FP32,
- * or tiles above 256) run as step-synchronous launches, each covering one
- * step of every problem.  Either way the run is captured into a CUDA graph on
- * the first egs_batch_run and replayed afterwards.
+ * (every wait bounded: EGS_ERR_TIMEOUT if one runs out).  Other batches
+ * (EGS_MIX_FP32, or tiles above 256) run as step-synchronous launches, each
+ * covering one step of every problem.  Either way the run is captured into a
+ * CUDA graph on the first egs_batch_run and replayed afterwards.
  *
  * egs_batch_create  plan for nprob problems of sizes n[0..nprob) with one tile
  *                   size for the batch (0 = the tile egs_batch_autotune found

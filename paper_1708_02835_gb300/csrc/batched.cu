@@ -465,16 +465,17 @@ struct egs_batch {
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     int launches_per_run = 0;
-    // tensor-core batch: step-synchronous launches of the FP64 tensor-core factorisation over
-    // all problems (by falling T, so that the ones with a step k are the first active[k])
+    // problems on the tensor cores: step-synchronous launches of the FP64 factorisation over
+    // them (by falling T, so that the ones with a step k are the first active[k])
     bool tc = false;
+    std::vector<char> big;  // which ones
     F64Prob *d_f64 = nullptr;
     F64Maps maps;
     std::vector<int> active;
     unsigned long long *d_f64ctr = nullptr;
     size_t f64ctr = 0;
-    // persistent scheduler (other FP64 batches with tile <= 256): one launch over
-    // the task list of every problem
+    // persistent scheduler (the other problems of FP64 batches with tile <= 256): one launch
+    // over the task list of all of them
     bool dag = false;
     int4 *d_tasks = nullptr;
     long long ntasks = 0;
@@ -534,14 +535,17 @@ void plan_launches(egs_batch *B, std::vector<int64_t> &prefix)
     auto band_of = [&](int q) { return B->mixed ? std::min(kBatchBand, B->T[q]) : B->T[q]; };
     auto nb_of = [&](int q, int k) { return (int64_t)std::min(band_of(q) - 1, B->T[q] - k - 1); };
     auto vec_items = [&](int q) { return ((int64_t)B->T[q] * b + 255) / 256; };
-    add(L_GEN, 0, 0, [&](int q) { return (int64_t)B->T[q] * (B->T[q] + 1) / 2 * nsub * nsub; });
+    auto gen_items = [&](int q) { return (int64_t)B->T[q] * (B->T[q] + 1) / 2 * nsub * nsub; };
     if (B->tc) {
-        add(L_PAD, 0, 0, vec_items);
-        add(L_FACTOR64, 0, 0, [&](int) { return (int64_t)1; });
-        add(L_LDQ, 0, 0, [&](int q) { return (int64_t)B->T[q]; });
-        add(L_FINAL, 0, 0, [&](int) { return (int64_t)1; });
+        auto of_big = [&](auto count) { return [=](int q) { return B->big[q] ? (int64_t)count(q) : (int64_t)0; }; };
+        add(L_GEN, 0, 0, of_big(gen_items));
+        add(L_PAD, 0, 0, of_big(vec_items));
+        add(L_FACTOR64, 0, 0, of_big([](int) { return 1; }));
+        add(L_LDQ, 0, 0, of_big([B](int q) { return B->T[q]; }));
+        add(L_FINAL, 0, 0, of_big([](int) { return 1; }));
         return;
     }
+    add(L_GEN, 0, 0, gen_items);
     for (int k = 0; k < Tmax; ++k) {
         for (int p = 0; p < b; p += kIB) {
             const int64_t nrest = (b - p - kIB) / 16, n32 = (b - p - kIB) / 32;
@@ -618,15 +622,15 @@ cudaError_t enqueue_all(egs_batch *B, cudaStream_t s)
 {
     cudaError_t et = launch_batch_tables(B->d_probs, B->ntab, s);
     if (et != cudaSuccess) return et;
+    int count = 1;  // the local polynomials
     if (B->dag) {
         cudaError_t e = cudaMemsetAsync(B->d_cnt, 0, B->ncnt * sizeof(unsigned), s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(B->d_ctl, B->h_ctl, sizeof(DagCtl), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = dag_enqueue(B->d_tasks, B->ntasks, B->d_probs, B->d_ctl, B->b, B->grid, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(B->h_ctl + 1, B->d_ctl, sizeof(DagCtl), cudaMemcpyDeviceToHost, s);
-        B->launches_per_run = 2;  // the local polynomials, then the persistent launch
-        return e;
+        if (e != cudaSuccess) return e;
+        ++count;
     }
-    int count = 1;
     for (const auto &L : B->launches) {
         if (L.items <= 0) continue;
         BatchArgs a{B->d_probs, B->d_prefix + L.prefix_off, B->nprob, B->b};
@@ -666,12 +670,15 @@ cudaError_t enqueue_all(egs_batch *B, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// A batch takes the tensor cores when its largest problem does as a single evaluation, with
-// all its problems (96 problems of 256 to 4,096 rows, tile 128: 607 ms as one persistent
-// launch of DFMA tasks, 76 ms so); without such a problem it stays on the persistent launch,
-// whose results equal single evaluations bit for bit.  any_size (the independent-blocks
-// approximation, whose blocks are no single evaluations): whatever the sizes.  once: the batch
-// lives for one call, its memory comes from the pool.
+// Each problem of an FP64 batch with tile <= 256 takes the route it takes as a single evaluation,
+// so that its l is that evaluation's bit for bit whatever its companions are: those of more than
+// 2,048 rows the tensor cores, step by step with a grid row per problem, the others the persistent
+// launch.  96 problems of 256 to 4,096 rows, 41 of them up to 2,048, tile 128: 607 ms as one
+// persistent launch, 115 ms so; 76 ms with all of them on the tensor cores, where a small problem's
+// last digits would depend on its companions.  Tiles above 256 have no persistent launch: all
+// problems take the tensor cores if one does.  any_size (the independent-blocks approximation, whose
+// blocks are no single evaluations): whatever the sizes.  once: the batch lives for one call, its
+// memory comes from the pool.
 egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_precision p, bool any_size, bool once,
                         egs_batch **out)
 {
@@ -690,9 +697,23 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     B->nprob = B->ntab = nprob;
     B->b = tile;
     B->mixed = (p == EGS_MIX_FP32);
-    if (!B->mixed && nprob <= 65535) {  // a grid row per problem
-        B->tc = any_size;
-        for (int i = 0; i < nprob && !B->tc; ++i) B->tc = tc64_applies(n[i], tile, (int)((n[i] + tile - 1) / tile));
+    B->big.assign((size_t)nprob, 0);
+    if (!B->mixed) {
+        int nbig = 0;
+        for (int i = 0; i < nprob; ++i) {
+            B->big[i] = any_size || tc64_applies(n[i], tile, (int)((n[i] + tile - 1) / tile));
+            nbig += B->big[i];
+        }
+        if (nbig > 0 && tile > 256) {
+            B->big.assign((size_t)nprob, 1);
+            nbig = nprob;
+        }
+        if (nbig > 65535) {  // a grid row per problem
+            B->big.assign((size_t)nprob, 0);
+            nbig = 0;
+        }
+        B->tc = nbig > 0;
+        B->dag = nbig < nprob && tile <= 256;
     }
     size_t off = 0;
     std::vector<size_t> tiles_off(nprob), zpad_off(nprob), part_off(nprob), f32_off(nprob), sig_off(nprob),
@@ -721,7 +742,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
         part_off[i] = off;
         off += a256((size_t)2 * T * sizeof(double));
         winv_offs[i] = off;
-        if (!B->mixed && !B->tc) off += a256((size_t)T * (tile / 64) * kWinvDoubles * sizeof(double));
+        if (!B->mixed && !B->big[i]) off += a256((size_t)T * (tile / 64) * kWinvDoubles * sizeof(double));
         mtab_off[i] = off;
         off += a256(EGS_MT_SCRATCH_DOUBLES * sizeof(double));
         B->in_off.push_back(in_doubles);
@@ -735,15 +756,16 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     off += a256(sizeof(DevStatus) * nprob);
     const size_t inputs_off = off;
     off += a256(in_doubles * sizeof(double));
-    // tensor-core batch: the slices of all problems in two arrays, problem order[i] from row
+    // the slices of the problems on the tensor cores in two arrays, problem order[i] from row
     // prow[i] / irow[i] on
     std::vector<int> order;
     std::vector<size_t> prow, irow, fctr;
     size_t R = 0, R1 = 0;
     if (B->tc) {
-        for (int i = 0; i < nprob; ++i) order.push_back(i);
+        for (int i = 0; i < nprob; ++i)
+            if (B->big[i]) order.push_back(i);
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return B->T[x] > B->T[y]; });
-        for (int i = 0; i < nprob; ++i) {
+        for (size_t i = 0; i < order.size(); ++i) {
             const int T = B->T[order[i]];
             prow.push_back(R);
             irow.push_back(R1);
@@ -753,11 +775,11 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
             B->f64ctr += tc64_counters(tile, T);
         }
         B->active.assign((size_t)B->T[order[0]], 0);
-        for (int i = 0; i < nprob; ++i)
-            for (int k = 0; k < B->T[i]; ++k) ++B->active[k];
+        for (int q : order)
+            for (int k = 0; k < B->T[q]; ++k) ++B->active[k];
     }
     const size_t f64_off = off;
-    if (B->tc) off += a256(sizeof(F64Prob) * nprob);
+    off += a256(sizeof(F64Prob) * order.size());
     const size_t psl_off = off;
     off += a256(R * tile * kF64Slices * sizeof(uint16_t));
     const size_t pex_off = off;
@@ -769,21 +791,22 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     const size_t fctr_off = off;
     off += a256(B->f64ctr * sizeof(unsigned long long));
     const size_t winv_off = off;
-    if (B->tc) off += a256((size_t)nprob * 2 * kWinvDoubles * sizeof(double));
+    off += a256(order.size() * 2 * kWinvDoubles * sizeof(double));
     std::vector<int64_t> prefix;
     std::vector<int4> tasks;
     std::vector<size_t> cnt_off;
-    B->dag = !B->mixed && !B->tc && tile <= 256;
     if (B->dag) {
-        egs_status sc = dag_plan(B->T, tile, tasks, cnt_off, B->ncnt);
+        std::vector<int> T = B->T;  // no tasks for the problems on the tensor cores
+        for (int i = 0; i < nprob; ++i)
+            if (B->big[i]) T[i] = 0;
+        egs_status sc = dag_plan(T, tile, tasks, cnt_off, B->ncnt);
         if (sc != EGS_OK) {
             delete B;
             return sc;
         }
         B->ntasks = (long long)tasks.size();
-    } else {
-        plan_launches(B, prefix);
     }
+    if (B->tc || !B->dag) plan_launches(B, prefix);
     const size_t prefix_off = off;
     off += a256(prefix.size() * sizeof(int64_t));
     const size_t tasks_off = off;
@@ -870,19 +893,19 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     }
     e = cudaMemcpy(B->d_probs, B->h_probs, sizeof(BatchProblem) * nprob, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && B->tc) {
-        std::vector<F64Prob> fp((size_t)nprob);
+        std::vector<F64Prob> fp(order.size());
         B->d_f64 = (F64Prob *)(B->ws + f64_off);
         B->d_f64ctr = (unsigned long long *)(B->ws + fctr_off);
-        for (int i = 0; i < nprob; ++i) {
+        for (size_t i = 0; i < order.size(); ++i) {
             const BatchProblem &pr = B->h_probs[order[i]];
-            F64Prob &P = fp[(size_t)i];
+            F64Prob &P = fp[i];
             P.tl = Tiles{pr.tiles, nullptr, tile, pr.T, pr.T};
             P.st = pr.st;
             P.z = pr.zpad;
             P.panel = F64Rows{(uint16_t *)(B->ws + psl_off), (int *)(B->ws + pex_off), R, prow[i]};
             P.inner = F64Rows{(uint16_t *)(B->ws + isl_off), (int *)(B->ws + iex_off), R1, irow[i]};
             P.ctr = B->d_f64ctr + fctr[i];
-            P.winv = (double *)(B->ws + winv_off) + (size_t)i * 2 * kWinvDoubles;
+            P.winv = (double *)(B->ws + winv_off) + i * 2 * kWinvDoubles;
         }
         e = make_f64_maps(fp[0].panel, fp[0].inner, tile, &B->maps);
         if (e == cudaSuccess) e = cudaMemcpy(B->d_f64, fp.data(), fp.size() * sizeof(F64Prob), cudaMemcpyHostToDevice);
