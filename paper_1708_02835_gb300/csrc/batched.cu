@@ -679,8 +679,10 @@ cudaError_t enqueue_all(egs_batch *B, cudaStream_t s)
 // problems take the tensor cores if one does.  any_size (the independent-blocks approximation, whose
 // blocks are no single evaluations): whatever the sizes.  once: the batch lives for one call, its
 // memory comes from the pool.
+// tensor = false: no problem on the tensor cores, whose slices then need no memory (taken when the
+// plan does not fit otherwise; a caller's allocator is asked once).
 egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_precision p, bool any_size, bool once,
-                        egs_batch **out)
+                        egs_batch **out, bool tensor = true)
 {
     if (!out || !n || nprob < 1) return set_error(EGS_ERR_ARG, "egs_batch_create: bad arguments");
     *out = nullptr;
@@ -700,7 +702,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     B->big.assign((size_t)nprob, 0);
     if (!B->mixed) {
         int nbig = 0;
-        for (int i = 0; i < nprob; ++i) {
+        for (int i = 0; i < nprob && tensor; ++i) {
             B->big[i] = any_size || tc64_applies(n[i], tile, (int)((n[i] + tile - 1) / tile));
             nbig += B->big[i];
         }
@@ -827,8 +829,11 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
         if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     }
     if (e != cudaSuccess) {
+        const bool smaller = e == cudaErrorMemoryAllocation && B->tc && !B->alloc.alloc;
         delete B;
-        return cuda_error(e, "egs_batch_create workspace");
+        if (!smaller) return cuda_error(e, "egs_batch_create workspace");
+        cudaGetLastError();
+        return batch_create(nprob, n, tile, p, any_size, once, out, false);
     }
     B->d_probs = (BatchProblem *)(B->ws + probs_off);
     B->d_params = (egs_matern_params *)(B->ws + params_off);
