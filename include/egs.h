@@ -369,18 +369,21 @@ egs_status egs_batch_autotune(int32_t nprob, const int64_t *n, const double *con
 /* Tile stored by egs_batch_autotune for batches whose largest n is nmax, or 0. */
 int32_t egs_batch_tuned_tile(int64_t nmax, egs_precision p);
 
-/* Tasks in the persistent launch of a batch (0 for a step-synchronous batch). */
+/* Tasks of a batch that a bounded wait depends on: those of the persistent
+ * launch, then one per step of each problem on the tensor cores (its trailing
+ * update).  0 for a batch without either. */
 int64_t egs_batch_tasks(const egs_batch *batch);
 /*
- * egs_batch_set_wait_limit - failure detection of the persistent launch:
- * every dependency wait gives up after limit_ns nanoseconds (default 10 s)
- * and the run returns EGS_ERR_TIMEOUT (all per_status EGS_ERR_TIMEOUT, out
- * NaN) with the batch still usable.  withhold_task in [0, egs_batch_tasks)
- * makes the launch never signal that task's completion, so that the waits
- * on it run out (for tests of this path); -1 signals every task.  Applies to
- * the following runs.  A tensor-core batch has no tasks: it accepts a limit,
- * and its waits keep their own of 2 s.  EGS_ERR_UNIMPLEMENTED for another
- * step-synchronous batch.
+ * egs_batch_set_wait_limit - failure detection of a batch: every dependency
+ * wait of the persistent launch and every pipeline wait of the tensor-core
+ * steps gives up after limit_ns nanoseconds (default 10 s) and the run returns
+ * EGS_ERR_TIMEOUT (all per_status EGS_ERR_TIMEOUT, out NaN) with the batch
+ * still usable.  withhold_task in [0, egs_batch_tasks) makes the launch never
+ * signal that task's completion (of a tensor-core step: of its first output
+ * block), so that the waits on it run out (for tests of this path); -1 signals
+ * every task.  Applies to the following runs.  EGS_ERR_UNIMPLEMENTED for a
+ * batch with neither (EGS_MIX_FP32, or tiles above 256 without a problem of
+ * more than 2048 rows).
  */
 egs_status egs_batch_set_wait_limit(egs_batch *batch, int64_t limit_ns, int64_t withhold_task);
 

@@ -410,12 +410,13 @@ class egs_batch:
 
     @property
     def tasks(self) -> int:
-        """Tasks of the persistent launch (0 for a step-synchronous batch)."""
+        """Tasks that a bounded wait depends on: the persistent launch's, then one per
+        step of each problem on the tensor cores (0 for a batch without either)."""
         return load_library().egs_batch_tasks(self._h)
 
     def set_wait_limit(self, limit_ns: int, withhold_task: int = -1):
-        """Bound of every dependency wait of the persistent launch; a task
-        whose completion is withheld (failure tests), or -1."""
+        """Bound of every wait of the following runs; a task whose completion is
+        withheld (failure tests), or -1."""
         _check(load_library().egs_batch_set_wait_limit(self._h, int(limit_ns), int(withhold_task)))
 
     def run(self, locs, z, thetas, stream=None, raise_on_not_pd=False):

@@ -474,6 +474,9 @@ struct egs_batch {
     std::vector<int> active;
     unsigned long long *d_f64ctr = nullptr;
     size_t f64ctr = 0;
+    std::vector<int> f64T;      // their tiles per side, in that order
+    int64_t f64tasks = 0;       // their trailing updates: T - 1 each
+    F64Ctl *d_f64ctl = nullptr, *h_f64ctl = nullptr;
     // persistent scheduler (the other problems of FP64 batches with tile <= 256): one launch
     // over the task list of all of them
     bool dag = false;
@@ -600,6 +603,7 @@ cudaError_t enqueue_factor64(egs_batch *B, cudaStream_t s, int *count)
 {
     KernelTimer kt;
     cudaError_t e = cudaMemsetAsync(B->d_f64ctr, 0, B->f64ctr * sizeof(unsigned long long), s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(B->d_f64ctl, B->h_f64ctl, sizeof(F64Ctl), cudaMemcpyHostToDevice, s);
     const int Tmax = (int)B->active.size();
     for (int k = 0; k < Tmax && e == cudaSuccess; ++k) {
         F64Set set{};
@@ -607,6 +611,7 @@ cudaError_t enqueue_factor64(egs_batch *B, cudaStream_t s, int *count)
         set.count = B->active[k];
         set.b = B->b;
         set.Tmax = Tmax;
+        set.ctl = B->d_f64ctl;
         e = launch_panel64(B->maps, set, k, nullptr, s, &kt);
         if (k + 1 < Tmax) {
             set.count = B->active[k + 1];
@@ -769,6 +774,8 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return B->T[x] > B->T[y]; });
         for (size_t i = 0; i < order.size(); ++i) {
             const int T = B->T[order[i]];
+            B->f64T.push_back(T);
+            B->f64tasks += T - 1;
             prow.push_back(R);
             irow.push_back(R1);
             fctr.push_back(B->f64ctr);
@@ -792,6 +799,8 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     off += a256(R1 * sizeof(int));
     const size_t fctr_off = off;
     off += a256(B->f64ctr * sizeof(unsigned long long));
+    const size_t fctl_off = off;
+    if (B->tc) off += a256(sizeof(F64Ctl));
     const size_t winv_off = off;
     off += a256(order.size() * 2 * kWinvDoubles * sizeof(double));
     std::vector<int64_t> prefix;
@@ -848,6 +857,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     if (e == cudaSuccess) e = host((void **)&B->h_probs, sizeof(BatchProblem) * nprob);
     if (e == cudaSuccess) e = host((void **)&B->h_params, sizeof(egs_matern_params) * nprob);
     if (e == cudaSuccess) e = host((void **)&B->h_status, sizeof(DevStatus) * nprob);
+    if (e == cudaSuccess && B->tc) e = host((void **)&B->h_f64ctl, sizeof(F64Ctl));
     if (e == cudaSuccess && !prefix.empty())
         e = cudaMemcpy(B->d_prefix, prefix.data(), prefix.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
     if (B->dag) {
@@ -901,6 +911,7 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
         std::vector<F64Prob> fp(order.size());
         B->d_f64 = (F64Prob *)(B->ws + f64_off);
         B->d_f64ctr = (unsigned long long *)(B->ws + fctr_off);
+        B->d_f64ctl = (F64Ctl *)(B->ws + fctl_off);
         for (size_t i = 0; i < order.size(); ++i) {
             const BatchProblem &pr = B->h_probs[order[i]];
             F64Prob &P = fp[i];
@@ -941,6 +952,16 @@ cudaError_t run_staged(egs_batch *B, cudaStream_t us, cudaError_t e)
         std::memset(B->h_ctl, 0, 2 * sizeof(DagCtl));
         B->h_ctl[0].limit_ns = B->limit_ns;
         B->h_ctl[0].withhold = B->withhold;
+    }
+    if (B->tc) {
+        B->h_f64ctl[0] = F64Ctl{B->limit_ns, -1, -1};
+        int64_t t = B->withhold - (int64_t)B->ntasks;  // tasks after the persistent launch's
+        for (size_t i = 0; t >= 0 && i < B->f64T.size(); t -= B->f64T[i++] - 1)
+            if (t < B->f64T[i] - 1) {
+                B->h_f64ctl->prob = (int)i;
+                B->h_f64ctl->step = (int)t;
+                break;
+            }
     }
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(B->d_params, B->h_params, sizeof(egs_matern_params) * B->nprob, cudaMemcpyHostToDevice, B->cs);
@@ -1022,15 +1043,13 @@ egs_status egs_batch_run(egs_batch *B, const double *const *locs, const double *
 
 int32_t egs_batch_launches(const egs_batch *B) { return B ? B->launches_per_run : 0; }
 
-int64_t egs_batch_tasks(const egs_batch *B) { return B && B->dag ? (int64_t)B->ntasks : 0; }
+int64_t egs_batch_tasks(const egs_batch *B) { return B ? (int64_t)B->ntasks + B->f64tasks : 0; }
 
 egs_status egs_batch_set_wait_limit(egs_batch *B, int64_t limit_ns, int64_t withhold_task)
 {
     if (!B) return set_error(EGS_ERR_ARG, "egs_batch_set_wait_limit: NULL batch");
-    // a tensor-core batch accepts a limit, but its waits (within one SM) keep their own, and it
-    // has no task to withhold
-    if (!B->dag && !B->tc) return set_error(EGS_ERR_UNIMPLEMENTED, "egs_batch_set_wait_limit: not a persistent batch");
-    if (limit_ns < 1 || withhold_task < -1 || withhold_task >= (int64_t)B->ntasks)
+    if (!B->dag && !B->tc) return set_error(EGS_ERR_UNIMPLEMENTED, "egs_batch_set_wait_limit: no bounded waits in this batch");
+    if (limit_ns < 1 || withhold_task < -1 || withhold_task >= egs_batch_tasks(B))
         return set_error(EGS_ERR_ARG, "egs_batch_set_wait_limit: limit %lld ns or task %lld out of range",
                          (long long)limit_ns, (long long)withhold_task);
     B->limit_ns = (unsigned long long)limit_ns;
@@ -1102,7 +1121,7 @@ egs_status egs_batch_destroy(egs_batch *B)
         if (!B->pooled) cudaFree(B->ws);
         else dev_free(B->alloc, B->ws, B->ws_bytes, nullptr);
     }
-    for (void *p : {(void *)B->h_probs, (void *)B->h_params, (void *)B->h_status, (void *)B->h_ctl}) {
+    for (void *p : {(void *)B->h_probs, (void *)B->h_params, (void *)B->h_status, (void *)B->h_ctl, (void *)B->h_f64ctl}) {
         if (B->once) std::free(p);
         else if (p) cudaFreeHost(p);
     }

@@ -277,6 +277,7 @@ __global__ void __launch_bounds__(256) k_winv_rows(const __grid_constant__ F64Se
 
 struct F64Item {
     int m, n, rb, cb;  // output tile, 128-row block, 64-column block; m < 0 ends
+    int hold;          // its accumulators are never signalled (failure tests)
 };
 
 // F64_TRAIL: output tiles (m, n), n = col0 .. col1 - 1, m = n .. T - 1, visited by blocks of
@@ -453,7 +454,9 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
     __shared__ uint64_t rfull[FRING], rempty[FRING];
     __shared__ F64Item ring[FRING];
     __shared__ uint32_t tmem_base;
-    __shared__ int abort_flag, stop, loaded;
+    __shared__ int abort_flag, stop, loaded, hold_first;
+    __shared__ uint64_t mdone;
+    __shared__ unsigned long long limit;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -471,8 +474,11 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             tc::mbar_init(&rfull[r], 1);
             tc::mbar_init(&rempty[r], 1 + 8);
         }
+        tc::mbar_init(&mdone, 1);
         abort_flag = 0;
         loaded = 0;
+        limit = set.ctl ? set.ctl->limit_ns : tc::kWaitNs;
+        hold_first = mode == F64_TRAIL && set.ctl && set.ctl->prob == (int)blockIdx.y && set.ctl->step == k;
         stop = failed(st) ? 1 : 0;
         tc::fence_mbar_init();
     }
@@ -501,8 +507,9 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                     continue;
                 }
                 const int slot = r % FRING;
-                if (!tc::mbar_wait(&rempty[slot], ((uint32_t)(r / FRING) & 1u) ^ 1u, &abort_flag)) break;
+                if (!tc::mbar_wait(&rempty[slot], ((uint32_t)(r / FRING) & 1u) ^ 1u, &abort_flag, limit)) break;
                 if (!valid) wi.m = -1;
+                wi.hold = hold_first && claimed == 0;
                 ring[slot] = wi;
                 tc::mbar_arrive(&rfull[slot]);
                 ++r;
@@ -513,12 +520,12 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                 const int kchunks = work.kchunks(wi.cb);
                 for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
                     const int bb = g & 1;
-                    if (!tc::mbar_wait(&bempty[bb], ((uint32_t)(g >> 1) & 1u) ^ 1u, &abort_flag)) break;
+                    if (!tc::mbar_wait(&bempty[bb], ((uint32_t)(g >> 1) & 1u) ^ 1u, &abort_flag, limit)) break;
                     tc::mbar_arrive_expect_tx(&bfull[bb], FB_BUF);
                     tma_load_3d(&mapB, &bfull[bb], sb + bb * FB_BUF, c * FKC, yb, 0);
                     int i = 0;
                     for (; i < kF64Slices; ++i) {
-                        if (!tc::mbar_wait(&aempty[i], ((uint32_t)g & 1u) ^ 1u, &abort_flag)) break;
+                        if (!tc::mbar_wait(&aempty[i], ((uint32_t)g & 1u) ^ 1u, &abort_flag, limit)) break;
                         tc::mbar_arrive_expect_tx(&afull[i], FA_SL);
                         tma_load_3d(&mapA, &afull[i], sa + i * FA_SL, c * FKC, ya, i);
                     }
@@ -534,23 +541,23 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             uint32_t f = 0;  // flush groups issued
             while (!abort_flag) {
                 const int slot = r % FRING;
-                if (!tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag)) break;
-                const int m = ring[slot].m, kchunks = work.kchunks(ring[slot].cb);
+                if (!tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag, limit)) break;
+                const int m = ring[slot].m, kchunks = work.kchunks(ring[slot].cb), hold = ring[slot].hold;
                 tc::mbar_arrive(&rempty[slot]);
                 ++r;
                 if (m < 0) break;
                 for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
                     const bool first = c % FLUSH == 0;
                     if (first) {
-                        if (!tc::mbar_wait(&tempty, (f & 1u) ^ 1u, &abort_flag)) break;
+                        if (!tc::mbar_wait(&tempty, (f & 1u) ^ 1u, &abort_flag, limit)) break;
                         tc::tc_fence_after();
                     }
                     const int bb = g & 1;
-                    if (!tc::mbar_wait(&bfull[bb], (uint32_t)(g >> 1) & 1u, &abort_flag)) break;
+                    if (!tc::mbar_wait(&bfull[bb], (uint32_t)(g >> 1) & 1u, &abort_flag, limit)) break;
                     const uint32_t b0 = tc::smem_u32(sb + bb * FB_BUF);
 #pragma unroll
                     for (int i = 0; i < kF64Slices; ++i) {
-                        if (!tc::mbar_wait(&afull[i], (uint32_t)g & 1u, &abort_flag)) break;
+                        if (!tc::mbar_wait(&afull[i], (uint32_t)g & 1u, &abort_flag, limit)) break;
                         tc::tc_fence_after();
                         const uint32_t a0 = tc::smem_u32(sa + i * FA_SL);
                         const int n = kF64Slices - i;  // B slices 0 .. n - 1
@@ -572,11 +579,12 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                     }
                     tc::mma_commit(&bempty[bb]);
                     if (c % FLUSH == FLUSH - 1 || c == kchunks - 1) {
-                        tc::mma_commit(&tfull);
+                        if (!hold) tc::mma_commit(&tfull);
                         ++f;
                     }
                 }
             }
+            tc::mma_commit(&mdone);  // every MMA issued, whatever way the loop ended
         }
     } else {
         // warp w: TMEM lanes 32 (w % 4) .. + 31 (rows of the block), columns 32 half .. + 31
@@ -587,7 +595,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
         bool run = true;
         while (run) {
             const int slot = r % FRING;
-            const bool got = tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag);
+            const bool got = tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag, limit);
             if (!__all_sync(0xffffffffu, got && !abort_flag)) break;
             const F64Item wi = ring[slot];
             __syncwarp();
@@ -598,7 +606,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             const int up = nflush > 2 ? 1 : 0;  // the sum over the flushes stays below 2^63
             long long acc[32];
             for (int fl = 0; fl < nflush; ++fl, ++f) {
-                const bool ok = tc::mbar_wait(&tfull, f & 1u, &abort_flag);
+                const bool ok = tc::mbar_wait(&tfull, f & 1u, &abort_flag, limit);
                 tc::tc_fence_after();
                 if (!__all_sync(0xffffffffu, ok && !abort_flag)) {
                     run = false;
@@ -675,6 +683,10 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
         }
         atomicExch(&st->timeout, 1);
         atomicMin(&st->fail_index, 0ull);  // stops the rest of the evaluation
+    }
+    if (threadIdx.x == 0) {  // and every MMA finish before TMEM goes (long done but after an abort)
+        volatile int dummy = 0;
+        tc::mbar_wait(&mdone, 0, &dummy);
     }
     tc::tc_fence_after();
     __syncthreads();

@@ -40,6 +40,13 @@ struct F64Prob {
     double *winv;             // inverses of the block's eight 8 x 8 diagonal blocks, two of kWinvDoubles (j & 1)
 };
 
+// Failure detection of a batch (egs_batch_set_wait_limit): the bound of k_tc_f64's waits, and the
+// problem and step whose trailing update never signals its first output block (-1: none).
+struct F64Ctl {
+    unsigned long long limit_ns;
+    int prob, step;
+};
+
 // The problems of a launch (one per grid row): one, or count of them in device memory with
 // Tmax tiles at most.
 struct F64Set {
@@ -48,6 +55,7 @@ struct F64Set {
     int count, b, Tmax;
     int solo;  // 1: the diagonal tile of a step alone (launch_panel64 is its POTRF and, with vinv, its
                // inverse: V_k as further rows of the panel, row r at inner slice row b + r)
+    const F64Ctl *ctl;  // in device memory, or NULL: 2 s, none
     __device__ const F64Prob &get(int i) const { return arr ? arr[i] : one; }
 };
 
