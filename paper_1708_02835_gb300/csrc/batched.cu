@@ -793,6 +793,8 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
     off += a256(R * tile * kF64Slices * sizeof(uint16_t));
     const size_t pex_off = off;
     off += a256(R * sizeof(int));
+    const size_t pdn_off = off;
+    off += a256(R);
     const size_t isl_off = off;
     off += a256(R1 * kF64Panel * kF64Slices * sizeof(uint16_t));
     const size_t iex_off = off;
@@ -918,8 +920,8 @@ egs_status batch_create(int32_t nprob, const int64_t *n, int32_t tile, egs_preci
             P.tl = Tiles{pr.tiles, nullptr, tile, pr.T, pr.T};
             P.st = pr.st;
             P.z = pr.zpad;
-            P.panel = F64Rows{(uint16_t *)(B->ws + psl_off), (int *)(B->ws + pex_off), R, prow[i]};
-            P.inner = F64Rows{(uint16_t *)(B->ws + isl_off), (int *)(B->ws + iex_off), R1, irow[i]};
+            P.panel = F64Rows{(uint16_t *)(B->ws + psl_off), (int *)(B->ws + pex_off), R, prow[i], (uint8_t *)(B->ws + pdn_off)};
+            P.inner = F64Rows{(uint16_t *)(B->ws + isl_off), (int *)(B->ws + iex_off), R1, irow[i], nullptr};
             P.ctr = B->d_f64ctr + fctr[i];
             P.winv = (double *)(B->ws + winv_off) + i * 2 * kWinvDoubles;
         }

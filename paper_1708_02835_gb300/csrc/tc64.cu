@@ -14,11 +14,16 @@
 // and the levels L = 0..6 (28 pairs) are kept.  The dropped ones and the rounding of the
 // last digit amount to about 2^-53.8 sqrt(K / 512) of |x|_max |y|_max, below the rounding
 // of a length-K chain of DFMAs.
-// Each level has its own FP32 accumulator in TMEM, flushed to FP64 every K = 256 columns.
-// Levels 0 and 1 stay below 2^24 units, so they are exact; level 2 could pass 2^24 units
-// only if |2 q_0 q_2 + q_1^2| averaged over 80% of its maximum, in phase, over 256 columns
-// (and level 3 over 67%), which the pseudo-random lower digits of a factor never do; from
-// level 4 on the FP32 rounding is below 2^-50 of the level-0 range even then.
+// Each level has its own FP32 accumulator in TMEM, flushed to FP64 every K = 256 columns, and a sum
+// of integers in units of its level is exact as long as it stays within 2^24 of them.  Over 256
+// columns levels 0 and 1 always do.  With S the largest sum of |q_0| over such 256 columns in either
+// row, level 2 is at most 128 * 2 S + 2^22 and level 3 at most 128 * 2 S + 2^23, so both are exact for
+// S <= 32,768 = half of what 256 digits can sum to, which the rows of a covariance's factor keep far
+// below.  The slicing marks the rows that do not; an output block with such a row is flushed every
+// 128 columns, where every level up to 5 is within 2^24 whatever the digits (rows with all leading
+// digits large, of one sign: off by 1.9e-9 of 250 without, 2.8e-14 so; n = 16,900
+// without such rows: 69.6 and 70.4 ms).  Of the levels from 4 on, the
+// FP32 rounding over 256 columns is below 2^-50 of the level-0 range.
 //
 // Kernel: persistent, one CTA per SM, 320 threads, output blocks of 128 x 64.  A K chunk
 // of 64 is 7 A boxes (128 rows) and one B box of all 7 slices (64 rows each, back to
@@ -51,6 +56,8 @@ constexpr int FSMEM = kF64Slices * FA_SL + 2 * FB_BUF + 1024;
 constexpr int FTHREADS = 320;      // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
 constexpr int FRING = 4;           // work items posted ahead by the producer
 constexpr int FLUSH = 256 / FKC;   // K chunks per accumulator flush
+constexpr int FLUSH_DENSE = 128 / FKC;  // with a dense row
+constexpr int kDenseSum = 32768;   // sum of |q_0| over 256 columns above which a row is dense
 constexpr uint32_t FTMEM = 512;
 constexpr int kBadRow = 1 << 20;   // exponent of a row holding an infinity or a NaN
 
@@ -72,9 +79,10 @@ __device__ __forceinline__ long long fixed57(double x, int e)
     return bits < 0 ? -f : f;
 }
 
-// The seven digits of f (balanced base 256) as BF16 bit patterns q_i 2^-8i.
-__device__ __forceinline__ void digits7(long long f, uint32_t (&d)[kF64Slices])
+// The seven digits of f (balanced base 256) as BF16 bit patterns q_i 2^-8i; returns |q_0|.
+__device__ __forceinline__ int digits7(long long f, uint32_t (&d)[kF64Slices])
 {
+    int lead = 0;
 #pragma unroll
     for (int i = kF64Slices - 1; i >= 0; --i) {
         int q;
@@ -83,16 +91,19 @@ __device__ __forceinline__ void digits7(long long f, uint32_t (&d)[kF64Slices])
             f = (f - q) >> 8;
         } else {
             q = (int)f;
+            lead = abs(q);
         }
         const float v = __int_as_float(0x4B400000 + q) - 12582912.0f;  // (float)q, |q| <= 256
         d[i] = __float_as_uint(v * __int_as_float((127 - 8 * i) << 23)) >> 16;  // exact: 8 significant bits
     }
+    return lead;
 }
 
 // One warp slices one row of b doubles (b <= 1024, a multiple of 64): slice i of the row
-// to dst[i * stride + c], the exponent to *ep.  Lanes take two consecutive columns.
+// to dst[i * stride + c], the exponent to *ep, whether it is dense to *dense.  Lanes take two
+// consecutive columns.
 __device__ __forceinline__ void slice7_row(const double *__restrict__ src, int b, uint16_t *__restrict__ dst,
-                                           size_t stride, int *ep)
+                                           size_t stride, int *ep, uint8_t *dense)
 {
     const int lane = threadIdx.x & 31;
     unsigned mh = 0;
@@ -106,15 +117,21 @@ __device__ __forceinline__ void slice7_row(const double *__restrict__ src, int b
     const bool bad = emax == 0x7FF;
     const int e = mh == 0 ? 0 : max(emax, 1) - 1022;
     if (lane == 0) *ep = bad ? kBadRow : e;
+    int lead = 0, most = 0;  // sum of |q_0| over the 256 columns at hand, the largest so far
     for (int c = 2 * lane; c < b; c += 64) {
         const double2 v = make_double2(src[c], src[c + 1]);
         uint32_t d0[kF64Slices], d1[kF64Slices];
-        digits7(bad || mh == 0 ? 0ll : fixed57(v.x, e), d0);
-        digits7(bad || mh == 0 ? 0ll : fixed57(v.y, e), d1);
+        lead += digits7(bad || mh == 0 ? 0ll : fixed57(v.x, e), d0);
+        lead += digits7(bad || mh == 0 ? 0ll : fixed57(v.y, e), d1);
 #pragma unroll
         for (int i = 0; i < kF64Slices; ++i)
             *reinterpret_cast<uint32_t *>(dst + (size_t)i * stride + c) = d0[i] | (d1[i] << 16);
+        if ((c >> 6 & 3) == 3 || c + 64 >= b) {
+            most = max(most, __reduce_add_sync(0xffffffffu, lead));
+            lead = 0;
+        }
     }
+    if (lane == 0) *dense = most > kDenseSum;
 }
 
 // Panel rows of step k (tiles m0 .. T - 1 of column k) -> slices; one warp per row.
@@ -127,7 +144,8 @@ __global__ void __launch_bounds__(256) k_slice_panel64(const __grid_constant__ F
     const int64_t pr = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (pr >= (int64_t)(tl.T - 1 - k) * b || failed(P.st)) return;
     const size_t r = P.panel.row0 + pr;
-    slice7_row(tl.t64(k + 1 + (int)(pr / b), k) + (pr % b) * b, b, P.panel.sl + r * b, P.panel.rows * b, P.panel.ex + r);
+    slice7_row(tl.t64(k + 1 + (int)(pr / b), k) + (pr % b) * b, b, P.panel.sl + r * b, P.panel.rows * b, P.panel.ex + r,
+               P.panel.dense + r);
 }
 
 // ---- the panel ----------------------------------------------------------------
@@ -263,7 +281,7 @@ __global__ void __launch_bounds__(256) k_winv_rows(const __grid_constant__ F64Se
     __syncthreads();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, c = c0 + w;
     const double *row = wrow + w * ld;
-    slice7_row(row, b, P.w.sl + (size_t)c * b, (size_t)b * b, P.w.ex + c);
+    slice7_row(row, b, P.w.sl + (size_t)c * b, (size_t)b * b, P.w.ex + c, P.w.dense + c);
     if (!wsp) return;
     float *out = wsp + (size_t)c * 2 * b;
     for (int i = lane; i < b; i += 32) {
@@ -278,7 +296,20 @@ __global__ void __launch_bounds__(256) k_winv_rows(const __grid_constant__ F64Se
 struct F64Item {
     int m, n, rb, cb;  // output tile, 128-row block, 64-column block; m < 0 ends
     int hold;          // its accumulators are never signalled (failure tests)
+    int flush;         // K chunks per accumulator flush
 };
+
+// Any of n (64 or 128) rows' marks set.
+__device__ __forceinline__ bool any_dense(const uint8_t *rows, int n)
+{
+    uint4 o = make_uint4(0, 0, 0, 0);
+    for (int i = 0; i < n; i += 16) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(rows + i);
+        o.x |= v.x | v.y;
+        o.y |= v.z | v.w;
+    }
+    return (o.x | o.y) != 0;
+}
 
 // F64_TRAIL: output tiles (m, n), n = col0 .. col1 - 1, m = n .. T - 1, visited by blocks of
 // kF64Cols columns (the block's triangle, then every lower row), so that the CTAs working side
@@ -510,6 +541,13 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                 if (!tc::mbar_wait(&rempty[slot], ((uint32_t)(r / FRING) & 1u) ^ 1u, &abort_flag, limit)) break;
                 if (!valid) wi.m = -1;
                 wi.hold = hold_first && claimed == 0;
+                wi.flush = FLUSH;
+                if (valid && rows.dense && work.kchunks(wi.cb) > FLUSH_DENSE) {
+                    // the block's rows of the tile, at most 128
+                    const uint8_t *da = rows.dense + yrow0 + work.slice_row(wi.m) + wi.rb * FM;
+                    const uint8_t *db = brows.dense + ybrow0 + (mode == F64_BAND ? 0 : work.slice_row(wi.n)) + wi.cb * FN;
+                    if (any_dense(da, min(FM, b - wi.rb * FM)) || any_dense(db, FN)) wi.flush = FLUSH_DENSE;
+                }
                 ring[slot] = wi;
                 tc::mbar_arrive(&rfull[slot]);
                 ++r;
@@ -543,11 +581,12 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                 const int slot = r % FRING;
                 if (!tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag, limit)) break;
                 const int m = ring[slot].m, kchunks = work.kchunks(ring[slot].cb), hold = ring[slot].hold;
+                const int flush = ring[slot].flush;
                 tc::mbar_arrive(&rempty[slot]);
                 ++r;
                 if (m < 0) break;
                 for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
-                    const bool first = c % FLUSH == 0;
+                    const bool first = c % flush == 0;
                     if (first) {
                         if (!tc::mbar_wait(&tempty, (f & 1u) ^ 1u, &abort_flag, limit)) break;
                         tc::tc_fence_after();
@@ -578,7 +617,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                         tc::mma_commit(&aempty[i]);
                     }
                     tc::mma_commit(&bempty[bb]);
-                    if (c % FLUSH == FLUSH - 1 || c == kchunks - 1) {
+                    if (c % flush == flush - 1 || c == kchunks - 1) {
                         if (!hold) tc::mma_commit(&tfull);
                         ++f;
                     }
@@ -602,8 +641,8 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             if (lane == 0) tc::mbar_arrive(&rempty[slot]);
             ++r;
             if (wi.m < 0) break;
-            const int nflush = (work.kchunks(wi.cb) + FLUSH - 1) / FLUSH;
-            const int up = nflush > 2 ? 1 : 0;  // the sum over the flushes stays below 2^63
+            const int kchunks = work.kchunks(wi.cb), nflush = (kchunks + wi.flush - 1) / wi.flush;
+            const int up = kchunks > 2 * FLUSH ? 1 : 0;  // the sum over the flushes stays below 2^63
             long long acc[32];
             for (int fl = 0; fl < nflush; ++fl, ++f) {
                 const bool ok = tc::mbar_wait(&tfull, f & 1u, &abort_flag, limit);
@@ -742,7 +781,7 @@ static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 size_t tc64_scratch_bytes(int b, int T)
 {
     const size_t R = (size_t)(T - 1) * (size_t)b, R1 = R + b;
-    return a256(R * b * kF64Slices * sizeof(uint16_t)) + a256(R * sizeof(int)) +
+    return a256(R * b * kF64Slices * sizeof(uint16_t)) + a256(R * sizeof(int)) + a256(R) +
            a256(R1 * PW * kF64Slices * sizeof(uint16_t)) + a256(R1 * sizeof(int)) +
            a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(2 * kWinvDoubles * sizeof(double));
 }
@@ -762,6 +801,7 @@ F64Prob tc64_problem(void *scratch, const Tiles &tl, DevStatus *st, double *z)
     P.z = z;
     P.panel.sl = (uint16_t *)take(R * tl.b * kF64Slices * sizeof(uint16_t));
     P.panel.ex = (int *)take(R * sizeof(int));
+    P.panel.dense = (uint8_t *)take(R);
     P.panel.rows = R;
     P.inner.sl = (uint16_t *)take(R1 * PW * kF64Slices * sizeof(uint16_t));
     P.inner.ex = (int *)take(R1 * sizeof(int));
@@ -785,10 +825,10 @@ cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64
 
 size_t tc64_solo_bytes(int b, int T, int nb)
 {
-    const size_t bb = (size_t)b * b;
-    return a256((size_t)nb * bb * kF64Slices * sizeof(uint16_t)) + a256((size_t)nb * b * sizeof(int)) +
-           a256((size_t)2 * b * PW * kF64Slices * sizeof(uint16_t)) + a256((size_t)2 * b * sizeof(int)) +
-           a256(bb * kF64Slices * sizeof(uint16_t)) + a256((size_t)b * sizeof(int)) +
+    auto rows = [](size_t n, size_t K) {  // as tc64_solo_problem
+        return a256(n * K * kF64Slices * sizeof(uint16_t)) + a256(n * sizeof(int)) + a256(n);
+    };
+    return rows((size_t)nb * b, b) + rows((size_t)2 * b, PW) + rows((size_t)b, b) +
            a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(2 * kWinvDoubles * sizeof(double));
 }
 
@@ -805,6 +845,7 @@ F64Prob tc64_solo_problem(void *scratch, const Tiles &tl, DevStatus *st, double 
         F64Rows r{};
         r.sl = (uint16_t *)take(n * K * kF64Slices * sizeof(uint16_t));
         r.ex = (int *)take(n * sizeof(int));
+        r.dense = (uint8_t *)take(n);
         r.rows = n;
         return r;
     };
@@ -814,6 +855,7 @@ F64Prob tc64_solo_problem(void *scratch, const Tiles &tl, DevStatus *st, double 
     P.vinv = vinv;
     P.panel = rows((size_t)nb * b, b);
     P.inner = rows(2 * b, PW);
+    P.inner.dense = nullptr;  // one chunk: never flushed in between
     P.w = rows(b, b);
     P.ctr = (unsigned long long *)take(tc64_counters(tl.b, tl.T) * sizeof(unsigned long long));
     P.winv = (double *)take(2 * kWinvDoubles * sizeof(double));

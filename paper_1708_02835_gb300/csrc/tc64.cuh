@@ -25,6 +25,7 @@ struct F64Rows {
     uint16_t *sl;
     int *ex;
     size_t rows, row0;
+    uint8_t *dense;  // K = b: 1 for a row whose level sums need the short flush (tc64.cu); NULL for K = 64
 };
 
 // One problem as the kernels see it.
