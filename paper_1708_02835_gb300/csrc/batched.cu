@@ -616,7 +616,7 @@ cudaError_t enqueue_factor64(egs_batch *B, cudaStream_t s, int *count)
         if (k + 1 < Tmax) {
             set.count = B->active[k + 1];
             if (e == cudaSuccess) e = launch_slice_panel64(set, k, s, &kt);
-            if (e == cudaSuccess) e = launch_update_tc64(B->maps, set, k, 0, 0, s, &kt);
+            if (e == cudaSuccess) e = launch_update_tc64(B->maps, set, k, s, &kt);
         }
     }
     *count += kt.launches;

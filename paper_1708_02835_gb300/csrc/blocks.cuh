@@ -35,20 +35,16 @@ __device__ __forceinline__ void tri_decode(int64_t t, int &i, int &j)
 // applied through 1 / sqrt(d) (one reciprocal square root per column, then
 // multiplications).  A pivot that is not positive records row0 + its row in
 // st->fail_index and returns false; the strict upper triangle is zeroed.
-// The same routine serves NB = 32.
 // ---------------------------------------------------------------------------
-template <int NB>
-struct PotrfSmem {
-    double S[NB][NB + 1];
-    double rd[NB];  // 1 / L_jj
+struct Potrf64Smem {
+    double S[64][65];
+    double rd[64];  // 1 / L_jj
     int fail_j;
 };
-using Potrf64Smem = PotrfSmem<64>;
 
-// NB x NB block (NB = 32 or 64), as described above.
-template <int NB>
-__device__ __forceinline__ bool potrf_smem_s(PotrfSmem<NB> &sm, double *A, int ld, int64_t row0, DevStatus *st)
+__device__ __forceinline__ bool potrf64_smem_s(Potrf64Smem &sm, double *A, int ld, int64_t row0, DevStatus *st)
 {
+    constexpr int NB = 64;
     double(&S)[NB][NB + 1] = sm.S;
     int &fail_j = sm.fail_j;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -124,11 +120,6 @@ __device__ __forceinline__ bool potrf_smem_s(PotrfSmem<NB> &sm, double *A, int l
         A[(size_t)i * ld + j] = (j <= i) ? S[i][j] : 0.0;
     }
     return true;
-}
-
-__device__ __forceinline__ bool potrf64_smem_s(Potrf64Smem &sm, double *A, int ld, int64_t row0, DevStatus *st)
-{
-    return potrf_smem_s<64>(sm, A, ld, row0, st);
 }
 
 __device__ __forceinline__ bool potrf64_smem(double *A, int ld, int64_t row0, DevStatus *st)
@@ -466,12 +457,11 @@ __device__ __forceinline__ void gemm_sub32(const EA *Am, int lda, const EB *An, 
 }
 
 // ---------------------------------------------------------------------------
-// X L^T = A for RB rows (RB in {8, 16, 64}): X and A at Xp (row stride ldx,
+// X L^T = A for RB rows (RB in {16, 64}): X and A at Xp (row stride ldx,
 // ncols columns), L lower ncols x ncols at Lp (row stride ldl).  32-column
 // blocks: a GEMM-style update with the already-solved columns, then a
 // 32-wide substitution in shared memory.  256 threads; fewer rows per CTA put
-// more SMs on a panel when the panel is short.  cstart (a multiple of 32):
-// the columns before it are zero in A, hence in X, and are skipped.  TX =
+// more SMs on a panel when the panel is short.  TX =
 // float: X and all arithmetic in FP32 (L rounded to FP32 as it is staged).
 // ---------------------------------------------------------------------------
 template <int RB, typename TX>
@@ -484,7 +474,7 @@ struct TrsmSmem {
 
 template <int RB, typename TX = double>
 __device__ __forceinline__ void trsm_rows_s(TrsmSmem<RB, TX> &sm, const double *Lp, int ldl, TX *Xp, int ldx,
-                                            int ncols, int cstart = 0)
+                                            int ncols)
 {
     constexpr int RPG = RB / 8;  // rows per thread group (8 groups of 32 threads)
     TX(&Xs)[RB][kPW + 1] = sm.Xs;
@@ -492,11 +482,11 @@ __device__ __forceinline__ void trsm_rows_s(TrsmSmem<RB, TX> &sm, const double *
     TX(&Ab)[RB][33] = sm.Ab;
     TX(&Ld)[32][33] = sm.Ld;
     const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
-    for (int c0 = cstart; c0 < ncols; c0 += 32) {
+    for (int c0 = 0; c0 < ncols; c0 += 32) {
         TX acc[RPG];
 #pragma unroll
         for (int i = 0; i < RPG; ++i) acc[i] = Xp[(size_t)(ty * RPG + i) * ldx + c0 + tx];
-        for (int p = cstart; p < c0; p += kPW) {
+        for (int p = 0; p < c0; p += kPW) {
             for (int e = tid; e < RB * kPW; e += 256) {
                 const int r = e >> 4, l = e & 15;
                 Xs[r][l] = Xp[(size_t)r * ldx + p + l];
@@ -536,10 +526,10 @@ __device__ __forceinline__ void trsm_rows_s(TrsmSmem<RB, TX> &sm, const double *
 }
 
 template <int RB, typename TX = double>
-__device__ __forceinline__ void trsm_rows(const double *Lp, int ldl, TX *Xp, int ldx, int ncols, int cstart = 0)
+__device__ __forceinline__ void trsm_rows(const double *Lp, int ldl, TX *Xp, int ldx, int ncols)
 {
     __shared__ TrsmSmem<RB, TX> sm;
-    trsm_rows_s<RB, TX>(sm, Lp, ldl, Xp, ldx, ncols, cstart);
+    trsm_rows_s<RB, TX>(sm, Lp, ldl, Xp, ldx, ncols);
 }
 
 // ---------------------------------------------------------------------------

@@ -69,16 +69,16 @@ __global__ void __launch_bounds__(256) k_update_f64_32(Tiles tl, int k, DevStatu
                tl.t64(m, nc) + (size_t)sr * 32 * b + sc * 32, b);
 }
 
-cudaError_t launch_update_f64(const Tiles &tl, int k, int64_t ntri, DevStatus *st, cudaStream_t s, KernelTimer *kt,
-                              int cls)
+static cudaError_t launch_update_f64(const Tiles &tl, int k, int64_t ntri, DevStatus *st, cudaStream_t s,
+                                     KernelTimer *kt)
 {
     if (ntri <= 0) return cudaSuccess;
     const int nsub = tl.b / 64;
     if (ntri * nsub * (nsub + 1) / 2 < 304) {
         const int n32 = tl.b / 32;
-        EGS_LAUNCH(kt, cls, s, k_update_f64_32<<<dim3((unsigned)ntri, (unsigned)(n32 * n32)), 256, 0, s>>>(tl, k, st));
+        EGS_LAUNCH(kt, KC_UPDATE, s, k_update_f64_32<<<dim3((unsigned)ntri, (unsigned)(n32 * n32)), 256, 0, s>>>(tl, k, st));
     } else {
-        EGS_LAUNCH(kt, cls, s, k_update_f64<<<dim3((unsigned)ntri, (unsigned)(nsub * nsub)), 256, 0, s>>>(tl, k, st));
+        EGS_LAUNCH(kt, KC_UPDATE, s, k_update_f64<<<dim3((unsigned)ntri, (unsigned)(nsub * nsub)), 256, 0, s>>>(tl, k, st));
     }
     return cudaGetLastError();
 }
@@ -101,7 +101,7 @@ cudaError_t launch_potrf_tiles_f64(double *tiles, const TileGeom &g, DevStatus *
             if (kt) kt->step = k;
             e = launch_panel64(maps, set, k, &fork, s, kt);
             if (e == cudaSuccess) e = launch_slice_panel64(set, k, s, kt);
-            if (e == cudaSuccess) e = launch_update_tc64(maps, set, k, 0, 0, s, kt);
+            if (e == cudaSuccess) e = launch_update_tc64(maps, set, k, s, kt);
         }
     } else {
         const F64Set set{nullptr, dfma_problem(winv, tl, st, z), 1, g.b, T, 0};

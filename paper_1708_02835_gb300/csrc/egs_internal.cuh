@@ -67,7 +67,7 @@ struct TileGeom {
 };
 
 // Kernel classes for per-class device timing.
-// KC_UPDATE64: the FP64 update launches of the mixed-precision factorisation.
+// KC_UPDATE64: the FP64-accurate update launches of the mixed-precision factorisation.
 enum KernelClass { KC_GEN = 0, KC_POTRF, KC_TRSM, KC_UPDATE, KC_TRSV, KC_OTHER, KC_UPDATE64, KC_COUNT };
 
 // Counts launches and, when enabled, brackets each launch with a CUDA event
@@ -272,9 +272,6 @@ bool mixed_result_ok(const EvalSetup &es, const DevStatus &h);
 int32_t default_tile(int64_t n, egs_precision p);
 
 // Building blocks shared by the FP64 and mixed drivers.
-// FP64 update of the first ntri tiles of step k's trailing triangle (row order).
-cudaError_t launch_update_f64(const Tiles &tl, int k, int64_t ntri, DevStatus *st, cudaStream_t s, KernelTimer *kt,
-                              int cls = KC_UPDATE);
 // FP32 mixed mode: FP64-accurate updates of the band tiles whose panel
 // operands are not both FP64 band tiles, by exact BF16 slicing on tcgen05
 // (ozaki.cu).  The TRSM stage writes the slices of every panel row.

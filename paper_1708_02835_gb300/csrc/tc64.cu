@@ -876,16 +876,16 @@ cudaError_t make_f64_solo_maps(const F64Prob &P, F64Maps *maps)
 }
 
 // CTAs of a problem's update launch: the whole GPU for one problem, a share for each of many.
-static unsigned tc64_ctas(const F64Set &set, int64_t items, int reserve)
+static unsigned tc64_ctas(const F64Set &set, int64_t items)
 {
-    int64_t c = device_sms() - reserve;
+    int64_t c = device_sms();
     if (set.count > 1) c = (c * 4 + set.count - 1) / set.count;
     c = items < c ? items : c;
     return (unsigned)(c > 1 ? c : 1);
 }
 
 static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, const F64Set &set, int k, int c0, int c1,
-                                 int mode, int slot, int reserve, cudaStream_t s, KernelTimer *kt)
+                                 int mode, int slot, cudaStream_t s, KernelTimer *kt)
 {
     cudaError_t e = cudaFuncSetAttribute(k_tc_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
     if (e != cudaSuccess) return e;
@@ -895,7 +895,7 @@ static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, con
     const bool in = mode == F64_INNER;
     const F64Work w{tl, T, k, in ? c0 : k + c0, in ? c1 : (k + c1 < T ? k + c1 : T), mode};
     if (w.col0 >= w.col1) return cudaSuccess;
-    const dim3 grid(tc64_ctas(set, w.items(), reserve), (unsigned)set.count);
+    const dim3 grid(tc64_ctas(set, w.items()), (unsigned)set.count);
     // of a mixed factorisation's diagonal tile: part of its POTRF; its band: the FP64 update class
     const int cls = mode == F64_BAND ? KC_TRSM : (!set.solo ? KC_UPDATE : (in ? KC_POTRF : KC_UPDATE64));
     EGS_LAUNCH(kt, cls, s,
@@ -987,7 +987,7 @@ cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, F64For
             e = cudaGetLastError();
             if (fork && e == cudaSuccess) e = cudaStreamWaitEvent(bs, fork->next, 0);
             if (e == cudaSuccess)
-                e = launch_tc_f64(maps.ia, maps.ib, set, k, j + 1, nj, F64_INNER, k * (2 + nj) + 2 + j, 0, bs, kt);
+                e = launch_tc_f64(maps.ia, maps.ib, set, k, j + 1, nj, F64_INNER, k * (1 + nj) + 1 + j, bs, kt);
         }
         if (fork && e == cudaSuccess) e = cudaEventRecord(fork->aux.done, bs);
     }
@@ -1005,11 +1005,9 @@ cudaError_t launch_slice_panel64(const F64Set &set, int k, cudaStream_t s, Kerne
     return cudaGetLastError();
 }
 
-cudaError_t launch_update_tc64(const F64Maps &maps, const F64Set &set, int k, int part, int reserve, cudaStream_t s,
-                               KernelTimer *kt)
+cudaError_t launch_update_tc64(const F64Maps &maps, const F64Set &set, int k, cudaStream_t s, KernelTimer *kt)
 {
-    return launch_tc_f64(maps.a, maps.b, set, k, part == 2 ? 2 : 1, part == 1 ? 2 : set.Tmax, F64_TRAIL,
-                         k * (2 + set.b / PW) + (part == 2 ? 1 : 0), reserve, s, kt);
+    return launch_tc_f64(maps.a, maps.b, set, k, 1, set.Tmax, F64_TRAIL, k * (1 + set.b / PW), s, kt);
 }
 
 cudaError_t launch_solo_init(const F64Set &set, cudaStream_t s, KernelTimer *kt)
@@ -1036,7 +1034,7 @@ cudaError_t launch_band_solve(const F64Maps &maps, const F64Set &set, int k, int
     EGS_LAUNCH(kt, KC_TRSM, s, k_slice_panel64<<<dim3((unsigned)((size_t)nb * set.b / 8), 1), 256, 0, s>>>(set, k));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_tc_f64(maps.a, maps.b, set, k, 1, 1 + nb, F64_BAND, k * (2 + set.b / PW), 0, s, kt);
+    return launch_tc_f64(maps.a, maps.b, set, k, 1, 1 + nb, F64_BAND, k * (1 + set.b / PW), s, kt);
 }
 
 cudaError_t launch_band_update(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt)
@@ -1045,7 +1043,7 @@ cudaError_t launch_band_update(const F64Maps &maps, const F64Set &set, int k, in
     EGS_LAUNCH(kt, KC_TRSM, s, k_slice_panel64<<<dim3((unsigned)((size_t)nb * set.b / 8), 1), 256, 0, s>>>(set, k));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_tc_f64(maps.a, maps.pb, set, k, 1, 1 + nb, F64_TRAIL, k * (2 + set.b / PW) + 1, 0, s, kt);
+    return launch_tc_f64(maps.a, maps.pb, set, k, 1, 1 + nb, F64_TRAIL, (k + 1) * (1 + set.b / PW) - 1, s, kt);
 }
 
 }  // namespace egs

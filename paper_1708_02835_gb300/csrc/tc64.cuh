@@ -60,8 +60,10 @@ struct F64Set {
     __device__ const F64Prob &get(int i) const { return arr ? arr[i] : one; }
 };
 
-// Work counters of a problem: two trailing updates and b / 64 inner ones per step.
-inline size_t tc64_counters(int b, int T) { return (size_t)T * (2 + b / kF64Panel); }
+// Work counters of a problem: per step one for the trailing update (a mixed factorisation: the band
+// solve) and one for each 64-column block's inner update; the last block has none, and its counter
+// is a mixed factorisation's band update's.
+inline size_t tc64_counters(int b, int T) { return (size_t)T * (1 + b / kF64Panel); }
 
 struct F64Maps {
     CUtensorMap a, b, ia, ib;  // panel slices, inner slices; diagonal tiles alone: b is W's, pb the panel's
@@ -108,9 +110,7 @@ cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, F64For
 cudaError_t launch_band_update(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt);
 // Slices of the solved panel tiles (k + 1 .. T - 1, k).
 cudaError_t launch_slice_panel64(const F64Set &set, int k, cudaStream_t s, KernelTimer *kt);
-// C_mn -= P_m P_n^T, m = n .. T - 1.  part 0: n = k + 1 .. T - 1; 1: n = k + 1; 2: the rest.
-// reserve: SMs left to other streams.
-cudaError_t launch_update_tc64(const F64Maps &maps, const F64Set &set, int k, int part, int reserve, cudaStream_t s,
-                               KernelTimer *kt);
+// C_mn -= P_m P_n^T for k < n <= m < T.
+cudaError_t launch_update_tc64(const F64Maps &maps, const F64Set &set, int k, cudaStream_t s, KernelTimer *kt);
 
 }  // namespace egs
