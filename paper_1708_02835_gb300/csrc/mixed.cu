@@ -461,9 +461,9 @@ cudaError_t factor_mixed(const MixedBuffers &mb, const CUtensorMap *ma, const CU
     for (cudaEvent_t *ev : {&ev_panel, &ev_col, &ev_diag})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     // POTRF of a diagonal tile and its inverse V_k = L_kk^-T: the FP64 path's 64-column blocks on
-    // that tile alone with V_k's rows below it; the band rows by multiplication with W = V_k^T on
-    // the tensor cores (tc64.cu).  Tile 512: 1.05 ms of POTRF, 0.32 of inversion and 0.22 of band
-    // solve as task graph, column and row substitutions; 0.85 and 0.05 ms so
+    // that tile alone with V_k's rows below it; the band rows by products with W = V_k^T on the
+    // tensor cores and one correction (tc64.cu).  Tile 512: 1.05 ms of POTRF, 0.32 of inversion and
+    // 0.22 of band solve as task graph, column and row substitutions; 0.85 and 0.15 ms so
     const F64Set diag{nullptr, tc64_solo_problem(mb.dpan, tl, st, mb.vinv, band_tiles(tl)), 1, b, T, 1};
     F64Maps dmaps;
     F64Fork fork;  // joined to the chain's stream, which is joined to s

@@ -136,16 +136,18 @@ __device__ __forceinline__ void slice7_row(const double *__restrict__ src, int b
 
 // Panel rows of step k (tiles m0 .. T - 1 of column k) -> slices; one warp per row.
 // Memory bound: 8 bytes read (twice, the second time from L1 / L2) and 14 written per entry.
-__global__ void __launch_bounds__(256) k_slice_panel64(const __grid_constant__ F64Set set, int k)
+// src: 0 the tiles of column k; 1 the band rows' Y; 2 the rows of L_kk, into their own slices.
+__global__ void __launch_bounds__(256) k_slice_panel64(const __grid_constant__ F64Set set, int k, int src)
 {
     const F64Prob &P = set.get(blockIdx.y);
     const Tiles &tl = P.tl;
     const int b = tl.b;
     const int64_t pr = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (pr >= (int64_t)(tl.T - 1 - k) * b || failed(P.st)) return;
-    const size_t r = P.panel.row0 + pr;
-    slice7_row(tl.t64(k + 1 + (int)(pr / b), k) + (pr % b) * b, b, P.panel.sl + r * b, P.panel.rows * b, P.panel.ex + r,
-               P.panel.dense + r);
+    if ((src != 2 && pr >= (int64_t)(tl.T - 1 - k) * b) || failed(P.st)) return;
+    const F64Rows &to = src == 2 ? P.l : P.panel;
+    const size_t r = to.row0 + pr;
+    const double *x = src == 0 ? tl.t64(k + 1 + (int)(pr / b), k) + (pr % b) * b : (src == 1 ? P.y : tl.t64(k, k)) + pr * b;
+    slice7_row(x, b, to.sl + r * b, to.rows * b, to.ex + r, to.dense + r);
 }
 
 // ---- the panel ----------------------------------------------------------------
@@ -318,20 +320,29 @@ __device__ __forceinline__ bool any_dense(const uint8_t *rows, int n)
 // F64_INNER, inside a panel: the 64-column blocks col0 .. col1 - 1 of tile column k, all rows
 // from each block's diagonal down; slice row (m - k) b + r, K = 64.  Tile k + 1 of a diagonal
 // tile alone is V_k, its rows below 64 col0 as far as they are nonzero.
-// F64_BAND: the tiles k + 1 .. col1 - 1 of column k times W^T (B operand: the rows of W; lower
-// triangular, so column block c needs K = 64 (c + 1) only), stored in their place.
-enum F64Mode { F64_TRAIL = 0, F64_INNER, F64_BAND };
+// The band solve of a mixed factorisation, X L_kk^T = A for the tiles k + 1 .. col1 - 1 of column k
+// with W = L_kk^-1 (B operands the rows of W or L_kk; lower triangular, so column block c needs
+// K = 64 (c + 1) only), in three products on those rows' slices:
+//   F64_BAND  Y = A W^T;
+//   F64_RES   the tiles become R = A - Y L_kk^T;
+//   F64_CORR  the tiles become X = Y + R W^T.
+// A product with the inverse alone leaves a residual that grows with the condition of L_kk: rms of
+// Y L^T - A 4.5 (nu = 1/2, range 0.1), 11 (nu = 1.3, range 0.2) and 58 times (nu = 5/2) a substitution's at
+// tile 512, X's 0.46, 0.10 and 0.10 times.  Tile 512: 0.05 ms a step alone, 0.15 with the correction
+// (n = 25,600: 63.1 and 68.2 ms; a row substitution took 0.22 ms a step).
+enum F64Mode { F64_TRAIL = 0, F64_INNER, F64_BAND, F64_RES, F64_CORR };
 constexpr int kF64Cols = 8;
 struct F64Work {
     const Tiles &tl;
     int T, k, col0, col1, mode;
     __host__ __device__ int row_blocks() const { return (tl.b + FM - 1) / FM; }
-    __device__ int kchunks(int cb) const { return mode == F64_INNER ? 1 : (mode == F64_BAND ? cb + 1 : tl.b / FKC); }
+    __host__ __device__ bool band() const { return mode >= F64_BAND; }
+    __device__ int kchunks(int cb) const { return mode == F64_INNER ? 1 : (band() ? cb + 1 : tl.b / FKC); }
     __host__ __device__ int64_t items() const
     {
         const int64_t c = col1 - col0;
         if (mode == F64_INNER) return c * row_blocks() * (T - k);
-        if (mode == F64_BAND) return c * row_blocks() * (tl.b / FN);
+        if (band()) return c * row_blocks() * (tl.b / FN);
         const int64_t h = T - col0;
         return (c * h - c * (c - 1) / 2) * row_blocks() * (tl.b / FN);
     }
@@ -352,7 +363,7 @@ struct F64Work {
         const int blk = (int)(item % per);
         w.rb = blk / ncb;
         w.cb = blk % ncb;
-        if (mode == F64_BAND) {
+        if (band()) {
             w.m = col0 + (int)t;
             w.n = k;
             return true;
@@ -476,7 +487,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
     if ((int64_t)blockIdx.x >= nitems) return;
     unsigned long long *next = P.ctr + slot;
     DevStatus *st = P.st;
-    const F64Rows &rows = mode == F64_INNER ? P.inner : P.panel, &brows = mode == F64_BAND ? P.w : rows;
+    const F64Rows &rows = mode == F64_INNER ? P.inner : P.panel, &brows = !work.band() ? rows : (mode == F64_RES ? P.l : P.w);
     const int *__restrict__ ex = rows.ex + rows.row0, *__restrict__ exb = brows.ex + brows.row0;
     const int yrow0 = (int)rows.row0, ybrow0 = (int)brows.row0;
     extern __shared__ uint8_t smem_raw[];
@@ -545,7 +556,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                 if (valid && rows.dense && work.kchunks(wi.cb) > FLUSH_DENSE) {
                     // the block's rows of the tile, at most 128
                     const uint8_t *da = rows.dense + yrow0 + work.slice_row(wi.m) + wi.rb * FM;
-                    const uint8_t *db = brows.dense + ybrow0 + (mode == F64_BAND ? 0 : work.slice_row(wi.n)) + wi.cb * FN;
+                    const uint8_t *db = brows.dense + ybrow0 + (work.band() ? 0 : work.slice_row(wi.n)) + wi.cb * FN;
                     if (any_dense(da, min(FM, b - wi.rb * FM)) || any_dense(db, FN)) wi.flush = FLUSH_DENSE;
                 }
                 ring[slot] = wi;
@@ -554,7 +565,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                 if (!valid) break;
                 claimed = (int64_t)atomicAdd(next, 1ull);  // overlaps the loads below
                 const int ya = yrow0 + (int)work.slice_row(wi.m) + wi.rb * FM;
-                const int yb = ybrow0 + (mode == F64_BAND ? 0 : (int)work.slice_row(wi.n)) + wi.cb * FN;
+                const int yb = ybrow0 + (work.band() ? 0 : (int)work.slice_row(wi.n)) + wi.cb * FN;
                 const int kchunks = work.kchunks(wi.cb);
                 for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
                     const int bb = g & 1;
@@ -673,21 +684,28 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             if (row >= work.r0(wi) && row < work.r1(wi, solo)) {
                 const int col = wi.cb * FN + half * 32;
                 const int ea = ex[work.slice_row(wi.m) + row] - 16;
-                const int *eb = exb + (mode == F64_BAND ? 0 : work.slice_row(wi.n)) + col;
+                const int *eb = exb + (work.band() ? 0 : work.slice_row(wi.n)) + col;
                 double *C = (solo && mode == F64_INNER && wi.m > k ? P.vinv + (size_t)k * work.tl.bb()
                                                                    : work.tl.t64(wi.m, wi.n)) + (size_t)row * b + col;
+                const double *Cin = C;  // what the product is added to or subtracted from
+                const bool add = mode == F64_BAND || mode == F64_CORR;
+                if (add) {
+                    double *y = P.y + (size_t)(wi.m - k - 1) * work.tl.bb() + (size_t)row * b + col;
+                    Cin = y;
+                    if (mode == F64_BAND) C = y;
+                }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     double2 cv[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
                         cv[j] = mode == F64_BAND ? make_double2(0.0, 0.0)
-                                                 : *reinterpret_cast<const double2 *>(C + 16 * h + 2 * j);
+                                                 : *reinterpret_cast<const double2 *>(Cin + 16 * h + 2 * j);
                     double *cd = reinterpret_cast<double *>(cv);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const int s = ea + __ldg(eb + 16 * h + j);
-                        const double d = fixed_to_f64(mode == F64_BAND ? -acc[16 * h + j] : acc[16 * h + j], up);
+                        const double d = fixed_to_f64(add ? -acc[16 * h + j] : acc[16 * h + j], up);
                         if (s >= -960 && s <= 1000) {
                             cd[j] = fma(-pow2(s), d, cd[j]);
                         } else if (s > 1000) {
@@ -828,7 +846,8 @@ size_t tc64_solo_bytes(int b, int T, int nb)
     auto rows = [](size_t n, size_t K) {  // as tc64_solo_problem
         return a256(n * K * kF64Slices * sizeof(uint16_t)) + a256(n * sizeof(int)) + a256(n);
     };
-    return rows((size_t)nb * b, b) + rows((size_t)2 * b, PW) + rows((size_t)b, b) +
+    return rows((size_t)nb * b, b) + rows((size_t)2 * b, PW) + 2 * rows((size_t)b, b) +
+           a256((size_t)nb * b * b * sizeof(double)) +
            a256(tc64_counters(b, T) * sizeof(unsigned long long)) + a256(2 * kWinvDoubles * sizeof(double));
 }
 
@@ -857,6 +876,8 @@ F64Prob tc64_solo_problem(void *scratch, const Tiles &tl, DevStatus *st, double 
     P.inner = rows(2 * b, PW);
     P.inner.dense = nullptr;  // one chunk: never flushed in between
     P.w = rows(b, b);
+    P.l = rows(b, b);
+    P.y = (double *)take((size_t)nb * b * b * sizeof(double));
     P.ctr = (unsigned long long *)take(tc64_counters(tl.b, tl.T) * sizeof(unsigned long long));
     P.winv = (double *)take(2 * kWinvDoubles * sizeof(double));
     return P;
@@ -870,6 +891,7 @@ cudaError_t make_f64_solo_maps(const F64Prob &P, F64Maps *maps)
     if (P.panel.rows) e = make_map3(&maps->a, P.panel.sl, P.panel.rows, b, FM, 1);
     if (e == cudaSuccess && P.panel.rows) e = make_map3(&maps->pb, P.panel.sl, P.panel.rows, b, FN, kF64Slices);
     if (e == cudaSuccess) e = make_map3(&maps->b, P.w.sl, P.w.rows, b, FN, kF64Slices);
+    if (e == cudaSuccess) e = make_map3(&maps->lb, P.l.sl, P.l.rows, b, FN, kF64Slices);
     if (e == cudaSuccess) e = make_map3(&maps->ia, P.inner.sl, P.inner.rows, PW, FM, 1);
     if (e == cudaSuccess) e = make_map3(&maps->ib, P.inner.sl, P.inner.rows, PW, FN, kF64Slices);
     return e;
@@ -897,7 +919,7 @@ static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, con
     if (w.col0 >= w.col1) return cudaSuccess;
     const dim3 grid(tc64_ctas(set, w.items()), (unsigned)set.count);
     // of a mixed factorisation's diagonal tile: part of its POTRF; its band: the FP64 update class
-    const int cls = mode == F64_BAND ? KC_TRSM : (!set.solo ? KC_UPDATE : (in ? KC_POTRF : KC_UPDATE64));
+    const int cls = mode >= F64_BAND ? KC_TRSM : (!set.solo ? KC_UPDATE : (in ? KC_POTRF : KC_UPDATE64));
     EGS_LAUNCH(kt, cls, s,
                k_tc_f64<<<grid, FTHREADS, FSMEM, s>>>(a, b, set, k, c0, c1, mode, slot));
     return cudaGetLastError();
@@ -987,7 +1009,8 @@ cudaError_t launch_panel64(const F64Maps &maps, const F64Set &set, int k, F64For
             e = cudaGetLastError();
             if (fork && e == cudaSuccess) e = cudaStreamWaitEvent(bs, fork->next, 0);
             if (e == cudaSuccess)
-                e = launch_tc_f64(maps.ia, maps.ib, set, k, j + 1, nj, F64_INNER, k * (1 + nj) + 1 + j, bs, kt);
+                e = launch_tc_f64(maps.ia, maps.ib, set, k, j + 1, nj, F64_INNER,
+                                  tc64_slot(set.b, k, 4 + j), bs, kt);
         }
         if (fork && e == cudaSuccess) e = cudaEventRecord(fork->aux.done, bs);
     }
@@ -1001,13 +1024,13 @@ cudaError_t launch_slice_panel64(const F64Set &set, int k, cudaStream_t s, Kerne
     if (k + 1 >= set.Tmax) return cudaSuccess;
     EGS_LAUNCH(kt, KC_TRSM, s,
                k_slice_panel64<<<dim3((unsigned)((size_t)(set.Tmax - k - 1) * set.b / 8), (unsigned)set.count), 256, 0,
-                                 s>>>(set, k));
+                                 s>>>(set, k, 0));
     return cudaGetLastError();
 }
 
 cudaError_t launch_update_tc64(const F64Maps &maps, const F64Set &set, int k, cudaStream_t s, KernelTimer *kt)
 {
-    return launch_tc_f64(maps.a, maps.b, set, k, 1, set.Tmax, F64_TRAIL, k * (1 + set.b / PW), s, kt);
+    return launch_tc_f64(maps.a, maps.b, set, k, 1, set.Tmax, F64_TRAIL, tc64_slot(set.b, k, 0), s, kt);
 }
 
 cudaError_t launch_solo_init(const F64Set &set, cudaStream_t s, KernelTimer *kt)
@@ -1019,31 +1042,41 @@ cudaError_t launch_solo_init(const F64Set &set, cudaStream_t s, KernelTimer *kt)
     return cudaGetLastError();
 }
 
+static cudaError_t launch_slice_band(const F64Set &set, int k, int rows, int src, cudaStream_t s, KernelTimer *kt)
+{
+    EGS_LAUNCH(kt, KC_TRSM, s, k_slice_panel64<<<dim3((unsigned)(rows / 8), 1), 256, 0, s>>>(set, k, src));
+    return cudaGetLastError();
+}
+
 cudaError_t launch_winv(const F64Set &set, int k, float *wsp, cudaStream_t s, KernelTimer *kt)
 {
     const size_t sm = (size_t)8 * (set.b + 1) * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_winv_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * 1025 * sizeof(double));
     if (e != cudaSuccess) return e;
     EGS_LAUNCH(kt, KC_TRSM, s, k_winv_rows<<<(unsigned)(set.b / 8), 256, sm, s>>>(set, k, wsp));
-    return cudaGetLastError();
+    e = cudaGetLastError();
+    return e == cudaSuccess ? launch_slice_band(set, k, set.b, 2, s, kt) : e;
 }
 
 cudaError_t launch_band_solve(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt)
 {
     if (nb <= 0) return cudaSuccess;
-    EGS_LAUNCH(kt, KC_TRSM, s, k_slice_panel64<<<dim3((unsigned)((size_t)nb * set.b / 8), 1), 256, 0, s>>>(set, k));
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_tc_f64(maps.a, maps.b, set, k, 1, 1 + nb, F64_BAND, k * (1 + set.b / PW), s, kt);
+    const int rows = nb * set.b;
+    cudaError_t e = launch_slice_band(set, k, rows, 0, s, kt);
+    if (e == cudaSuccess) e = launch_tc_f64(maps.a, maps.b, set, k, 1, 1 + nb, F64_BAND, tc64_slot(set.b, k, 1), s, kt);
+    if (e == cudaSuccess) e = launch_slice_band(set, k, rows, 1, s, kt);
+    if (e == cudaSuccess) e = launch_tc_f64(maps.a, maps.lb, set, k, 1, 1 + nb, F64_RES, tc64_slot(set.b, k, 2), s, kt);
+    if (e == cudaSuccess) e = launch_slice_band(set, k, rows, 0, s, kt);
+    if (e == cudaSuccess) e = launch_tc_f64(maps.a, maps.b, set, k, 1, 1 + nb, F64_CORR, tc64_slot(set.b, k, 3), s, kt);
+    return e;
 }
 
 cudaError_t launch_band_update(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt)
 {
     if (nb <= 0) return cudaSuccess;
-    EGS_LAUNCH(kt, KC_TRSM, s, k_slice_panel64<<<dim3((unsigned)((size_t)nb * set.b / 8), 1), 256, 0, s>>>(set, k));
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_slice_band(set, k, nb * set.b, 0, s, kt);
     if (e != cudaSuccess) return e;
-    return launch_tc_f64(maps.a, maps.pb, set, k, 1, 1 + nb, F64_TRAIL, (k + 1) * (1 + set.b / PW) - 1, s, kt);
+    return launch_tc_f64(maps.a, maps.pb, set, k, 1, 1 + nb, F64_TRAIL, tc64_slot(set.b, k, 0), s, kt);
 }
 
 }  // namespace egs

@@ -36,7 +36,8 @@ struct F64Prob {
     double *vinv;             // diagonal tiles alone: V_k = L_kk^-T (T b x b, identities before), or NULL
     F64Rows panel;            // K = b: row r of tile m at row0 + (m - k - 1) b + r
     F64Rows inner;            // K = 64, the current 64-column block: row0 + (m - k) b + r; sl NULL: no slices
-    F64Rows w;                // diagonal tiles alone: K = b, the rows of L_kk^-1
+    F64Rows w, l;             // diagonal tiles alone: K = b, the rows of L_kk^-1 and of L_kk
+    double *y;                // diagonal tiles alone: the band rows' first solution, nb b x b
     unsigned long long *ctr;  // tc64_counters(b, T) zeroed work counters
     double *winv;             // inverses of the block's eight 8 x 8 diagonal blocks, two of kWinvDoubles (j & 1)
 };
@@ -60,14 +61,14 @@ struct F64Set {
     __device__ const F64Prob &get(int i) const { return arr ? arr[i] : one; }
 };
 
-// Work counters of a problem: per step one for the trailing update (a mixed factorisation: the band
-// solve) and one for each 64-column block's inner update; the last block has none, and its counter
-// is a mixed factorisation's band update's.
-inline size_t tc64_counters(int b, int T) { return (size_t)T * (1 + b / kF64Panel); }
+// Work counters of a problem, per step: the trailing update (a mixed factorisation: the band update),
+// the three products of a mixed factorisation's band solve, then each 64-column block's inner update.
+inline int tc64_slot(int b, int k, int i) { return k * (4 + b / kF64Panel) + i; }
+inline size_t tc64_counters(int b, int T) { return (size_t)tc64_slot(b, T, 0); }
 
 struct F64Maps {
-    CUtensorMap a, b, ia, ib;  // panel slices, inner slices; diagonal tiles alone: b is W's, pb the panel's
-    CUtensorMap pb;
+    CUtensorMap a, b, ia, ib;  // panel slices, inner slices; diagonal tiles alone: b is W's, pb the panel's, lb L_kk's
+    CUtensorMap pb, lb;
 };
 // Over slice arrays of rows (K = b) and irows (K = 64) rows.
 cudaError_t make_f64_maps(const F64Rows &panel, const F64Rows &inner, int b, F64Maps *maps);
@@ -84,10 +85,10 @@ F64Prob tc64_solo_problem(void *scratch, const Tiles &tl, DevStatus *st, double 
 cudaError_t make_f64_solo_maps(const F64Prob &p, F64Maps *maps);
 // Identities into V, the counters.
 cudaError_t launch_solo_init(const F64Set &set, cudaStream_t s, KernelTimer *kt);
-// The rows of W = L_kk^-1 = V_k^T: slices, and (wsp not NULL) the split-TF32 layout of the
-// off-band solve, row c: [hi | lo] of (float)W[c][.].
+// The rows of W = L_kk^-1 = V_k^T and of L_kk: slices, and (wsp not NULL) the split-TF32 layout of
+// the off-band solve, row c: [hi | lo] of (float)W[c][.].
 cudaError_t launch_winv(const F64Set &set, int k, float *wsp, cudaStream_t s, KernelTimer *kt);
-// Tiles (k + 1 .. k + nb, k): X = A W^T, in place.
+// Tiles (k + 1 .. k + nb, k): X L_kk^T = A, in place, by products with W and one correction.
 cudaError_t launch_band_solve(const F64Maps &maps, const F64Set &set, int k, int nb, cudaStream_t s, KernelTimer *kt);
 
 // The same without slices, for the DFMA updates; winv: 2 kWinvDoubles of scratch.
