@@ -173,7 +173,9 @@ __global__ void __launch_bounds__(256) k_diag64(const __grid_constant__ F64Set s
     __shared__ Chol64Smem sm;
     const F64Prob &P = set.get(blockIdx.y);
     const Tiles &tl = P.tl;
-    if (k >= tl.T || failed(P.st)) return;
+    // one answer for the CTA: work on the other stream may give up meanwhile, and the block's warps
+    // hand each other indexes
+    if (k >= tl.T || __syncthreads_or(failed(P.st))) return;
     const int b = tl.b;
     diag64_block(sm, tl.t64(k, k) + (size_t)j * PW * (b + 1), b, b - (j + 1) * PW,
                  P.z ? P.z + (size_t)k * b + j * PW : nullptr, P.winv + (j & 1) * kWinvDoubles,
