@@ -409,8 +409,9 @@ egs_status egs_predict(const double *locs_obs, const double *z_obs, int64_t n, c
  * tiles of tile x tile) is set to zero, so Sigma is block diagonal over
  * consecutive runs of super_tiles * tile locations (the last run holds the
  * rest), and l_IND = sum over the blocks of Eq. 1 on each block's locations
- * and measurements.  FP64; the blocks run as one batch of the batched
- * scheduler (one CUDA graph).  Sums over the blocks are in block order.
+ * and measurements.  FP64; the blocks run as one batch on the tensor cores,
+ * each launch covering one step of every block.  Sums over the blocks are in
+ * block order.  A single block is egs_loglik_ex's evaluation with this tile.
  *   locs  2n doubles (x then y), device or host;  z  n doubles, device or host
  *   tile  0 = 128;  super_tiles >= 1 (super_tiles * tile >= n gives exact l)
  *   info  loglik, logdet, quad summed over the blocks; band = super_tiles

@@ -1161,11 +1161,26 @@ egs_status egs_loglik_ind(const double *locs, const double *z, const double thet
     const int64_t bs = (int64_t)super_tiles * tile;
     const int64_t nblk = (n + bs - 1) / bs;
     if (nblk > (1 << 20)) return set_error(EGS_ERR_ARG, "egs_loglik_ind: too many blocks");
+    if (nblk == 1) {  // the exact likelihood
+        egs_opts o{};
+        o.tile = tile;
+        egs_info one{};
+        double l1 = NAN;
+        const egs_status st = egs_loglik_ex(locs, z, theta, n, EGS_FP64, &o, &l1, &one, stream);
+        if (st != EGS_OK && st != EGS_ERR_NOT_PD) return st;
+        if (info) {
+            *info = one;
+            info->band = super_tiles;
+        }
+        if (st != EGS_OK)
+            return set_error(st, "egs_loglik_ind: not positive definite at row %lld", (long long)one.fail_index);
+        if (out_loglik) *out_loglik = l1;
+        return EGS_OK;
+    }
     std::vector<int64_t> ns((size_t)nblk);
     for (int64_t i = 0; i < nblk; ++i) ns[(size_t)i] = std::min(bs, n - i * bs);
     egs_batch *B = nullptr;
-    // one block is the exact likelihood, and equals egs_loglik bit for bit
-    egs_status sc = batch_create((int32_t)nblk, ns.data(), tile, EGS_FP64, nblk > 1, true, &B);
+    egs_status sc = batch_create((int32_t)nblk, ns.data(), tile, EGS_FP64, true, true, &B);
     if (sc != EGS_OK) return sc;
     for (int i = 0; i < B->nprob; ++i) B->h_params[i] = P;
     cudaStream_t us = (cudaStream_t)stream;
