@@ -138,7 +138,8 @@ __device__ __forceinline__ bool potrf64_smem(double *A, int ld, int64_t row0, De
 // sub-partition, not latency:
 //  - L D L^T (no square root between pivots): with y ~ 1 / d from the hardware's approximation,
 //    e = 1 - d y, the column a / d = a y (1 + e + e^2) (Newton's iteration one order up) costs
-//    four instructions; the square roots are taken for all 64 columns at the end;
+//    four instructions; the square roots are taken for all 64 columns at the end.  A pivot whose
+//    reciprocal leaves the normal doubles is divided by instead;
 //  - panels of 4 columns: warps 0 .. 2 each factor the 4 x 4 block in lanes 0 .. 3, redundantly
 //    (each has a sub-partition of its own), while lanes 4 .. 31 carry 28 rows below it, so that
 //    the rows below cost no instruction;
@@ -157,10 +158,17 @@ struct Chol64Smem {
     int fail_j, claim;
 };
 
-// 1 / sqrt(d) for normal d > 0: the hardware's approximation and one step of Householder's
-// third-order iteration.
+// Positive with a biased exponent of 2 .. 2044: 1 / d and its approximation are normal numbers too.
+__device__ __forceinline__ bool recip_normal(double d)
+{
+    return (unsigned)__double2hiint(d) - 0x00200000u < 0x7FB00000u;
+}
+
+// 1 / sqrt(d), d > 0: the hardware's approximation and one step of Householder's third-order
+// iteration.
 __device__ __forceinline__ double rsqrt_iter(double d)
 {
+    if (!recip_normal(d)) return 1.0 / sqrt(d);
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
     const double e = fma(-(d * y), y, 1.0);
@@ -171,18 +179,11 @@ __device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld
                                          DevStatus *st)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // a block far from 1 is scaled by 4^h, so that the reciprocals stay in range
-    const int e0 = ((__double2hiint(A[0]) >> 20) & 0x7FF) - 1023;
-    const int h = (e0 > 400 || e0 < -400) && e0 != 1024 ? -(e0 >> 1) : 0;
     double v[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
         const int e = tid + 256 * q;
         v[q] = (e & 63) <= (e >> 6) ? A[(size_t)(e >> 6) * ld + (e & 63)] : 0.0;
-    }
-    if (h != 0) {
-#pragma unroll
-        for (int q = 0; q < 16; ++q) v[q] = scalbn(v[q], 2 * h);
     }
 #pragma unroll
     for (int q = 0; q < 16; ++q) sm.S[(tid + 256 * q) >> 6][tid & 63] = v[q];
@@ -209,16 +210,19 @@ __device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const double d = __shfl_sync(0xffffffffu, a[j], j);
-                // normal and positive by its high word, the rest by an FP64 comparison
-                if ((unsigned)__double2hiint(d) - 0x00100000u >= 0x7FE00000u && ok && !(d > 0.0)) {
-                    ok = false;
-                    if (tid == 0) sm.fail_j = p0 + j;
+                if (recip_normal(d)) {
+                    double y;
+                    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+                    const double e = fma(-d, y, 1.0);
+                    const double ay = a[j] * y, u = fma(e, e, e);
+                    w[j] = fma(ay, u, ay);
+                } else {
+                    if (ok && !(d > 0.0)) {
+                        ok = false;
+                        if (tid == 0) sm.fail_j = p0 + j;
+                    }
+                    w[j] = a[j] / d;
                 }
-                double y;
-                asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-                const double e = fma(-d, y, 1.0);
-                const double ay = a[j] * y, u = fma(e, e, e);
-                w[j] = fma(ay, u, ay);
 #pragma unroll
                 for (int c = j + 1; c < 4; ++c) a[c] = fma(-a[j], __shfl_sync(0xffffffffu, w[j], c), a[c]);
             }
@@ -284,14 +288,6 @@ __device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld
     const int jc = tid & 63;
     const double rj = sm.rd[jc];
     for (int i = tid >> 6; i < 64 + zr; i += 4) sm.S[i][jc] = jc <= i ? sm.S[i][jc] * rj : 0.0;
-    if (h != 0) {
-        __syncthreads();
-        for (int i = tid >> 6; i < 64; i += 4) sm.S[i][jc] = scalbn(sm.S[i][jc], -h);
-        if (tid < 64) {
-            sm.rd[tid] = scalbn(sm.rd[tid], h);
-            if (z) sm.S[64][tid] = scalbn(sm.S[64][tid], h);
-        }
-    }
     __syncthreads();
     return true;
 }
