@@ -148,8 +148,8 @@ __device__ __forceinline__ bool potrf64_smem(double *A, int ld, int64_t row0, De
 // 64 pivots x 22 / 4 instructions of panels, about 400 of updates: 43 us with the launch (115 us
 // with 16-column panels, a thread per row below them and a square root per pivot).
 //
-// Leaves L (zero upper half), y in row 64 and 1 / L_jj in sm; false if a pivot is not positive
-// (its row is recorded as row0 + j).
+// Leaves L (zero upper half), y in row 64 and 1 / L_jj in sm; false if a pivot is not positive and
+// finite (its row is recorded as row0 + j).
 // ---------------------------------------------------------------------------
 struct Chol64Smem {
     double S[65][65];
@@ -217,7 +217,7 @@ __device__ __forceinline__ bool chol64_s(Chol64Smem &sm, const double *A, int ld
                     const double ay = a[j] * y, u = fma(e, e, e);
                     w[j] = fma(ay, u, ay);
                 } else {
-                    if (ok && !(d > 0.0)) {
+                    if (ok && !(d > 0.0 && d < __longlong_as_double(0x7FF0000000000000ll))) {
                         ok = false;
                         if (tid == 0) sm.fail_j = p0 + j;
                     }
