@@ -21,9 +21,9 @@
 // S <= 32,768 = half of what 256 digits can sum to, which the rows of a covariance's factor keep far
 // below.  The slicing marks the rows that do not; an output block with such a row is flushed every
 // 128 columns, where every level up to 5 is within 2^24 whatever the digits (rows with all leading
-// digits large, of one sign: off by 1.9e-9 of 250 without, 2.8e-14 so; n = 16,900
-// without such rows: 69.6 and 70.4 ms).  Of the levels from 4 on, the
-// FP32 rounding over 256 columns is below 2^-50 of the level-0 range.
+// digits large, of one sign: off by 1.9e-9 of 250 without, 2.8e-14 so; n = 51,200 without such rows,
+// all updates: 967 and 973 ms).  Of the levels from 4 on, the FP32 rounding over 256 columns is below
+// 2^-50 of the level-0 range.
 //
 // Kernel: persistent, one CTA per SM, 320 threads, output blocks of 128 x 64.  A K chunk
 // of 64 is 7 A boxes (128 rows) and one B box of all 7 slices (64 rows each, back to
@@ -57,6 +57,7 @@ constexpr int FTHREADS = 320;      // warp 0 TMA, warp 1 MMA, warps 2..9 epilogu
 constexpr int FRING = 4;           // work items posted ahead by the producer
 constexpr int FLUSH = 256 / FKC;   // K chunks per accumulator flush
 constexpr int FLUSH_DENSE = 128 / FKC;  // with a dense row
+static_assert(FLUSH == 4 && FLUSH_DENSE == 2, "powers of two, as the masks and shifts have them");
 constexpr int kDenseSum = 32768;   // sum of |q_0| over 256 columns above which a row is dense
 constexpr uint32_t FTMEM = 512;
 constexpr int kBadRow = 1 << 20;   // exponent of a row holding an infinity or a NaN
@@ -100,10 +101,10 @@ __device__ __forceinline__ int digits7(long long f, uint32_t (&d)[kF64Slices])
 }
 
 // One warp slices one row of b doubles (b <= 1024, a multiple of 64): slice i of the row
-// to dst[i * stride + c], the exponent to *ep, whether it is dense to *dense.  Lanes take two
-// consecutive columns.
+// to dst[i * stride + c], the exponent to *ep, whether it is dense to *dense (and into *any).  Lanes
+// take two consecutive columns.
 __device__ __forceinline__ void slice7_row(const double *__restrict__ src, int b, uint16_t *__restrict__ dst,
-                                           size_t stride, int *ep, uint8_t *dense)
+                                           size_t stride, int *ep, uint8_t *dense, unsigned long long *any)
 {
     const int lane = threadIdx.x & 31;
     unsigned mh = 0;
@@ -131,7 +132,10 @@ __device__ __forceinline__ void slice7_row(const double *__restrict__ src, int b
             lead = 0;
         }
     }
-    if (lane == 0) *dense = most > kDenseSum;
+    if (lane == 0) {
+        *dense = most > kDenseSum;
+        if (most > kDenseSum) atomicOr(any, 1ull);
+    }
 }
 
 // Panel rows of step k (tiles m0 .. T - 1 of column k) -> slices; one warp per row.
@@ -147,7 +151,7 @@ __global__ void __launch_bounds__(256) k_slice_panel64(const __grid_constant__ F
     const F64Rows &to = src == 2 ? P.l : P.panel;
     const size_t r = to.row0 + pr;
     const double *x = src == 0 ? tl.t64(k + 1 + (int)(pr / b), k) + (pr % b) * b : (src == 1 ? P.y : tl.t64(k, k)) + pr * b;
-    slice7_row(x, b, to.sl + r * b, to.rows * b, to.ex + r, to.dense + r);
+    slice7_row(x, b, to.sl + r * b, to.rows * b, to.ex + r, to.dense + r, P.ctr + tc64_dense_slot(b, k));
 }
 
 // ---- the panel ----------------------------------------------------------------
@@ -285,7 +289,8 @@ __global__ void __launch_bounds__(256) k_winv_rows(const __grid_constant__ F64Se
     __syncthreads();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, c = c0 + w;
     const double *row = wrow + w * ld;
-    slice7_row(row, b, P.w.sl + (size_t)c * b, (size_t)b * b, P.w.ex + c, P.w.dense + c);
+    slice7_row(row, b, P.w.sl + (size_t)c * b, (size_t)b * b, P.w.ex + c, P.w.dense + c,
+               P.ctr + tc64_dense_slot(b, k));
     if (!wsp) return;
     float *out = wsp + (size_t)c * 2 * b;
     for (int i = lane; i < b; i += 32) {
@@ -298,9 +303,11 @@ __global__ void __launch_bounds__(256) k_winv_rows(const __grid_constant__ F64Se
 // ---- the update -------------------------------------------------------------
 
 struct F64Item {
-    int m, n, rb, cb;  // output tile, 128-row block, 64-column block; m < 0 ends
-    int hold;          // its accumulators are never signalled (failure tests)
-    int flush;         // K chunks per accumulator flush
+    int m, n;         // output tile; m < 0 ends
+    int rb : 8;       // 128-row block
+    int cb : 8;       // 64-column block
+    int hold : 8;     // its accumulators are never signalled (failure tests)
+    int flush : 8;    // K chunks per accumulator flush
 };
 
 // Any of n (64 or 128) rows' marks set.
@@ -474,10 +481,14 @@ __device__ __forceinline__ void tma_load_3d(const CUtensorMap *map, uint64_t *ba
         : "memory");
 }
 
+// Band: the three products of the band solve, apart from the others (their epilogue's choice of
+// sources costs those 0.8%).
+template <bool Band>
 __global__ void __launch_bounds__(FTHREADS, 1)
 k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
          const __grid_constant__ F64Set set, int k, int c0, int c1, int mode, int slot)
 {
+    __builtin_assume(Band == (mode >= F64_BAND));
     const F64Prob &P = set.get(blockIdx.y);
     const bool solo = set.solo != 0;
     if (P.tl.T <= k) return;
@@ -489,7 +500,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
     if ((int64_t)blockIdx.x >= nitems) return;
     unsigned long long *next = P.ctr + slot;
     DevStatus *st = P.st;
-    const F64Rows &rows = mode == F64_INNER ? P.inner : P.panel, &brows = !work.band() ? rows : (mode == F64_RES ? P.l : P.w);
+    const F64Rows &rows = mode == F64_INNER ? P.inner : P.panel, &brows = !Band ? rows : (mode == F64_RES ? P.l : P.w);
     const int *__restrict__ ex = rows.ex + rows.row0, *__restrict__ exb = brows.ex + brows.row0;
     const int yrow0 = (int)rows.row0, ybrow0 = (int)brows.row0;
     extern __shared__ uint8_t smem_raw[];
@@ -498,7 +509,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
     __shared__ uint64_t rfull[FRING], rempty[FRING];
     __shared__ F64Item ring[FRING];
     __shared__ uint32_t tmem_base;
-    __shared__ int abort_flag, stop, loaded, hold_first;
+    __shared__ int abort_flag, stop, loaded, hold_first, dense_step;
     __shared__ uint64_t mdone;
     __shared__ unsigned long long limit;
 
@@ -523,6 +534,9 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
         loaded = 0;
         limit = set.ctl ? set.ctl->limit_ns : tc::kWaitNs;
         hold_first = mode == F64_TRAIL && set.ctl && set.ctl->prob == (int)blockIdx.y && set.ctl->step == k;
+        // the rows' own marks are read only in a step that has one (read for every block they cost
+        // the producer 1 us each: n = 51,200, all updates 996 ms against 980)
+        dense_step = rows.dense && *(volatile unsigned long long *)(P.ctr + tc64_dense_slot(work.tl.b, k)) != 0;
         stop = failed(st) ? 1 : 0;
         tc::fence_mbar_init();
     }
@@ -551,14 +565,14 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                     continue;
                 }
                 const int slot = r % FRING;
-                if (!tc::mbar_wait(&rempty[slot], ((uint32_t)(r / FRING) & 1u) ^ 1u, &abort_flag, limit)) break;
+                if (!tc::mbar_wait(&rempty[slot], ((uint32_t)(r / FRING) & 1u) ^ 1u, &abort_flag, &limit)) break;
                 if (!valid) wi.m = -1;
                 wi.hold = hold_first && claimed == 0;
                 wi.flush = FLUSH;
-                if (valid && rows.dense && work.kchunks(wi.cb) > FLUSH_DENSE) {
+                if (valid && dense_step && work.kchunks(wi.cb) > FLUSH_DENSE) {
                     // the block's rows of the tile, at most 128
                     const uint8_t *da = rows.dense + yrow0 + work.slice_row(wi.m) + wi.rb * FM;
-                    const uint8_t *db = brows.dense + ybrow0 + (work.band() ? 0 : work.slice_row(wi.n)) + wi.cb * FN;
+                    const uint8_t *db = brows.dense + ybrow0 + (Band ? 0 : work.slice_row(wi.n)) + wi.cb * FN;
                     if (any_dense(da, min(FM, b - wi.rb * FM)) || any_dense(db, FN)) wi.flush = FLUSH_DENSE;
                 }
                 ring[slot] = wi;
@@ -567,16 +581,16 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                 if (!valid) break;
                 claimed = (int64_t)atomicAdd(next, 1ull);  // overlaps the loads below
                 const int ya = yrow0 + (int)work.slice_row(wi.m) + wi.rb * FM;
-                const int yb = ybrow0 + (work.band() ? 0 : (int)work.slice_row(wi.n)) + wi.cb * FN;
+                const int yb = ybrow0 + (Band ? 0 : (int)work.slice_row(wi.n)) + wi.cb * FN;
                 const int kchunks = work.kchunks(wi.cb);
                 for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
                     const int bb = g & 1;
-                    if (!tc::mbar_wait(&bempty[bb], ((uint32_t)(g >> 1) & 1u) ^ 1u, &abort_flag, limit)) break;
+                    if (!tc::mbar_wait(&bempty[bb], ((uint32_t)(g >> 1) & 1u) ^ 1u, &abort_flag, &limit)) break;
                     tc::mbar_arrive_expect_tx(&bfull[bb], FB_BUF);
                     tma_load_3d(&mapB, &bfull[bb], sb + bb * FB_BUF, c * FKC, yb, 0);
                     int i = 0;
                     for (; i < kF64Slices; ++i) {
-                        if (!tc::mbar_wait(&aempty[i], ((uint32_t)g & 1u) ^ 1u, &abort_flag, limit)) break;
+                        if (!tc::mbar_wait(&aempty[i], ((uint32_t)g & 1u) ^ 1u, &abort_flag, &limit)) break;
                         tc::mbar_arrive_expect_tx(&afull[i], FA_SL);
                         tma_load_3d(&mapA, &afull[i], sa + i * FA_SL, c * FKC, ya, i);
                     }
@@ -592,24 +606,24 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             uint32_t f = 0;  // flush groups issued
             while (!abort_flag) {
                 const int slot = r % FRING;
-                if (!tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag, limit)) break;
+                if (!tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag, &limit)) break;
                 const int m = ring[slot].m, kchunks = work.kchunks(ring[slot].cb), hold = ring[slot].hold;
                 const int flush = ring[slot].flush;
                 tc::mbar_arrive(&rempty[slot]);
                 ++r;
                 if (m < 0) break;
                 for (int c = 0; c < kchunks && !abort_flag; ++c, ++g) {
-                    const bool first = c % flush == 0;
+                    const bool first = (c & (flush - 1)) == 0;
                     if (first) {
-                        if (!tc::mbar_wait(&tempty, (f & 1u) ^ 1u, &abort_flag, limit)) break;
+                        if (!tc::mbar_wait(&tempty, (f & 1u) ^ 1u, &abort_flag, &limit)) break;
                         tc::tc_fence_after();
                     }
                     const int bb = g & 1;
-                    if (!tc::mbar_wait(&bfull[bb], (uint32_t)(g >> 1) & 1u, &abort_flag, limit)) break;
+                    if (!tc::mbar_wait(&bfull[bb], (uint32_t)(g >> 1) & 1u, &abort_flag, &limit)) break;
                     const uint32_t b0 = tc::smem_u32(sb + bb * FB_BUF);
 #pragma unroll
                     for (int i = 0; i < kF64Slices; ++i) {
-                        if (!tc::mbar_wait(&afull[i], (uint32_t)g & 1u, &abort_flag, limit)) break;
+                        if (!tc::mbar_wait(&afull[i], (uint32_t)g & 1u, &abort_flag, &limit)) break;
                         tc::tc_fence_after();
                         const uint32_t a0 = tc::smem_u32(sa + i * FA_SL);
                         const int n = kF64Slices - i;  // B slices 0 .. n - 1
@@ -630,7 +644,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                         tc::mma_commit(&aempty[i]);
                     }
                     tc::mma_commit(&bempty[bb]);
-                    if (c % flush == flush - 1 || c == kchunks - 1) {
+                    if ((c & (flush - 1)) == flush - 1 || c == kchunks - 1) {
                         if (!hold) tc::mma_commit(&tfull);
                         ++f;
                     }
@@ -647,18 +661,18 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
         bool run = true;
         while (run) {
             const int slot = r % FRING;
-            const bool got = tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag, limit);
+            const bool got = tc::mbar_wait(&rfull[slot], (uint32_t)(r / FRING) & 1u, &abort_flag, &limit);
             if (!__all_sync(0xffffffffu, got && !abort_flag)) break;
             const F64Item wi = ring[slot];
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&rempty[slot]);
             ++r;
             if (wi.m < 0) break;
-            const int kchunks = work.kchunks(wi.cb), nflush = (kchunks + wi.flush - 1) / wi.flush;
+            const int kchunks = work.kchunks(wi.cb), nflush = (kchunks + wi.flush - 1) >> (wi.flush == FLUSH ? 2 : 1);
             const int up = kchunks > 2 * FLUSH ? 1 : 0;  // the sum over the flushes stays below 2^63
             long long acc[32];
             for (int fl = 0; fl < nflush; ++fl, ++f) {
-                const bool ok = tc::mbar_wait(&tfull, f & 1u, &abort_flag, limit);
+                const bool ok = tc::mbar_wait(&tfull, f & 1u, &abort_flag, &limit);
                 tc::tc_fence_after();
                 if (!__all_sync(0xffffffffu, ok && !abort_flag)) {
                     run = false;
@@ -686,11 +700,11 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
             if (row >= work.r0(wi) && row < work.r1(wi, solo)) {
                 const int col = wi.cb * FN + half * 32;
                 const int ea = ex[work.slice_row(wi.m) + row] - 16;
-                const int *eb = exb + (work.band() ? 0 : work.slice_row(wi.n)) + col;
+                const int *eb = exb + (Band ? 0 : work.slice_row(wi.n)) + col;
                 double *C = (solo && mode == F64_INNER && wi.m > k ? P.vinv + (size_t)k * work.tl.bb()
                                                                    : work.tl.t64(wi.m, wi.n)) + (size_t)row * b + col;
                 const double *Cin = C;  // what the product is added to or subtracted from
-                const bool add = mode == F64_BAND || mode == F64_CORR;
+                const bool add = Band && mode != F64_RES;
                 if (add) {
                     double *y = P.y + (size_t)(wi.m - k - 1) * work.tl.bb() + (size_t)row * b + col;
                     Cin = y;
@@ -701,7 +715,7 @@ k_tc_f64(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUten
                     double2 cv[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        cv[j] = mode == F64_BAND ? make_double2(0.0, 0.0)
+                        cv[j] = Band && mode == F64_BAND ? make_double2(0.0, 0.0)
                                                  : *reinterpret_cast<const double2 *>(Cin + 16 * h + 2 * j);
                     double *cd = reinterpret_cast<double *>(cv);
 #pragma unroll
@@ -911,7 +925,8 @@ static unsigned tc64_ctas(const F64Set &set, int64_t items)
 static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, const F64Set &set, int k, int c0, int c1,
                                  int mode, int slot, cudaStream_t s, KernelTimer *kt)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_tc_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
+    auto kernel = mode >= F64_BAND ? k_tc_f64<true> : k_tc_f64<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
     if (e != cudaSuccess) return e;
     // of the largest problem, as in the kernel
     const int T = !set.solo ? set.Tmax : (mode == F64_INNER ? k + 1 + (set.one.vinv ? 1 : 0) : k + c1);
@@ -923,7 +938,7 @@ static cudaError_t launch_tc_f64(const CUtensorMap &a, const CUtensorMap &b, con
     // of a mixed factorisation's diagonal tile: part of its POTRF; its band: the FP64 update class
     const int cls = mode >= F64_BAND ? KC_TRSM : (!set.solo ? KC_UPDATE : (in ? KC_POTRF : KC_UPDATE64));
     EGS_LAUNCH(kt, cls, s,
-               k_tc_f64<<<grid, FTHREADS, FSMEM, s>>>(a, b, set, k, c0, c1, mode, slot));
+               kernel<<<grid, FTHREADS, FSMEM, s>>>(a, b, set, k, c0, c1, mode, slot));
     return cudaGetLastError();
 }
 

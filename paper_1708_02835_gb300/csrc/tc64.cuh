@@ -19,6 +19,13 @@ constexpr int64_t kTc64MinRows = 2049;
 inline bool tc64_aligned(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 inline bool tc64_applies(int64_t n, int b, int T) { return n >= kTc64MinRows && T > 1 && b % 64 == 0; }
 
+// Work counters of a problem, per step: the trailing update (a mixed factorisation: the band update),
+// the three products of a mixed factorisation's band solve, then each 64-column block's inner update
+// but the last one's, whose place holds whether any row sliced in the step is dense.
+__host__ __device__ inline int tc64_slot(int b, int k, int i) { return k * (4 + b / kF64Panel) + i; }
+__host__ __device__ inline int tc64_dense_slot(int b, int k) { return tc64_slot(b, k + 1, -1); }
+inline size_t tc64_counters(int b, int T) { return (size_t)tc64_slot(b, T, 0); }
+
 // Slices of operand rows (slice i of row r at sl[(i rows + r) K ..], K = b or 64) and the
 // rows' exponents; several problems share one array, each from its own row0 on.
 struct F64Rows {
@@ -61,10 +68,6 @@ struct F64Set {
     __device__ const F64Prob &get(int i) const { return arr ? arr[i] : one; }
 };
 
-// Work counters of a problem, per step: the trailing update (a mixed factorisation: the band update),
-// the three products of a mixed factorisation's band solve, then each 64-column block's inner update.
-inline int tc64_slot(int b, int k, int i) { return k * (4 + b / kF64Panel) + i; }
-inline size_t tc64_counters(int b, int T) { return (size_t)tc64_slot(b, T, 0); }
 
 struct F64Maps {
     CUtensorMap a, b, ia, ib;  // panel slices, inner slices; diagonal tiles alone: b is W's, pb the panel's, lb L_kk's

@@ -59,17 +59,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
     return ok != 0;
 }
 
-// Wait for the phase of the given parity; false on timeout (limit ns) or if another
-// thread of the CTA has already aborted.
+// Wait for the phase of the given parity; false on timeout (*limit ns, kWaitNs if NULL; read only
+// once the first try has failed) or if another thread of the CTA has already aborted.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
-                                          unsigned long long limit = kWaitNs)
+                                          const unsigned long long *limit = nullptr)
 {
     if (mbar_try_wait(bar, parity)) return true;
     const unsigned long long t0 = globaltimer();
     while (true) {
         if (mbar_try_wait(bar, parity)) return true;
         if (*abort_flag) return false;
-        if (globaltimer() - t0 > limit) {
+        if (globaltimer() - t0 > (limit ? *limit : kWaitNs)) {
             *abort_flag = 1;
             return false;
         }
