@@ -374,10 +374,16 @@ def run_batched(a, egs):
              "persistent_tasks": B.tasks, "autotune_ms": {str(k): v for k, v in tune.items()},
              "potrf_tflops_equiv": tfl, "failed": int(np.sum(stat != 0)), "workspace_gb": B.workspace_bytes / 1e9}
         if prec == "fp64":
-            r["roofline"] = {"bound": "alu", "kernel": "kb_dag (persistent FP64 batch: generation, tile Cholesky, "
-                                                       "forward solve)",
-                             "achieved": tfl, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": tfl / FP64_PEAK_TFLOPS,
-                             "note": "sum of n^3/3 over the problems / batch time; generation and solve time included"}
+            # problems of up to 2,048 rows run on the FP64 pipe, the others' updates as slice products
+            small = sum(n ** 3 / 3.0 for n in ns if n <= 2048)
+            pk = f64_tensor_peak()
+            floor = small / FP64_PEAK_TFLOPS + (flops - small) / pk["tflops"]
+            peak = flops / floor
+            r["roofline"] = {"bound": "alu", "kernel": "kb_dag (n <= 2,048: persistent launch on the FP64 pipe), k_tc_f64 "
+                                                       "and k_solve64 (larger problems)",
+                             "achieved": tfl, "peak": peak, "unit": "TFLOP/s", "frac": tfl / peak,
+                             "note": "sum of n^3/3 over the problems / batch time, generation and solves included; peak: "
+                                     "the FP64 pipe for problems of up to 2,048 rows, " + pk["source"] + " for the others"}
         B.close()
         return r, out
 

@@ -78,8 +78,8 @@ typedef enum {
     EGS_FP64 = 0,     /* everything in double */
     EGS_MIX_FP32 = 1, /* FP64 band; off-band tiles FP32; updates of band tiles
                          (and of the tiles within egs_opts.xband of the
-                         diagonal) FP64-accurate (DFMA, or exact BF16 slice
-                         products on tcgen05), of the other off-band tiles on
+                         diagonal) FP64-accurate (exact BF16 slice products
+                         on tcgen05), of the other off-band tiles on
                          tcgen05 as split FP16 (lo hi' + hi lo' + hi hi' of
                          row-scaled FP16 halves, FP32-accurate products); the
                          off-band TRSM as the split-TF32 product with the
@@ -104,8 +104,8 @@ typedef struct {
      * egs_opts.timing is set).  timing = 1: per phase; timing = 2: also the
      * summed duration of each kernel class (one event pair per launch). */
     double ms_generate;   /* Sigma generation */
-    double ms_factor;     /* tile Cholesky */
-    double ms_solve;      /* solve, refinement and reductions */
+    double ms_factor;     /* tile Cholesky; EGS_FP64: with the forward solve */
+    double ms_solve;      /* reductions; mixed precisions: solves and refinement too */
     double ms_total;      /* whole evaluation */
     double ms_potrf;      /* timing = 2: diagonal-tile POTRF kernels */
     double ms_trsm;       /* timing = 2: panel TRSM kernels */
@@ -124,7 +124,11 @@ typedef struct {
     int32_t timing;        /* nonzero: record per-phase CUDA events into egs_info;
                               >= 3: also keep a per-launch trace (egs_trace_last) */
     void *workspace;       /* caller-owned device workspace, or NULL (library allocates) */
-    size_t workspace_bytes;
+    size_t workspace_bytes;/* egs_loglik_workspace_bytes.  EGS_FP64 above 2048 rows: with less
+                              (2% less is enough for the matrix), or a workspace that is not
+                              on a 16-byte boundary, the call takes the FP64-pipe update
+                              instead of the tensor-core one, as it does when its own
+                              allocation fails: n = 102,400 then takes 288 s instead of 8 */
     int32_t distance;      /* 0: Euclidean on (x, y); 1: great-circle distance on
                               (longitude, latitude) in degrees by the haversine
                               formula (Section 7.4) on a sphere of 6371 km, so
@@ -229,7 +233,12 @@ egs_status egs_matern_tiles(const double *locs, int64_t n, const double theta[3]
  * diagonal tile, TRSM on the panel, SYRK/GEMM on the trailing tiles).
  *   tiles       device, lower tiles of Sigma in EGS_FP64 layout; on return L.
  *               Above 2048 rows the tensor-core update needs a 16-byte
- *               boundary; tiles without it take the slower FP64-pipe update
+ *               boundary; tiles without it take the slower FP64-pipe update.
+ *               Its products are accurate relative to the largest entries of
+ *               their two rows (about 2^-53.8 of their product), as the
+ *               backward error of a Cholesky factorisation is: an entry of L
+ *               far below sqrt(Sigma_ii) is accurate to 1e-16 of that, not of
+ *               itself
  *   fail_index  host; first failing row or -1.  The call synchronises stream.
  * EGS_ERR_ARG if tiles is not device memory.
  */

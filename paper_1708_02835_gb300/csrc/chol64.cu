@@ -15,8 +15,8 @@
 // (tc64_applies).  Every output element is updated by exactly one thread in a
 // fixed order, so results are bitwise reproducible, and the persistent batch
 // (batched_dag.cu) runs the same operations on every element.  n = 777 (tile
-// 128): 4.51 ms with 32 x 32 task-graph POTRFs and whole-tile solves, 1.63 ms now;
-// n = 1,600 (tile 320): 7.44 and 3.42 ms.
+// 128): 4.51 ms with 32 x 32 task-graph POTRFs and whole-tile solves, 1.60 ms now;
+// n = 1,600 (tile 320): 7.44 and 3.37 ms.
 #include "blocks.cuh"
 #include "tc64.cuh"
 

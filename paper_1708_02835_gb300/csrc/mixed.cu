@@ -3,8 +3,9 @@
 // Storage: tiles with i - j < band (the diagonal band) stay FP64; the others
 // are FP32.  Per step k of the right-looking tile Cholesky (Section 5.2):
 //   POTRF  L_kk in FP64;
-//   TRSM   band rows (m - k < band) in FP64; the other rows in the FP32
-//          mode as the product with W = L_kk^-1 (inverted in FP64) on tcgen05
+//   TRSM   band rows (m - k < band) FP64-accurate, by products with
+//          W = L_kk^-1 and a correction (tc64.cu); the other rows in the FP32
+//          mode as the product with W on tcgen05
 //          in split TF32, in the TF32 / BF16 modes in FP32 arithmetic with
 //          L_kk rounded to FP32; every solved tile is also written to the
 //          panel buffer in the tensor-core operand format (TF32-rounded FP32,
@@ -16,8 +17,8 @@
 //          from the others.  FP32 mode (split TF32): each update takes the
 //          precision of its output tile, as in a mixed-precision tile
 //          Cholesky that keeps the band in double -- band outputs in FP64 on
-//          the stored FP32 / FP64 values (band x band on DFMA, the others as
-//          exact BF16 slice products on tcgen05, ozaki.cu), off-band outputs
+//          the stored FP32 / FP64 values (exact BF16 slice products on
+//          tcgen05, ozaki.cu), off-band outputs
 //          on tcgen05 as lo hi^T + hi lo^T + hi hi^T (FP32-accurate products).
 // The log-determinant 2 sum log L_ii is reduced in FP64 from the FP64
 // diagonal tiles.  The quadratic form Z^T Sigma^-1 Z is won back in FP64 by

@@ -13,7 +13,11 @@
 //   x . y = 2^(ex + ey - 16) sum_L 2^-8L sum_{i+j=L} q_i(x) . q_j(y)
 // and the levels L = 0..6 (28 pairs) are kept.  The dropped ones and the rounding of the
 // last digit amount to about 2^-53.8 sqrt(K / 512) of |x|_max |y|_max, below the rounding
-// of a length-K chain of DFMAs.
+// of a length-K chain of DFMAs.  That bound is relative to the rows' largest entries, i.e. to
+// sqrt(a_mm a_nn), as Cholesky's backward error is; relative to |x| . |y| of the entry itself a
+// DFMA chain keeps more where that is far smaller (n = 4,096, range 0.03: absolute error 8.5e-17 against
+// 3.4e-16, relative to |x| . |y| up to 8e-4 against 3e-15), so entries of L far below
+// sqrt(a_mm) have their digits relative to it and not to themselves.
 // Each level has its own FP32 accumulator in TMEM, flushed to FP64 every K = 256 columns, and a sum
 // of integers in units of its level is exact as long as it stays within 2^24 of them.  Over 256
 // columns levels 0 and 1 always do.  With S the largest sum of |q_0| over such 256 columns in either
@@ -30,14 +34,15 @@
 // back).  A slice i multiplies B slices 0 .. 6-i in one or two MMAs (N <= 256) whose D
 // address is shifted by 64 i columns, so the block of B slice j lands in level i + j:
 // each A slice is read from shared memory once or twice per K step instead of once per
-// pair.  Shared memory (reads by the MMAs 96 KB and TMA writes 42 KB per 16-column K
-// step of 896 tensor clocks, at 128 B / clock) is what bounds the kernel; 128 x 64
-// with 7 x 64 accumulator columns is the largest block that fits TMEM.
+// pair; 128 x 64 with 7 x 64 accumulator columns is the largest block that fits TMEM.
 // A slots are freed slice by slice (7 slots of 16 KB), B is double buffered (2 x 56 KB).
+// What bounds it (ncu, n = 8,192, K = 512): the tensor pipe is busy 56% of the time and shared
+// memory 48%; the rest is the A slices' single buffering, a slot being refilled 21 of 28 product
+// units before its next use, and the epilogue before the accumulators are free.
 // Measured (n = 16,900, tile 512, all 33 updates): 1,361 ms with DFMA, 40.8 ms here with FP64
 // additions in the epilogue, 33 ms with integer ones, i.e. 53 TFLOP/s of FP64-equivalent work,
-// 1,490 executed on the tensor cores.  Error of the factor, rms of Sigma - L L^T in twice the precision (n = 2,304, tile 256): 2.5e-17 against
-// 3.2e-17 with DFMA (theta = (1, 0.1, 0.5)), 2.9e-17 / 6.3e-17 (nu = 1.3), 9.9e-18 / 1.0e-17
+// 1,490 executed on the tensor cores.  Error of the factor, rms of Sigma - L L^T in twice the
+// precision (n = 2,304, tile 256): 2.5e-17 against 3.2e-17 with DFMA (theta = (1, 0.1, 0.5)), 2.9e-17 / 6.3e-17 (nu = 1.3), 9.9e-18 / 1.0e-17
 // (range 0.03).
 #include "blocks.cuh"
 #include "tc_common.cuh"

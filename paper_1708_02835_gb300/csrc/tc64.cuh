@@ -9,10 +9,11 @@ namespace egs {
 constexpr int kF64Slices = 7;
 constexpr int kF64Panel = 64;  // width of the blocks a tile column is factored in
 
-// FP64 factorisations take the tensor cores above this many rows.  Below it the chain of
-// diagonal blocks sets the time (n = 1,600: DFMA trailing updates 1.1 of 3.4 ms), and the
-// persistent batch, which runs the DFMA routines, stays bit for bit equal to a single evaluation;
-// above it the updates do (n = 5,000: 36.4 ms by DFMA, 2.5 here).
+// FP64 factorisations take the tensor cores above this many rows.  The line is the persistent
+// batch's: it runs the DFMA routines and equals single evaluations bit for bit.  The tensor cores
+// alone would win from about 700 rows on (evaluations by DFMA / by slice products, default tile:
+// n = 500 0.88 / 0.89 ms, 777 1.58 / 1.44, 1,600 3.67 / 2.55, 2,048 5.42 / 3.16, 2,049 6.11 / 3.36,
+// 4,096 25.3 / 7.05).
 constexpr int64_t kTc64MinRows = 2049;
 // They also need memory that starts on a 16-byte boundary (tc64_aligned: TMA boxes, pairs of doubles
 // in the update's epilogue); a caller's tiles or workspace without that take the DFMA update.

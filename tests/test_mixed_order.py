@@ -26,7 +26,7 @@ def test_every_tile_access_is_ordered(tmp_path):
     assert int(v["seen"]) > 100_000 and int(v["races"]) == 0 and int(v["wrong"]) == 0, out
 
 
-def test_the_driver_follows_the_rule():
+def test_factor_mixed_follows_the_rule():
     """The order of the calls in factor_mixed that the model restates."""
     src = open(os.path.join(CSRC, "mixed.cu")).read()
     body = src[src.index("cudaError_t factor_mixed("):src.index("// out = L^-1 rhs with the inverted diagonal tiles")]
