@@ -54,6 +54,15 @@ constexpr int kMaxDevices = 64;
 static std::mutex g_pool_mu;
 static cudaMemPool_t g_pools[kMaxDevices] = {};
 
+// Making or trimming a pool is no stream operation, but the runtime counts both among the calls that
+// a capture on this thread forbids (egs_matern_tiles may be captured, as the first call too); in this
+// mode it allows them.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 static cudaError_t lib_pool(cudaMemPool_t *pool)
 {
     int dev = 0;
@@ -62,6 +71,7 @@ static cudaError_t lib_pool(cudaMemPool_t *pool)
     if (dev >= kMaxDevices) return cudaDeviceGetDefaultMemPool(pool, dev);
     std::lock_guard<std::mutex> lk(g_pool_mu);
     if (!g_pools[dev]) {
+        RelaxedCapture relaxed;
         cudaMemPoolProps props{};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
@@ -86,7 +96,10 @@ void dev_trim()
 {
     std::lock_guard<std::mutex> lk(g_pool_mu);
     for (cudaMemPool_t q : g_pools)
-        if (q) cudaMemPoolTrimTo(q, 0);
+        if (q) {
+            RelaxedCapture relaxed;
+            cudaMemPoolTrimTo(q, 0);
+        }
 }
 
 cudaError_t dev_alloc(const Allocator &A, void **p, size_t bytes, cudaStream_t s)
