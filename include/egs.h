@@ -327,7 +327,10 @@ egs_status egs_loglik_ex(const double *locs, const double *z, const double theta
  * its tile algorithm -- and the forward-solve tasks) form one list in a
  * dependency order checked when the plan is made, and each CTA claims the
  * next task and waits on per-tile device counters until its inputs are final
- * (every wait bounded: EGS_ERR_TIMEOUT if one runs out).  Other batches
+ * (every wait bounded: EGS_ERR_TIMEOUT if one runs out).  (A plan that the
+ * device has room for only without the tensor-core scratch runs all its
+ * problems in the persistent launch; l of the large ones then equals
+ * egs_loglik_ex's to rounding.)  Other batches
  * (EGS_MIX_FP32, or tiles above 256) run as step-synchronous launches, each
  * covering one step of every problem.  Either way the run is captured into a
  * CUDA graph on the first egs_batch_run and replayed afterwards.
